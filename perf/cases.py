@@ -162,6 +162,94 @@ def work(case):
     return {"bytes": packed + 2 * M * values, "flops": 2 * M * weights}
 
 
+def _s64(v):
+    return v - (1 << 64) if v >= 1 << 63 else v
+
+
+def _mix(z):
+    """splitmix64's output function on int64 tensors (products wrap, shifts are logical)."""
+    z = (z ^ ((z >> 30) & ((1 << 34) - 1))) * _s64(0xBF58476D1CE4E5B9)
+    z = (z ^ ((z >> 27) & ((1 << 37) - 1))) * _s64(0x94D049BB133111EB)
+    return z ^ ((z >> 31) & ((1 << 33) - 1))
+
+
+def _draws(seed, tensor, counter):
+    golden = 0x9E3779B97F4A7C15
+    key = _mix(torch.tensor([_s64((seed ^ (tensor * golden)) & (1 << 64) - 1)], device="cuda"))
+    return _mix(key + counter * _s64(golden))
+
+
+def _weights64(out, in_, K, g, seed, r0, r1):
+    """Rows r0..r1-1 of the weights that the seed stands for, in binary64 with nothing rounded: c0 + sum_i ci * bi of the
+    seeded planes (one draw per 32 columns) and binary16 coefficients (twelve 16-bit uniforms for c0, one 24-bit uniform else)."""
+    r = torch.arange(r0, r1, device="cuda", dtype=torch.int64)[:, None]
+    ng, nw = -(-in_ // g), in_ // 32
+    group = torch.arange(in_, device="cuda") // g
+    bit = torch.arange(32, device="cuda")
+    w = None
+    for i in range(K + 1):
+        e = (i * out + r) * ng + torch.arange(ng, device="cuda")[None, :]
+        if i == 0:
+            total = torch.zeros_like(e)
+            for part in range(3):
+                d = _draws(seed, 2, 4 * e + part)
+                for q in range(4):
+                    total += (d >> (16 * q)) & 0xFFFF
+            c = (total - 6 * 65535).float() * (float.fromhex("0x1.47ae14p-6") * 2.0 ** -16)
+        else:
+            u = ((_draws(seed, 2, 4 * e) >> 40) & 0xFFFFFF).float()
+            lo, span = ("0x1.47ae14p-8", "0x1.70a3d8p-5") if i <= 2 else ("0x1.0624dep-9", "0x1.26e978p-6")
+            c = u * (float.fromhex(span) * 2.0 ** -24) + float.fromhex(lo)
+        c = c.half().double()[:, group]
+        if i == 0:
+            w = c
+        else:
+            word = _draws(seed, 1, ((i - 1) * out + r) * nw + torch.arange(nw, device="cuda")[None, :]) >> 32
+            w += c * ((word[:, :, None] >> bit) & 1).reshape(r1 - r0, in_)
+    return w
+
+
+def exact(case, seed):
+    """run()'s outputs in binary64 from Eq. 1 as it stands (no rounding of weights, sums or the unit).  The rebuilt weights of
+    the dequantisation have a definition of their own, bit by bit, and are compared as they are."""
+    M, K, g, kind = case["M"], case["K"], case["group"], case["kind"]
+    if kind == "dequant":
+        return None
+    lins = _linears(case)
+    seeds = {n: (seed << 8) + k for k, n in enumerate(lins)}
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+
+    def acts(n):
+        return torch.randn((M, n), generator=gen, device="cuda", dtype=torch.float32).half().double()
+
+    def linear(n, x):
+        out, in_ = lins[n]
+        return torch.cat([x @ _weights64(out, in_, K, g, seeds[n], r, min(out, r + 2048)).T for r in range(0, out, 2048)], 1)
+
+    if kind == "linear":
+        return linear("w", acts(case["in"]))
+    rs = np.random.RandomState(seed % 2 ** 32)
+    bias, perm = {}, {}
+    if case["bias"]:
+        bias = {n: torch.from_numpy(rs.randn(lins[n][0]).astype(np.float16)).cuda().double() for n in ("q", "k", "v")}
+    if case["perm"]:
+        perm = {n: torch.from_numpy(rs.permutation(lins[n][1])).cuda() for n in NAMES}
+
+    def full(n, x):
+        y = linear(n, x[:, perm[n]] if n in perm else x)
+        return y + bias[n] if n in bias else y
+
+    if kind == "layer_host":
+        xs = [acts(lins[n][1]) for n in NAMES]
+        return [full(n, x).cpu() for n, x in zip(NAMES, xs)]
+    x, attn, mid = acts(case["hidden"]), acts(case["hidden"]), acts(case["hidden"])
+    y = {n: full(n, x) for n in ("q", "k", "v")}
+    y["o"] = full("o", attn)
+    y["unit"] = torch.nn.functional.silu(full("gate", mid)) * full("up", mid)
+    y["down"] = full("down", y["unit"])
+    return y
+
+
 def tolerance(case):
     """Rebuilt weights are defined bit by bit.  Everything else: weights may enter the sums rounded to binary16 or unrounded,
     sums may be taken in any order in binary32, outputs are binary16.  Against binary64 sums of the rounded weights the layers'
