@@ -313,8 +313,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                         asm volatile("ld.shared.u16 %0, [%1];" : "=h"(cbits[gg][i])
                                      : "r"(psrc + C::kPlaneBytes + gg * C::kCoefBytes + i * (BM * 2) + rl * 2));
                 }
-            __syncwarp();                                // every lane's loads have returned (their results were used above)
-            if (lane == 0) mbar_arrive(empty_p(sp));     // the block's packed bytes are in registers: its slot may be refilled
             bpdq::ByteTables<K> tab;
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
@@ -346,7 +344,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                                  "r"(v8[ch].x), "r"(v8[ch].y), "r"(v8[ch].z), "r"(v8[ch].w) : "memory");
                 fence_proxy_async();                     // make the generic-proxy stores visible to the MMA's reads
                 __syncwarp();
-                if (lane == 0) mbar_arrive(full_a(sa));  // one arrival per warp, after all its lanes' stores and fences
+                if (lane == 0) {
+                    mbar_arrive(full_a(sa));             // one arrival per warp, after all its lanes' stores and fences
+                    // The slot may be refilled once the loads from it have RETURNED, not when they have been issued: the
+                    // refill is an asynchronous write that does not queue behind them.  They have returned where a stored
+                    // stage was computed from them (both groups' coefficients: the second half's).
+                    if (half == ng - 1) mbar_arrive(empty_p(sp));
+                }
             }
         }
         // ---------------- epilogue: each decode group takes half of the token columns (all of them when there are only 16) ----------------

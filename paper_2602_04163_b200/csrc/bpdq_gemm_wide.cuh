@@ -181,8 +181,6 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                         asm volatile("ld.shared.u16 %0, [%1];" : "=h"(cbits[gg][i])
                                      : "r"(psrc + C::kPlaneBytes + gg * C::kCoefBytes + i * (BM * 2) + rl * 2));
                 }
-            __syncwarp();                                // every lane's loads have returned (their results were used above)
-            if (lane == 0) mbar_arrive(empty_p(sp));     // the block's packed bytes are in registers: its slot may be refilled
             bpdq::ByteTables<K> tab;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {                // the block's four 32-column stages
@@ -209,7 +207,10 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                                  "r"(v8[ch].x), "r"(v8[ch].y), "r"(v8[ch].z), "r"(v8[ch].w) : "memory");
                 fence_proxy_async();                     // make the generic-proxy stores visible to the MMA's reads
                 __syncwarp();
-                if (lane == 0) mbar_arrive(full_a(s));   // one arrival per warp, after all its lanes' stores and fences
+                if (lane == 0) {
+                    mbar_arrive(full_a(s));              // one arrival per warp, after all its lanes' stores and fences
+                    if (q == 2 * (ng - 1)) mbar_arrive(empty_p(sp));   // a stored stage has used the last loads from the packed slot: it may be refilled
+                }
             }
         }
     } else {

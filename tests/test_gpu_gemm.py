@@ -88,3 +88,19 @@ def test_gemm_full_size_sampled(name, out, in_, K, M):
                                  synth.coefficients(950 + K, out, in_, K, g, rows), x, g)
     G.assert_linear_close(y[:, rows], y_ref, a_ref, name)
     assert np.all(np.isfinite(y))
+
+
+@pytest.mark.parametrize("K,g,M", [(2, 128, 48), (2, 256, 100), (3, 64, 40), (4, 128, 128), (3, 64, 300)])
+def test_gemm_packed_ring_under_load(K, g, M):
+    """A layer that keeps every SM's packed ring turning, several launches: a slot that is refilled before the last load from it
+    has returned shows as rows that are off by a few columns' worth.  Weights from bpdq_dequant, sums in binary32."""
+    import torch
+    out, in_ = 18944, 3584
+    h = binding.Handle(out, in_, K, g, None, 17, M)
+    x = synth.activations(18, M, in_)
+    w = torch.from_numpy(G.run_dequant(h).view(np.float16)).cuda().float()
+    ref = (G.x_tensor(x).float() @ w.T).cpu().numpy()
+    for _ in range(8):
+        y = G.run_linear(h, x, binding.KERNEL_GEMM)
+        # binary16 rounding of the result (2^-11) and binary32 sums of 3584 terms of size up to 0.2 in another order
+        assert np.all(np.abs(y - ref) <= 2.0 ** -10 * np.abs(ref) + 2e-3)
