@@ -191,7 +191,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
     unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * (kBars + 1));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform, and known to be
     const int row0 = blockIdx.x * BM;          // first output row of this CTA
     const int tok0 = blockIdx.y * BN;          // first token of this CTA
     const int kb0 = blockIdx.z * p.kb_per;           // this CTA's stages: [kb0, kb1) of the in / 64 stages of the row
@@ -260,24 +260,28 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
         }
     } else if (warp <= 2) {
         // ---------------- MMA issuers: warp 1 + j takes the stages it % NI == j, into accumulator j ----------------
-        if (lane == 0 && warp <= NI) {
+        if (warp <= NI) {
             constexpr unsigned idesc = instr_desc_f16(BM, BN);
             const int j = warp - 1;
             for (int it = j; it < nst; it += NI) {
                 const int sa = it % SA, sb = it % SB;
-                if (!mbar_wait(full_a(sa), (unsigned)(it / SA) & 1u, abort_flag, p.status) ||
-                    !mbar_wait(full_b(sb), (unsigned)(it / SB) & 1u, abort_flag, p.status))
+                if (!mbar_wait_warp(full_a(sa), (unsigned)(it / SA) & 1u, abort_flag, p.status) ||
+                    !mbar_wait_warp(full_b(sb), (unsigned)(it / SB) & 1u, abort_flag, p.status))
                     break;
                 tc_fence_after();
                 const uint64_t adesc = smem_desc_sw128(a_base + sa * kATileBytes);
                 const uint64_t bdesc = smem_desc_sw128(b_base + sb * C::kBTileBytes);
+                if (elect_one()) {
 #pragma unroll
-                for (int k4 = 0; k4 < BK / 16; ++k4)     // 16 columns = 32 bytes further along the swizzled row
-                    umma_f16(tmem_d + (unsigned)(j * BN), adesc + 2u * k4, bdesc + 2u * k4, idesc, (it >= NI || k4 != 0) ? 1u : 0u);
-                umma_commit(empty_a(sa));                // each frees its slot once these MMAs have read it
-                umma_commit(empty_b(sb));
+                    for (int k4 = 0; k4 < BK / 16; ++k4) // 16 columns = 32 bytes further along the swizzled row
+                        umma_f16(tmem_d + (unsigned)(j * BN), adesc + 2u * k4, bdesc + 2u * k4, idesc, (it >= NI || k4 != 0) ? 1u : 0u);
+                    umma_commit(empty_a(sa));            // each frees its slot once these MMAs have read it
+                    umma_commit(empty_b(sb));
+                }
+                __syncwarp();
             }
-            umma_commit(acc_full);                       // arrives when every MMA of this issuer has completed
+            if (elect_one()) umma_commit(acc_full);      // arrives when every MMA of this issuer has completed
+            __syncwarp();
         }
     } else {
         // ---------------- decode warps (thread = output row), then epilogue ----------------
@@ -450,7 +454,7 @@ gemm_persistent_kernel(const __grid_constant__ CUtensorMap x_map, const GemmPara
     unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * (4 * S + 4));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform, and known to be
     const int nkb = p.in / BK;
     const int nrt = (p.out + BM - 1) / BM;            // row tiles
     const int ntt = (p.M + BN - 1) / BN;              // token tiles
@@ -512,30 +516,34 @@ gemm_persistent_kernel(const __grid_constant__ CUtensorMap x_map, const GemmPara
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
+        {
             constexpr unsigned idesc = instr_desc_f16(BM, BN);
             int it = 0, j = 0;                           // stage sequence number; tiles done by this CTA
             bool ok = true;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++j) {
                 const int buf = j & 1;
                 // the epilogue must have drained this accumulator (two tiles ago)
-                if (!mbar_wait(acc_empty(buf), ((unsigned)(j >> 1) & 1u) ^ 1u, abort_flag, p.status)) break;
+                if (!mbar_wait_warp(acc_empty(buf), ((unsigned)(j >> 1) & 1u) ^ 1u, abort_flag, p.status)) break;
                 tc_fence_after();
                 const unsigned d = tmem_d + (unsigned)(buf * BN);
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % S;
                     const unsigned ph = (unsigned)(it / S) & 1u;
-                    ok = mbar_wait(full_a(s), ph, abort_flag, p.status) && mbar_wait(full_b(s), ph, abort_flag, p.status);
+                    ok = mbar_wait_warp(full_a(s), ph, abort_flag, p.status) && mbar_wait_warp(full_b(s), ph, abort_flag, p.status);
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t adesc = smem_desc_sw128(a_base + s * kATileBytes);
                     const uint64_t bdesc = smem_desc_sw128(b_base + s * C::kBTileBytes);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k4 = 0; k4 < BK / 16; ++k4)
-                        umma_f16(d, adesc + 2u * k4, bdesc + 2u * k4, idesc, (kb | k4) != 0 ? 1u : 0u);
-                    umma_commit(empty(s));
+                        for (int k4 = 0; k4 < BK / 16; ++k4)
+                            umma_f16(d, adesc + 2u * k4, bdesc + 2u * k4, idesc, (kb | k4) != 0 ? 1u : 0u);
+                        umma_commit(empty(s));
+                    }
+                    __syncwarp();
                 }
-                if (ok) umma_commit(acc_full(buf));
+                if (ok && elect_one()) umma_commit(acc_full(buf));
+                __syncwarp();
             }
         }
     } else if (warp < 2 + 4 * kDecodeGroups) {

@@ -62,7 +62,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * (3 * S + 2 * SP + 2));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int nkb = p.in / kWideBK;                  // stages per tile
     const int nblk = p.in / 128;                     // packed blocks per tile (four stages each)
     const int nrt = (p.out + BM - 1) / BM;
@@ -118,7 +118,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         }
     } else if (warp <= 2) {
         // ---------------- MMA issuers: warp 1 + h multiplies every stage with x half h into accumulator h ----------------
-        if (lane == 0) {
+        {
             constexpr unsigned idesc = instr_desc_f16(BM, 256);
             const int h = warp - 1;
             const unsigned d = tmem_d + (unsigned)(h * 256);
@@ -126,23 +126,27 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             bool ok = true;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++j) {
                 // the epilogue must have drained the accumulators of the tile before
-                if (!mbar_wait(acc_empty, ((unsigned)j & 1u) ^ 1u, abort_flag, p.status)) break;
+                if (!mbar_wait_warp(acc_empty, ((unsigned)j & 1u) ^ 1u, abort_flag, p.status)) break;
                 tc_fence_after();
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % S;
                     const unsigned ph = (unsigned)(it / S) & 1u;
-                    ok = mbar_wait(full_a(s), ph, abort_flag, p.status) && mbar_wait(full_b(s), ph, abort_flag, p.status);
+                    ok = mbar_wait_warp(full_a(s), ph, abort_flag, p.status) && mbar_wait_warp(full_b(s), ph, abort_flag, p.status);
                     if (!ok) break;
                     tc_fence_after();
                     const unsigned a_addr = st_base + s * kWideStage;
                     const uint64_t adesc = smem_desc_sw64(a_addr);
                     const uint64_t bdesc = smem_desc_sw64(a_addr + kWideATile + h * kWideBHalf);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k2 = 0; k2 < kWideBK / 16; ++k2)    // 16 columns = 32 bytes further along the swizzled row
-                        umma_f16(d, adesc + 2u * k2, bdesc + 2u * k2, idesc, (kb | k2) != 0 ? 1u : 0u);
-                    umma_commit(empty(s));
+                        for (int k2 = 0; k2 < kWideBK / 16; ++k2)    // 16 columns = 32 bytes further along the swizzled row
+                            umma_f16(d, adesc + 2u * k2, bdesc + 2u * k2, idesc, (kb | k2) != 0 ? 1u : 0u);
+                        umma_commit(empty(s));
+                    }
+                    __syncwarp();
                 }
-                if (ok) umma_commit(acc_full);
+                if (ok && elect_one()) umma_commit(acc_full);
+                __syncwarp();
             }
         }
     } else if (warp < 3 + 4 * kDecodeGroups) {

@@ -62,6 +62,19 @@ constexpr unsigned long long kWaitNanos = 2000000000ull;       // two seconds: f
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatile int* abort_flag, int* status) {
     return mbar_wait_ns(bar, parity, abort_flag, status, kWaitNanos);
 }
+// One lane of a converged warp.  Code behind it (unlike behind "lane == 0") is known to run in a single thread of a
+// warp that is otherwise together, so the operands of a tcgen05.mma stay in uniform registers: the issue loops of the
+// tensor-core kernels then keep up with the pipe (four 72B-shaped launches with 48 tokens, K = 2: 367 -> 329 us, a
+// 7B-shaped layer with 777 tokens 785 -> 724 us, a 72B-shaped layer with 4096 tokens 6.92 -> 6.71 ms).
+__device__ __forceinline__ bool elect_one() {
+    unsigned is;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(is));
+    return is != 0;
+}
+// The bounded wait by a whole warp: the same answer in every lane, also when the wait of some lanes ran out.
+__device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned parity, volatile int* abort_flag, int* status) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status)) != 0;
+}
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 
