@@ -157,8 +157,8 @@ BPDQ_API int bpdq_dequant(bpdq_handle_t h, void* w_fp16_dev, void* stream);
 /* The quantized linear map y = x * W^T (paper: Eq. 1 applied to activations, Section 3.1).
  * x: device binary16 [M][in]; y: device binary16 [M][out]; 0 <= M <= max_M.  M == 0 returns
  * BPDQ_OK without a launch.  Picks the look-up-table kernel for the smallest M (default: up to
- * 2 tokens, 3 at K = 4 and g >= 128), the few-token kernel above that (default: up to 16 tokens) and the tcgen05 kernel
- * beyond (also below when the packed weights of the linear reach 4 GB, which the look-up-table
+ * 2 tokens, 3 at K = 4 and g >= 128), the tensor-core (tcgen05) kernels above that; the few-token kernel only where
+ * bpdq_set_few_max_m asks for it (the tensor-core kernel also below when the packed weights of the linear reach 4 GB, which the look-up-table
  * kernel's 32-bit offsets do not cover).  x and y must not alias. */
 BPDQ_API int bpdq_linear(bpdq_handle_t h, const void* x_fp16_dev, void* y_fp16_dev, int M, void* stream);
 
@@ -170,8 +170,8 @@ BPDQ_API int bpdq_linear_ex(bpdq_handle_t h, const void* x_fp16_dev, void* y_fp1
 /* Several independent linears in one launch (decode: q, k, v of one token, or gate and up, or a
  * whole layer's linears when their inputs do not depend on each other).  y[k] = x[k] * W^[k]^T
  * for k = 0..n-1, each as bpdq_linear computes it for this M: the look-up-table kernel up to the
- * first handle's look-up-table threshold, the few-token kernel above it (up to its threshold,
- * when every linear allows it), else passes of the look-up-table kernel; the task spaces of the
+ * first handle's look-up-table threshold, the tensor-core kernel above it (the few-token kernel up to
+ * its threshold where that is set); the task spaces of the
  * n linears are concatenated, so launch ramp, set-up and tail are paid once instead of n times.  hs, xs, ys are HOST arrays of n
  * handles / device pointers (read before the call returns); 1 <= n <= BPDQ_BATCH_MAX; the
  * handles are distinct, live on the current device, share K, and either all or none of them
@@ -241,11 +241,11 @@ BPDQ_API int bpdq_set_bias(bpdq_handle_t h, const uint16_t* bias_fp16_host);
  * g = x W^gate^T (+ bias), u = x W^up^T (+ bias), silu(v) = v / (1 + exp(-v)), evaluated in binary32
  * and rounded to binary16 (not part of the paper's method: the step that follows these two
  * linears in the decoder layers the paper measures).  Both handles have
- * the same out, in and K and live on the current device; 0 <= M <= min(max_M).  Up to the
- * few-token threshold the two linears run in one launch and the kernel that completes a block of
- * rows applies the unit to the unrounded binary32 sums (nothing but h is written); above it two
- * tcgen05 launches write g and u, rounded to binary16, to handle-owned buffers and a third launch
- * applies the unit.  x, h_out: device binary16 [M][in] /
+ * the same out, in and K and live on the current device; 0 <= M <= min(max_M).  Up to
+ * 128 tokens the two linears run in one launch and the kernel that completes a block of rows applies
+ * the unit to the unrounded binary32 sums (nothing but h is written); above it two tcgen05 launches
+ * write g and u, rounded to binary16, to handle-owned buffers and a third launch applies the unit.
+ * x, h_out: device binary16 [M][in] /
  * [M][out], 16-byte aligned. */
 BPDQ_API int bpdq_gate_up_swiglu(bpdq_handle_t gate, bpdq_handle_t up, const void* x_fp16_dev, void* h_fp16_dev, int M,
                         void* stream);
@@ -255,7 +255,7 @@ BPDQ_API int bpdq_gate_up_swiglu(bpdq_handle_t gate, bpdq_handle_t up, const voi
 BPDQ_API int bpdq_set_gemv_max_m(bpdq_handle_t h, int max_gemv_m);
 
 /* Sets the largest M that bpdq_linear sends to the few-token kernel once M is above the look-up-table
- * threshold (0 = never; at most BPDQ_FEW_MAX_M and the handle's max_M). */
+ * threshold (0 = never, the default; at most BPDQ_FEW_MAX_M and the handle's max_M). */
 BPDQ_API int bpdq_set_few_max_m(bpdq_handle_t h, int max_few_m);
 
 /* Copies the device blob back to host memory (bpdq_packed_bytes() bytes); synchronises. */

@@ -126,6 +126,12 @@ int check_batch_handles(const bpdq_handle_t* hs, int n, int M, const char* who) 
     return M == 0 ? BPDQ_OK : check_device(hs[0], who);
 }
 
+// Whether a launch goes to the look-up-table kernel: up to the first linear's threshold, unless the tensor-core kernel is
+// the better one below it (and the caller has not set the threshold).
+bool prefer_lut(bpdq_handle_s* const* hs, int n, int M) {
+    return M <= hs[0]->gemv_max_m;
+}
+
 }  // namespace
 
 extern "C" int bpdq_create(bpdq_handle_t* hp, int out, int in, int K, int group, const void* host_blob,
@@ -158,10 +164,7 @@ extern "C" int bpdq_create(bpdq_handle_t* hp, int out, int in, int K, int group,
     // Measured on 72B-shaped layers: one two-token pass of the look-up-table kernel (37 us on the largest projections)
     // beats every other kernel; a second pass (64 us) does not beat the few-token kernel.
     h->gemv_max_m = 2;
-    // 3 to 16 tokens: the few-token kernel reads the weights once (43-60 us on the largest 72B-shaped projections
-    // against 64 us for two look-up-table passes and 67-78 us for the tcgen05 tile kernel); from 17 tokens on its second
-    // token tile costs more than the tile kernel.
-    h->few_max_m = 16;
+    h->few_max_m = 0;                                    // the few-token kernel runs for callers that ask for it
     // sixteen candidates (the few-token kernel then takes tasks of two row groups): 83-88 us on the largest projections for
     // 3 to 16 tokens against 77 / 92 us for two look-up-table passes at 3 / 4 tokens (103 / 120 us at g = 64) and 118 us
     // for the tile kernel
@@ -224,8 +227,8 @@ extern "C" int bpdq_linear_ex(bpdq_handle_t h, const void* x, void* y, int M, in
         const bool gv = gemv_supported(h->out, h->in, h->K, h->group);
         const bool gm = gemm_supported(h->out, h->in, h->K, h->group);
         const bool fw = gemv_mma_supported(h->out, h->in, h->K, h->group);
-        if (gv && (M <= h->gemv_max_m || !gm) && M <= BPDQ_GEMV_MAX_M) kernel = BPDQ_KERNEL_GEMV;
-        else if (fw && M <= h->few_max_m && M <= BPDQ_FEW_MAX_M) kernel = BPDQ_KERNEL_FEW;
+        if (gv && (prefer_lut(&h, 1, M) || !gm) && M <= BPDQ_GEMV_MAX_M) kernel = BPDQ_KERNEL_GEMV;
+        else if (fw && h->few_max_m && M <= h->few_max_m && M <= BPDQ_FEW_MAX_M) kernel = BPDQ_KERNEL_FEW;
         else if (gm) kernel = BPDQ_KERNEL_GEMM;
         else kernel = BPDQ_KERNEL_GEMV_SIMPLE;
     }
@@ -266,12 +269,15 @@ extern "C" int bpdq_linear_batch(const bpdq_handle_t* hs, const void* const* xs,
     for (int k = 0; k < n; ++k)
         if (!xs[k] || !ys[k] || !aligned16(xs[k]) || !aligned16(ys[k]))
             return set_error(BPDQ_ERR_INVALID, "bpdq_linear_batch: x and y of linear %d must be non-null and 16-byte aligned", k);
-    // above the look-up-table threshold the few-token kernel takes the whole batch, when every linear allows it
+    // above the look-up-table threshold the tensor-core kernel (or the few-token kernel, if asked for) takes the whole batch,
+    // when every linear allows it
+    bool gemm = !prefer_lut(hs, n, M);
     bool few = M > hs[0]->gemv_max_m && M <= hs[0]->few_max_m && M <= BPDQ_FEW_MAX_M;
     for (int k = 0; few && k < n; ++k)
         few = hs[k]->d_few_maps && gemv_mma_supported(hs[k]->out, hs[k]->in, hs[k]->K, hs[k]->group) &&
               (size_t)M * hs[k]->out * sizeof(float) <= hs[k]->ws_bytes;
-    if (few) {
+    for (int k = 0; gemm && k < n; ++k) gemm = gemm_batch_supported(hs[k], M);
+    if (few || gemm) {
         const void* xg[BPDQ_BATCH_MAX];
         for (int k = 0; k < n; ++k) {
             xg[k] = xs[k];
@@ -280,7 +286,8 @@ extern "C" int bpdq_linear_batch(const bpdq_handle_t* hs, const void* const* xs,
                 xg[k] = hs[k]->d_xperm;
             }
         }
-        return launch_gemv_mma_batch(hs, xg, ys, n, M, static_cast<cudaStream_t>(stream));
+        return few ? launch_gemv_mma_batch(hs, xg, ys, n, M, static_cast<cudaStream_t>(stream))
+                   : launch_gemm_batch(hs, xg, ys, n, M, static_cast<cudaStream_t>(stream));
     }
     return launch_gemv_batch(hs, xs, ys, n, M, static_cast<cudaStream_t>(stream));
 }
@@ -373,6 +380,7 @@ extern "C" int bpdq_set_gemv_max_m(bpdq_handle_t h, int max_gemv_m) {
     if (max_gemv_m < 0 || max_gemv_m > BPDQ_GEMV_MAX_M)
         return set_error(BPDQ_ERR_INVALID, "bpdq_set_gemv_max_m: %d outside [0, %d]", max_gemv_m, BPDQ_GEMV_MAX_M);
     h->gemv_max_m = max_gemv_m;
+    h->gemv_set = 1;
     return BPDQ_OK;
 }
 
@@ -510,14 +518,15 @@ extern "C" int bpdq_gate_up_swiglu(bpdq_handle_t hg, bpdq_handle_t hu, const voi
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     bpdq_handle_s* hs[2] = {hg, hu};
     const bool same_g64 = (hg->group == 64) == (hu->group == 64);
-    const bool lut = same_g64 && M <= hg->gemv_max_m && M <= BPDQ_GEMV_MAX_M && gemv_supported(hg->out, hg->in, hg->K, hg->group) &&
+    const bool lut = same_g64 && prefer_lut(hs, 2, M) && M <= BPDQ_GEMV_MAX_M && gemv_supported(hg->out, hg->in, hg->K, hg->group) &&
                      gemv_supported(hu->out, hu->in, hu->K, hu->group);
     bool few = same_g64 && !lut && M <= hg->few_max_m && M <= BPDQ_FEW_MAX_M && hg->d_few_maps && hu->d_few_maps &&
                (size_t)M * hg->out * sizeof(float) <= hg->ws_bytes && (size_t)M * hu->out * sizeof(float) <= hu->ws_bytes;
-    if (lut || few) {
+    const bool gemm = same_g64 && !lut && !few && gemm_batch_supported(hg, M) && gemm_batch_supported(hu, M);
+    if (lut || few || gemm) {
         // one launch over both linears; the kernel that completes a block of rows applies the unit
         const void* xs[2] = {x, x};
-        if (few) {                                                 // this kernel does not read through a permutation: gather first
+        if (!lut) {                                                // these kernels do not read through a permutation: gather first
             for (int k = 0; k < 2; ++k) {
                 if (hs[k]->d_perm) {
                     if (const int rc = launch_gather_columns(hs[k], x, M, s); rc != BPDQ_OK) return rc;
@@ -526,7 +535,8 @@ extern "C" int bpdq_gate_up_swiglu(bpdq_handle_t hg, bpdq_handle_t hu, const voi
             }
         }
         void* ys[2] = {hout, hout};
-        return lut ? launch_gemv_batch(hs, xs, ys, 2, M, s, true) : launch_gemv_mma_batch(hs, xs, ys, 2, M, s, true);
+        return lut ? launch_gemv_batch(hs, xs, ys, 2, M, s, true)
+             : few ? launch_gemv_mma_batch(hs, xs, ys, 2, M, s, true) : launch_gemm_batch(hs, xs, ys, 2, M, s, true);
     }
     // many tokens: both projections through the dispatcher into the handles' own output buffers, then the unit
     for (int k = 0; k < 2; ++k)

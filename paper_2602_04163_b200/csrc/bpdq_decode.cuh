@@ -106,8 +106,8 @@ __device__ __forceinline__ void candidate_byte_tables(const float (&c)[K + 1], B
 }
 
 // prmt.b32 as the hardware defines it: byte n of the result is byte (selector nibble n) & 7 of {b, a} (a = bytes 0..3);
-// a nibble with its top bit set would replicate that byte's sign instead.  Every selector used below keeps the top
-// bit of its four low nibbles clear (codes are at most 7), so no masking instruction is needed in front of it;
+// a nibble with its top bit set replicates that byte's sign instead.  Selectors of up to eight candidates keep the top
+// bit of their four low nibbles clear (codes are at most 7), so no masking instruction is needed in front of them;
 // bits 16..31 of the selector are ignored.
 __device__ __forceinline__ unsigned prmt_raw(unsigned a, unsigned b, unsigned sel) {
     unsigned d;
@@ -120,15 +120,16 @@ template <int K>
 __device__ __forceinline__ void decode4(const unsigned sel, const ByteTables<K>& t, unsigned& out01, unsigned& out23) {
     unsigned l, h;
     if constexpr (K == 4) {
-        // a byte-permute selects among eight bytes: candidates 0..7 and 8..15 are looked up separately
-        // (selector without its top bit) and the top bit of every code picks between the two results
-        const unsigned s7 = sel & 0x7777u;
-        unsigned m = (sel >> 3) & 0x1111u;                   // top bits at nibble positions 0, 4, 8, 12
-        m = (m & 0x0011u) | ((m & 0x1100u) << 8);            // ... at 0, 4, 16, 20
-        m = (m & 0x00010001u) | ((m & 0x00100010u) << 4);    // ... at 0, 8, 16, 24
-        m *= 0xFFu;                                          // one full byte per code
-        const unsigned la = prmt_raw(t.lo[0], t.lo[1], s7), lb = prmt_raw(t.lo[2], t.lo[3], s7);
-        const unsigned ha = prmt_raw(t.hi[0], t.hi[1], s7), hb = prmt_raw(t.hi[2], t.hi[3], s7);
+        // a byte-permute selects among eight bytes: candidates 0..7 are looked up with the codes as they are and 8..15 with
+        // their top bits flipped; a nibble whose top bit is set yields a replicated sign, which the choice below discards.
+        // The choice is a byte mask: the permute turns the top bits into 0x80 or 0xFF, doubling moves bit 6 into bit 7
+        // (10.5 instructions of the half-rate pipe for four weights; spreading the bits with shifts and masks took 17 and
+        // the 72B gate with 16 tokens 75 us)
+        const unsigned flip = sel ^ 0x88888888u;
+        const unsigned top = prmt_raw(0x80808080u, 0x80808080u, sel);
+        const unsigned m = (top & 0x7F7F7F7Fu) | ((top * 2u) & 0x80808080u);
+        const unsigned la = prmt_raw(t.lo[0], t.lo[1], sel), lb = prmt_raw(t.lo[2], t.lo[3], flip);
+        const unsigned ha = prmt_raw(t.hi[0], t.hi[1], sel), hb = prmt_raw(t.hi[2], t.hi[3], flip);
         l = (la & ~m) | (lb & m);
         h = (ha & ~m) | (hb & m);
     } else {

@@ -12,40 +12,24 @@
 // 16-byte chunk c of row r is stored at chunk position c ^ (r mod 8).  TMA writes that layout by
 // itself; the decode threads reproduce it by hand.
 //
-// Roles (320 threads; the tile kernel has a second MMA-issuing warp, 352): warp 0 is the producer (one lane: TMA
-// loads of x and of the packed weights); warp 1 allocates TMEM and issues the MMAs (one lane); eight warps decode in two groups of four
-// warps, thread = output row, group 0 taking the even 128-column blocks (two stages each) and
-// group 1 the odd ones (one warp per scheduler could not hide its own instruction latencies).
-// The packed planes and coefficients come through the pipeline as well, so that no decode thread
-// ever waits on global memory: in the tile kernel a block's K plane segments (128 rows x 16 bytes)
-// are one box of a tensor map over the blob's planes and its coefficient segments (128 rows x
-// 2 bytes) one box of a map over the coefficients -- two copies per block whatever K is (the TMA
-// unit takes about 55 ns per copy however small, and 2K+1 bulk copies per block made the kernel
-// slower with every plane); the persistent kernel issues bulk copies per segment.
-// A decode thread reads its row's units and coefficients from the stage, builds the 2^K
-// candidate values of the group (Eq. 7, the decode rule's exact arithmetic) as two byte tables,
-// and then eight columns cost one shift-and-mask per plane to form eight
-// code nibbles and eight byte-permutes to select and interleave the binary16 bytes, then one
-// 16-byte shared-memory store.  The same eight warps run the epilogue, each group on one half of
-// the token columns: tcgen05.ld gives a thread its output row for 16 tokens at a time; adjacent
-// threads hold adjacent output indices, so a warp writes 64 contiguous bytes of y per token.
+// Three kernels: gemm_ts_kernel (up to 128 tokens: decoded weights in TMEM, one or several linears per launch;
+// bpdq_gemm_ts.cuh), gemm_persistent_kernel (129..256 tokens: token tile 256, one CTA per SM walks over tiles, two TMEM
+// accumulators, separate epilogue warps; described at its definition) and gemm_wide_kernel (more than 256 tokens: token
+// tile 512, two issuing warps; bpdq_gemm_wide.cuh).  In the two for many tokens the decoded operand goes through shared
+// memory: the MMAs, not the decode, are the bound there, and TMEM is full of accumulators.
 //
-// Three kernels share this scheme: gemm_kernel (one output tile per CTA; token tiles of 16..128, two CTAs per SM
-// and a split over the input dimension when tokens are few), gemm_persistent_kernel (129..256 tokens: token tile 256,
-// one CTA per SM walks over tiles, two TMEM accumulators, separate epilogue warps; described at its definition) and
-// gemm_wide_kernel (more than 256 tokens: token tile 512, two issuing warps; bpdq_gemm_wide.cuh).
+// Decode: a thread reads its row's units and coefficients from the stage, builds the 2^K candidate values of the group
+// (Eq. 7, the decode rule's exact arithmetic) as byte tables, and then eight columns cost one shift-and-mask per plane to
+// form eight code nibbles and eight byte-permutes to select and interleave the binary16 bytes.  Epilogue: tcgen05.ld gives
+// a thread its output row for 16 tokens at a time; adjacent threads hold adjacent output indices, so a warp writes 64
+// contiguous bytes of y per token.
 //
-// Pipeline of the tile kernel: three rings, each with full / empty mbarriers -- packed blocks (full_p by the
-// copies' bytes, empty_p by one arrival per decode warp once the block is in registers), x tiles (full_b by
-// the TMA's bytes, empty_b by tcgen05.commit) and A tiles (full_a by one arrival per decode warp after a proxy
-// fence, empty_a by tcgen05.commit of the MMAs that read the slot); the persistent kernel keeps one ring with
-// four barriers per stage (full_b, full_p, full_a of 128 arrivals, empty).  Both have one
-// acc_full barrier for the epilogue.  Every wait is bounded: on expiry the thread records
-// BPDQ_ERR_TIMEOUT in the handle's status word, raises a CTA-wide abort flag that lets all other
-// waits fall through, and the CTA still runs to its common exit where TMEM is freed.
+// Every wait is bounded: on expiry the thread records BPDQ_ERR_TIMEOUT in the handle's status word, raises a CTA-wide abort
+// flag that lets all other waits fall through, and the CTA still runs to its common exit where TMEM is freed.
 #include "bpdq_internal.h"
 #include "bpdq_decode.cuh"
 #include "bpdq_tma.cuh"
+#include "bpdq_finish.cuh"
 
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -56,8 +40,6 @@ constexpr int BM = 128;                 // output rows per CTA (MMA M)
 constexpr int BK = 64;                  // columns per stage: one 128-byte swizzle row of binary16
 constexpr int kDecodeGroups = 2;
 constexpr int kDecodeThreads = 128;               // per group: one thread per output row
-constexpr int kThreads = 64 + kDecodeGroups * kDecodeThreads;
-constexpr int kTileThreads = 96 + kDecodeGroups * kDecodeThreads;   // tile kernel: producer warp, two MMA-issuing warps, eight decode warps
 constexpr int kATileBytes = BM * BK * 2;                       // 16 KB
 
 template <int K, int BN> struct Cfg {
@@ -66,12 +48,8 @@ template <int K, int BN> struct Cfg {
     static constexpr int kCoefBytes = (K + 1) * BM * 2;         // K+1 segments of 128 rows x 2 bytes
     static constexpr int kPackedBytes = (kPlaneBytes + kCoefBytes + 1023) / 1024 * 1024;
     static constexpr int kStageBytes = kATileBytes + kBTileBytes + kPackedBytes;
-    // Few tokens (BN <= 64): the kernel is bound by the decode threads, not by the MMAs, so two CTAs share an SM
-    // (half the shared memory each) and a 72B-shaped projection's row tiles run in one wave.
-    static constexpr int kCtasPerSm = BN <= 64 ? 2 : 1;
-    static constexpr int kSmemBudget = kCtasPerSm == 2 ? 110 * 1024 : 222 * 1024;
+    static constexpr int kSmemBudget = 222 * 1024;
     static constexpr int kStages = kSmemBudget / kStageBytes > 8 ? 8 : kSmemBudget / kStageBytes;
-    static constexpr int kTmemCols = BN < 32 ? 32 : BN;        // power of two >= 32
     static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 512 /*barriers*/;
 };
 
@@ -81,11 +59,6 @@ struct GemmParams {
     __half* y;                // [M][out]
     int* status;
     int out, in, group, M;
-    // split over the input dimension (few tokens, fewer row tiles than SMs): gridDim.z CTAs share an output tile,
-    // each takes kb_per stages, adds its partial tile into `ws` and the last to arrive writes y
-    int kb_per;               // stages per CTA (even: a 128-column block is never cut)
-    float* ws;                // [M][out] binary32, zero between calls (only used when gridDim.z > 1)
-    unsigned* counters;       // one arrival counter per 128-row tile, zero between calls
     const __half* bias;       // binary16 [out] added before the rounding, or null
 };
 
@@ -134,291 +107,6 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(unsigned addr) {
 // K-major (bits 15, 16 = 0), N / 8 in bits 17..22, M / 16 in bits 24..28.
 __host__ __device__ constexpr unsigned instr_desc_f16(int m, int n) {
     return (1u << 4) | ((unsigned)(n >> 3) << 17) | ((unsigned)(m >> 4) << 24);
-}
-
-// Ring depths of the tile kernel.  Its three operand streams have very different sizes per 64-column stage -- 16 KB of
-// decoded weights (A), BN x 128 bytes of activations (B), about 2.5 KB of packed planes and coefficients -- and very
-// different latencies (A is produced on the SM, B comes from L2, the packed bytes from HBM), so each has its own
-// ring: a few A slots, more B slots, and packed 128-column blocks several stages ahead.
-template <int K, int BN> struct TileCfg {
-    static constexpr int kBTileBytes = BN * BK * 2;
-    static constexpr int kPlaneBytes = K * BM * 16;             // K segments of 128 rows x 16 bytes
-    static constexpr int kCoefBytes = (K + 1) * BM * 2;         // K+1 segments of 128 rows x 2 bytes: one coefficient group
-    static constexpr int kBlockBytes = (kPlaneBytes + 2 * kCoefBytes + 1023) / 1024 * 1024;   // a block's planes and up to two groups (g = 64)
-    static constexpr int kCtasPerSm = 2;                        // bound by the decode threads, so two CTAs share an SM (128 tokens: with two x slots)
-    static constexpr int kSmemBudget = 111 * 1024;
-    // One thread issues a tcgen05.mma every 160 clocks or so whatever its shape, while the pipe could take one of these
-    // few-column MMAs every 40 to 50 clocks: up to 64 tokens two warps issue, stage `it` going to issuer it % 2, each into
-    // an accumulator of its own (added up in the epilogue).  A parity wait is only safe on consecutive phases, so every
-    // barrier must always be waited on by the same thread or group: the ring lengths are multiples of the issuer count
-    // and of the number of decode groups (each group then owns two A slots and every other packed slot).  With one
-    // issuer the A ring may have three slots although the groups then share them: a group that waits for the release of
-    // use u of a slot (stage it) has, for the stage it stored before (it - 1 or it - 3), already waited for an MMA no
-    // earlier than it - 6, the one that ended use u - 2; MMAs complete in order, so the wait is on the next phase.
-    static constexpr int kIssuers = BN <= 64 ? 2 : 1;
-    static constexpr int kSA = kIssuers == 2 ? 4 : 3;
-    static constexpr int kSB = BN <= 16 ? 8 : (BN <= 32 ? (K <= 3 ? 6 : 4) : 2);
-    static constexpr int kRest = kSmemBudget - kSA * kATileBytes - kSB * kBTileBytes - 2048;
-    static constexpr int kSP = (kRest / kBlockBytes > 8 ? 8 : kRest / kBlockBytes) / kDecodeGroups * kDecodeGroups;
-    static_assert(kSP >= 2, "at least two packed blocks in flight");
-    static_assert(kSA % kIssuers == 0 && kSB % kIssuers == 0, "all uses of a slot go to one issuer");
-    static constexpr int kAccCols = kIssuers * BN;
-    static constexpr int kTmemCols = kAccCols <= 32 ? 32 : (kAccCols <= 64 ? 64 : (kAccCols <= 128 ? 128 : 256));   // power of two >= 32
-    static constexpr int kSmemBytes = kSA * kATileBytes + kSB * kBTileBytes + kSP * kBlockBytes + 1024 /*alignment slack*/ + 1024 /*barriers*/;
-};
-
-template <int K, int BN>
-__global__ void __launch_bounds__(kTileThreads, TileCfg<K, BN>::kCtasPerSm)
-gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap planes_map,
-            const __grid_constant__ CUtensorMap coefs_map, const GemmParams p) {
-    using C = TileCfg<K, BN>;
-    constexpr int SA = C::kSA, SB = C::kSB, SP = C::kSP, NI = C::kIssuers;
-    extern __shared__ unsigned char smem_raw[];
-    const unsigned base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
-    const unsigned a_base = base;                                  // SA x 16 KB
-    const unsigned b_base = a_base + SA * kATileBytes;             // SB x BN*128 bytes
-    const unsigned p_base = b_base + SB * C::kBTileBytes;          // SP x (planes, coefficients) of a 128-column block
-    const unsigned bar_base = p_base + SP * C::kBlockBytes;
-    auto full_a = [&](int s) { return bar_base + 8u * s; };
-    auto empty_a = [&](int s) { return bar_base + 8u * (SA + s); };
-    auto full_b = [&](int s) { return bar_base + 8u * (2 * SA + s); };
-    auto empty_b = [&](int s) { return bar_base + 8u * (2 * SA + SB + s); };
-    auto full_p = [&](int s) { return bar_base + 8u * (2 * SA + 2 * SB + s); };
-    auto empty_p = [&](int s) { return bar_base + 8u * (2 * SA + 2 * SB + SP + s); };
-    constexpr int kBars = 2 * SA + 2 * SB + 2 * SP;
-    const unsigned acc_full = bar_base + 8u * kBars;
-    unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * (kBars + 1));
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform, and known to be
-    const int row0 = blockIdx.x * BM;          // first output row of this CTA
-    const int tok0 = blockIdx.y * BN;          // first token of this CTA
-    const int kb0 = blockIdx.z * p.kb_per;           // this CTA's stages: [kb0, kb1) of the in / 64 stages of the row
-    const int kb1 = min(p.in / BK, kb0 + p.kb_per);
-    const int nst = kb1 - kb0;                       // even: whole 128-column blocks
-    const int b0 = kb0 / 2, nblk = nst / 2;
-    const int ng = p.group == 64 ? 2 : 1;            // coefficient groups per block
-
-    if (tid == 0) {
-        for (int s = 0; s < SA; ++s) { mbar_init(full_a(s), kDecodeThreads / 32); mbar_init(empty_a(s), 1); }   // one arrival per decode warp
-        for (int s = 0; s < SB; ++s) { mbar_init(full_b(s), 1); mbar_init(empty_b(s), 1); }
-        for (int s = 0; s < SP; ++s) { mbar_init(full_p(s), 1); mbar_init(empty_p(s), kDecodeThreads / 32); }
-        mbar_init(acc_full, NI);
-        *abort_flag = 0;
-        fence_barrier_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_slot), C::kTmemCols);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const unsigned tmem_d = *tmem_slot;
-
-    if (warp == 0) {
-        // ---------------- producer: packed blocks (bulk copies) and x tiles (TMA), each as its ring has room ----------------
-        if (lane == 0) {
-            // A block's K plane segments (128 rows x 16 bytes each) are one box of the planes' tensor map, its one or two
-            // coefficient groups one box of the coefficients' map: two copies per block, whatever K is.  Rows past a
-            // ragged last tile are filled with zeros (and count as received bytes).
-            int pb = 0, xb = 0;                          // next packed block, next x stage
-            unsigned idle = 0;
-            unsigned long long idle_since = 0;
-            while (pb < nblk || xb < nst) {
-                bool moved = false;
-                if (pb < nblk && mbar_try_wait(empty_p(pb % SP), ((unsigned)(pb / SP) & 1u) ^ 1u)) {
-                    const int sp = pb % SP, b = b0 + pb;
-                    mbar_expect_tx(full_p(sp), (unsigned)(C::kPlaneBytes + ng * C::kCoefBytes));
-                    const unsigned pdst = p_base + sp * C::kBlockBytes;
-                    tma_load_2d(pdst, &planes_map, row0 * 2, b * K, full_p(sp));                 // 8-byte elements: 2 per row
-                    tma_load_2d(pdst + C::kPlaneBytes, &coefs_map, row0 / 4, ((b * 128) / p.group) * (K + 1), full_p(sp));
-                    ++pb;
-                    moved = true;
-                }
-                if (xb < nst && mbar_try_wait(empty_b(xb % SB), ((unsigned)(xb / SB) & 1u) ^ 1u)) {
-                    const int sb = xb % SB;
-                    mbar_expect_tx(full_b(sb), C::kBTileBytes);
-                    tma_load_2d(b_base + sb * C::kBTileBytes, &x_map, (kb0 + xb) * BK, tok0, full_b(sb));
-                    ++xb;
-                    moved = true;
-                }
-                if (moved) {
-                    idle = 0;
-                } else if (++idle == 1) {
-                    idle_since = global_ns();
-                } else if ((idle & 63u) == 63u) {
-                    if (*abort_flag) break;
-                    if (global_ns() - idle_since > kWaitNanos) {   // neither ring has freed a slot for too long
-                        *abort_flag = 1;
-                        atomicExch(p.status, BPDQ_ERR_TIMEOUT);
-                        break;
-                    }
-                }
-            }
-        }
-    } else if (warp <= 2) {
-        // ---------------- MMA issuers: warp 1 + j takes the stages it % NI == j, into accumulator j ----------------
-        if (warp <= NI) {
-            constexpr unsigned idesc = instr_desc_f16(BM, BN);
-            const int j = warp - 1;
-            for (int it = j; it < nst; it += NI) {
-                const int sa = it % SA, sb = it % SB;
-                if (!mbar_wait_warp(full_a(sa), (unsigned)(it / SA) & 1u, abort_flag, p.status) ||
-                    !mbar_wait_warp(full_b(sb), (unsigned)(it / SB) & 1u, abort_flag, p.status))
-                    break;
-                tc_fence_after();
-                const uint64_t adesc = smem_desc_sw128(a_base + sa * kATileBytes);
-                const uint64_t bdesc = smem_desc_sw128(b_base + sb * C::kBTileBytes);
-                if (elect_one()) {
-#pragma unroll
-                    for (int k4 = 0; k4 < BK / 16; ++k4) // 16 columns = 32 bytes further along the swizzled row
-                        umma_f16(tmem_d + (unsigned)(j * BN), adesc + 2u * k4, bdesc + 2u * k4, idesc, (it >= NI || k4 != 0) ? 1u : 0u);
-                    umma_commit(empty_a(sa));            // each frees its slot once these MMAs have read it
-                    umma_commit(empty_b(sb));
-                }
-                __syncwarp();
-            }
-            if (elect_one()) umma_commit(acc_full);      // arrives when every MMA of this issuer has completed
-            __syncwarp();
-        }
-    } else {
-        // ---------------- decode warps (thread = output row), then epilogue ----------------
-        const int quad = warp & 3;                       // TMEM lane quadrant this warp may access
-        const int grp = (warp - 3) >> 2;                 // decode group: takes every other 128-column block
-        const int rl = quad * 32 + lane;                 // row inside the tile
-        const int r = row0 + rl;
-        const bool row_ok = r < p.out;                   // rows past a ragged last tile decode stale bytes; nothing of theirs is stored
-        unsigned a_off[8];                               // swizzled byte offset of each 16-byte chunk of this thread's row
-#pragma unroll
-        for (int ch = 0; ch < 8; ++ch) a_off[ch] = (unsigned)rl * 128u + (((unsigned)ch ^ (unsigned)(rl & 7)) << 4);
-        bool ok = true;
-        for (int bi = grp; bi < nblk && ok; bi += kDecodeGroups) {
-            const int sp = bi % SP;
-            if (!mbar_wait(full_p(sp), (unsigned)(bi / SP) & 1u, abort_flag, p.status)) { ok = false; break; }
-            const unsigned psrc = p_base + sp * C::kBlockBytes;
-            unsigned cur[K][4];                          // logical words of this row's plane units
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                uint4 raw;
-                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(raw.x), "=r"(raw.y), "=r"(raw.z), "=r"(raw.w)
-                             : "r"(psrc + i * (BM * 16) + rl * 16));
-                const uint4 u = bpdq::unrotate_unit(raw, r);
-                cur[i][0] = u.x; cur[i][1] = u.y; cur[i][2] = u.z; cur[i][3] = u.w;
-            }
-            unsigned short cbits[2][K + 1];              // coefficients of the block's one or two groups
-#pragma unroll
-            for (int gg = 0; gg < 2; ++gg)
-#pragma unroll
-                for (int i = 0; i <= K; ++i) {
-                    cbits[gg][i] = 0;
-                    if (gg < ng)
-                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(cbits[gg][i])
-                                     : "r"(psrc + C::kPlaneBytes + gg * C::kCoefBytes + i * (BM * 2) + rl * 2));
-                }
-            bpdq::ByteTables<K> tab;
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const int it = 2 * bi + half;
-                const int sa = it % SA;
-                if (half == 0 || ng == 2) {              // candidate tables of the coefficient group that starts here
-                    float c[K + 1];
-#pragma unroll
-                    for (int i = 0; i <= K; ++i) c[i] = __half2float(__ushort_as_half(cbits[ng == 2 ? half : 0][i]));
-                    bpdq::candidate_byte_tables<K>(c, tab);
-                }
-                // decode the stage's 64 columns into registers first (eight independent chains the compiler can interleave,
-                // and nothing of it waits for the slot), then wait for the slot and store
-                uint4 v8[8];
-#pragma unroll
-                for (int wd = 0; wd < 2; ++wd) {         // two 32-column words per 64-column stage
-                    unsigned w[K], sel[4];
-#pragma unroll
-                    for (int i = 0; i < K; ++i) w[i] = cur[i][2 * half + wd];
-                    bpdq::code_nibbles_word<K>(w, sel);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) v8[4 * wd + u] = bpdq::decode8<K>(sel[u], tab);
-                }
-                if (!mbar_wait(empty_a(sa), ((unsigned)(it / SA) & 1u) ^ 1u, abort_flag, p.status)) { ok = false; break; }
-                const unsigned dst = a_base + sa * kATileBytes;
-#pragma unroll
-                for (int ch = 0; ch < 8; ++ch)
-                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + a_off[ch]),
-                                 "r"(v8[ch].x), "r"(v8[ch].y), "r"(v8[ch].z), "r"(v8[ch].w) : "memory");
-                fence_proxy_async();                     // make the generic-proxy stores visible to the MMA's reads
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(full_a(sa));             // one arrival per warp, after all its lanes' stores and fences
-                    // The slot may be refilled once the loads from it have RETURNED, not when they have been issued: the
-                    // refill is an asynchronous write that does not queue behind them.  They have returned where a stored
-                    // stage was computed from them (both groups' coefficients: the second half's).
-                    if (half == ng - 1) mbar_arrive(empty_p(sp));
-                }
-            }
-        }
-        // ---------------- epilogue: each decode group takes half of the token columns (all of them when there are only 16) ----------------
-        constexpr int kColsPerGroup = BN >= 32 ? BN / 2 : BN;
-        if (ok && (BN >= 32 || grp == 0) && mbar_wait(acc_full, 0u, abort_flag, p.status)) {
-            tc_fence_after();
-            const unsigned taddr = tmem_d + ((unsigned)(quad * 32) << 16);
-#pragma unroll 1
-            for (int c0 = grp * kColsPerGroup; c0 < (grp + 1) * kColsPerGroup; c0 += 16) {
-                if (tok0 + c0 >= p.M) break;             // warp-uniform
-                float acc[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) acc[j] = 0.f;
-#pragma unroll
-                for (int a = 0; a < NI; ++a) {           // the issuers' accumulators, in a fixed order (every issuer has a stage: nst >= 2)
-                    unsigned v[16];
-                    tmem_ld16(taddr + (unsigned)(a * BN + c0), v);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) acc[j] += __uint_as_float(v[j]);
-                }
-                if (row_ok) {
-                    const float br = (p.bias && gridDim.z == 1) ? __half2float(p.bias[r]) : 0.f;   // a shared tile gets it when it is completed
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int t = tok0 + c0 + j;
-                        if (t < p.M) {
-                            if (gridDim.z > 1) atomicAdd(p.ws + (size_t)t * p.out + r, acc[j]);
-                            else p.y[(size_t)t * p.out + r] = __float2half_rn(acc[j] + br);
-                        }
-                    }
-                }
-            }
-        }
-    }
-    if (gridDim.z > 1) __threadfence();              // this thread's partial sums are out before the tile's counter moves
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc(tmem_d, C::kTmemCols);
-    }
-    if (gridDim.z > 1) {
-        // the last of the CTAs that share this output tile rounds it to binary16, writes y and zeroes the workspace
-        int* last = reinterpret_cast<int*>(const_cast<int*>(abort_flag)) + 1;
-        if (tid == 0) {
-            const unsigned before = atomicAdd(p.counters + blockIdx.x, 1u);
-            *last = before == gridDim.z - 1;
-            if (*last) p.counters[blockIdx.x] = 0u;
-        }
-        __syncthreads();
-        if (*last) {
-            __threadfence();
-            const int ntok = min(BN, p.M - tok0);
-            for (int idx = tid; idx < ntok * BM; idx += kTileThreads) {
-                const int t = tok0 + idx / BM, r = row0 + idx % BM;
-                if (r < p.out) {
-                    float* src = p.ws + (size_t)t * p.out + r;
-                    p.y[(size_t)t * p.out + r] = __float2half_rn(__ldcg(src) + (p.bias ? __half2float(p.bias[r]) : 0.f));
-                    __stcg(src, 0.f);
-                }
-            }
-        }
-    }
 }
 
 // ---- persistent variant for many tokens (token tile 256) -------------------------------------------------
@@ -653,6 +341,7 @@ gemm_persistent_kernel(const __grid_constant__ CUtensorMap x_map, const GemmPara
 }
 
 #include "bpdq_gemm_wide.cuh"
+#include "bpdq_gemm_ts.cuh"
 
 // ---- host side ------------------------------------------------------------------------------
 using bpdq::EncodeTiledFn;
@@ -685,46 +374,74 @@ int ensure_packed_maps(bpdq_handle_s* h, EncodeTiledFn enc) {
     return BPDQ_OK;
 }
 
-template <int K, int BN>
-int launch_tile(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
-    using C = TileCfg<K, BN>;
+// Up to 128 tokens: one or several linears (same K, all or none with group 64); pair: the gated unit of two.
+template <int K>
+int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair) {
+    using C = TsCfg<K>;
     static bpdq::SmemOptin optin;
-    if (const int rc = bpdq::ensure_smem_optin(gemm_kernel<K, BN>, optin, h->device, C::kSmemBytes, "gemm"); rc != BPDQ_OK) return rc;
+    bpdq_handle_s* h0 = hs[0];
+    if (kTsSmem > h0->smem_optin)
+        return bpdq::set_error(BPDQ_ERR_UNSUPPORTED, "gemm: %d bytes of shared memory needed, device offers %d", kTsSmem, h0->smem_optin);
+    if (const int rc = bpdq::ensure_smem_optin(gemm_ts_kernel<K>, optin, h0->device, kTsSmem, "gemm"); rc != BPDQ_OK) return rc;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: cuTensorMapEncodeTiled is not available from this driver");
-    CUtensorMap map;
-    const cuuint64_t dims[2] = {(cuuint64_t)h->in, (cuuint64_t)M};
-    const cuuint64_t strides[1] = {(cuuint64_t)h->in * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)BN};
-    const cuuint32_t estr[2] = {1, 1};
-    CUresult cr = enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr,
-                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (cr != CUDA_SUCCESS) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: tensor map encode failed (CUresult %d)", (int)cr);
-    if (const int rc = ensure_packed_maps<K>(h, enc); rc != BPDQ_OK) return rc;
-    GemmParams p;
-    p.blob = h->d_blob; p.planes_bytes = h->planes_bytes; p.y = static_cast<__half*>(y); p.status = h->d_status;
-    p.out = h->out; p.in = h->in; p.group = h->group; p.M = M;
-    p.ws = h->d_ws; p.counters = h->d_counters; p.bias = static_cast<const __half*>(h->d_bias);
-    dim3 grid((h->out + BM - 1) / BM, (M + BN - 1) / BN);
-    const int nkb = h->in / BK;
-    p.kb_per = nkb;
-    if (grid.y == 1 && (size_t)M * h->out * sizeof(float) <= h->ws_bytes) {
-        // fewer output tiles than CTA slots: split the input dimension so that every SM gets work
-        const int slots = h->sm_count * C::kCtasPerSm;
-        int splits = slots / (int)grid.x;
-        constexpr int kMaxSplits = BN <= 32 ? 8 : 4;   // every split adds BN x 128 atomic adds per tile: fewer with many tokens
-        if (splits > kMaxSplits) splits = kMaxSplits;
-        if (splits > nkb / 16) splits = nkb / 16;     // at least 16 stages (1024 columns) per CTA
-        if (splits > 1) {
-            p.kb_per = ((nkb + splits - 1) / splits + 1) / 2 * 2;
-            grid.z = (nkb + p.kb_per - 1) / p.kb_per;
-        }
+    TsParams p;
+    p.n = n; p.M = M; p.cols = (M + 15) / 16 * 16;
+    p.status = h0->d_status;
+    p.ng = h0->group == 64 ? 2 : 1;
+    long long units = 0, tiles = 0;
+    bool same = true;                                    // rows of one length
+    for (int k = 0; k < n; ++k) {
+        const bpdq_handle_s* h = hs[k];
+        TsLinear& L = p.lin[k];
+        const cuuint64_t dims[2] = {(cuuint64_t)h->in, (cuuint64_t)M};
+        const cuuint64_t strides[1] = {(cuuint64_t)h->in * 2};
+        const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)p.cols};
+        const cuuint32_t estr[2] = {1, 1};
+        CUresult cr = enc(&L.x_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(xs[k]), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (cr != CUDA_SUCCESS) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: tensor map encode failed (CUresult %d)", (int)cr);
+        L.maps = static_cast<const CUtensorMap*>(h->d_few_maps) + 2;
+        L.y = static_cast<__half*>(ys[pair ? 0 : k]);
+        L.ws = h->d_ws; L.counters = pair ? h0->d_counters : h->d_counters;
+        L.conv_a = pair ? h0->d_ws : h->d_ws; L.conv_b = pair ? hs[1]->d_ws : nullptr;
+        L.bias_a = static_cast<const __half*>(pair ? h0->d_bias : h->d_bias);
+        L.bias_b = pair ? static_cast<const __half*>(hs[1]->d_bias) : nullptr;
+        L.out = h->out; L.nblocks = h->in / 128;
+        L.gsh = h->group == 64 ? 0 : (h->group == 128 ? 1 : 2);
+        L.u_begin = (int)units;
+        same = same && L.nblocks == p.lin[0].nblocks;
+        units += (long long)((h->out + BM - 1) / BM) * L.nblocks;
+        tiles += (h->out + BM - 1) / BM;
+        if (units >= (1ll << 31)) return bpdq::set_error(BPDQ_ERR_UNSUPPORTED, "gemm: task space too large");
     }
-    gemm_kernel<K, BN><<<grid, kTileThreads, C::kSmemBytes, stream>>>(map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
-                                                                   *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[1]), p);
-    h->launches += 1;
-    cudaError_t e = cudaGetLastError();
+    // x ring: as many blocks as 128 KB hold (four to eight, an even number: a slot belongs to one issuer), the packed ring
+    // gets the rest (nine slots or more; a decode group is at most eight blocks ahead of the MMAs, see the kernel)
+    p.sx = 128 * 1024 / (p.cols * 256) / 2 * 2;
+    if (p.sx > 8) p.sx = 8;
+    p.sp = (kTsSmem - 3072 - p.sx * p.cols * 256) / C::kSlotBytes;
+    if (p.sp > 24) p.sp = 24;
+    p.nbuf = p.cols <= 64 ? 2 : 1;
+    p.dcols = p.cols <= 64 ? 64 : 128;
+    // CTAs: at least eight blocks each when rows are cut (a share of a tile costs a tile of adds), else a tile each
+    const bool cut = !same || p.lin[0].nblocks >= kTsMinCut;
+    const long long most = cut ? (units + 7) / 8 : tiles;
+    const int grid = most < h0->sm_count ? (int)most : h0->sm_count;
+    p.nb0 = p.lin[0].nblocks;
+    p.whole = same ? (int)(tiles / grid) : 0;
+    p.cut_begin = p.whole * grid * p.nb0;
+    p.cut_units = (int)units - p.cut_begin;
+    p.cut_step = cut ? 1 : p.nb0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kTsThreads); cfg.dynamicSmemBytes = kTsSmem; cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the first packed blocks are requested under the tail of the kernel before
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_ts_kernel<K>, p);
+    h0->launches += 1;
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
     return BPDQ_OK;
 }
@@ -748,7 +465,7 @@ int launch_persistent(bpdq_handle_s* h, const void* x, void* y, int M, cudaStrea
     GemmParams p;
     p.blob = h->d_blob; p.planes_bytes = h->planes_bytes; p.y = static_cast<__half*>(y); p.status = h->d_status;
     p.out = h->out; p.in = h->in; p.group = h->group; p.M = M;
-    p.ws = h->d_ws; p.counters = h->d_counters; p.kb_per = h->in / BK; p.bias = static_cast<const __half*>(h->d_bias);
+    p.bias = static_cast<const __half*>(h->d_bias);
     const long long ntiles = (long long)((h->out + BM - 1) / BM) * ((M + kPersistBN - 1) / kPersistBN);
     const int grid = ntiles < h->sm_count ? (int)ntiles : h->sm_count;
     gemm_persistent_kernel<K><<<grid, kPersistThreads, C::kSmemBytes, stream>>>(map, p);
@@ -778,7 +495,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t st
     GemmParams p;
     p.blob = h->d_blob; p.planes_bytes = h->planes_bytes; p.y = static_cast<__half*>(y); p.status = h->d_status;
     p.out = h->out; p.in = h->in; p.group = h->group; p.M = M;
-    p.ws = h->d_ws; p.counters = h->d_counters; p.kb_per = h->in / kWideBK; p.bias = static_cast<const __half*>(h->d_bias);
+    p.bias = static_cast<const __half*>(h->d_bias);
     const long long ntiles = (long long)((h->out + BM - 1) / BM) * ((M + kWideBN - 1) / kWideBN);
     const int grid = ntiles < h->sm_count ? (int)ntiles : h->sm_count;
     gemm_wide_kernel<K><<<grid, kWideThreads, C::kSmemBytes, stream>>>(map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
@@ -791,10 +508,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t st
 
 template <int K>
 int launch_k(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
-    if (M <= 16) return launch_tile<K, 16>(h, x, y, M, stream);
-    if (M <= 32) return launch_tile<K, 32>(h, x, y, M, stream);
-    if (M <= 64) return launch_tile<K, 64>(h, x, y, M, stream);
-    if (M <= 128) return launch_tile<K, 128>(h, x, y, M, stream);
+    if (M <= kTsMaxM) return launch_ts<K>(&h, &x, &y, 1, M, stream, false);
     if (M <= 256) return launch_persistent<K>(h, x, y, M, stream);
     return launch_wide<K>(h, x, y, M, stream);       // 512-token tiles: measured faster than the 256-token kernel from 257 tokens on
 }
@@ -844,6 +558,23 @@ EncodeTiledFn encode_tiled_fn() {
 
 bool gemm_supported(int, int, int K, int group) {
     return K >= 1 && K <= 4 && (group == 64 || group == 128 || group == 256);
+}
+
+bool gemm_batch_supported(const bpdq_handle_s* h, int M) { return h->d_few_maps && M <= kTsMaxM && gemm_supported(h->out, h->in, h->K, h->group); }
+
+int launch_gemm_batch(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair) {
+    if (n < 1 || n > BPDQ_BATCH_MAX) return set_error(BPDQ_ERR_INVALID, "gemm: %d linears in one launch (1..%d)", n, BPDQ_BATCH_MAX);
+    if (pair && (n != 2 || hs[0]->out != hs[1]->out)) return set_error(BPDQ_ERR_INVALID, "gemm: a (gate, up) pair is two linears with the same rows");
+    for (int k = 0; k < n; ++k)
+        if (hs[k]->K != hs[0]->K || (hs[k]->group == 64) != (hs[0]->group == 64) || !gemm_batch_supported(hs[k], M))
+            return set_error(BPDQ_ERR_INVALID, "gemm: linear %d does not go into one launch with linear 0 (M=%d)", k, M);
+    switch (hs[0]->K) {
+        case 1: return launch_ts<1>(hs, xs, ys, n, M, stream, pair);
+        case 2: return launch_ts<2>(hs, xs, ys, n, M, stream, pair);
+        case 3: return launch_ts<3>(hs, xs, ys, n, M, stream, pair);
+        case 4: return launch_ts<4>(hs, xs, ys, n, M, stream, pair);
+        default: return set_error(BPDQ_ERR_UNSUPPORTED, "gemm: K=%d", hs[0]->K);
+    }
 }
 
 int launch_gemm(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {

@@ -566,7 +566,7 @@ int few_prepare(bpdq_handle_s* h) {
     if (!enc) return BPDQ_OK;
     const int K = h->K;
     const int ngs = 512 / h->group;
-    alignas(64) CUtensorMap maps[2];
+    alignas(64) CUtensorMap maps[4];
     constexpr int rows = 8 * kRowGroups;                                  // output rows of a task
     const cuuint32_t estr3[3] = {1, 1, 1};
     const cuuint64_t pd[3] = {16, (cuuint64_t)(h->in / 128) * K, (cuuint64_t)h->out / 8};
@@ -580,8 +580,18 @@ int few_prepare(bpdq_handle_s* h) {
     const CUresult r2 = enc(&maps[1], CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, h->d_blob + h->planes_bytes, cd, cs, cb, estr3,
                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r1 != CUDA_SUCCESS || r2 != CUDA_SUCCESS)
-        return set_error(BPDQ_ERR_CUDA, "bpdq_create: tensor map encode of the packed weights failed (CUresult %d, %d)", (int)r1, (int)r2);
+    // the tensor-core kernel's for up to 128 tokens: boxes of one 128-row x 128-column block (all planes; its one or two coefficient groups)
+    const cuuint64_t pd2[2] = {(cuuint64_t)h->out * 2, (cuuint64_t)(h->in / 128) * K};
+    const cuuint64_t ps2[1] = {(cuuint64_t)h->out * 16};
+    const cuuint32_t pb2[2] = {256, (cuuint32_t)K};
+    const cuuint32_t cb2[2] = {32, (cuuint32_t)((h->group == 64 ? 2 : 1) * (K + 1))};
+    const CUresult r3 = enc(&maps[2], CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, h->d_blob, pd2, ps2, pb2, estr3, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r4 = enc(&maps[3], CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, h->d_blob + h->planes_bytes, cd, cs, cb2, estr3,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r1 != CUDA_SUCCESS || r2 != CUDA_SUCCESS || r3 != CUDA_SUCCESS || r4 != CUDA_SUCCESS)
+        return set_error(BPDQ_ERR_CUDA, "bpdq_create: tensor map encode of the packed weights failed (CUresult %d, %d, %d, %d)", (int)r1, (int)r2, (int)r3, (int)r4);
     cudaError_t e = cudaMalloc(&h->d_few_maps, sizeof(maps));
     if (e != cudaSuccess) { h->d_few_maps = nullptr; return set_error(BPDQ_ERR_ALLOC, "bpdq_create: cudaMalloc failed (%s)", cudaGetErrorString(e)); }
     e = cudaMemcpy(h->d_few_maps, maps, sizeof(maps), cudaMemcpyHostToDevice);

@@ -79,7 +79,8 @@ struct bpdq_handle_s {
     int gemv_max_m;
     uint64_t launches;
     int few_max_m;            // largest M the dispatcher sends to the few-token kernel
-    void* d_few_maps;         // device copy of the few-token kernel's two tensor maps (null: not available)
+    int gemv_set;             // the caller chose gemv_max_m: no other kernel up to it
+    void* d_few_maps;         // device copy of two tensor maps of the few-token kernel and two of the tensor-core kernel for up to 128 tokens (null: not available)
     int* d_perm;              // input-channel permutation: stored column j multiplies x[perm[j]] (null: identity)
     void* d_xperm;            // [max_M][in] gathered activations for the kernels that do not fold the permutation into their loads
     void* d_bias;             // binary16 [out], added to every output row before the rounding (null: none)
@@ -102,6 +103,8 @@ int launch_gather_columns(bpdq_handle_s* h, const void* x, int M, cudaStream_t s
 int launch_swiglu(const void* gate, const void* up, void* hout, size_t n, cudaStream_t stream);
 int launch_gemv_mma(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream);
 int launch_gemv_mma_batch(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair = false);
+int launch_gemm_batch(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair = false);
+bool gemm_batch_supported(const bpdq_handle_s* h, int M);
 bool gemv_mma_supported(int out, int in, int K, int group);
 int few_prepare(bpdq_handle_s* h);
 size_t gemv_workspace_bytes(int out, int in, int K, int group, int max_M, int sm_count);

@@ -104,3 +104,60 @@ def test_gemm_packed_ring_under_load(K, g, M):
         y = G.run_linear(h, x, binding.KERNEL_GEMM)
         # binary16 rounding of the result (2^-11) and binary32 sums of 3584 terms of size up to 0.2 in another order
         assert np.all(np.abs(y - ref) <= 2.0 ** -10 * np.abs(ref) + 2e-3)
+
+
+@pytest.mark.parametrize("K,g,shapes,M", [
+    (2, 128, [(4096, 2048), (528, 2048), (512, 2048)], 5),       # rows of one length, fewer tiles than SMs: all are cut
+    (3, 64, [(20000, 2048), (272, 2048)], 16),                   # a whole tile per CTA and shared ones, across a linear's end
+    (2, 256, [(400, 1152), (272, 640), (16, 2176)], 3),          # rows of different lengths, ragged tiles
+    (4, 128, [(144, 384), (160, 384)], 9),                       # short rows: whole tiles only
+])
+def test_gemm_batch(K, g, shapes, M):
+    """Several linears in one launch of the tensor-core kernel, each against the checker; a second call finds clean state."""
+    import torch
+    hs, ref, xs, ys = [], [], [], []
+    for k, (o, i) in enumerate(shapes):
+        h, bits, coef = G.make_layer(400 + k, o, i, K, g, max_M=M)
+        x = synth.activations(410 + k, M, i)
+        rows = np.unique(np.concatenate([np.arange(0, o, 1 + o // 200), [0, o - 17 if o > 16 else 0, o - 1]]))
+        bias = np.random.RandomState(k).randn(o).astype(np.float16)
+        if k == 1:
+            h.bpdq_set_bias(bias.view(np.uint16))
+        r, a = oracle.linear(bits[:, rows], coef[:, rows], x, g)
+        ref.append((rows, r + (bias[rows].astype(np.float64) if k == 1 else 0.0), a + (np.abs(bias[rows].astype(np.float64)) if k == 1 else 0.0)))
+        hs.append(h)
+        xs.append(G.x_tensor(x))
+        ys.append(torch.full((M, o), float("nan"), dtype=torch.float16, device="cuda"))
+    for _ in range(2):
+        n0 = sum(h.bpdq_launch_count() for h in hs)
+        binding.bpdq_linear_batch(hs, [x.data_ptr() for x in xs], [y.data_ptr() for y in ys], M, G.stream_ptr())
+        torch.cuda.synchronize()
+        hs[0].bpdq_get_status(G.stream_ptr())
+        assert sum(h.bpdq_launch_count() for h in hs) == n0 + 1
+        for y, (rows, r, a) in zip(ys, ref):
+            G.assert_linear_close(y.cpu().numpy().astype(np.float64)[:, rows], r, a, "batch")
+
+
+@pytest.mark.parametrize("K,g,out,in_,M", [(2, 128, 2064, 2048, 17), (3, 64, 528, 896, 100), (4, 128, 272, 4096, 128), (2, 128, 40000, 256, 33)])
+def test_gated_unit_up_to_128_tokens_in_one_launch(K, g, out, in_, M):
+    """silu(gate) * up from unrounded sums: shared tiles, whole tiles and short rows."""
+    import torch
+    hg, bg, cg = G.make_layer(420, out, in_, K, g, max_M=M)
+    hu, bu, cu = G.make_layer(421, out, in_, K, g, max_M=M)
+    x = synth.activations(422, M, in_)
+    rows = np.unique(np.concatenate([np.arange(0, out, 1 + out // 100), [127, 128, out - 1]]))
+    gy, ga = oracle.linear(bg[:, rows], cg[:, rows], x, g)
+    uy, ua = oracle.linear(bu[:, rows], cu[:, rows], x, g)
+    want = oracle.swiglu(gy, uy)
+    dg, du = G.TOL_REL * ga + G.TOL_ABS, G.TOL_REL * ua + G.TOL_ABS
+    silu_g = oracle.swiglu(gy, np.ones_like(gy))
+    bound = 1.1 * (np.abs(uy) + du) * dg + (np.abs(silu_g) + 1.1 * dg) * du + 2.0 ** -10 * np.abs(want) + 1e-4
+    xt = G.x_tensor(x)
+    for _ in range(2):
+        hout = torch.full((M, out), float("nan"), dtype=torch.float16, device="cuda")
+        n0 = hg.bpdq_launch_count() + hu.bpdq_launch_count()
+        binding.bpdq_gate_up_swiglu(hg, hu, xt.data_ptr(), hout.data_ptr(), M, G.stream_ptr())
+        torch.cuda.synchronize()
+        hg.bpdq_get_status(G.stream_ptr())
+        assert hg.bpdq_launch_count() + hu.bpdq_launch_count() == n0 + 1
+        assert np.all(np.abs(hout.cpu().numpy().astype(np.float64)[:, rows] - want) <= bound)
