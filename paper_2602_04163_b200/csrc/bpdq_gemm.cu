@@ -12,11 +12,10 @@
 // 16-byte chunk c of row r is stored at chunk position c ^ (r mod 8).  TMA writes that layout by
 // itself; the decode threads reproduce it by hand.
 //
-// Three kernels: gemm_ts_kernel (up to 128 tokens: decoded weights in TMEM, one or several linears per launch;
-// bpdq_gemm_ts.cuh), gemm_persistent_kernel (129..256 tokens: token tile 256, one CTA per SM walks over tiles, two TMEM
-// accumulators, separate epilogue warps; described at its definition) and gemm_wide_kernel (more than 256 tokens: token
-// tile 512, two issuing warps; bpdq_gemm_wide.cuh).  In the two for many tokens the decoded operand goes through shared
-// memory: the MMAs, not the decode, are the bound there, and TMEM is full of accumulators.
+// Two kernels: gemm_ts_kernel (up to 128 tokens: decoded weights in TMEM, one or several linears per launch;
+// bpdq_gemm_ts.cuh) and gemm_wide_kernel (more than 128 tokens: token tiles of up to 512, two issuing warps;
+// bpdq_gemm_wide.cuh).  In the second the decoded operand goes through shared memory: there the MMAs, not the decode, are
+// the bound, and TMEM is full of accumulators.
 //
 // Decode: a thread reads its row's units and coefficients from the stage, builds the 2^K candidate values of the group
 // (Eq. 7, the decode rule's exact arithmetic) as byte tables, and then eight columns cost one shift-and-mask per plane to
@@ -38,20 +37,6 @@ namespace {
 
 constexpr int BM = 128;                 // output rows per CTA (MMA M)
 constexpr int BK = 64;                  // columns per stage: one 128-byte swizzle row of binary16
-constexpr int kDecodeGroups = 2;
-constexpr int kDecodeThreads = 128;               // per group: one thread per output row
-constexpr int kATileBytes = BM * BK * 2;                       // 16 KB
-
-template <int K, int BN> struct Cfg {
-    static constexpr int kBTileBytes = BN * BK * 2;
-    static constexpr int kPlaneBytes = K * BM * 16;             // K segments of 128 rows x 16 bytes
-    static constexpr int kCoefBytes = (K + 1) * BM * 2;         // K+1 segments of 128 rows x 2 bytes
-    static constexpr int kPackedBytes = (kPlaneBytes + kCoefBytes + 1023) / 1024 * 1024;
-    static constexpr int kStageBytes = kATileBytes + kBTileBytes + kPackedBytes;
-    static constexpr int kSmemBudget = 222 * 1024;
-    static constexpr int kStages = kSmemBudget / kStageBytes > 8 ? 8 : kSmemBudget / kStageBytes;
-    static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 512 /*barriers*/;
-};
 
 struct GemmParams {
     const uint8_t* blob;
@@ -107,237 +92,6 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(unsigned addr) {
 // K-major (bits 15, 16 = 0), N / 8 in bits 17..22, M / 16 in bits 24..28.
 __host__ __device__ constexpr unsigned instr_desc_f16(int m, int n) {
     return (1u << 4) | ((unsigned)(n >> 3) << 17) | ((unsigned)(m >> 4) << 24);
-}
-
-// ---- persistent variant for many tokens (token tile 256) -------------------------------------------------
-// One CTA per SM walks over output tiles (row tile fastest, so that the CTAs running together share one
-// 256-token slab of x in L2).  TMEM holds two 128 x 256 accumulators: while four epilogue warps drain one, the
-// MMA warp fills the other, and the producer and decode warps run straight on into the next tile's stages.
-// Roles (448 threads): warp 0 producer, warp 1 MMA, warps 2..9 decode (two groups, as above), warps 10..13
-// epilogue.  Barriers: the four per-stage barriers of the kernel above, used over one stage sequence that
-// continues across tiles, plus acc_full[2] (tcgen05.commit after a tile's last MMA) and acc_empty[2]
-// (128 epilogue threads after they have read the accumulator).
-constexpr int kPersistThreads = 64 + kDecodeGroups * kDecodeThreads + 128;
-constexpr int kPersistBN = 256;
-
-template <int K>
-__global__ void __launch_bounds__(kPersistThreads, 1)
-gemm_persistent_kernel(const __grid_constant__ CUtensorMap x_map, const GemmParams p) {
-    constexpr int BN = kPersistBN;
-    using C = Cfg<K, BN>;
-    constexpr int S = C::kStages;
-    extern __shared__ unsigned char smem_raw[];
-    const unsigned base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
-    const unsigned a_base = base;
-    const unsigned b_base = base + S * kATileBytes;
-    const unsigned p_base = b_base + S * C::kBTileBytes;
-    const unsigned bar_base = p_base + S * C::kPackedBytes;
-    auto full_b = [&](int s) { return bar_base + 8u * s; };
-    auto full_a = [&](int s) { return bar_base + 8u * (S + s); };
-    auto empty = [&](int s) { return bar_base + 8u * (2 * S + s); };
-    auto full_p = [&](int s) { return bar_base + 8u * (3 * S + s); };
-    auto acc_full = [&](int b) { return bar_base + 8u * (4 * S + b); };
-    auto acc_empty = [&](int b) { return bar_base + 8u * (4 * S + 2 + b); };
-    unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * (4 * S + 4));
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform, and known to be
-    const int nkb = p.in / BK;
-    const int nrt = (p.out + BM - 1) / BM;            // row tiles
-    const int ntt = (p.M + BN - 1) / BN;              // token tiles
-    const int ntiles = nrt * ntt;
-
-    if (tid == 0) {
-        for (int s = 0; s < S; ++s) {
-            mbar_init(full_b(s), 1);
-            mbar_init(full_a(s), kDecodeThreads);
-            mbar_init(empty(s), 1);
-            mbar_init(full_p(s), 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(acc_full(b), 1);
-            mbar_init(acc_empty(b), 128);
-        }
-        *abort_flag = 0;
-        fence_barrier_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_slot), 512);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const unsigned tmem_d = *tmem_slot;
-
-    if (warp == 0) {
-        // ---------------- producer ----------------
-        if (lane == 0) {
-            const uint8_t* cbase = p.blob + p.planes_bytes;
-            int it = 0;                                  // stage sequence number, continues across tiles
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-                const int row0 = (tile % nrt) * BM, tok0 = (tile / nrt) * BN;
-                const int nrows = min(BM, p.out - row0);
-                const unsigned seg_p = (unsigned)nrows * 16u, seg_c = (unsigned)nrows * 2u;
-                for (int kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = it % S;
-                    const unsigned ph = (unsigned)(it / S) & 1u;
-                    if (!mbar_wait(empty(s), ph ^ 1u, abort_flag, p.status)) { ok = false; break; }
-                    const bool first_half = (kb & 1) == 0;
-                    mbar_expect_tx(full_p(s), (first_half ? (unsigned)K * seg_p : 0u) + (unsigned)(K + 1) * seg_c);
-                    const unsigned pdst = p_base + s * C::kPackedBytes;
-                    const int b = kb >> 1, G = (kb * BK) / p.group;
-                    if (first_half) {
-#pragma unroll
-                        for (int i = 0; i < K; ++i)
-                            bulk_load(pdst + i * (BM * 16), p.blob + (((size_t)b * K + i) * p.out + row0) * 16, seg_p, full_p(s));
-                    }
-#pragma unroll
-                    for (int i = 0; i <= K; ++i)
-                        bulk_load(pdst + C::kPlaneBytes + i * (BM * 2), cbase + (((size_t)G * (K + 1) + i) * p.out + row0) * 2, seg_c, full_p(s));
-                    mbar_expect_tx(full_b(s), C::kBTileBytes);
-                    tma_load_2d(b_base + s * C::kBTileBytes, &x_map, kb * BK, tok0, full_b(s));
-                }
-            }
-        }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
-        {
-            constexpr unsigned idesc = instr_desc_f16(BM, BN);
-            int it = 0, j = 0;                           // stage sequence number; tiles done by this CTA
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++j) {
-                const int buf = j & 1;
-                // the epilogue must have drained this accumulator (two tiles ago)
-                if (!mbar_wait_warp(acc_empty(buf), ((unsigned)(j >> 1) & 1u) ^ 1u, abort_flag, p.status)) break;
-                tc_fence_after();
-                const unsigned d = tmem_d + (unsigned)(buf * BN);
-                for (int kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = it % S;
-                    const unsigned ph = (unsigned)(it / S) & 1u;
-                    ok = mbar_wait_warp(full_a(s), ph, abort_flag, p.status) && mbar_wait_warp(full_b(s), ph, abort_flag, p.status);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t adesc = smem_desc_sw128(a_base + s * kATileBytes);
-                    const uint64_t bdesc = smem_desc_sw128(b_base + s * C::kBTileBytes);
-                    if (elect_one()) {
-#pragma unroll
-                        for (int k4 = 0; k4 < BK / 16; ++k4)
-                            umma_f16(d, adesc + 2u * k4, bdesc + 2u * k4, idesc, (kb | k4) != 0 ? 1u : 0u);
-                        umma_commit(empty(s));
-                    }
-                    __syncwarp();
-                }
-                if (ok && elect_one()) umma_commit(acc_full(buf));
-                __syncwarp();
-            }
-        }
-    } else if (warp < 2 + 4 * kDecodeGroups) {
-        // ---------------- decode warps (thread = output row) ----------------
-        const int quad = warp & 3;
-        const int grp = (warp - 2) >> 2;
-        const int rl = quad * 32 + lane;
-        unsigned a_off[8];
-#pragma unroll
-        for (int ch = 0; ch < 8; ++ch) a_off[ch] = (unsigned)rl * 128u + (((unsigned)ch ^ (unsigned)(rl & 7)) << 4);
-        const int nblocks = nkb / 2;
-        int it0 = 0;                                     // stage sequence number of the current tile's first stage
-        bool ok = true;
-        for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, it0 += nkb) {
-            const int r = (tile % nrt) * BM + rl;        // rows past a ragged last tile decode stale bytes; nothing of theirs is stored
-            // A group keeps to every other block of the stage sequence ACROSS tiles (with an odd number of blocks per
-            // tile its parity inside the tile flips): its waits then follow the sequence two stages at a time and
-            // never run a whole ring ahead of a barrier's phase, which a parity wait could not tell from "ready".
-            static_assert(kDecodeGroups == 2, "two groups alternate blocks");
-            for (int b = grp ^ ((it0 >> 1) & 1); b < nblocks && ok; b += kDecodeGroups) {
-                unsigned cur[K][4];
-                bpdq::ByteTables<K> tab;
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const int it = it0 + 2 * b + half;
-                    const int s = it % S;
-                    const unsigned ph = (unsigned)(it / S) & 1u;
-                    if (!mbar_wait(full_p(s), ph, abort_flag, p.status)) { ok = false; break; }
-                    const unsigned psrc = p_base + s * C::kPackedBytes;
-                    if (half == 0) {
-#pragma unroll
-                        for (int i = 0; i < K; ++i) {
-                            uint4 raw;
-                            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(raw.x), "=r"(raw.y), "=r"(raw.z), "=r"(raw.w)
-                                         : "r"(psrc + i * (BM * 16) + rl * 16));
-                            const uint4 u = bpdq::unrotate_unit(raw, r);
-                            cur[i][0] = u.x; cur[i][1] = u.y; cur[i][2] = u.z; cur[i][3] = u.w;
-                        }
-                    }
-                    if (half == 0 || p.group == 64) {
-                        float c[K + 1];
-#pragma unroll
-                        for (int i = 0; i <= K; ++i) {
-                            unsigned short hbits;
-                            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(hbits) : "r"(psrc + C::kPlaneBytes + i * (BM * 2) + rl * 2));
-                            c[i] = __half2float(__ushort_as_half(hbits));
-                        }
-                        bpdq::candidate_byte_tables<K>(c, tab);
-                    }
-                    const unsigned dst = a_base + s * kATileBytes;
-#pragma unroll
-                    for (int wd = 0; wd < 2; ++wd) {
-                        unsigned w[K], sel[4];
-#pragma unroll
-                        for (int i = 0; i < K; ++i) w[i] = cur[i][2 * half + wd];
-                        bpdq::code_nibbles_word<K>(w, sel);
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const uint4 v8 = bpdq::decode8<K>(sel[u], tab);
-                            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + a_off[4 * wd + u]),
-                                         "r"(v8.x), "r"(v8.y), "r"(v8.z), "r"(v8.w) : "memory");
-                        }
-                    }
-                    fence_proxy_async();
-                    mbar_arrive(full_a(s));
-                }
-            }
-        }
-    } else {
-        // ---------------- epilogue warps: drain one accumulator while the other is being filled ----------------
-        const int quad = warp & 3;                       // TMEM lane quadrant this warp may access
-        const int rl = quad * 32 + lane;
-        int j = 0;
-        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++j) {
-            const int buf = j & 1;
-            if (!mbar_wait(acc_full(buf), (unsigned)(j >> 1) & 1u, abort_flag, p.status)) break;
-            tc_fence_after();
-            const int row0 = (tile % nrt) * BM, tok0 = (tile / nrt) * BN;
-            const int r = row0 + rl;
-            const bool row_ok = r < p.out;
-            const unsigned taddr = tmem_d + ((unsigned)(quad * 32) << 16) + (unsigned)(buf * BN);
-#pragma unroll 1
-            for (int c0 = 0; c0 < BN; c0 += 16) {
-                if (tok0 + c0 >= p.M) break;             // warp-uniform
-                unsigned v[16];
-                tmem_ld16(taddr + (unsigned)c0, v);
-                tmem_ld_wait();
-                if (row_ok) {
-                    const float br = p.bias ? __half2float(p.bias[r]) : 0.f;
-#pragma unroll
-                    for (int jj = 0; jj < 16; ++jj) {
-                        const int t = tok0 + c0 + jj;
-                        if (t < p.M) p.y[(size_t)t * p.out + r] = __float2half_rn(__uint_as_float(v[jj]) + br);
-                    }
-                }
-            }
-            tc_fence_before();
-            mbar_arrive(acc_empty(buf));                 // 128 arrivals: the accumulator may be overwritten
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc(tmem_d, 512);
-    }
 }
 
 #include "bpdq_gemm_wide.cuh"
@@ -446,60 +200,55 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
     return BPDQ_OK;
 }
 
-template <int K>
-int launch_persistent(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
-    using C = Cfg<K, kPersistBN>;
-    static bpdq::SmemOptin optin;
-    if (const int rc = bpdq::ensure_smem_optin(gemm_persistent_kernel<K>, optin, h->device, C::kSmemBytes, "gemm"); rc != BPDQ_OK) return rc;
-    EncodeTiledFn enc = encode_tiled_fn();
-    if (!enc) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: cuTensorMapEncodeTiled is not available from this driver");
-    CUtensorMap map;
-    const cuuint64_t dims[2] = {(cuuint64_t)h->in, (cuuint64_t)M};
-    const cuuint64_t strides[1] = {(cuuint64_t)h->in * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)kPersistBN};
-    const cuuint32_t estr[2] = {1, 1};
-    CUresult cr = enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr,
-                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (cr != CUDA_SUCCESS) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: tensor map encode failed (CUresult %d)", (int)cr);
-    GemmParams p;
-    p.blob = h->d_blob; p.planes_bytes = h->planes_bytes; p.y = static_cast<__half*>(y); p.status = h->d_status;
-    p.out = h->out; p.in = h->in; p.group = h->group; p.M = M;
-    p.bias = static_cast<const __half*>(h->d_bias);
-    const long long ntiles = (long long)((h->out + BM - 1) / BM) * ((M + kPersistBN - 1) / kPersistBN);
-    const int grid = ntiles < h->sm_count ? (int)ntiles : h->sm_count;
-    gemm_persistent_kernel<K><<<grid, kPersistThreads, C::kSmemBytes, stream>>>(map, p);
-    h->launches += 1;
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
-    return BPDQ_OK;
+// Tokens of a half tile: the cut of M tokens into equal tiles that takes the least time by a model of the kernel.  A 128-column
+// block takes 8.5 clocks per token of a half (the MMAs; 1.14 us with 512-token tiles), but no less than 1320 (the copies of its
+// stages and the decode; 1700 with sixteen candidates); a tile is paid for in whole rounds over the SMs.  Always 512 tokens per tile left most SMs idle
+// on short token counts: 3584 x 18944 (28 row tiles) with 777 tokens took 199 us in 56 tiles, in 140 it takes 121.
+int wide_half(int M, int nrt, int nblocks, int K, int sms) {
+    const long long least = K == 4 ? 1700 : 1320;
+    long long best = 0;
+    int half = kWideMaxHalf;
+    for (int ntt = (M + 2 * kWideMaxHalf - 1) / (2 * kWideMaxHalf); ntt <= (M + 31) / 32; ++ntt) {
+        const int h = ((M + ntt - 1) / ntt + 31) / 32 * 16;
+        const long long tiles = (long long)nrt * ((M + 2 * h - 1) / (2 * h)), rounds = (tiles + sms - 1) / sms;
+        const long long block = 17LL * h / 2 > least ? 17LL * h / 2 : least;
+        const long long cost = rounds * (nblocks * block + 2000 + 30LL * h);
+        if (best == 0 || cost < best) { best = cost; half = h; }
+    }
+    return half;
 }
 
 template <int K>
 int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
     using C = WideCfg<K>;
     static bpdq::SmemOptin optin;
-    if (const int rc = bpdq::ensure_smem_optin(gemm_wide_kernel<K>, optin, h->device, C::kSmemBytes, "gemm"); rc != BPDQ_OK) return rc;
+    if (const int rc = bpdq::ensure_smem_optin(gemm_wide_kernel<K>, optin, h->device, kWideSmem, "gemm"); rc != BPDQ_OK) return rc;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: cuTensorMapEncodeTiled is not available from this driver");
+    const int nrt = (h->out + BM - 1) / BM;
+    WideParams p;
+    p.half = wide_half(M, nrt, h->in / 128, K, h->sm_count);
+    const int stage = kWideATile + 2 * p.half * kWideBK * 2;
+    p.stages = C::kStageBudget / stage > kWideMaxStages ? kWideMaxStages : C::kStageBudget / stage;
+    p.sp = kWideMinSP + (C::kStageBudget - p.stages * stage) / C::kBlockBytes;
+    p.sp = p.sp > kWideMaxSP ? kWideMaxSP : p.sp / 2 * 2;
     CUtensorMap map;
     const cuuint64_t dims[2] = {(cuuint64_t)h->in, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)h->in * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kWideBK, 256};
+    const cuuint32_t box[2] = {(cuuint32_t)kWideBK, (cuuint32_t)(2 * p.half <= 256 ? 2 * p.half : p.half)};
     const cuuint32_t estr[2] = {1, 1};
     CUresult cr = enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr,
                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (cr != CUDA_SUCCESS) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: tensor map encode failed (CUresult %d)", (int)cr);
     if (const int rc = ensure_packed_maps<K>(h, enc); rc != BPDQ_OK) return rc;
-    GemmParams p;
-    p.blob = h->d_blob; p.planes_bytes = h->planes_bytes; p.y = static_cast<__half*>(y); p.status = h->d_status;
-    p.out = h->out; p.in = h->in; p.group = h->group; p.M = M;
-    p.bias = static_cast<const __half*>(h->d_bias);
-    const long long ntiles = (long long)((h->out + BM - 1) / BM) * ((M + kWideBN - 1) / kWideBN);
+    p.g.blob = h->d_blob; p.g.planes_bytes = h->planes_bytes; p.g.y = static_cast<__half*>(y); p.g.status = h->d_status;
+    p.g.out = h->out; p.g.in = h->in; p.g.group = h->group; p.g.M = M;
+    p.g.bias = static_cast<const __half*>(h->d_bias);
+    const long long ntiles = (long long)nrt * ((M + 2 * p.half - 1) / (2 * p.half));
     const int grid = ntiles < h->sm_count ? (int)ntiles : h->sm_count;
-    gemm_wide_kernel<K><<<grid, kWideThreads, C::kSmemBytes, stream>>>(map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
-                                                                      *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[1]), p);
+    gemm_wide_kernel<K><<<grid, kWideThreads, kWideSmem, stream>>>(map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
+                                                                  *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[1]), p);
     h->launches += 1;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
@@ -509,8 +258,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t st
 template <int K>
 int launch_k(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
     if (M <= kTsMaxM) return launch_ts<K>(&h, &x, &y, 1, M, stream, false);
-    if (M <= 256) return launch_persistent<K>(h, x, y, M, stream);
-    return launch_wide<K>(h, x, y, M, stream);       // 512-token tiles: measured faster than the 256-token kernel from 257 tokens on
+    return launch_wide<K>(h, x, y, M, stream);
 }
 
 // Diagnostic: the library's bounded wait on a barrier that nothing arrives at.  It must give up after its limit, record
