@@ -201,16 +201,17 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
 }
 
 // Tokens of a half tile: the cut of M tokens into equal tiles that takes the least time by a model of the kernel.  A 128-column
-// block takes 8.5 clocks per token of a half (the MMAs; 1.14 us with 512-token tiles), but no less than 1320 (the copies of its
-// stages and the decode; 1700 with sixteen candidates); a tile is paid for in whole rounds over the SMs.  Always 512 tokens per tile left most SMs idle
-// on short token counts: 3584 x 18944 (28 row tiles) with 777 tokens took 199 us in 56 tiles, in 140 it takes 121.
+// block takes 8.5 clocks per token of a half (the MMAs; 1.14 us with 512-token tiles), but no less than the decode and the
+// hand-over of its stages: 1150 clocks with 64-column stages, 1320 with 32-column ones (1600 and 1700 with sixteen candidates).
+// A tile is paid for in whole rounds over the SMs.  Always 512 tokens per tile left most SMs idle on short token counts:
+// 3584 x 18944 (28 row tiles) with 777 tokens took 199 us in 56 tiles, in 140 it takes 100.
 int wide_half(int M, int nrt, int nblocks, int K, int sms) {
-    const long long least = K == 4 ? 1700 : 1320;
     long long best = 0;
     int half = kWideMaxHalf;
     for (int ntt = (M + 2 * kWideMaxHalf - 1) / (2 * kWideMaxHalf); ntt <= (M + 31) / 32; ++ntt) {
         const int h = ((M + ntt - 1) / ntt + 31) / 32 * 16;
         const long long tiles = (long long)nrt * ((M + 2 * h - 1) / (2 * h)), rounds = (tiles + sms - 1) / sms;
+        const long long least = h <= kWideLongHalf ? (K == 4 ? 1600 : 1150) : (K == 4 ? 1700 : 1320);
         const long long block = 17LL * h / 2 > least ? 17LL * h / 2 : least;
         const long long cost = rounds * (nblocks * block + 2000 + 30LL * h);
         if (best == 0 || cost < best) { best = cost; half = h; }
@@ -218,27 +219,27 @@ int wide_half(int M, int nrt, int nblocks, int K, int sms) {
     return half;
 }
 
-template <int K>
-int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
-    using C = WideCfg<K>;
+template <int K, int BKW>
+int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaStream_t stream) {
+    using C = WideCfg<K, BKW>;
     static bpdq::SmemOptin optin;
-    if (const int rc = bpdq::ensure_smem_optin(gemm_wide_kernel<K>, optin, h->device, kWideSmem, "gemm"); rc != BPDQ_OK) return rc;
+    if (const int rc = bpdq::ensure_smem_optin(gemm_wide_kernel<K, BKW>, optin, h->device, kWideSmem, "gemm"); rc != BPDQ_OK) return rc;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: cuTensorMapEncodeTiled is not available from this driver");
     const int nrt = (h->out + BM - 1) / BM;
     WideParams p;
-    p.half = wide_half(M, nrt, h->in / 128, K, h->sm_count);
-    const int stage = kWideATile + 2 * p.half * kWideBK * 2;
+    p.half = half;
+    const int stage = C::stage_bytes(half);
     p.stages = C::kStageBudget / stage > kWideMaxStages ? kWideMaxStages : C::kStageBudget / stage;
     p.sp = kWideMinSP + (C::kStageBudget - p.stages * stage) / C::kBlockBytes;
     p.sp = p.sp > kWideMaxSP ? kWideMaxSP : p.sp / 2 * 2;
     CUtensorMap map;
     const cuuint64_t dims[2] = {(cuuint64_t)h->in, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)h->in * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kWideBK, (cuuint32_t)(2 * p.half <= 256 ? 2 * p.half : p.half)};
+    const cuuint32_t box[2] = {(cuuint32_t)BKW, (cuuint32_t)(2 * p.half <= 256 ? 2 * p.half : p.half)};
     const cuuint32_t estr[2] = {1, 1};
     CUresult cr = enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr,
-                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, BKW == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (cr != CUDA_SUCCESS) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: tensor map encode failed (CUresult %d)", (int)cr);
     if (const int rc = ensure_packed_maps<K>(h, enc); rc != BPDQ_OK) return rc;
@@ -247,7 +248,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t st
     p.g.bias = static_cast<const __half*>(h->d_bias);
     const long long ntiles = (long long)nrt * ((M + 2 * p.half - 1) / (2 * p.half));
     const int grid = ntiles < h->sm_count ? (int)ntiles : h->sm_count;
-    gemm_wide_kernel<K><<<grid, kWideThreads, kWideSmem, stream>>>(map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
+    gemm_wide_kernel<K, BKW><<<grid, kWideThreads, kWideSmem, stream>>>(map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
                                                                   *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[1]), p);
     h->launches += 1;
     cudaError_t e = cudaGetLastError();
@@ -258,7 +259,8 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t st
 template <int K>
 int launch_k(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
     if (M <= kTsMaxM) return launch_ts<K>(&h, &x, &y, 1, M, stream, false);
-    return launch_wide<K>(h, x, y, M, stream);
+    const int half = wide_half(M, (h->out + BM - 1) / BM, h->in / 128, K, h->sm_count);
+    return half <= kWideLongHalf ? launch_wide<K, 64>(h, x, y, M, half, stream) : launch_wide<K, 32>(h, x, y, M, half, stream);
 }
 
 // Diagnostic: the library's bounded wait on a barrier that nothing arrives at.  It must give up after its limit, record

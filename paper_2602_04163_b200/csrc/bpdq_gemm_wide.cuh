@@ -9,20 +9,21 @@
 // is lifted.  TMEM is full with one tile, so the epilogue no longer overlaps the next tile's MMAs (about 3 % of a
 // 72B-shaped tile's time); producer and decode warps run ahead into the next tile's stages meanwhile.
 //
-// Stages are 32 columns (64-byte swizzle rows): 8 KB of decoded weights and two halves of activations per stage, five stages
-// of the widest tile, up to twelve of narrower ones; packed 128-column blocks (two tensor-map boxes each) in a ring of two
-// to eight.  Roles (640 threads): warps 0 and 3 producers (x, packed), warps 1-2 MMA issuers (half 0, half 1), warps 4-11 decode (two groups of
-// four warps, thread = output row, alternating 128-column blocks of the stage sequence, which continues across tiles), warps
-// 12-19 epilogue (four per half).  Barriers per stage: full (both x halves' bytes and one arrival per warp of the owning
-// decode group), empty (one tcgen05.commit per issuer); per packed slot: full_p, empty_p; acc_full (one commit per issuer),
-// acc_empty (one arrival per epilogue warp).  All waits are bounded.
-constexpr int kWideBK = 32;                                   // columns per stage: one 64-byte swizzle row of binary16
+// Stages are 64 columns (128-byte swizzle rows) while four of them fit, i.e. for halves of up to 128 tokens, else 32 columns
+// (64-byte rows: five stages of the widest tile): a stage costs its issuers about 330 clocks beside the decode warps that
+// share their schedulers, a block of four 32-column ones 1320, which is more than the MMAs of halves below 160 tokens take.
+// Packed 128-column blocks (two tensor-map boxes each) come in a ring of two to eight.  Roles (640 threads): warps 0 and 3
+// producers (x, packed), warps 1-2 MMA issuers (half 0, half 1), warps 4-11 decode (two groups of four warps, thread =
+// output row, alternating 128-column blocks of the stage sequence, which continues across tiles), warps 12-19 epilogue (four
+// per half).  Barriers per stage: full (both x halves' bytes and one arrival per warp of the owning decode group), empty (one
+// tcgen05.commit per issuer); per packed slot: full_p, empty_p; acc_full (one commit per issuer), acc_empty (one arrival per
+// epilogue warp).  All waits are bounded.
 constexpr int kWideMaxHalf = 256;                             // most tokens of a half
+constexpr int kWideLongHalf = 128;                            // ... with 64-column stages
 constexpr int kWideEpiWarps = 8;
 constexpr int kWideGroups = 2;                                // decode groups, alternating blocks
 constexpr int kWideFirstDecode = 4, kWideFirstEpi = kWideFirstDecode + 4 * kWideGroups;
 constexpr int kWideThreads = 32 * (kWideFirstEpi + kWideEpiWarps);
-constexpr int kWideATile = BM * kWideBK * 2;                  // 8 KB
 constexpr int kWideMinSP = 2, kWideMaxSP = 8;                  // packed blocks in flight (an even number: a slot belongs to one group)
 constexpr int kWideSmem = 227 * 1024;
 constexpr int kWideMaxStages = 12;
@@ -33,12 +34,18 @@ struct WideParams {
     int stages, sp;            // slots of the stage ring and of the packed ring
 };
 
-template <int K> struct WideCfg {
+// BKW: columns per stage, 32 (64-byte swizzle rows) or 64 (128-byte ones).
+template <int K, int BKW> struct WideCfg {
+    static constexpr int kATile = BM * BKW * 2;                // 8 or 16 KB
+    static constexpr int kPerBlock = 128 / BKW;                // stages per packed block
+    // a decode group waits for stage it after stage it - (kPerBlock + 1): the ring has to be at least that long (see there)
+    static constexpr int kMinStages = kPerBlock + 1;
+    static constexpr int stage_bytes(int half) { return kATile + 2 * half * BKW * 2; }
     static constexpr int kPlaneBytes = K * BM * 16;
     static constexpr int kCoefBytes = (K + 1) * BM * 2;
     static constexpr int kBlockBytes = (kPlaneBytes + 2 * kCoefBytes + 1023) / 1024 * 1024;
     static constexpr int kStageBudget = kWideSmem - kWideMinSP * kBlockBytes - 1024 /*alignment slack*/ - 1024 /*barriers*/;
-    static_assert(kStageBudget >= 5 * (kWideATile + 2 * kWideMaxHalf * kWideBK * 2), "five stages of the widest tile");
+    static_assert(BKW == 64 || kStageBudget >= kMinStages * stage_bytes(kWideMaxHalf), "the widest tile");
 };
 
 // Shared-memory matrix descriptor of a K-major tile with 64-byte swizzle whose rows are 64 bytes apart: start address
@@ -49,14 +56,15 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(unsigned addr) {
            ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
-template <int K>
+template <int K, int BKW>
 __global__ void __launch_bounds__(kWideThreads, 1)
 gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap planes_map,
                  const __grid_constant__ CUtensorMap coefs_map, const WideParams wp) {
     const GemmParams& p = wp.g;
-    using C = WideCfg<K>;
+    using C = WideCfg<K, BKW>;
+    constexpr int kPerBlock = C::kPerBlock;
     const int S = wp.stages, SP = wp.sp, half = wp.half;
-    const unsigned bhalf = (unsigned)half * (kWideBK * 2), stage = kWideATile + 2u * bhalf;
+    const unsigned bhalf = (unsigned)half * (BKW * 2), stage = C::kATile + 2u * bhalf;
     extern __shared__ unsigned char smem_raw[];
     const unsigned base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
@@ -72,7 +80,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    const int nkb = p.in / kWideBK;                  // stages per tile
+    const int nkb = p.in / BKW;                  // stages per tile
     const int nblk = p.in / 128;                     // packed blocks per tile (four stages each)
     const int nrt = (p.out + BM - 1) / BM;
     const int ntt = (p.M + 2 * half - 1) / (2 * half);
@@ -113,9 +121,9 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 for (int kb = 0; kb < nkb; ++kb) {
                     if (!mbar_wait(empty(s), ph, abort_flag, p.status)) { ok = false; break; }
                     mbar_expect_tx(full(s), 2u * bhalf);
-                    const unsigned bdst = st_base + (unsigned)s * stage + kWideATile;
-                    tma_load_2d(bdst, &x_map, kb * kWideBK, tok0, full(s));
-                    if (boxes == 2) tma_load_2d(bdst + bhalf, &x_map, kb * kWideBK, tok0 + half, full(s));
+                    const unsigned bdst = st_base + (unsigned)s * stage + C::kATile;
+                    tma_load_2d(bdst, &x_map, kb * BKW, tok0, full(s));
+                    if (boxes == 2) tma_load_2d(bdst + bhalf, &x_map, kb * BKW, tok0 + half, full(s));
                     if (++s == S) { s = 0; ph ^= 1u; }
                 }
             }
@@ -160,10 +168,12 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                     if (!ok) break;
                     tc_fence_after();
                     const unsigned a_addr = st_base + (unsigned)s * stage;
-                    const uint64_t adesc = smem_desc_sw64(a_addr);
-                    const uint64_t bdesc = smem_desc_sw64(a_addr + kWideATile + (unsigned)h * bhalf);
-                    umma_f16(d, adesc, bdesc, idesc, more);
-                    umma_f16(d, adesc + 2u, bdesc + 2u, idesc, 1u);   // 16 columns = 32 bytes further along the swizzled row
+                    const unsigned b_addr = a_addr + C::kATile + (unsigned)h * bhalf;
+                    const uint64_t adesc = BKW == 32 ? smem_desc_sw64(a_addr) : smem_desc_sw128(a_addr);
+                    const uint64_t bdesc = BKW == 32 ? smem_desc_sw64(b_addr) : smem_desc_sw128(b_addr);
+#pragma unroll
+                    for (int k = 0; k < BKW / 16; ++k)                // 16 columns = 32 bytes further along the swizzled row
+                        umma_f16(d, adesc + 2u * k, bdesc + 2u * k, idesc, k == 0 ? more : 1u);
                     umma_commit(empty(s));
                     more = 1u;
                     if (++s == S) { s = 0; ph ^= 1u; }
@@ -176,21 +186,22 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         // ---------------- decode warps: thread = output row; a group takes every other block ----------------
         const int grp = (warp - kWideFirstDecode) >> 2;
         const int rl = ((warp - kWideFirstDecode) & 3) * 32 + lane;     // row inside the tile; row tiles start at multiples of 128
-        unsigned a_off[4];                               // swizzled byte offset of each 16-byte chunk of this thread's 64-byte row
+        unsigned a_off[BKW / 8];                         // swizzled byte offset of each 16-byte chunk of this thread's 64- or 128-byte row
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) a_off[ch] = (unsigned)rl * 64u + (((unsigned)ch ^ (unsigned)((rl >> 1) & 3)) << 4);
+        for (int ch = 0; ch < BKW / 8; ++ch)
+            a_off[ch] = (unsigned)rl * (BKW * 2u) + (((unsigned)ch ^ (unsigned)(BKW == 32 ? (rl >> 1) & 3 : rl & 7)) << 4);
         const unsigned wrot = (unsigned)(rl >> 2) & 3u, sh = (unsigned)(rl & 3) * 8u;
         unsigned off[4];                                 // logical word k takes the bytes of physical words k - wrot and k - wrot - 1
 #pragma unroll
         for (unsigned k = 0; k < 4; ++k) off[k] = p_base + (unsigned)rl * 16u + (((k - wrot) & 3u) << 2);
         // Stage slots are shared by the groups; a wait by parity needs the release two uses back to be over.  A group that
-        // waits for stage it has waited for a stage no earlier than it - 5 before, i.e. for an MMA no earlier than
-        // it - 5 - S, and MMAs complete in order: enough for S >= 5.
+        // waits for stage it has waited for a stage no earlier than it - (kPerBlock + 1) before, i.e. for an MMA no earlier
+        // than S stages before that one, and MMAs complete in order: enough for S >= kPerBlock + 1.
         const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
         int s = 0, sp = grp;
         unsigned ph = 1u, pp = 0u;
         auto advance = [&](int n) { s += n; while (s >= S) { s -= S; ph ^= 1u; } };
-        advance(4 * grp);
+        advance(kPerBlock * grp);
         bool ok = true;
         const long long nbseq = (long long)my_tiles * nblk;
         for (long long bseq = grp; bseq < nbseq && ok; bseq += kWideGroups) {
@@ -203,39 +214,44 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 for (int k = 0; k < 4; ++k) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(a[i][k]) : "r"(so + i * (BM * 16) + off[k]));
             bpdq::ByteTables<K> tab;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {                // the block's four 32-column stages
-                if (q == 0 || (ng == 2 && q == 2)) {     // candidate tables of the coefficient group that starts here
+            for (int st = 0; st < kPerBlock; ++st) {     // the block's stages
+                constexpr int kWords = BKW / 32;         // 32-column words per stage
+                if (st == 0 || (ng == 2 && st * kWords == 2)) {   // candidate tables of the coefficient group that starts here
                     float c[K + 1];
 #pragma unroll
                     for (int i = 0; i <= K; ++i) {
                         unsigned short hb;
-                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(hb) : "r"(p_base + so + C::kPlaneBytes + (q / 2) * C::kCoefBytes + i * (BM * 2) + rl * 2));
+                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(hb) : "r"(p_base + so + C::kPlaneBytes + (st * kWords / 2) * C::kCoefBytes + i * (BM * 2) + rl * 2));
                         c[i] = __half2float(__ushort_as_half(hb));
                     }
                     bpdq::candidate_byte_tables<K>(c, tab);
                 }
-                unsigned w[K], sel[4];
+                uint4 v8[BKW / 8];                       // decode first (nothing of it waits for the slot), then wait and store
 #pragma unroll
-                for (int i = 0; i < K; ++i) w[i] = __funnelshift_l(a[i][(q + 3) & 3], a[i][q], sh);
-                bpdq::code_nibbles_word<K>(w, sel);
-                uint4 v8[4];                             // decode first (nothing of it waits for the slot), then wait and store
+                for (int e = 0; e < kWords; ++e) {
+                    const int q = st * kWords + e;
+                    unsigned w[K], sel[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) v8[u] = bpdq::decode8<K>(sel[u], tab);
+                    for (int i = 0; i < K; ++i) w[i] = __funnelshift_l(a[i][(q + 3) & 3], a[i][q], sh);
+                    bpdq::code_nibbles_word<K>(w, sel);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) v8[4 * e + u] = bpdq::decode8<K>(sel[u], tab);
+                }
                 if (!mbar_wait(empty(s), ph, abort_flag, p.status)) { ok = false; break; }
                 const unsigned dst = st_base + (unsigned)s * stage;
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch)
+                for (int ch = 0; ch < BKW / 8; ++ch)
                     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + a_off[ch]),
                                  "r"(v8[ch].x), "r"(v8[ch].y), "r"(v8[ch].z), "r"(v8[ch].w) : "memory");
                 fence_proxy_async();                     // make the generic-proxy stores visible to the MMA's reads
                 __syncwarp();
                 if (lane == 0) {
                     mbar_arrive(full(s));                // one arrival per warp, after all its lanes' stores and fences
-                    if (q == 2 * (ng - 1)) mbar_arrive(empty_p(sp));   // a stored stage has used the last loads from the packed slot: it may be refilled
+                    if (st == (ng - 1) * (kPerBlock / 2)) mbar_arrive(empty_p(sp));   // a stored stage has used the last loads from the packed slot: it may be refilled
                 }
                 advance(1);
             }
-            advance(4 * (kWideGroups - 1));              // the other group's block
+            advance(kPerBlock * (kWideGroups - 1));              // the other group's block
             sp += kWideGroups;
             if (sp >= SP) { sp -= SP; pp ^= 1u; }
         }
