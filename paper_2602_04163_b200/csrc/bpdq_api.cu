@@ -55,24 +55,58 @@ __global__ void gather_kernel(const __grid_constant__ GatherParams p) {
     }
 }
 
-// Activations in stored-column order: dst[m][j] = src[m][perm[j]], eight columns (sixteen bytes) per thread.
-__global__ void gather_columns_kernel(const __half* __restrict__ src, const int* __restrict__ perm, __half* __restrict__ dst,
-                                      int M, int in) {
+// Activations in stored-column order: dst[m][j] = src[m][perm[j]].  A CTA takes a token: its row comes in once with full
+// lines and is picked apart in shared memory (2-byte reads from global memory at random took 45 us for 777 x 18944 values).
+// Rows that do not fit shared memory are read from L2.
+template <bool STAGED>
+__global__ void __launch_bounds__(512) gather_columns_kernel(const __half* __restrict__ src, const int* __restrict__ perm, __half* __restrict__ dst,
+                                                             int M, int in) {
+    extern __shared__ __align__(16) unsigned char gather_smem[];
+    const __half* staged = reinterpret_cast<const __half*>(gather_smem);
     const int chunks = in / 8;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)M * chunks; i += (long long)gridDim.x * blockDim.x) {
-        const int m = (int)(i / chunks), c = (int)(i % chunks);
-        const int4 p0 = *reinterpret_cast<const int4*>(perm + c * 8), p1 = *reinterpret_cast<const int4*>(perm + c * 8 + 4);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");            // the kernel before this one may have written src, or still read dst
+    for (int m = blockIdx.x; m < M; m += gridDim.x) {
         const __half* row = src + (size_t)m * in;
-        __align__(16) __half v[8] = {row[p0.x], row[p0.y], row[p0.z], row[p0.w], row[p1.x], row[p1.y], row[p1.z], row[p1.w]};
-        *reinterpret_cast<uint4*>(dst + (size_t)m * in + c * 8) = *reinterpret_cast<const uint4*>(v);
+        if (STAGED) {
+            for (int c = threadIdx.x; c < chunks; c += blockDim.x)
+                reinterpret_cast<uint4*>(gather_smem)[c] = __ldcg(reinterpret_cast<const uint4*>(row) + c);
+            __syncthreads();
+        }
+        const __half* from = STAGED ? staged : row;
+        for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
+            const int4 p0 = __ldg(reinterpret_cast<const int4*>(perm + c * 8)), p1 = __ldg(reinterpret_cast<const int4*>(perm + c * 8 + 4));
+            __align__(16) __half v[8] = {from[p0.x], from[p0.y], from[p0.z], from[p0.w], from[p1.x], from[p1.y], from[p1.z], from[p1.w]};
+            *reinterpret_cast<uint4*>(dst + (size_t)m * in + c * 8) = *reinterpret_cast<const uint4*>(v);
+        }
+        if (STAGED) __syncthreads();
     }
 }
 
-// h = silu(gate) * up on rounded binary16 inputs (the many-token path of bpdq_gate_up_swiglu), two values per thread.
-__global__ void swiglu_kernel(const __half2* __restrict__ gate, const __half2* __restrict__ up, __half2* __restrict__ hout, size_t n2) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
-        const float2 g = __half22float2(gate[i]), u = __half22float2(up[i]);
-        hout[i] = __floats2half2_rn(bpdq::silu_f32(g.x) * u.x, bpdq::silu_f32(g.y) * u.y);
+// h = silu(gate) * up on rounded binary16 inputs (the many-token path of bpdq_gate_up_swiglu), eight values per thread and
+// access (two took 23 us for 777 x 18944 values).
+__global__ void swiglu_kernel(const uint4* gate, const uint4* up, uint4* hout, size_t n8) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const size_t step = gridDim.x * (size_t)blockDim.x;
+    for (size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i0 < n8; i0 += 2 * step) {
+        uint4 gv[2], uv[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (i0 + k * step < n8) { gv[k] = __ldcg(gate + i0 + k * step); uv[k] = __ldcg(up + i0 + k * step); }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (i0 + k * step >= n8) break;
+            const unsigned g4[4] = {gv[k].x, gv[k].y, gv[k].z, gv[k].w}, u4[4] = {uv[k].x, uv[k].y, uv[k].z, uv[k].w};
+            unsigned o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 g = __half22float2(*reinterpret_cast<const __half2*>(&g4[e])), u = __half22float2(*reinterpret_cast<const __half2*>(&u4[e]));
+                const __half2 h = __floats2half2_rn(bpdq::silu_f32(g.x) * u.x, bpdq::silu_f32(g.y) * u.y);
+                o[e] = *reinterpret_cast<const unsigned*>(&h);
+            }
+            hout[i0 + k * step] = make_uint4(o[0], o[1], o[2], o[3]);
+        }
     }
 }
 
@@ -427,23 +461,45 @@ extern "C" int bpdq_launch_count(bpdq_handle_t h, uint64_t* count) {
 
 namespace bpdq {
 
+// Launch configuration of a small kernel between two large ones: it may be scheduled under the tail of the kernel before.
+struct PdlConfig {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    PdlConfig(unsigned grid, unsigned block, size_t smem, cudaStream_t stream) {
+        cfg.gridDim = dim3(grid); cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+    }
+};
+
 int launch_gather_columns(bpdq_handle_s* h, const void* x, int M, cudaStream_t stream) {
-    const long long items = (long long)M * (h->in / 8);
-    long long blocks = (items + 255) / 256;
-    if (blocks > 4LL * h->sm_count) blocks = 4LL * h->sm_count;
-    gather_columns_kernel<<<(unsigned)blocks, 256, 0, stream>>>(static_cast<const __half*>(x), h->d_perm, static_cast<__half*>(h->d_xperm), M, h->in);
-    const cudaError_t e = cudaGetLastError();
+    const size_t smem = (size_t)h->in * 2;
+    const bool staged = smem <= (size_t)h->smem_optin && smem <= 200 * 1024;
+    unsigned blocks = 4u * (unsigned)h->sm_count;
+    if ((long long)M < (long long)blocks) blocks = (unsigned)M;
+    static SmemOptin optin;
+    if (staged)
+        if (const int rc = ensure_smem_optin(gather_columns_kernel<true>, optin, h->device, (int)smem, "gather"); rc != BPDQ_OK) return rc;
+    PdlConfig c(blocks, 512, staged ? smem : 0, stream);
+    const __half* src = static_cast<const __half*>(x);
+    __half* dst = static_cast<__half*>(h->d_xperm);
+    const int* perm = h->d_perm;
+    cudaError_t e = staged ? cudaLaunchKernelEx(&c.cfg, gather_columns_kernel<true>, src, perm, dst, M, h->in)
+                           : cudaLaunchKernelEx(&c.cfg, gather_columns_kernel<false>, src, perm, dst, M, h->in);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(BPDQ_ERR_CUDA, "gather launch: %s", cudaGetErrorString(e));
     h->launches += 1;
     return BPDQ_OK;
 }
 
 int launch_swiglu(const void* gate, const void* up, void* hout, size_t n, cudaStream_t stream) {
-    const size_t n2 = n / 2;                                      // out is a multiple of 16: an even count
-    size_t blocks = (n2 + 255) / 256;
+    const size_t n8 = n / 8;                                      // out is a multiple of 16
+    size_t blocks = (n8 + 255) / 256;
     if (blocks > 1184) blocks = 1184;
-    swiglu_kernel<<<(unsigned)blocks, 256, 0, stream>>>(static_cast<const __half2*>(gate), static_cast<const __half2*>(up), static_cast<__half2*>(hout), n2);
-    const cudaError_t e = cudaGetLastError();
+    PdlConfig c((unsigned)blocks, 256, 0, stream);
+    cudaError_t e = cudaLaunchKernelEx(&c.cfg, swiglu_kernel, static_cast<const uint4*>(gate), static_cast<const uint4*>(up), static_cast<uint4*>(hout), n8);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(BPDQ_ERR_CUDA, "gated unit launch: %s", cudaGetErrorString(e));
     return BPDQ_OK;
 }

@@ -248,10 +248,18 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaS
     p.g.bias = static_cast<const __half*>(h->d_bias);
     const long long ntiles = (long long)nrt * ((M + 2 * p.half - 1) / (2 * p.half));
     const int grid = ntiles < h->sm_count ? (int)ntiles : h->sm_count;
-    gemm_wide_kernel<K, BKW><<<grid, kWideThreads, kWideSmem, stream>>>(map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
-                                                                  *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[1]), p);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kWideThreads); cfg.dynamicSmemBytes = kWideSmem; cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    // Short launches: SMs that the kernel before has left set up and fetch packed blocks.  Long ones run into the power limit,
+    // and CTAs that wait beside them cost more than the start they save (72B-shaped layer with 4096 tokens: 6.24 ms, 6.40 with).
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = ntiles <= 4LL * h->sm_count ? 1 : 0;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_wide_kernel<K, BKW>, map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
+                                       *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[1]), p);
     h->launches += 1;
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
     return BPDQ_OK;
 }

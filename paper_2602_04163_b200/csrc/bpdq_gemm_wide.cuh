@@ -105,12 +105,15 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // only now: a CTA of the next kernel that took this SM's TMEM first and then waited for this kernel would keep it
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned tmem_d = *tmem_slot;
 
     if (warp == 0) {
         // ---------------- x tiles of every stage ----------------
         // A thread needs 100 clocks or more per copy, so packed blocks have a producer of their own, and two halves of up to
         // 128 tokens come as one box.
+        asm volatile("griddepcontrol.wait;" ::: "memory");   // the kernel before this one may have written x
         if (elect_one()) {
             const int boxes = 2 * half <= 256 ? 1 : 2;
             int s = 0;                                   // stage slot, continuing across tiles
@@ -261,6 +264,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         const int rl = quad * 32 + lane;
         const unsigned taddr = tmem_d + ((unsigned)(quad * 32) << 16) + (unsigned)(h * 256);
         const size_t out = (size_t)p.out;
+        asm volatile("griddepcontrol.wait;" ::: "memory");   // ... or may still be reading what y overwrites
         int j = 0;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++j) {
             if (!mbar_wait_warp(acc_full, (unsigned)j & 1u, abort_flag, p.status)) break;

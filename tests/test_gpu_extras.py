@@ -159,3 +159,20 @@ def test_data_free_weights_through_every_kernel(K, g):
     y_q, _ = oracle.linear(bits, coef, x, g)
     y_w = x.view(np.float16).astype(np.float64) @ w.astype(np.float64).T
     assert np.sqrt(np.mean((y_q - y_w) ** 2)) < (0.45, 0.45, 0.25, 0.13)[K - 1] * np.sqrt(np.mean(y_w ** 2))
+
+
+@pytest.mark.parametrize("in_,M", [(128, 1), (1152, 700), (102400, 3), (102528, 130)])
+def test_permuted_rows_staged_and_not(in_, M):
+    """The gather ahead of the tensor-core kernels: rows up to the shared-memory limit (102400 columns) and beyond; a permuted
+    linear equals the plain one on permuted activations, bit for bit where one CTA sums a row."""
+    K, g, out = 2, 128, 16
+    h = binding.Handle(out, in_, K, g, None, 77, M)
+    x = synth.activations(78, M, in_)
+    perm = np.random.RandomState(79).permutation(in_).astype(np.int32)
+    want = G.run_linear(h, np.ascontiguousarray(x[:, perm]), binding.KERNEL_GEMM)
+    h.bpdq_set_input_permutation(perm)
+    got = G.run_linear(h, x, binding.KERNEL_GEMM)
+    if M > 128 or in_ < 2048:
+        assert np.array_equal(got, want)
+    else:
+        assert np.allclose(got, want, rtol=2.0 ** -9, atol=1e-4)
