@@ -13,7 +13,8 @@
 // delivers the last block of the two tiles applies the gated unit.
 //
 // Roles (768 threads): warp 0 packed blocks (TMA), warp 3 x tiles (TMA), warps 1 and 2 MMA issuers, four groups of four
-// decode warps (thread = row, groups take every fourth block), four epilogue warps.  One issuer needs about 500 clocks per
+// decode warps (thread = row, groups take every fourth block), four epilogue warps, which
+// the decode warps join for a CTA's last piece (nothing else is left to do then; with 100 tokens four warps took 12 us).  One issuer needs about 500 clocks per
 // block beside the decode warps that share its scheduler (two waits, eight instructions with their operands, a commit), so
 // blocks alternate between two, each with an accumulator of its own; up to 64 tokens there are two such pairs, and one is
 // drained while the other is being filled.  Rings, each with full / empty barriers: packed blocks, x tiles (one block: two
@@ -26,6 +27,7 @@ constexpr int kTsGroups = 4;
 constexpr int kTsDecodeWarps = 4 * kTsGroups, kTsFirstDecode = 4, kTsFirstEpi = kTsFirstDecode + kTsDecodeWarps;
 constexpr int kTsThreads = 32 * (kTsFirstEpi + 4);
 constexpr int kTsACols = 64 * kTsGroups;              // A slots: one per decode group
+constexpr int kTsJoint = 32 * (kTsDecodeWarps + 4);    // threads that drain a CTA's last piece
 constexpr int kTsSmem = 227 * 1024;
 constexpr int kTsMaxM = 128;
 constexpr int kTsMinCut = 16;                         // blocks per row from which tiles are shared between CTAs
@@ -87,6 +89,7 @@ template <int K> struct TsCfg {
     static constexpr int kSlotBytes = kPlaneBytes + 2 * kCoefBytes;
 };
 
+__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 __device__ __forceinline__ void umma_f16_ts(unsigned d, unsigned a, uint64_t bdesc, unsigned idesc, unsigned accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -123,7 +126,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_con
     const int nbars = 2 * NA + 4 + 2 * SX + 2 * SP;
     unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + bar_off + 8 * nbars);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    int* finish = reinterpret_cast<int*>(tmem_slot + 2);
+    volatile int* finish = reinterpret_cast<volatile int*>(tmem_slot + 2);
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int ng = p.ng;
@@ -150,6 +153,103 @@ __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_con
     const unsigned tmem = *tmem_slot, tmem_d = tmem + kTsACols;
     const unsigned quad_lanes = (unsigned)((warp & 3) * 32) << 16;     // TMEM lane quadrant this warp may access
 
+    // ---- a finished piece: thread = row.  A whole tile goes to y, a part of one (or of a pair) into the workspace.  `parts`
+    // sets of four warps share the token columns; this thread belongs to set `part` and is number et of all ----
+    auto drain = [&](const TsPiece& c, const int seq, const int buf, const bool ok, const int part, const int parts, const int et) {
+        // (local copies: the compiler would load launch parameters again behind every store)
+        const TsLinear& L = p.lin[c.li];
+        const int rl = (warp & 3) * 32 + lane, M = p.M, out = L.out, nblocks = L.nblocks;
+        float* const ws = L.ws;
+        float* const conv_b = L.conv_b;
+        __half* const y = L.y;
+        unsigned* const counter = L.counters + c.tile;
+        const bool whole = c.n == nblocks, pair = conv_b != nullptr;
+        const int row0 = c.tile * 128, r = row0 + rl;
+        const bool row_ok = r < out;
+        const float br = (whole && !pair && row_ok && L.bias_a) ? __half2float(L.bias_a[r]) : 0.f;
+        // a part of one block has one issuer's sum only: it is taken for both and halved (exactly)
+        const float half = c.n > 1 ? 1.f : 0.5f;
+        const unsigned d = tmem_d + quad_lanes + (unsigned)(2 * buf * p.dcols);
+        const unsigned d_first = c.n > 1 ? d : d + (unsigned)((seq & 1) * p.dcols), d_second = c.n > 1 ? d + (unsigned)p.dcols : d_first;
+        size_t at = (size_t)r + (size_t)(16 * part) * out;
+#pragma unroll 1
+        for (int c0 = 16 * part; c0 < N && ok; c0 += 16 * parts, at += (size_t)(16 * parts) * out) {
+            unsigned v[16], v2[16];
+            tmem_ld16(d_first + (unsigned)c0, v);
+            tmem_ld16(d_second + (unsigned)c0, v2);
+            tmem_ld_wait();
+            if (row_ok) {
+                const int nt = M - c0;                   // tokens left
+                float* wp = ws + at;
+                if (!whole) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j, wp += out)
+                        if (j < nt) asm volatile("red.global.add.f32 [%0], %1;" ::"l"(wp), "f"((__uint_as_float(v[j]) + __uint_as_float(v2[j])) * half));
+                } else if (pair) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j, wp += out)
+                        if (j < nt) __stcg(wp, (__uint_as_float(v[j]) + __uint_as_float(v2[j])) * half);
+                } else {
+                    __half* yp = y + at;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j, yp += out)
+                        if (j < nt) *yp = __float2half_rn((__uint_as_float(v[j]) + __uint_as_float(v2[j])) * half + br);
+                }
+            }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (parts == 1 && lane == 0) mbar_arrive(acc_empty + 8u * buf);   // (nothing follows the last piece)
+        if (!whole || pair) {
+            __threadfence();                             // this thread's parts are out before the tile's counter moves
+            bar_sync(1, 128 * parts);
+            if (et == 0) {
+                const unsigned before = atomicAdd(counter, (unsigned)c.n);
+                *finish = before + (unsigned)c.n == (unsigned)(pair ? 2 * nblocks : nblocks);
+                if (*finish) *counter = 0u;
+            }
+            bar_sync(1, 128 * parts);
+            if (*finish) {                               // the last part of the tile: finish it, write y, zero the workspace
+                __threadfence();
+                // a thread keeps its four rows and walks over the tokens
+                const int q = row0 + (et & 31) * 4;
+                float* const conv_a = const_cast<float*>(L.conv_a);
+                const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+                float4 ba = zero, bb = zero;
+                if (q < out && L.bias_a) ba = bpdq::bias_quad(L.bias_a, q);
+                if (q < out && L.bias_b) bb = bpdq::bias_quad(L.bias_b, q);
+                constexpr int kAhead = 4;
+                const int step = 4 * parts;
+                for (int t0 = et >> 5; q < out && t0 < M; t0 += step * kAhead) {
+                    float4 v[kAhead], vb[kAhead];
+#pragma unroll
+                    for (int e = 0; e < kAhead; ++e)
+                        if (t0 + step * e < M) {
+                            v[e] = __ldcg(reinterpret_cast<const float4*>(conv_a + (size_t)(t0 + step * e) * out + q));
+                            if (pair) vb[e] = __ldcg(reinterpret_cast<const float4*>(conv_b + (size_t)(t0 + step * e) * out + q));
+                        }
+#pragma unroll
+                    for (int e = 0; e < kAhead; ++e)
+                        if (t0 + step * e < M) {
+                            const size_t to = (size_t)(t0 + step * e) * out + q;
+                            float4 a = make_float4(v[e].x + ba.x, v[e].y + ba.y, v[e].z + ba.z, v[e].w + ba.w);
+                            if (pair) {
+                                a.x = bpdq::silu_f32(a.x) * (vb[e].x + bb.x); a.y = bpdq::silu_f32(a.y) * (vb[e].y + bb.y);
+                                a.z = bpdq::silu_f32(a.z) * (vb[e].z + bb.z); a.w = bpdq::silu_f32(a.w) * (vb[e].w + bb.w);
+                                __stcg(reinterpret_cast<float4*>(conv_b + to), zero);
+                            }
+                            const __half2 h01 = __floats2half2_rn(a.x, a.y), h23 = __floats2half2_rn(a.z, a.w);
+                            uint2 o;
+                            o.x = *reinterpret_cast<const unsigned*>(&h01);
+                            o.y = *reinterpret_cast<const unsigned*>(&h23);
+                            *reinterpret_cast<uint2*>(y + to) = o;
+                            __stcg(reinterpret_cast<float4*>(conv_a + to), zero);
+                        }
+                }
+            }
+            bar_sync(1, 128 * parts);                    // *finish has been read by all
+        }
+    };
     if (warp == 0) {
         // ---------------- packed blocks ----------------
         if (elect_one()) {
@@ -292,120 +392,43 @@ __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_con
                 if (++sl == SP) { sl = 0; ph ^= 1u; }
         }
     } else if (warp >= kTsFirstEpi) {
-        // ---------------- epilogue warps: thread = row; a whole tile goes to y, a part of one into the workspace ----------------
+        // ---------------- epilogue warps: every piece, the last one together with the decode warps ----------------
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        const int rl = (warp & 3) * 32 + lane, et = tid - 32 * kTsFirstEpi;
         int buf = 0, seq = 0;                            // seq: blocks before this piece
         unsigned pacc = 0u;
-        const int M = p.M;
-        while (ts_next(p, work, pc)) {
-            // (local copies: the compiler would load launch parameters again behind every store)
-            const TsLinear& L = p.lin[pc.li];
-            const int out = L.out, nblocks = L.nblocks;
-            float* const ws = L.ws;
-            float* const conv_b = L.conv_b;
-            __half* const y = L.y;
-            unsigned* const counter = L.counters + pc.tile;
-            const bool whole = pc.n == nblocks, pair = conv_b != nullptr;
-            const int row0 = pc.tile * 128, r = row0 + rl;
-            const bool row_ok = r < out;
-            const float br = (whole && !pair && row_ok && L.bias_a) ? __half2float(L.bias_a[r]) : 0.f;
-            // a part of one block has one issuer's sum only: it is taken for both and halved (exactly)
-            const float half = pc.n > 1 ? 1.f : 0.5f;
-            unsigned d = tmem_d + quad_lanes + (unsigned)(2 * buf * p.dcols);
-            const unsigned d_first = pc.n > 1 ? d : d + (unsigned)((seq & 1) * p.dcols), d_second = pc.n > 1 ? d + (unsigned)p.dcols : d_first;
+        bool more = ts_next(p, work, pc);
+        while (more) {
             const bool ok = mbar_wait_warp(acc_full + 8u * buf, pacc, abort_flag, p.status);
             tc_fence_after();
-            size_t at = (size_t)r;
-#pragma unroll 1
-            for (int c0 = 0; c0 < N && ok; c0 += 16, at += (size_t)16 * out) {
-                unsigned v[16], v2[16];
-                tmem_ld16(d_first + (unsigned)c0, v);
-                tmem_ld16(d_second + (unsigned)c0, v2);
-                tmem_ld_wait();
-                if (row_ok) {
-                    const int nt = M - c0;               // tokens left
-                    float* wp = ws + at;
-                    if (!whole) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j, wp += out)
-                            if (j < nt) asm volatile("red.global.add.f32 [%0], %1;" ::"l"(wp), "f"((__uint_as_float(v[j]) + __uint_as_float(v2[j])) * half));
-                    } else if (pair) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j, wp += out)
-                            if (j < nt) __stcg(wp, (__uint_as_float(v[j]) + __uint_as_float(v2[j])) * half);
-                    } else {
-                        __half* yp = y + at;
-#pragma unroll
-                        for (int j = 0; j < 16; ++j, yp += out)
-                            if (j < nt) *yp = __float2half_rn((__uint_as_float(v[j]) + __uint_as_float(v2[j])) * half + br);
-                    }
-                }
+            const TsPiece now = pc;
+            more = ts_next(p, work, pc);
+            if (!more) {
+                if (tid == 32 * kTsFirstEpi) *finish = ok;
+                tc_fence_before();
+                bar_sync(2, kTsJoint);
+                tc_fence_after();
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty + 8u * buf);
-            if (!whole || pair) {
-                __threadfence();                         // this thread's parts are out before the tile's counter moves
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (et == 0) {
-                    const unsigned before = atomicAdd(counter, (unsigned)pc.n);
-                    *finish = before + (unsigned)pc.n == (unsigned)(pair ? 2 * nblocks : nblocks);
-                    if (*finish) *counter = 0u;
-                }
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (*finish) {                           // the last part of the tile: finish it, write y, zero the workspace
-                    __threadfence();
-                    // a thread keeps its four rows and walks over the tokens
-                    const int q = row0 + (et & 31) * 4;
-                    float* const conv_a = const_cast<float*>(L.conv_a);
-                    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-                    float4 ba = zero, bb = zero;
-                    if (q < out && L.bias_a) ba = bpdq::bias_quad(L.bias_a, q);
-                    if (q < out && L.bias_b) bb = bpdq::bias_quad(L.bias_b, q);
-                    constexpr int kAhead = 8;
-                    for (int t0 = et >> 5; q < out && t0 < M; t0 += 4 * kAhead) {
-                        float4 v[kAhead];
-#pragma unroll
-                        for (int e = 0; e < kAhead; ++e)
-                            if (t0 + 4 * e < M) v[e] = __ldcg(reinterpret_cast<const float4*>(conv_a + (size_t)(t0 + 4 * e) * out + q));
-                        if (pair) {
-#pragma unroll
-                            for (int e0 = 0; e0 < kAhead; e0 += 4) {
-                                float4 vb[4];
-#pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    if (t0 + 4 * (e0 + e) < M) vb[e] = __ldcg(reinterpret_cast<const float4*>(conv_b + (size_t)(t0 + 4 * (e0 + e)) * out + q));
-#pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    if (t0 + 4 * (e0 + e) < M) {
-                                        float4& a = v[e0 + e];
-                                        a.x = bpdq::silu_f32(a.x + ba.x) * (vb[e].x + bb.x); a.y = bpdq::silu_f32(a.y + ba.y) * (vb[e].y + bb.y);
-                                        a.z = bpdq::silu_f32(a.z + ba.z) * (vb[e].z + bb.z); a.w = bpdq::silu_f32(a.w + ba.w) * (vb[e].w + bb.w);
-                                        __stcg(reinterpret_cast<float4*>(conv_b + (size_t)(t0 + 4 * (e0 + e)) * out + q), zero);
-                                    }
-                            }
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < kAhead; ++e) { v[e].x += ba.x; v[e].y += ba.y; v[e].z += ba.z; v[e].w += ba.w; }
-                        }
-#pragma unroll
-                        for (int e = 0; e < kAhead; ++e)
-                            if (t0 + 4 * e < M) {
-                                const size_t to = (size_t)(t0 + 4 * e) * out + q;
-                                const __half2 h01 = __floats2half2_rn(v[e].x, v[e].y), h23 = __floats2half2_rn(v[e].z, v[e].w);
-                                uint2 o;
-                                o.x = *reinterpret_cast<const unsigned*>(&h01);
-                                o.y = *reinterpret_cast<const unsigned*>(&h23);
-                                *reinterpret_cast<uint2*>(y + to) = o;
-                                __stcg(reinterpret_cast<float4*>(conv_a + to), zero);
-                            }
-                    }
-                }
-                asm volatile("bar.sync 1, 128;" ::: "memory");   // *finish has been read by all
-            }
+            drain(now, seq, buf, ok, more ? 0 : kTsGroups, more ? 1 : kTsGroups + 1, tid - 32 * (more ? kTsFirstEpi : kTsFirstDecode));
             if (++buf == p.nbuf) { buf = 0; pacc ^= 1u; }
-            seq += pc.n;
+            seq += now.n;
+        }
+    }
+    if (warp >= kTsFirstDecode && warp < kTsFirstEpi) {
+        // the last piece: the epilogue warps have waited for its sums (barrier 2), twenty warps read them
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        int buf = -1, seq = 0, n = 0;
+        TsPiece last = {0, 0, 0, 0};
+        while (ts_next(p, work, pc)) {
+            seq += n;
+            last = pc;
+            n = pc.n;
+            buf = buf + 1 == p.nbuf ? 0 : buf + 1;
+        }
+        if (n > 0) {
+            bar_sync(2, kTsJoint);
+            const bool ok = *finish != 0;
+            tc_fence_after();
+            drain(last, seq, buf, ok, (warp - kTsFirstDecode) >> 2, kTsGroups + 1, tid - 32 * kTsFirstDecode);
         }
     }
     tc_fence_before();
