@@ -160,11 +160,9 @@ int check_batch_handles(const bpdq_handle_t* hs, int n, int M, const char* who) 
     return M == 0 ? BPDQ_OK : check_device(hs[0], who);
 }
 
-// Whether a launch goes to the look-up-table kernel: up to the first linear's threshold, unless the tensor-core kernel is
-// the better one below it (and the caller has not set the threshold).
-bool prefer_lut(bpdq_handle_s* const* hs, int n, int M) {
-    return M <= hs[0]->gemv_max_m;
-}
+// Whether a launch goes to the look-up-table kernel: up to the first linear's threshold.  (Two tokens at K = 3, g = 64 are
+// faster through the tensor-core kernel, but it rounds the weights to binary16 and this one does not.)
+bool prefer_lut(bpdq_handle_s* const* hs, int M) { return M <= hs[0]->gemv_max_m; }
 
 }  // namespace
 
@@ -261,7 +259,7 @@ extern "C" int bpdq_linear_ex(bpdq_handle_t h, const void* x, void* y, int M, in
         const bool gv = gemv_supported(h->out, h->in, h->K, h->group);
         const bool gm = gemm_supported(h->out, h->in, h->K, h->group);
         const bool fw = gemv_mma_supported(h->out, h->in, h->K, h->group);
-        if (gv && (prefer_lut(&h, 1, M) || !gm) && M <= BPDQ_GEMV_MAX_M) kernel = BPDQ_KERNEL_GEMV;
+        if (gv && (prefer_lut(&h, M) || !gm) && M <= BPDQ_GEMV_MAX_M) kernel = BPDQ_KERNEL_GEMV;
         else if (fw && h->few_max_m && M <= h->few_max_m && M <= BPDQ_FEW_MAX_M) kernel = BPDQ_KERNEL_FEW;
         else if (gm) kernel = BPDQ_KERNEL_GEMM;
         else kernel = BPDQ_KERNEL_GEMV_SIMPLE;
@@ -305,7 +303,7 @@ extern "C" int bpdq_linear_batch(const bpdq_handle_t* hs, const void* const* xs,
             return set_error(BPDQ_ERR_INVALID, "bpdq_linear_batch: x and y of linear %d must be non-null and 16-byte aligned", k);
     // above the look-up-table threshold the tensor-core kernel (or the few-token kernel, if asked for) takes the whole batch,
     // when every linear allows it
-    bool gemm = !prefer_lut(hs, n, M);
+    bool gemm = !prefer_lut(hs, M);
     bool few = M > hs[0]->gemv_max_m && M <= hs[0]->few_max_m && M <= BPDQ_FEW_MAX_M;
     for (int k = 0; few && k < n; ++k)
         few = hs[k]->d_few_maps && gemv_mma_supported(hs[k]->out, hs[k]->in, hs[k]->K, hs[k]->group) &&
@@ -414,7 +412,6 @@ extern "C" int bpdq_set_gemv_max_m(bpdq_handle_t h, int max_gemv_m) {
     if (max_gemv_m < 0 || max_gemv_m > BPDQ_GEMV_MAX_M)
         return set_error(BPDQ_ERR_INVALID, "bpdq_set_gemv_max_m: %d outside [0, %d]", max_gemv_m, BPDQ_GEMV_MAX_M);
     h->gemv_max_m = max_gemv_m;
-    h->gemv_set = 1;
     return BPDQ_OK;
 }
 
@@ -574,7 +571,7 @@ extern "C" int bpdq_gate_up_swiglu(bpdq_handle_t hg, bpdq_handle_t hu, const voi
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     bpdq_handle_s* hs[2] = {hg, hu};
     const bool same_g64 = (hg->group == 64) == (hu->group == 64);
-    const bool lut = same_g64 && prefer_lut(hs, 2, M) && M <= BPDQ_GEMV_MAX_M && gemv_supported(hg->out, hg->in, hg->K, hg->group) &&
+    const bool lut = same_g64 && prefer_lut(hs, M) && M <= BPDQ_GEMV_MAX_M && gemv_supported(hg->out, hg->in, hg->K, hg->group) &&
                      gemv_supported(hu->out, hu->in, hu->K, hu->group);
     bool few = same_g64 && !lut && M <= hg->few_max_m && M <= BPDQ_FEW_MAX_M && hg->d_few_maps && hu->d_few_maps &&
                (size_t)M * hg->out * sizeof(float) <= hg->ws_bytes && (size_t)M * hu->out * sizeof(float) <= hu->ws_bytes;

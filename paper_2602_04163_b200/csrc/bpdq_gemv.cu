@@ -124,15 +124,6 @@ __device__ __forceinline__ unsigned short ldg_stream2(const uint8_t* p) {
 __device__ __forceinline__ void red_add(float* p, float v) {
     asm volatile("red.global.add.f32 [%0], %1;" :: "l"(p), "f"(v) : "memory");
 }
-// Table load.  Not volatile: its address is computed from plane bytes that were read after the
-// barrier that published the tables, so it cannot move above that barrier, and the compiler may
-// interleave the independent look-ups of a plane unit freely.
-template <int IMM>
-__device__ __forceinline__ float lds_table(unsigned addr) {
-    float v;
-    asm("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(addr), "n"(IMM));
-    return v;
-}
 // prmt.b32 in its generic form: selector nibble n picks byte n of {b, a} (a = bytes 0..3); with its top bit set
 // the byte's sign is replicated instead
 __device__ __forceinline__ unsigned prmt(unsigned a, unsigned b, unsigned sel) {
@@ -143,10 +134,8 @@ __device__ __forceinline__ unsigned prmt(unsigned a, unsigned b, unsigned sel) {
 __device__ __forceinline__ unsigned word_of(const uint4& v, int k) {
     return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w;
 }
-// A pair of binary32 accumulators in one 64-bit register: (lo, hi) += (a, b) as one packed add.
-__device__ __forceinline__ void add2(unsigned long long& acc, float a, float b) {
-    asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %2};\n\tadd.rn.f32x2 %0, %0, t;\n\t}" : "+l"(acc) : "f"(a), "f"(b));
-}
+// (Not volatile: addresses come from plane bytes that were read after the barrier that published the tables, so the loads
+// cannot move above it, and the compiler may interleave the independent look-ups of a plane unit freely.)
 // Two table look-ups and their packed add in one statement, so that the two loaded values are born as the
 // register pair the packed add reads (separate loads would each need a move into the pair).
 template <int IMM0, int IMM1>
@@ -157,16 +146,6 @@ __device__ __forceinline__ void lookup2_add(unsigned long long& acc, unsigned ad
         "mov.b64 t, {a, b};\n\t"
         "add.rn.f32x2 %0, %0, t;\n\t}"
         : "+l"(acc) : "r"(addr0), "r"(addr1), "n"(IMM0), "n"(IMM1));
-}
-// The same, and the two loaded values are handed back (g = 64 adds them to the first group's partial sums as well).
-template <int IMM0, int IMM1>
-__device__ __forceinline__ void lookup2v_add(unsigned long long& acc, unsigned addr0, unsigned addr1, float& a, float& b) {
-    asm("{\n\t.reg .b64 t;\n\t"
-        "ld.shared.f32 %1, [%3+%5];\n\t"
-        "ld.shared.f32 %2, [%4+%6];\n\t"
-        "mov.b64 t, {%1, %2};\n\t"
-        "add.rn.f32x2 %0, %0, t;\n\t}"
-        : "+l"(acc), "=&f"(a), "=&f"(b) : "r"(addr0), "r"(addr1), "n"(IMM0), "n"(IMM1));
 }
 __device__ __forceinline__ float2 unpack2(unsigned long long v) {
     float2 f;
@@ -219,15 +198,22 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
             const int s = 3 * j + e;
-            if (s < 16) slots[j] |= (4u * ((s + a) & 15) + 64u * h) << (8 * (e + 1));
+            // g = 64: the eight steps of each half stay in one 64-column half of the block, lanes a < 8 beginning with the
+            // first and the others with the second, so that the sixteen lanes still meet sixteen chunks at every step
+            const unsigned chunk = G64 ? ((s + a) & 7) + 8 * (((a >> 3) ^ (s >> 3)) & 1) : (s + a) & 15;
+            if (s < 16) slots[j] |= (4u * chunk + 64u * h) << (8 * (e + 1));
         }
     }
 #pragma unroll
     for (int j = 0; j < 6; ++j) asm volatile("" : "+r"(slots[j]));   // opaque: kept in registers instead of being recomputed at every use
-    // steps at which this lane's chunk (logical byte (s + a) mod 16) lies in the block's first 64 columns
-    unsigned lo_steps = 0;
+    // g = 64: that order takes physical byte s or (s + 8) mod 16 at step s; the bytes s < 8 that trade places with s + 8 are
+    // those with s + a mod 8 >= 8, masks of the unit's words 0 and 1
+    unsigned swap0 = 0u, swap1 = 0u;
 #pragma unroll
-    for (int s = 0; s < 16; ++s) lo_steps |= (((s + a) & 15) < 8 ? 1u : 0u) << s;
+    for (int e = 0; e < 4; ++e) {
+        swap0 |= (e + (a & 7) >= 8 ? 0xFFu : 0u) << (8 * e);
+        swap1 |= (4 + e + (a & 7) >= 8 ? 0xFFu : 0u) << (8 * e);
+    }
 
     // contiguous share of the concatenated (linear, slice, row group) task space, cut by the host
     const int bid = blockIdx.x;
@@ -459,11 +445,29 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                 unsigned long long acc[NP][2];
 #pragma unroll
                 for (int j = 0; j < NP; ++j) acc[j][0] = acc[j][1] = 0ull;
-                float held = 0.f;                     // odd stream count: the last stream pairs two steps
-                unsigned held_addr = 0u;
-                float Slo[NS];                        // g = 64: the part of every stream that falls into the block's first 64 columns
+                unsigned held_addr = 0u;              // odd stream count: the last stream pairs two steps
+                float Sfirst[NS];                     // g = 64: the sums of the first eight steps, i.e. of one half of the block
+                if constexpr (G64) {
 #pragma unroll
-                for (int j = 0; j < NS; ++j) Slo[j] = 0.f;
+                    for (int i = 0; i < K; ++i) {
+                        uint4& u = tk.pl[q][i];
+                        const unsigned x = u.x, y = u.y;
+                        u.x = (x & ~swap0) | (u.z & swap0); u.z = (u.z & ~swap0) | (x & swap0);
+                        u.y = (y & ~swap1) | (u.w & swap1); u.w = (u.w & ~swap1) | (y & swap1);
+                    }
+                }
+                auto sums = [&](float (&S)[NS]) {     // the accumulators' sums per stream
+#pragma unroll
+                    for (int j = 0; j < NS / 2; ++j) {
+                        const float2 e = unpack2(acc[j][0]), o = unpack2(acc[j][1]);
+                        S[2 * j] = e.x + o.x;
+                        S[2 * j + 1] = e.y + o.y;
+                    }
+                    if (NS & 1) {
+                        const float2 e = unpack2(acc[NP - 1][0]), o = unpack2(acc[NP - 1][1]);
+                        S[NS - 1] = (e.x + e.y) + (o.x + o.y);
+                    }
+                };
 #pragma unroll
                 for (int st = 0; st < 16; ++st) {
                     // address = slot address with the plane byte in bits 8..15
@@ -472,29 +476,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                     for (int i = 0; i < K; ++i)
                         addr[i] = prmt(word_of(tk.pl[q][i], st >> 2), slots[st / 3], 0xC400u | ((st & 3) << 4) | (5 + st % 3));   // the selector is a constant once the step loop is unrolled
                     constexpr int QI = 128;               // the block pair and the token's table go into the immediate
-                    if constexpr (G64) {
-                        // pairs as below (two planes of one token, or the two tokens of a plane); the loaded values also go, on
-                        // the steps of the block's first 64 columns, into the first group's partial sums
-                        const bool lo = ((lo_steps >> st) & 1u) != 0u;
-#pragma unroll
-                        for (int j = 0; j < NS / 2; ++j) {
-                            float va, vb;
-                            if constexpr (MT == 2) {
-                                if (q == 0) lookup2v_add<0, kTableBytes>(acc[j][st & 1], addr[j], addr[j], va, vb);
-                                else lookup2v_add<QI, kTableBytes + QI>(acc[j][st & 1], addr[j], addr[j], va, vb);
-                            } else {
-                                if (q == 0) lookup2v_add<0, 0>(acc[j][st & 1], addr[2 * j], addr[2 * j + 1], va, vb);
-                                else lookup2v_add<QI, QI>(acc[j][st & 1], addr[2 * j], addr[2 * j + 1], va, vb);
-                            }
-                            if (lo) { Slo[2 * j] += va; Slo[2 * j + 1] += vb; }
-                        }
-                        if (NS & 1) {                     // one token, odd K: the last plane pairs two consecutive steps
-                            const float vl = q == 0 ? lds_table<0>(addr[K - 1]) : lds_table<QI>(addr[K - 1]);
-                            if (lo) Slo[NS - 1] += vl;
-                            if ((st & 1) == 0) held = vl;
-                            else add2(acc[NP - 1][(st >> 1) & 1], held, vl);
-                        }
-                    } else if constexpr (MT == 2) {
+                    if constexpr (MT == 2) {
                         // pair = the two tokens of one plane: one address, two tables
 #pragma unroll
                         for (int i = 0; i < K; ++i) {
@@ -514,18 +496,16 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                             else lookup2_add<QI, QI>(acc[NP - 1][(st >> 1) & 1], held_addr, addr[K - 1]);
                         }
                     }
+                    if constexpr (G64) {
+                        if (st == 7) {
+                            sums(Sfirst);
+#pragma unroll
+                            for (int j = 0; j < NP; ++j) acc[j][0] = acc[j][1] = 0ull;
+                        }
+                    }
                 }
                 float S[NS];
-#pragma unroll
-                for (int j = 0; j < NS / 2; ++j) {
-                    const float2 e = unpack2(acc[j][0]), o = unpack2(acc[j][1]);
-                    S[2 * j] = e.x + o.x;
-                    S[2 * j + 1] = e.y + o.y;
-                }
-                if (NS & 1) {
-                    const float2 e = unpack2(acc[NP - 1][0]), o = unpack2(acc[NP - 1][1]);
-                    S[NS - 1] = (e.x + e.y) + (o.x + o.y);
-                }
+                sums(S);
                 const int blk = 2 * q + h;
                 if constexpr (G64) {
                     // swap with the pair's other lane: word = (even row, odd row) of one group; this lane's row is half a & 1
@@ -544,11 +524,10 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                         yacc[m] = fmaf(c0h, xsum[(m * kSliceBlocks + blk) * 2 + 1], fmaf(c0l, xsum[(m * kSliceBlocks + blk) * 2], yacc[m]));
 #pragma unroll
                     for (int i = 0; i < K; ++i) {
-                        const float cil = cl[i + 1];
-                        const float cih = ch[i + 1];
+                        const float c1 = (a & 8) ? ch[i + 1] : cl[i + 1], c2 = (a & 8) ? cl[i + 1] : ch[i + 1];   // of the half summed first, second
 #pragma unroll
                         for (int m = 0; m < MT; ++m)
-                            yacc[m] = fmaf(cih, S[i * MT + m] - Slo[i * MT + m], fmaf(cil, Slo[i * MT + m], yacc[m]));
+                            yacc[m] = fmaf(c2, S[i * MT + m], fmaf(c1, Sfirst[i * MT + m], yacc[m]));
                     }
                 } else {
                     const float c0 = __half2float(__ushort_as_half(tk.cf[q][0]));
