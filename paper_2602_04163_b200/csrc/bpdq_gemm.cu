@@ -29,6 +29,7 @@
 #include "bpdq_decode.cuh"
 #include "bpdq_tma.cuh"
 #include "bpdq_finish.cuh"
+#include "bpdq_rings.h"
 
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -131,7 +132,6 @@ int ensure_packed_maps(bpdq_handle_s* h, EncodeTiledFn enc) {
 // Up to 128 tokens: one or several linears (same K, all or none with group 64); pair: the gated unit of two.
 template <int K>
 int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair) {
-    using C = TsCfg<K>;
     static bpdq::SmemOptin optin;
     bpdq_handle_s* h0 = hs[0];
     if (kTsSmem > h0->smem_optin)
@@ -170,12 +170,9 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
         tiles += (h->out + BM - 1) / BM;
         if (units >= (1ll << 31)) return bpdq::set_error(BPDQ_ERR_UNSUPPORTED, "gemm: task space too large");
     }
-    // x ring: as many blocks as 128 KB hold (four to eight, an even number: a slot belongs to one issuer), the packed ring
-    // gets the rest (nine slots or more; a decode group is at most eight blocks ahead of the MMAs, see the kernel)
-    p.sx = 128 * 1024 / (p.cols * 256) / 2 * 2;
-    if (p.sx > 8) p.sx = 8;
-    p.sp = (kTsSmem - 3072 - p.sx * p.cols * 256) / C::kSlotBytes;
-    if (p.sp > 24) p.sp = 24;
+    const bpdq::TsRings rings = bpdq::ts_rings(K, p.cols);
+    p.sx = rings.sx;
+    p.sp = rings.sp;
     p.nbuf = p.cols <= 64 ? 2 : 1;
     p.dcols = p.cols <= 64 ? 64 : 128;
     // CTAs: at least eight blocks each when rows are cut (a share of a tile costs a tile of adds), else a tile each

@@ -19,16 +19,16 @@
 // blocks alternate between two, each with an accumulator of its own; up to 64 tokens there are two such pairs, and one is
 // drained while the other is being filled.  Rings, each with full / empty barriers: packed blocks, x tiles (one block: two
 // 64-column tiles of N rows), A slots (one block: 64 TMEM columns).  A wait by parity has to follow its barrier phase by
-// phase: A and x slots belong to one decode group and one issuer (ring lengths are multiples of their numbers); a packed
-// slot is waited on by different groups in turn, but the use before has landed by then, because a group only gets past its
-// A slot when the MMAs are within two rounds of the groups, and the ring is longer than that.  Bound: the pipe that executes byte-permutes, masks and
+// phase: A slots belong to one decode group and one issuer, x slots to one issuer; a packed slot is waited on by different
+// groups in turn, but its length is even, so that its blocks share an issuer (the argument is at ts_rings, bpdq_rings.h).
+// Bound: the pipe that executes byte-permutes, masks and
 // shifts (half rate): 220 to 300 of its instructions per lane and block.
-constexpr int kTsGroups = 4;
+using bpdq::kTsGroups;
+using bpdq::kTsSmem;
 constexpr int kTsDecodeWarps = 4 * kTsGroups, kTsFirstDecode = 4, kTsFirstEpi = kTsFirstDecode + kTsDecodeWarps;
 constexpr int kTsThreads = 32 * (kTsFirstEpi + 4);
 constexpr int kTsACols = 64 * kTsGroups;              // A slots: one per decode group
 constexpr int kTsJoint = 32 * (kTsDecodeWarps + 4);    // threads that drain a CTA's last piece
-constexpr int kTsSmem = 227 * 1024;
 constexpr int kTsMaxM = 128;
 constexpr int kTsMinCut = 16;                         // blocks per row from which tiles are shared between CTAs
 
@@ -85,8 +85,8 @@ __device__ __forceinline__ bool ts_next(const TsParams& p, TsPieces& w, TsPiece&
 }
 
 template <int K> struct TsCfg {
-    static constexpr int kPlaneBytes = K * 2048, kCoefBytes = (K + 1) * 256;
-    static constexpr int kSlotBytes = kPlaneBytes + 2 * kCoefBytes;
+    static constexpr int kPlaneBytes = bpdq::ts_plane_bytes(K), kCoefBytes = bpdq::ts_coef_bytes(K);
+    static constexpr int kSlotBytes = bpdq::ts_slot_bytes(K);
 };
 
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }

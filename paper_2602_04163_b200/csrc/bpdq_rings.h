@@ -1,0 +1,36 @@
+// Host-side lengths of the rings in shared memory that the tensor-core kernels' roles hand blocks round in (plain C++, no CUDA).
+#pragma once
+
+namespace bpdq {
+
+constexpr int kTsGroups = 4;                          // decode groups of the kernel for up to 128 tokens; they take blocks in turn
+constexpr int kTsIssuers = 2;                         // its MMA issuers; blocks alternate between them
+constexpr int kTsSmem = 227 * 1024;
+constexpr int kTsMaxSX = 8, kTsMaxSP = 24;
+
+constexpr int ts_plane_bytes(int K) { return K * 2048; }
+constexpr int ts_coef_bytes(int K) { return (K + 1) * 256; }
+constexpr int ts_slot_bytes(int K) { return ts_plane_bytes(K) + 2 * ts_coef_bytes(K); }
+
+struct TsRings {
+    int sx, sp;                                       // slots of the x ring and of the packed ring
+};
+
+// `cols` token columns (a multiple of 16, at most 128).  The x ring takes as many blocks as 128 KB hold, four to eight, the
+// packed ring the rest of shared memory, eight slots or more.
+//
+// Both lengths are even.  A wait by parity is right only if the barrier's phase before the awaited one is over when the wait
+// begins; else it passes at once.  x slots: with an even length a slot belongs to one issuer, which has waited for every use of
+// it.  Packed slots: the group that waits for block q has seen its A slot free for block q - 4, so the MMAs of block q - 8 are
+// complete, and with them, in the order of its commits, every earlier block of THAT issuer: q - 8, q - 10, ...  With an even
+// length of at least eight the slot's last use, block q - sp, is among them, so its copy has landed.  With an odd one it
+// belongs to the other issuer, which may be any way behind when that block's copy is late (9 slots at K = 4 with 128 tokens).
+constexpr TsRings ts_rings(int K, int cols) {
+    int sx = 128 * 1024 / (cols * 256) / 2 * 2;
+    if (sx > kTsMaxSX) sx = kTsMaxSX;
+    int sp = (kTsSmem - 3072 - sx * cols * 256) / ts_slot_bytes(K) / 2 * 2;   // 3072: alignment slack, barriers
+    if (sp > kTsMaxSP) sp = kTsMaxSP;
+    return {sx, sp};
+}
+
+}  // namespace bpdq

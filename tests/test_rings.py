@@ -1,0 +1,111 @@
+"""Host logic of the tensor-core kernels: lengths of the rings that their roles hand blocks round in (csrc/bpdq_rings.h).
+
+A role that waits on an mbarrier by parity is let through at once when the barrier's phase BEFORE the awaited one is still
+open.  So for every wait that phase has to be over, by what the waiting role has itself waited for, whatever the copies' and the
+other roles' delays.  The kernels' order constraints are laid out as a graph, and the end of the phase before must be reachable
+from every wait; a copy may land arbitrarily late, also later than copies that were requested after it."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+HEADER_DIR = os.path.join(ROOT, "paper_2602_04163_b200", "csrc")
+
+DRIVER = r"""
+#include <cstdio>
+#include "bpdq_rings.h"
+int main() {
+    for (int K = 1; K <= 4; ++K)
+        for (int cols = 16; cols <= 128; cols += 16) {
+            const bpdq::TsRings r = bpdq::ts_rings(K, cols);
+            printf("ts %d %d %d %d %d\n", K, cols, r.sx, r.sp, bpdq::kTsSmem - r.sx * cols * 256 - r.sp * bpdq::ts_slot_bytes(K));
+        }
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rings(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rings")
+    src, exe = d / "driver.cpp", d / "driver"
+    src.write_text(DRIVER)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", HEADER_DIR, str(src), "-o", str(exe)], check=True)
+    rows = [line.split() for line in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.splitlines()]
+    return [(r[0], [int(v) for v in r[1:]]) for r in rows]
+
+
+class Order:
+    """Events with what must have happened before them; waits with the event that ends the phase before the awaited one."""
+
+    def __init__(self):
+        self.before, self.waits = {}, []
+
+    def event(self, name, *after):
+        self.before[name] = {a for a in after if a is not None}
+
+    def wait(self, role, after, previous):
+        """`role` begins to wait once `after` has happened; `previous` must be over then."""
+        self.waits.append((role, after, previous))
+
+    def _happened(self, name):
+        seen, todo = set(), [name]
+        while todo:
+            e = todo.pop()
+            if e in seen or e is None:
+                continue
+            seen.add(e)
+            todo += self.before[e]
+        return seen
+
+    def open_waits(self):
+        return [(role, previous) for role, after, previous in self.waits
+                if previous in self.before and (after is None or previous not in self._happened(after))]
+
+
+def ts_order(sx, sp, blocks, groups=4, issuers=2):
+    """gemm_ts_kernel: packed producer, x producer, decode groups (group q mod 4 takes block q), issuers (issuer q mod 2)."""
+    o = Order()
+
+    def ev(kind, q):
+        return (kind, q) if q >= 0 else None
+    for q in range(blocks):
+        # producers: one thread each, in block order; a slot is free once the block before in it has been decoded / multiplied
+        o.event(("packed asked", q), ev("packed asked", q - 1), ev("decoded", q - sp))
+        o.wait("packed producer", ev("packed asked", q - 1), ev("decoded", q - 2 * sp))
+        o.event(("packed landed", q), ("packed asked", q))
+        o.event(("x asked", q), ev("x asked", q - 1), ev("multiplied", q - sx))
+        o.wait("x producer", ev("x asked", q - 1), ev("multiplied", q - 2 * sx))
+        o.event(("x landed", q), ("x asked", q))
+        # a group: waits for the packed block, decodes into registers, waits for its A slot, stores and arrives
+        o.wait("group, packed", ev("decoded", q - groups), ev("packed landed", q - sp))
+        o.wait("group, A slot", ev("decoded", q - groups), ev("multiplied", q - 2 * groups))
+        o.event(("decoded", q), ev("decoded", q - groups), ("packed landed", q), ev("multiplied", q - groups))
+        # an issuer: waits for x, then for the A slot; its commits complete in order
+        o.wait("issuer, x", ev("issued", q - issuers), ev("x landed", q - sx))
+        o.wait("issuer, A slot", ev("issued", q - issuers), ev("decoded", q - groups))
+        o.event(("issued", q), ev("issued", q - issuers), ("x landed", q), ("decoded", q))
+        o.event(("multiplied", q), ("issued", q), ev("multiplied", q - issuers))
+    return o
+
+
+def test_rings_up_to_128_tokens(rings):
+    """Every K and number of token columns: no wait can pass by a phase that is still open, and the rings fit shared memory."""
+    seen = 0
+    for kind, r in rings:
+        if kind != "ts":
+            continue
+        K, cols, sx, sp, left = r
+        seen += 1
+        assert left >= 1024 + 8 * (2 * 4 + 4 + 2 * sx + 2 * sp) + 16, r      # alignment slack, barriers, TMEM address and flags
+        assert 4 <= sx <= 8 and 8 <= sp <= 24, r
+        assert ts_order(sx, sp, 2 * sp + 40).open_waits() == [], r
+    assert seen == 32
+
+
+def test_the_order_model_sees_an_odd_ring():
+    """The model itself: nine packed slots beside four of x (K = 4 with 128 tokens, were the length not rounded) leave a group's
+    wait for its packed block open."""
+    assert {role for role, _ in ts_order(4, 9, 60).open_waits()} == {"group, packed"}
+    assert ts_order(8, 23, 100).open_waits() == []           # an odd ring that the x ring covers
