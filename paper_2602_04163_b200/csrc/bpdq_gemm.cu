@@ -147,6 +147,8 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
     bool same = true;                                    // rows of one length
     for (int k = 0; k < n; ++k) {
         const bpdq_handle_s* h = hs[k];
+        if (!h->d_few_maps)
+            return bpdq::set_error(BPDQ_ERR_UNSUPPORTED, "gemm: linear %d has no tensor maps (the driver did not offer cuTensorMapEncodeTiled)", k);
         TsLinear& L = p.lin[k];
         const cuuint64_t dims[2] = {(cuuint64_t)h->in, (cuuint64_t)M};
         const cuuint64_t strides[1] = {(cuuint64_t)h->in * 2};
@@ -293,22 +295,6 @@ int launch_wait_limit_probe(bpdq_handle_s* h, cudaStream_t stream) {
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(BPDQ_ERR_CUDA, "probe launch: %s", cudaGetErrorString(e));
     return BPDQ_OK;
-}
-
-EncodeTiledFn encode_tiled_fn() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void* ptr = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(ptr);
-        else
-            cudaGetLastError();
-    }
-    return fn;
 }
 
 bool gemm_supported(int, int, int K, int group) {
