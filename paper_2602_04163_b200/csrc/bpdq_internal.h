@@ -2,6 +2,7 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <mutex>
 #include <cuda_runtime.h>
 
 #include "bpdq.h"
@@ -34,16 +35,22 @@ bool shape_supported(int out, int in, int K, int group);
 int set_error(int code, const char* fmt, ...);
 
 // Opt-in to more than 48 KB of dynamic shared memory is a per-device attribute of a kernel: one record per kernel
-// instantiation, indexed by device ordinal.  Setting the attribute twice is harmless, so concurrent first calls
-// need no lock; the record only saves the runtime call on later launches.
+// instantiation, indexed by device ordinal; it saves the runtime call on later launches.  Launches of one kernel may ask for
+// different sizes from different threads (the gather's rows): attribute and record move together under a lock and only grow.
 constexpr int kMaxDevices = 64;
 struct SmemOptin {
     int bytes[kMaxDevices];       // largest size opted in to on each device so far (zero-initialised as a static)
 };
+inline std::mutex& smem_optin_mutex() {
+    static std::mutex m;
+    return m;
+}
 template <typename Kernel>
 inline int ensure_smem_optin(Kernel kernel, SmemOptin& rec, int device, int bytes, const char* who) {
     if (device < 0 || device >= kMaxDevices) return set_error(BPDQ_ERR_UNSUPPORTED, "%s: device ordinal %d", who, device);
     if (__atomic_load_n(&rec.bytes[device], __ATOMIC_ACQUIRE) >= bytes) return BPDQ_OK;
+    const std::lock_guard<std::mutex> lock(smem_optin_mutex());
+    if (rec.bytes[device] >= bytes) return BPDQ_OK;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return set_error(BPDQ_ERR_CUDA, "%s: shared memory opt-in: %s", who, cudaGetErrorString(e));
     __atomic_store_n(&rec.bytes[device], bytes, __ATOMIC_RELEASE);
