@@ -250,7 +250,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 __syncwarp();
                 if (lane == 0) {
                     mbar_arrive(full(s));                // one arrival per warp, after all its lanes' stores and fences
-                    if (st == (ng - 1) * (kPerBlock / 2)) mbar_arrive(empty_p(sp));   // a stored stage has used the last loads from the packed slot: it may be refilled
+                    if (st == bpdq::wide_release_stage(kPerBlock)) mbar_arrive(empty_p(sp));   // stored stages have used everything loaded from the packed slot
                 }
                 advance(1);
             }

@@ -33,4 +33,10 @@ constexpr TsRings ts_rings(int K, int cols) {
     return {sx, sp};
 }
 
+// Prefill kernel: the stage of a 128-column block (of four 32-column or two 64-column ones) behind which a decode group gives the
+// block's packed slot back.  A refill does not queue behind loads that are still out, so every loaded word has to have gone into
+// a stored stage: column word q is put together from physical words q and q - 1 (mod 4), so the stage that holds word 2 is the
+// first by which all four are used; it also builds the tables of the second coefficient group of g = 64.
+constexpr int wide_release_stage(int stages_per_block) { return stages_per_block / 2; }
+
 }  // namespace bpdq

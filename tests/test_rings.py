@@ -21,6 +21,7 @@ int main() {
             const bpdq::TsRings r = bpdq::ts_rings(K, cols);
             printf("ts %d %d %d %d %d\n", K, cols, r.sx, r.sp, bpdq::kTsSmem - r.sx * cols * 256 - r.sp * bpdq::ts_slot_bytes(K));
         }
+    printf("release %d %d\n", bpdq::wide_release_stage(4), bpdq::wide_release_stage(2));
     return 0;
 }
 """
@@ -109,3 +110,18 @@ def test_the_order_model_sees_an_odd_ring():
     wait for its packed block open."""
     assert {role for role, _ in ts_order(4, 9, 60).open_waits()} == {"group, packed"}
     assert ts_order(8, 23, 100).open_waits() == []           # an odd ring that the x ring covers
+
+
+def test_prefill_slots_are_given_back_after_the_last_use(rings):
+    """The stage behind which a decode group of the prefill kernel gives a packed slot back: by then every plane word and every
+    coefficient group that it has loaded is part of a stored stage, for both stage widths and for one or two groups per block."""
+    (release,) = [r for kind, r in rings if kind == "release"]
+    for stages, at in zip((4, 2), release):
+        words = 4 // stages                                   # 32-column words per stage
+        for groups in (1, 2):
+            need = {("plane", k) for k in range(4)} | {("coefficients", c) for c in range(groups)}
+            for st in range(at + 1):
+                for q in range(st * words, (st + 1) * words):
+                    need -= {("plane", q), ("plane", (q + 3) % 4), ("coefficients", q // 2 if groups == 2 else 0)}
+            assert not need, (stages, groups, need)
+        assert at < stages
