@@ -208,7 +208,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         bool ok = true;
         const long long nbseq = (long long)my_tiles * nblk;
         for (long long bseq = grp; bseq < nbseq && ok; bseq += kWideGroups) {
-            if (!mbar_wait(full_p(sp), pp, abort_flag, p.status)) break;
+            if (!mbar_wait_warp(full_p(sp), pp, abort_flag, p.status)) break;
             const unsigned so = (unsigned)(sp * C::kBlockBytes);
             unsigned a[K][4];
 #pragma unroll
@@ -240,7 +240,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 #pragma unroll
                     for (int u = 0; u < 4; ++u) v8[4 * e + u] = bpdq::decode8<K>(sel[u], tab);
                 }
-                if (!mbar_wait(empty(s), ph, abort_flag, p.status)) { ok = false; break; }
+                if (!mbar_wait_warp(empty(s), ph, abort_flag, p.status)) { ok = false; break; }
                 const unsigned dst = st_base + (unsigned)s * stage;
 #pragma unroll
                 for (int ch = 0; ch < BKW / 8; ++ch)

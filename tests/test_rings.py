@@ -4,7 +4,9 @@ A role that waits on an mbarrier by parity is let through at once when the barri
 open.  So for every wait that phase has to be over, by what the waiting role has itself waited for, whatever the copies' and the
 other roles' delays.  The kernels' order constraints are laid out as a graph, and the end of the phase before must be reachable
 from every wait; a copy may land arbitrarily late, also later than copies that were requested after it."""
+import glob
 import os
+import re
 import subprocess
 
 import pytest
@@ -125,3 +127,37 @@ def test_prefill_slots_are_given_back_after_the_last_use(rings):
                     need -= {("plane", q), ("plane", (q + 3) % 4), ("coefficients", q // 2 if groups == 2 else 0)}
             assert not need, (stages, groups, need)
         assert at < stages
+
+
+def guarded_waits(text):
+    """(line, inside a block that one thread runs) for every per-thread wait whose answer decides what the thread does next."""
+    text = re.sub(r"//[^\n]*", "", text)
+    headers, at, found = [], 0, []
+    for m in re.finditer(r"[;{}]|\bmbar_wait\(", text):
+        if m.group() == "{":
+            headers.append(text[at:m.start()])
+        elif m.group() == "}":
+            headers.pop()
+        elif m.group() != ";":
+            statement = text[at:m.start()].strip()
+            if re.sub(r"[\w]+::", "", statement):          # a bare call's answer goes nowhere
+                one = any(re.search(r"elect_one\(\)|threadIdx\.x == 0|\blane == 0", h) for h in headers)
+                found.append((text.count("\n", 0, m.start()) + 1, one))
+            continue
+        at = m.end()
+    return found
+
+
+def test_warps_leave_a_wait_together():
+    """A bounded wait that ran out ends the role that waited.  Lanes that each decide for themselves may part there, some at the CTA's
+    last barrier and some in a warp-wide instruction, for good: code that a whole warp runs uses mbar_wait_warp (one answer for all
+    lanes), the per-thread wait stands only where a single thread runs."""
+    seen = 0
+    for path in glob.glob(os.path.join(HEADER_DIR, "*.cu*")):
+        if path.endswith("bpdq_tma.cuh"):
+            continue                                        # where the waits are defined
+        with open(path) as f:
+            for line, one in guarded_waits(f.read()):
+                assert one, f"{os.path.basename(path)}:{line}: a wait that lanes leave one by one"
+                seen += 1
+    assert seen >= 6
