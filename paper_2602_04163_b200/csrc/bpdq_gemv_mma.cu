@@ -180,6 +180,14 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_mma_kernel(const __grid_consta
         }
     };
 
+    // ... once every lane has read it.  The copies do not queue behind loads that are still out: each lane's loads come before
+    // them by its proxy fence.
+    auto refill = [&](const MmaLinear& L, const int rg, const int s) {
+        bpdq::tma::fence_proxy_async();
+        __syncwarp();
+        issue_task(L, rg, s);
+    };
+
     // ---- hand-over of a finished segment (its atomic adds are fenced, the CTA has passed a barrier) ----
     auto hand_over = [&](const MmaLinear& L, const int rg_begin, const int rg_end, const int nsl) {
         const int ck_begin = rg_begin / kChunkRgs, ck_end = (rg_end + kChunkRgs - 1) / kChunkRgs;
@@ -272,7 +280,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_mma_kernel(const __grid_consta
             asm volatile("griddepcontrol.wait;" ::: "memory");
             dep_waited = true;
         }
-        if (!early && q_begin < q_end) issue_task(L, rg, s_begin + sl);
+        if (!early && q_begin < q_end) refill(L, rg, s_begin + sl);
 
         // ---- stage the segment's activations as A fragments ----
         // item = (token tile and slice msl, 8-column chunk q8, token m_lo, block bt): sixteen bytes of x become four
@@ -363,8 +371,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_mma_kernel(const __grid_consta
                 tables_of(j, 0, tab[j]);
                 if (G64) tables_of(j, 1, tab2[G64 ? j : 0]);
             }
-            __syncwarp();                                            // every lane has read the landing area: it may be refilled
-            if (more) issue_task(L, rg, s_begin + sl);               // (rg, sl) already name the task after this one
+            if (more) refill(L, rg, s_begin + sl);                   // (rg, sl) already name the task after this one
 
             const unsigned xs = xs0 + (unsigned)sl_now * (32u * 512u) + (unsigned)lane * 16u;
 #pragma unroll
@@ -444,8 +451,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_mma_kernel(const __grid_consta
                     }
                 }
             }
-            __syncwarp();
-            if (more) issue_task(L, rg, s_begin + sl);
+            if (more) refill(L, rg, s_begin + sl);
         };
         for (int q = q_begin; q < q_end; ++q) {
             const int rg_now = rg, sl_now = sl;

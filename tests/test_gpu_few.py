@@ -112,3 +112,19 @@ def test_dispatcher_with_sixteen_candidates(g):
         passes = (M + 1) // 2 if M <= lut_max else 1      # the look-up-table kernel takes two tokens per pass
         assert h.bpdq_launch_count() - n0 == passes
     h.bpdq_destroy()
+
+
+@pytest.mark.parametrize("K,g,M", [(2, 128, 16), (4, 64, 9), (3, 128, 32)])
+def test_few_token_landing_areas_under_load(K, g, M):
+    """A layer that keeps every warp refilling its landing area, several launches: a copy that overtook the loads from the area would
+    show as rows off by a task's worth of columns.  Weights from bpdq_dequant, sums in binary32."""
+    import torch
+    out, in_ = 18944, 3584
+    h = binding.Handle(out, in_, K, g, None, 17, M)
+    x = synth.activations(18, M, in_)
+    w = torch.from_numpy(G.run_dequant(h).view(np.float16)).cuda().float()
+    ref = (G.x_tensor(x).float() @ w.T).cpu().numpy()
+    for _ in range(8):
+        y = G.run_linear(h, x, binding.KERNEL_FEW)
+        # binary16 rounding of the result (2^-11) and binary32 sums of 3584 terms of size up to 0.2 in another order
+        assert np.all(np.abs(y - ref) <= 2.0 ** -10 * np.abs(ref) + 2e-3)

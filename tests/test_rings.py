@@ -161,3 +161,13 @@ def test_warps_leave_a_wait_together():
                 assert one, f"{os.path.basename(path)}:{line}: a wait that lanes leave one by one"
                 seen += 1
     assert seen >= 6
+
+
+def test_landing_areas_are_refilled_behind_a_fence():
+    """The few-token kernel's warps copy the next task over the one they have just loaded: every copy but a warp's very first is asked
+    for behind a proxy fence of all its lanes."""
+    with open(os.path.join(HEADER_DIR, "bpdq_gemv_mma.cu")) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    calls = re.findall(r"([^;{}]*)\bissue_task\(", text)
+    assert len(calls) == 2 and sum("early &&" in c for c in calls) == 1       # the first copy, and the one in refill
+    assert re.search(r"auto refill = [^;]*\{\s*bpdq::tma::fence_proxy_async\(\);\s*__syncwarp\(\);\s*issue_task\(", text)
