@@ -170,8 +170,9 @@ BPDQ_API int bpdq_linear_ex(bpdq_handle_t h, const void* x_fp16_dev, void* y_fp1
 /* Several independent linears in one launch (decode: q, k, v of one token, or gate and up, or a
  * whole layer's linears when their inputs do not depend on each other).  y[k] = x[k] * W^[k]^T
  * for k = 0..n-1, each as bpdq_linear computes it for this M: the look-up-table kernel up to the
- * first handle's look-up-table threshold, the tensor-core kernel above it (the few-token kernel up to
- * its threshold where that is set); the task spaces of the
+ * first handle's look-up-table threshold, the tensor-core kernel above it.  Where bpdq_set_few_max_m has
+ * been called on the first handle: the few-token kernel up to that threshold and passes of the
+ * look-up-table kernel, which does not round the weights to binary16, above it.  The task spaces of the
  * n linears are concatenated, so launch ramp, set-up and tail are paid once instead of n times.  hs, xs, ys are HOST arrays of n
  * handles / device pointers (read before the call returns); 1 <= n <= BPDQ_BATCH_MAX; the
  * handles are distinct, live on the current device, share K, and either all or none of them
@@ -255,7 +256,8 @@ BPDQ_API int bpdq_gate_up_swiglu(bpdq_handle_t gate, bpdq_handle_t up, const voi
 BPDQ_API int bpdq_set_gemv_max_m(bpdq_handle_t h, int max_gemv_m);
 
 /* Sets the largest M that bpdq_linear sends to the few-token kernel once M is above the look-up-table
- * threshold (0 = never, the default; at most BPDQ_FEW_MAX_M and the handle's max_M). */
+ * threshold (0 = never, the default; at most BPDQ_FEW_MAX_M and the handle's max_M).  A call, with 0 too,
+ * also has bpdq_linear_batch take look-up-table passes above this threshold (see there). */
 BPDQ_API int bpdq_set_few_max_m(bpdq_handle_t h, int max_few_m);
 
 /* Copies the device blob back to host memory (bpdq_packed_bytes() bytes); synchronises. */

@@ -302,8 +302,9 @@ extern "C" int bpdq_linear_batch(const bpdq_handle_t* hs, const void* const* xs,
         if (!xs[k] || !ys[k] || !aligned16(xs[k]) || !aligned16(ys[k]))
             return set_error(BPDQ_ERR_INVALID, "bpdq_linear_batch: x and y of linear %d must be non-null and 16-byte aligned", k);
     // above the look-up-table threshold the tensor-core kernel (or the few-token kernel, if asked for) takes the whole batch,
-    // when every linear allows it
-    bool gemm = !prefer_lut(hs, M);
+    // when every linear allows it.  A caller who has set the few-token threshold has also set where the rounding of weights to
+    // binary16 ends: above it come passes of the look-up-table kernel, which does not round them.
+    bool gemm = !prefer_lut(hs, M) && !hs[0]->few_set;
     bool few = M > hs[0]->gemv_max_m && M <= hs[0]->few_max_m && M <= BPDQ_FEW_MAX_M;
     for (int k = 0; few && k < n; ++k)
         few = hs[k]->d_few_maps && gemv_mma_supported(hs[k]->out, hs[k]->in, hs[k]->K, hs[k]->group) &&
@@ -420,6 +421,7 @@ extern "C" int bpdq_set_few_max_m(bpdq_handle_t h, int max_few_m) {
     if (max_few_m < 0 || max_few_m > BPDQ_FEW_MAX_M)
         return set_error(BPDQ_ERR_INVALID, "bpdq_set_few_max_m: %d outside [0, %d]", max_few_m, BPDQ_FEW_MAX_M);
     h->few_max_m = max_few_m;
+    h->few_set = 1;
     return BPDQ_OK;
 }
 

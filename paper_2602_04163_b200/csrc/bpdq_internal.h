@@ -86,6 +86,7 @@ struct bpdq_handle_s {
     int gemv_max_m;
     uint64_t launches;
     int few_max_m;            // largest M the dispatcher sends to the few-token kernel
+    int few_set;              // the caller chose it (bpdq_set_few_max_m)
     void* d_few_maps;         // device copy of two tensor maps of the few-token kernel and two of the tensor-core kernel for up to 128 tokens (null: not available)
     int* d_perm;              // input-channel permutation: stored column j multiplies x[perm[j]] (null: identity)
     void* d_xperm;            // [max_M][in] gathered activations for the kernels that do not fold the permutation into their loads

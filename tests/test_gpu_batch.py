@@ -151,3 +151,21 @@ def test_single_host_call(M):
     yh = torch.full((M, out), float("nan"), dtype=torch.float16).pin_memory()
     h.bpdq_linear_host(xh.data_ptr(), yh.data_ptr(), M, G.stream_ptr())
     assert np.allclose(yh.numpy().astype(np.float64), want.astype(np.float64), rtol=2.0 ** -9, atol=1e-5)
+
+
+@pytest.mark.parametrize("few,M", [(0, 4), (0, 16), (8, 9)])
+def test_batch_above_a_chosen_few_token_threshold_does_not_round_the_weights(few, M):
+    """A caller who has set the few-token threshold gets look-up-table passes (two tokens each) above it, bit for bit: rows of one
+    512-column slice are summed by one CTA.  By default the batch goes to the tensor-core kernel, whose weights are binary16."""
+    K, g = 2, 128
+    layers = [G.make_layer(300 + k, o, 512, K, g, max_M=M) for k, o in enumerate((160, 272))]
+    handles = [L[0] for L in layers]
+    xs = [synth.activations(310 + k, M, 512) for k in range(2)]
+    rounded = _run_batch(handles, xs, M)
+    handles[0].bpdq_set_few_max_m(few)
+    n0 = handles[0].bpdq_launch_count()
+    ys = _run_batch(handles, xs, M)
+    assert handles[0].bpdq_launch_count() == n0 + (M + 1) // 2
+    for h, x, y, r in zip(handles, xs, ys, rounded):
+        assert np.array_equal(y, G.run_linear(h, x, binding.KERNEL_GEMV))
+        assert not np.array_equal(y, r)
