@@ -177,17 +177,11 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
     p.sp = rings.sp;
     p.nbuf = p.cols <= 64 ? 2 : 1;
     p.dcols = p.cols <= 64 ? 64 : 128;
-    // CTAs: at least eight blocks each when rows are cut (a share of a tile costs a tile of adds), else a tile each
-    const bool cut = !same || p.lin[0].nblocks >= kTsMinCut;
-    const long long most = cut ? (units + 7) / 8 : tiles;
-    const int grid = most < h0->sm_count ? (int)most : h0->sm_count;
+    const bpdq::TsSplit w = bpdq::ts_split((int)tiles, (int)units, same ? p.lin[0].nblocks : 0, h0->sm_count);
     p.nb0 = p.lin[0].nblocks;
-    p.whole = same ? (int)(tiles / grid) : 0;
-    p.cut_begin = p.whole * grid * p.nb0;
-    p.cut_units = (int)units - p.cut_begin;
-    p.cut_step = cut ? 1 : p.nb0;
+    p.whole = w.whole; p.cut_begin = w.cut_begin; p.cut_units = w.cut_units; p.cut_step = w.cut_step;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kTsThreads); cfg.dynamicSmemBytes = kTsSmem; cfg.stream = stream;
+    cfg.gridDim = dim3(w.grid); cfg.blockDim = dim3(kTsThreads); cfg.dynamicSmemBytes = kTsSmem; cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the first packed blocks are requested under the tail of the kernel before
     attr[0].val.programmaticStreamSerializationAllowed = 1;

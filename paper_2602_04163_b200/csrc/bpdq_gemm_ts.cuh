@@ -30,7 +30,6 @@ constexpr int kTsThreads = 32 * (kTsFirstEpi + 4);
 constexpr int kTsACols = 64 * kTsGroups;              // A slots: one per decode group
 constexpr int kTsJoint = 32 * (kTsDecodeWarps + 4);    // threads that drain a CTA's last piece
 constexpr int kTsMaxM = 128;
-constexpr int kTsMinCut = 16;                         // blocks per row from which tiles are shared between CTAs
 
 struct TsLinear {
     CUtensorMap x_map;         // [M][in], boxes of N rows x 64 columns

@@ -33,6 +33,32 @@ constexpr TsRings ts_rings(int K, int cols) {
     return {sx, sp};
 }
 
+// Work split of the kernel for up to 128 tokens.  `tiles` row tiles with `units` 128-column blocks in all; rows of one length have
+// `nb0` blocks, nb0 = 0 says that the linears differ in length.  CTA b of `grid` takes the units [share(b), share(b + 1)) of the cut
+// ones, share(s) = cut_begin + cut_units / cut_step * s / grid * cut_step, and the whole tiles b, b + grid, ... below cut_begin.
+struct TsSplit {
+    int grid, whole, cut_begin, cut_units, cut_step;
+};
+constexpr int kTsMinCut = 16;                         // blocks per row from which tiles are shared between CTAs
+constexpr int kTsMinShare = 8;                        // blocks of a share at least (a share of a tile costs a tile of adds)
+
+constexpr TsSplit ts_split(int tiles, int units, int nb0, int sms) {
+    const bool cut = nb0 == 0 || nb0 >= kTsMinCut;
+    int grid = cut ? (units - 1) / kTsMinShare + 1 : tiles;
+    // Few tiles: every tile in equally many shares, so that none lies across two tiles and pays for two.  512 x 3584 (four tiles
+    // of 28 blocks) with 4 tokens takes 6.3 us in sixteen shares of seven, 7.9 in fourteen of eight, the few-token kernel 6.5; a
+    // 7B-shaped W4-G128 layer with 100 tokens, whose pieces are drained one after the other, 133 us after 179.
+    if (cut && nb0 > 0) {
+        const long long even = (long long)tiles * ((nb0 - 1) / kTsMinShare + 1);
+        if (even <= sms) grid = (int)even;
+    }
+    if (grid > sms) grid = sms;
+    TsSplit w = {grid, nb0 > 0 ? tiles / grid : 0, 0, 0, cut ? 1 : nb0};
+    w.cut_begin = w.whole * grid * nb0;
+    w.cut_units = units - w.cut_begin;
+    return w;
+}
+
 // Prefill kernel: the stage of a 128-column block (of four 32-column or two 64-column ones) behind which a decode group gives the
 // block's packed slot back.  A refill does not queue behind loads that are still out, so every loaded word has to have gone into
 // a stored stage: column word q is put together from physical words q and q - 1 (mod 4), so the stage that holds word 2 is the

@@ -16,8 +16,14 @@ HEADER_DIR = os.path.join(ROOT, "paper_2602_04163_b200", "csrc")
 
 DRIVER = r"""
 #include <cstdio>
+#include <cstdlib>
 #include "bpdq_rings.h"
-int main() {
+int main(int argc, char** argv) {
+    if (argc == 5) {
+        const bpdq::TsSplit w = bpdq::ts_split(atoi(argv[1]), atoi(argv[2]), atoi(argv[3]), atoi(argv[4]));
+        printf("%d %d %d %d %d\n", w.grid, w.whole, w.cut_begin, w.cut_units, w.cut_step);
+        return 0;
+    }
     for (int K = 1; K <= 4; ++K)
         for (int cols = 16; cols <= 128; cols += 16) {
             const bpdq::TsRings r = bpdq::ts_rings(K, cols);
@@ -30,12 +36,17 @@ int main() {
 
 
 @pytest.fixture(scope="module")
-def rings(tmp_path_factory):
+def driver(tmp_path_factory):
     d = tmp_path_factory.mktemp("rings")
     src, exe = d / "driver.cpp", d / "driver"
     src.write_text(DRIVER)
     subprocess.run(["g++", "-O2", "-std=c++17", "-I", HEADER_DIR, str(src), "-o", str(exe)], check=True)
-    rows = [line.split() for line in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.splitlines()]
+    return str(exe)
+
+
+@pytest.fixture(scope="module")
+def rings(driver):
+    rows = [line.split() for line in subprocess.run([driver], check=True, capture_output=True, text=True).stdout.splitlines()]
     return [(r[0], [int(v) for v in r[1:]]) for r in rows]
 
 
@@ -171,3 +182,35 @@ def test_landing_areas_are_refilled_behind_a_fence():
     calls = re.findall(r"([^;{}]*)\bissue_task\(", text)
     assert len(calls) == 2 and sum("early &&" in c for c in calls) == 1       # the first copy, and the one in refill
     assert re.search(r"auto refill = [^;]*\{\s*bpdq::tma::fence_proxy_async\(\);\s*__syncwarp\(\);\s*issue_task\(", text)
+
+
+@pytest.mark.parametrize("tiles,nb0,sms", [(4, 28, 148), (28, 28, 148), (36, 28, 148), (32, 32, 148), (1, 16, 148), (9, 17, 148), (8, 64, 148),
+                                           (231, 64, 148), (64, 231, 148), (148, 28, 148), (296, 28, 148), (256, 4, 148), (3, 1, 148),
+                                           (149, 15, 148), (37, 31, 132), (1, 1, 1)])
+def test_the_work_split_covers_every_block_once(driver, tiles, nb0, sms):
+    """Shares of the cut units and whole tiles together are all blocks, once each; every CTA has work; where every tile can be cut into
+    shares of eight blocks at most, no share lies across two tiles."""
+    units = tiles * nb0
+    out = subprocess.run([driver, str(tiles), str(units), str(nb0), str(sms)], check=True, capture_output=True, text=True).stdout
+    grid, whole, cut_begin, cut_units, step = (int(v) for v in out.split())
+    assert 1 <= grid <= sms
+    taken = [(b + grid * f) * nb0 + k for b in range(grid) for f in range(whole) for k in range(nb0)]
+    shares = [cut_begin + cut_units // step * s // grid * step for s in range(grid + 1)]
+    assert shares[0] == cut_begin and shares[-1] == units
+    taken += range(shares[0], shares[-1])
+    assert sorted(taken) == list(range(units))
+    assert whole > 0 or all(a < b for a, b in zip(shares, shares[1:]))
+    per_tile = -(-nb0 // 8)
+    if nb0 >= 16 and tiles * per_tile <= sms:
+        assert grid == tiles * per_tile
+        assert all(a // nb0 == (b - 1) // nb0 for a, b in zip(shares, shares[1:]))
+    if nb0 < 16:
+        assert all(a % nb0 == 0 for a in shares)                # short rows are not cut
+
+
+@pytest.mark.parametrize("blocks,sms", [([64, 9, 5], 148), ([28, 231], 148), ([1], 4), ([200, 17], 3)])
+def test_the_work_split_of_rows_of_different_lengths(driver, blocks, sms):
+    units = sum(blocks)
+    out = subprocess.run([driver, str(len(blocks)), str(units), "0", str(sms)], check=True, capture_output=True, text=True).stdout
+    grid, whole, cut_begin, cut_units, step = (int(v) for v in out.split())
+    assert (whole, cut_begin, cut_units, step) == (0, 0, units, 1) and 1 <= grid <= min(sms, (units + 7) // 8)
