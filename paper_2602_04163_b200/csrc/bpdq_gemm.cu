@@ -259,7 +259,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaS
 
 template <int K>
 int launch_k(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
-    if (M <= kTsMaxM) return launch_ts<K>(&h, &x, &y, 1, M, stream, false);
+    if (M <= kTsMaxM && !bpdq::ts_drain_bound((h->out + BM - 1) / BM, h->in / 128, M, h->sm_count)) return launch_ts<K>(&h, &x, &y, 1, M, stream, false);
     const int half = wide_half(M, (h->out + BM - 1) / BM, h->in / 128, K, h->sm_count);
     return half <= kWideLongHalf ? launch_wide<K, 64>(h, x, y, M, half, stream) : launch_wide<K, 32>(h, x, y, M, half, stream);
 }

@@ -59,6 +59,15 @@ constexpr TsSplit ts_split(int tiles, int units, int nb0, int sms) {
     return w;
 }
 
+// Linears of up to 128 tokens that go to the prefill kernel all the same: more tiles than SMs with rows so short that a tile's
+// drain, by four warps and above 64 tokens with no second accumulator, takes longer than its blocks; the prefill kernel drains
+// with eight.  K = 2, us here and there: 20480 x 1024 (8 blocks) with 128 tokens 17.7 and 12.4, with 72 tokens 14.0 and 11.3; 20480 x 256 with
+// 56 tokens 8.8 and 5.0, with 17 tokens 7.3 and 4.5.  Between 3 and 8 blocks below 64 tokens and between 9 and 15 above either may be
+// the faster one, by a sixth at most.
+constexpr bool ts_drain_bound(int tiles, int nblocks, int M, int sms) {
+    return tiles > sms && M > 16 && nblocks <= (M > 64 ? 8 : 2);
+}
+
 // Prefill kernel: the stage of a 128-column block (of four 32-column or two 64-column ones) behind which a decode group gives the
 // block's packed slot back.  A refill does not queue behind loads that are still out, so every loaded word has to have gone into
 // a stored stage: column word q is put together from physical words q and q - 1 (mod 4), so the stage that holds word 2 is the

@@ -161,3 +161,21 @@ def test_gated_unit_up_to_128_tokens_in_one_launch(K, g, out, in_, M):
         hg.bpdq_get_status(G.stream_ptr())
         assert hg.bpdq_launch_count() + hu.bpdq_launch_count() == n0 + 1
         assert np.all(np.abs(hout.cpu().numpy().astype(np.float64)[:, rows] - want) <= bound)
+
+
+@pytest.mark.parametrize("K,g,in_,M", [(2, 128, 256, 17), (3, 64, 128, 64), (4, 128, 384, 64), (2, 256, 1024, 65), (3, 64, 896, 128), (2, 128, 1152, 100)])
+def test_short_rows_in_more_tiles_than_sms(K, g, in_, M):
+    """Either side of the lines where up to 128 tokens of short rows go to the prefill kernel; a tile more than SMs, the last one
+    ragged.  Weights from bpdq_dequant, sums in binary32."""
+    import torch
+    out = 128 * torch.cuda.get_device_properties(0).multi_processor_count + 48
+    h = binding.Handle(out, in_, K, g, None, 23, M)
+    bias = np.random.RandomState(3).randn(out).astype(np.float16)
+    h.bpdq_set_bias(bias.view(np.uint16))
+    x = synth.activations(24, M, in_)
+    w = torch.from_numpy(G.run_dequant(h).view(np.float16)).cuda().float()
+    ref = (G.x_tensor(x).float() @ w.T).cpu().numpy() + bias.astype(np.float32)
+    for kernel in (binding.KERNEL_AUTO, binding.KERNEL_GEMM):
+        y = G.run_linear(h, x, kernel)
+        # binary16 rounding of the result (2^-11) and binary32 sums of up to 1152 terms of size up to 0.2 in another order
+        assert np.all(np.abs(y - ref) <= 2.0 ** -10 * np.abs(ref) + 2e-3)
