@@ -40,8 +40,6 @@ constexpr int BM = 128;                 // output rows per CTA (MMA M)
 constexpr int BK = 64;                  // columns per stage: one 128-byte swizzle row of binary16
 
 struct GemmParams {
-    const uint8_t* blob;
-    size_t planes_bytes;
     __half* y;                // [M][out]
     int* status;
     int out, in, group, M;
@@ -108,7 +106,7 @@ template <int K>
 int ensure_packed_maps(bpdq_handle_s* h, EncodeTiledFn enc) {
     if (h->gemm_maps_ready) return BPDQ_OK;
     const cuuint32_t estr[2] = {1, 1};
-        // planes: rows (block, plane) of out x 16 bytes; coefficients: rows (group, coefficient) of out x 2 bytes; both
+    // planes: rows (block, plane) of out x 16 bytes; coefficients: rows (group, coefficient) of out x 2 bytes; both
     // as 8-byte elements, so that 128 output rows are 256 resp. 32 elements (a box dimension holds at most 256)
     const int ng = h->group == 64 ? 2 : 1;
     const cuuint64_t pd[2] = {(cuuint64_t)h->out * 2, (cuuint64_t)(h->in / 128) * K};
@@ -193,39 +191,18 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
     return BPDQ_OK;
 }
 
-// Tokens of a half tile: the cut of M tokens into equal tiles that takes the least time by a model of the kernel.  A 128-column
-// block takes 8.5 clocks per token of a half (the MMAs; 1.14 us with 512-token tiles), but no less than the decode and the
-// hand-over of its stages: 1150 clocks with 64-column stages, 1320 with 32-column ones (1600 and 1700 with sixteen candidates).
-// A tile is paid for in whole rounds over the SMs.  Always 512 tokens per tile left most SMs idle on short token counts:
-// 3584 x 18944 (28 row tiles) with 777 tokens took 199 us in 56 tiles, in 140 it takes 100.
-int wide_half(int M, int nrt, int nblocks, int K, int sms) {
-    long long best = 0;
-    int half = kWideMaxHalf;
-    for (int ntt = (M + 2 * kWideMaxHalf - 1) / (2 * kWideMaxHalf); ntt <= (M + 31) / 32; ++ntt) {
-        const int h = ((M + ntt - 1) / ntt + 31) / 32 * 16;
-        const long long tiles = (long long)nrt * ((M + 2 * h - 1) / (2 * h)), rounds = (tiles + sms - 1) / sms;
-        const long long least = h <= kWideLongHalf ? (K == 4 ? 1600 : 1150) : (K == 4 ? 1700 : 1320);
-        const long long block = 17LL * h / 2 > least ? 17LL * h / 2 : least;
-        const long long cost = rounds * (nblocks * block + 2000 + 30LL * h);
-        if (best == 0 || cost < best) { best = cost; half = h; }
-    }
-    return half;
-}
-
 template <int K, int BKW>
 int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaStream_t stream) {
-    using C = WideCfg<K, BKW>;
     static bpdq::SmemOptin optin;
     if (const int rc = bpdq::ensure_smem_optin(gemm_wide_kernel<K, BKW>, optin, h->device, kWideSmem, "gemm"); rc != BPDQ_OK) return rc;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: cuTensorMapEncodeTiled is not available from this driver");
     const int nrt = (h->out + BM - 1) / BM;
+    const bpdq::WideRings rings = bpdq::wide_rings(K, BKW, half);
     WideParams p;
     p.half = half;
-    const int stage = C::stage_bytes(half);
-    p.stages = C::kStageBudget / stage > kWideMaxStages ? kWideMaxStages : C::kStageBudget / stage;
-    p.sp = kWideMinSP + (C::kStageBudget - p.stages * stage) / C::kBlockBytes;
-    p.sp = p.sp > kWideMaxSP ? kWideMaxSP : p.sp / 2 * 2;
+    p.stages = rings.stages;
+    p.sp = rings.sp;
     CUtensorMap map;
     const cuuint64_t dims[2] = {(cuuint64_t)h->in, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)h->in * 2};
@@ -236,7 +213,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaS
                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (cr != CUDA_SUCCESS) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: tensor map encode failed (CUresult %d)", (int)cr);
     if (const int rc = ensure_packed_maps<K>(h, enc); rc != BPDQ_OK) return rc;
-    p.g.blob = h->d_blob; p.g.planes_bytes = h->planes_bytes; p.g.y = static_cast<__half*>(y); p.g.status = h->d_status;
+    p.g.y = static_cast<__half*>(y); p.g.status = h->d_status;
     p.g.out = h->out; p.g.in = h->in; p.g.group = h->group; p.g.M = M;
     p.g.bias = static_cast<const __half*>(h->d_bias);
     const long long ntiles = (long long)nrt * ((M + 2 * p.half - 1) / (2 * p.half));
@@ -244,8 +221,9 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaS
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kWideThreads); cfg.dynamicSmemBytes = kWideSmem; cfg.stream = stream;
     cudaLaunchAttribute attr[1];
-    // Short launches: SMs that the kernel before has left set up and fetch packed blocks.  Long ones run into the power limit,
-    // and CTAs that wait beside them cost more than the start they save (72B-shaped layer with 4096 tokens: 6.24 ms, 6.40 with).
+    // Short launches: SMs that the kernel before has left set up and fetch packed blocks (a permuted 7B-shaped layer with 777 tokens
+    // 512 us, 479 with this and what was changed beside it).  Long ones run into the power limit, and CTAs that wait beside them cost
+    // more than the start they save: 72B-shaped layer with 4096 tokens 6.50, 6.48, 6.53 ms, 6.54, 6.56, 6.56 with (three comparisons in turn).
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = ntiles <= 4LL * h->sm_count ? 1 : 0;
     cfg.attrs = attr; cfg.numAttrs = 1;
@@ -260,7 +238,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaS
 template <int K>
 int launch_k(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
     if (M <= kTsMaxM && !bpdq::ts_drain_bound((h->out + BM - 1) / BM, h->in / 128, M, h->sm_count)) return launch_ts<K>(&h, &x, &y, 1, M, stream, false);
-    const int half = wide_half(M, (h->out + BM - 1) / BM, h->in / 128, K, h->sm_count);
+    const int half = bpdq::wide_half(M, (h->out + BM - 1) / BM, h->in / 128, K, h->sm_count);
     return half <= kWideLongHalf ? launch_wide<K, 64>(h, x, y, M, half, stream) : launch_wide<K, 32>(h, x, y, M, half, stream);
 }
 

@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_con
     } else if (warp <= 2) {
         // ---------------- MMA issuers: blocks alternate between the two, each adds into an accumulator of its own ----------------
         const int me = warp - 1;
-        const unsigned idesc = (1u << 4) | ((unsigned)(N >> 3) << 17) | ((unsigned)(128 >> 4) << 24);
+        const unsigned idesc = instr_desc_f16(BM, N);
         int sx = 0, sa = 0, buf = 0;
         unsigned px = 0u, pa = 0u, pacc = 1u;
         bool ok = true;

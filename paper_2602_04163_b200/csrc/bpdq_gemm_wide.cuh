@@ -1,13 +1,10 @@
 // Included by bpdq_gemm.cu (inside its unnamed namespace, after the PTX wrappers): the prefill kernel for many tokens.
 //
-// gemm_wide_kernel: one decoded weight stage feeds TWO 256-token halves of a 512-token tile.  The persistent
-// 256-token kernel decodes every weight once per 256 tokens and one thread issues all of its MMAs; measured, a
-// single thread gets a tcgen05.mma out every 155-167 clocks whatever its shape while a 128 x 256 x 16 one occupies
-// the pipe for 128, and the decode's energy is what the 1 kW cap charges (every further plane costs 8-20 %).  Here
-// two warps issue, each into a 128 x 256 accumulator of its own (the two halves of TMEM's 512 columns) from the
-// same A stage and its own x half, so the decode work and the A-tile traffic per FLOP are halved and the issue cap
-// is lifted.  TMEM is full with one tile, so the epilogue no longer overlaps the next tile's MMAs (about 3 % of a
-// 72B-shaped tile's time); producer and decode warps run ahead into the next tile's stages meanwhile.
+// gemm_wide_kernel: one decoded weight stage feeds TWO halves (of up to 256 tokens each) of a token tile.  Two warps issue, each into
+// a 128 x half accumulator of its own (the two halves of TMEM's 512 columns) from the same A stage and its own x half, so a weight is
+// decoded once per tile: the decode's energy is what the 1 kW cap charges (every further plane costs 8-20 %).  TMEM is full with one
+// tile, so the epilogue does not overlap the next tile's MMAs (about 3 % of a 72B-shaped tile's time); producer and decode warps run
+// ahead into the next tile's stages meanwhile.
 //
 // Stages are 64 columns (128-byte swizzle rows) while four of them fit, i.e. for halves of up to 128 tokens, else 32 columns
 // (64-byte rows: five stages of the widest tile): a stage costs its issuers about 330 clocks beside the decode warps that
@@ -18,15 +15,13 @@
 // per half).  Barriers per stage: full (both x halves' bytes and one arrival per warp of the owning decode group), empty (one
 // tcgen05.commit per issuer); per packed slot: full_p, empty_p; acc_full (one commit per issuer), acc_empty (one arrival per
 // epilogue warp).  All waits are bounded.
-constexpr int kWideMaxHalf = 256;                             // most tokens of a half
-constexpr int kWideLongHalf = 128;                            // ... with 64-column stages
+using bpdq::kWideMaxHalf;
+using bpdq::kWideLongHalf;
+using bpdq::kWideSmem;
 constexpr int kWideEpiWarps = 8;
 constexpr int kWideGroups = 2;                                // decode groups, alternating blocks
 constexpr int kWideFirstDecode = 4, kWideFirstEpi = kWideFirstDecode + 4 * kWideGroups;
 constexpr int kWideThreads = 32 * (kWideFirstEpi + kWideEpiWarps);
-constexpr int kWideMinSP = 2, kWideMaxSP = 8;                  // packed blocks in flight (an even number: a slot belongs to one group)
-constexpr int kWideSmem = 227 * 1024;
-constexpr int kWideMaxStages = 12;
 
 struct WideParams {
     GemmParams g;
@@ -38,14 +33,9 @@ struct WideParams {
 template <int K, int BKW> struct WideCfg {
     static constexpr int kATile = BM * BKW * 2;                // 8 or 16 KB
     static constexpr int kPerBlock = 128 / BKW;                // stages per packed block
-    // a decode group waits for stage it after stage it - (kPerBlock + 1): the ring has to be at least that long (see there)
-    static constexpr int kMinStages = kPerBlock + 1;
-    static constexpr int stage_bytes(int half) { return kATile + 2 * half * BKW * 2; }
-    static constexpr int kPlaneBytes = K * BM * 16;
-    static constexpr int kCoefBytes = (K + 1) * BM * 2;
-    static constexpr int kBlockBytes = (kPlaneBytes + 2 * kCoefBytes + 1023) / 1024 * 1024;
-    static constexpr int kStageBudget = kWideSmem - kWideMinSP * kBlockBytes - 1024 /*alignment slack*/ - 1024 /*barriers*/;
-    static_assert(BKW == 64 || kStageBudget >= kMinStages * stage_bytes(kWideMaxHalf), "the widest tile");
+    static constexpr int kPlaneBytes = bpdq::wide_plane_bytes(K), kCoefBytes = bpdq::wide_coef_bytes(K);
+    static constexpr int kBlockBytes = bpdq::wide_block_bytes(K);
+    static_assert(kATile == bpdq::wide_a_bytes(BKW), "bytes of a stage's weights");
 };
 
 // Shared-memory matrix descriptor of a K-major tile with 64-byte swizzle whose rows are 64 bytes apart: start address
@@ -197,9 +187,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         unsigned off[4];                                 // logical word k takes the bytes of physical words k - wrot and k - wrot - 1
 #pragma unroll
         for (unsigned k = 0; k < 4; ++k) off[k] = p_base + (unsigned)rl * 16u + (((k - wrot) & 3u) << 2);
-        // Stage slots are shared by the groups; a wait by parity needs the release two uses back to be over.  A group that
-        // waits for stage it has waited for a stage no earlier than it - (kPerBlock + 1) before, i.e. for an MMA no earlier
-        // than S stages before that one, and MMAs complete in order: enough for S >= kPerBlock + 1.
+        // Stage slots are shared by the groups; why their waits by parity are safe stands at wide_rings (bpdq_rings.h).
         const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
         int s = 0, sp = grp;
         unsigned ph = 1u, pp = 0u;

@@ -1,4 +1,5 @@
-// Host-side lengths of the rings in shared memory that the tensor-core kernels' roles hand blocks round in (plain C++, no CUDA).
+// Host side of the tensor-core kernels (plain C++, no CUDA): lengths of the rings in shared memory that their roles hand blocks
+// round in, the split of the work over CTAs, the size of token tiles.
 #pragma once
 
 namespace bpdq {
@@ -46,7 +47,7 @@ constexpr TsSplit ts_split(int tiles, int units, int nb0, int sms) {
     const bool cut = nb0 == 0 || nb0 >= kTsMinCut;
     int grid = cut ? (units - 1) / kTsMinShare + 1 : tiles;
     // Few tiles: every tile in equally many shares, so that none lies across two tiles and pays for two.  512 x 3584 (four tiles
-    // of 28 blocks) with 4 tokens takes 6.3 us in sixteen shares of seven, 7.9 in fourteen of eight, the few-token kernel 6.5; a
+    // of 28 blocks) with 4 tokens takes 6.0 us in sixteen shares of seven, 7.9 in fourteen of eight, the few-token kernel 6.5; a
     // 7B-shaped W4-G128 layer with 100 tokens, whose pieces are drained one after the other, 133 us after 179.
     if (cut && nb0 > 0) {
         const long long even = (long long)tiles * ((nb0 - 1) / kTsMinShare + 1);
@@ -73,5 +74,59 @@ constexpr bool ts_drain_bound(int tiles, int nblocks, int M, int sms) {
 // a stored stage: column word q is put together from physical words q and q - 1 (mod 4), so the stage that holds word 2 is the
 // first by which all four are used; it also builds the tables of the second coefficient group of g = 64.
 constexpr int wide_release_stage(int stages_per_block) { return stages_per_block / 2; }
+
+constexpr int kWideMaxHalf = 256;                             // most tokens of a half tile
+constexpr int kWideLongHalf = 128;                            // ... with 64-column stages
+constexpr int kWideSmem = 227 * 1024;
+constexpr int kWideMinSP = 2, kWideMaxSP = 8, kWideMaxStages = 12;
+constexpr int wide_plane_bytes(int K) { return K * 2048; }
+constexpr int wide_coef_bytes(int K) { return (K + 1) * 256; }
+constexpr int wide_block_bytes(int K) { return (wide_plane_bytes(K) + 2 * wide_coef_bytes(K) + 1023) / 1024 * 1024; }
+constexpr int wide_a_bytes(int bkw) { return 128 * bkw * 2; }                              // a stage's weights
+constexpr int wide_stage_bytes(int bkw, int half) { return wide_a_bytes(bkw) + 2 * half * bkw * 2; }   // ... and both halves of x
+
+struct WideRings {
+    int stages, sp;                                   // slots of the stage ring and of the packed ring
+};
+
+// `bkw` columns per stage, 32 or 64.  Packed slots: an even number, so that a slot belongs to one of the two decode groups, which
+// has waited for every use of it.  Stage slots are shared by the groups: the group that waits for the release of stage it - S has
+// waited, for the last stage of its block before, it - (stages per block + 1), for MMAs no later than S stages before that one, and MMAs
+// complete in order; so the release before, of stage it - 2 S, is over if S >= stages per block + 1.  The narrowest ring is the
+// widest tile's at K = 4: five stages of 32 columns.
+constexpr WideRings wide_rings(int K, int bkw, int half) {
+    const int stage = wide_stage_bytes(bkw, half), budget = kWideSmem - kWideMinSP * wide_block_bytes(K) - 2048;   // 2048: alignment slack, barriers
+    int stages = budget / stage;
+    if (stages > kWideMaxStages) stages = kWideMaxStages;
+    int sp = kWideMinSP + (budget - stages * stage) / wide_block_bytes(K);
+    sp = sp > kWideMaxSP ? kWideMaxSP : sp / 2 * 2;
+    return {stages, sp};
+}
+static_assert(wide_rings(4, 32, kWideMaxHalf).stages >= 5 && wide_rings(4, 64, kWideLongHalf).stages >= 3, "the widest tiles");
+
+// Tokens of a half tile: the cut of M tokens into equal tiles that takes the least time by a model of the kernel.  A 128-column
+// block takes 8.5 clocks per token of a half (the MMAs), but no less than the decode and the hand-over of its stages: 1150 clocks
+// with 64-column stages, 1320 with 32-column ones (1600 and 1700 with sixteen candidates); a tile is paid for in whole rounds over
+// the SMs.  Measured, ns per block with one tile per SM, 12288 and 4096 columns, back to back (the 1 kW cap slows the larger halves; g = 128):
+//   half      16    48    80   112   128 |  144   160   192   224   256
+//   K = 1    479   524   697   764   825 | 1006  1055  1144  1326  1541
+//   K = 2    507   548   658   800   872 | 1179  1121  1232  1473  1602
+//   K = 3    830   866   779   948  1028 | 1311  1307  1324  1503  1722
+//   K = 4   1069  1078   974  1167  1517 | 1383  1453  1578  1632  1833
+// Always 512 tokens per tile left most SMs idle on short token counts: 3584 x 18944 (28 row tiles) with 777 tokens took 199 us in
+// 56 tiles, in 140 it takes 94.
+inline int wide_half(int M, int nrt, int nblocks, int K, int sms) {
+    long long best = 0;
+    int half = kWideMaxHalf;
+    for (int ntt = (M + 2 * kWideMaxHalf - 1) / (2 * kWideMaxHalf); ntt <= (M + 31) / 32; ++ntt) {
+        const int h = ((M + ntt - 1) / ntt + 31) / 32 * 16;
+        const long long tiles = (long long)nrt * ((M + 2 * h - 1) / (2 * h)), rounds = (tiles + sms - 1) / sms;
+        const long long least = h <= kWideLongHalf ? (K == 4 ? 1600 : 1150) : (K == 4 ? 1700 : 1320);
+        const long long block = 17LL * h / 2 > least ? 17LL * h / 2 : least;
+        const long long cost = rounds * (nblocks * block + 2000 + 30LL * h);
+        if (best == 0 || cost < best) { best = cost; half = h; }
+    }
+    return half;
+}
 
 }  // namespace bpdq

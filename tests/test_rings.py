@@ -24,6 +24,17 @@ int main(int argc, char** argv) {
         printf("%d %d %d %d %d\n", w.grid, w.whole, w.cut_begin, w.cut_units, w.cut_step);
         return 0;
     }
+    if (argc == 6) {
+        printf("%d\n", bpdq::wide_half(atoi(argv[1]), atoi(argv[2]), atoi(argv[3]), atoi(argv[4]), atoi(argv[5])));
+        return 0;
+    }
+    for (int K = 1; K <= 4; ++K)
+        for (int half = 16; half <= 256; half += 16) {
+            const int bkw = half <= bpdq::kWideLongHalf ? 64 : 32;
+            const bpdq::WideRings r = bpdq::wide_rings(K, bkw, half);
+            printf("wide %d %d %d %d %d %d\n", K, half, 128 / bkw, r.stages, r.sp,
+                   bpdq::kWideSmem - r.stages * bpdq::wide_stage_bytes(bkw, half) - r.sp * bpdq::wide_block_bytes(K));
+        }
     for (int K = 1; K <= 4; ++K)
         for (int cols = 16; cols <= 128; cols += 16) {
             const bpdq::TsRings r = bpdq::ts_rings(K, cols);
@@ -123,6 +134,62 @@ def test_the_order_model_sees_an_odd_ring():
     wait for its packed block open."""
     assert {role for role, _ in ts_order(4, 9, 60).open_waits()} == {"group, packed"}
     assert ts_order(8, 23, 100).open_waits() == []           # an odd ring that the x ring covers
+
+
+def wide_order(stages, sp, per_block, blocks, release):
+    """gemm_wide_kernel: x producer, packed producer, two decode groups (group b mod 2 takes block b), two issuers that multiply every
+    stage."""
+    o = Order()
+
+    def ev(kind, q):
+        return (kind, q) if q >= 0 else None
+    for b in range(blocks):
+        o.event(("packed asked", b), ev("packed asked", b - 1), ev("stored", (b - sp) * per_block + release) if b >= sp else None)
+        o.wait("packed producer", ev("packed asked", b - 1), ev("stored", (b - 2 * sp) * per_block + release) if b >= 2 * sp else None)
+        o.event(("packed landed", b), ("packed asked", b))
+        for it in range(b * per_block, (b + 1) * per_block):
+            o.event(("x asked", it), ev("x asked", it - 1), ev("multiplied", it - stages))
+            o.wait("x producer", ev("x asked", it - 1), ev("multiplied", it - 2 * stages))
+            o.event(("x landed", it), ("x asked", it))
+            before = ev("stored", it - 1) if it % per_block else ev("stored", (b - 1) * per_block - 1)    # the group's stage before
+            if it % per_block == 0:
+                o.wait("group, packed", before, ev("packed landed", b - sp))
+            o.wait("group, stage", before, ev("multiplied", it - 2 * stages))
+            o.event(("stored", it), before, ("packed landed", b), ev("multiplied", it - stages))
+            for i in range(2):
+                o.wait("issuer", ev(f"issued {i}", it - 1), ev("full", it - stages))
+                o.event((f"issued {i}", it), ev(f"issued {i}", it - 1), ("full", it))
+            o.event(("full", it), ("stored", it), ("x landed", it))
+            o.event(("multiplied", it), ("issued 0", it), ("issued 1", it), ev("multiplied", it - 1))
+    return o
+
+
+def test_rings_of_the_prefill_kernel(rings):
+    (release,) = [r for kind, r in rings if kind == "release"]
+    seen = 0
+    for kind, r in rings:
+        if kind != "wide":
+            continue
+        K, half, per_block, stages, sp, left = r
+        seen += 1
+        assert left >= 1024 + 8 * (2 * stages + 2 * sp + 2) + 8, r             # alignment slack, barriers, TMEM address and flag
+        assert wide_order(stages, sp, per_block, 2 * sp + 2 * stages + 4, release[0 if per_block == 4 else 1]).open_waits() == [], r
+    assert seen == 64
+    assert wide_order(4, 2, 4, 20, 2).open_waits()                              # four stages of 32 columns would not do
+
+
+@pytest.mark.parametrize("M,nrt,nblocks,K", [(129, 28, 28, 2), (777, 28, 148, 2), (777, 4, 28, 2), (4096, 231, 64, 3), (4096, 1, 1, 4), (513, 148, 32, 4),
+                                             (131, 64, 231, 1), (8192, 64, 64, 3), (17, 192, 1, 2), (128, 256, 8, 4), (300, 1, 8, 2)])
+def test_half_tiles(driver, M, nrt, nblocks, K):
+    """A half tile is a multiple of 16 tokens, at most 256, and its cut of M takes no more rounds over the SMs than 512-token tiles do."""
+    half = int(subprocess.run([driver, *map(str, (M, nrt, nblocks, K, 148))], check=True, capture_output=True, text=True).stdout)
+    assert half % 16 == 0 and 16 <= half <= 256
+
+    def clocks(h):
+        rounds = -(-nrt * -(-M // (2 * h)) // 148)
+        return rounds * (nblocks * max(8.5 * h, (1600 if K == 4 else 1150) if h <= 128 else (1700 if K == 4 else 1320)) + 2000 + 30 * h)
+    equal = [min(256, -(-(-(-M // n)) // 32) * 16) for n in range(-(-M // 512), -(-M // 32) + 1)]
+    assert half in equal and clocks(half) <= min(clocks(h) for h in equal) * 1.001
 
 
 def test_prefill_slots_are_given_back_after_the_last_use(rings):
