@@ -12,7 +12,7 @@ from tests import gpu_util as G
 pytestmark = pytest.mark.gpu
 
 KERNELS = [("lut", binding.KERNEL_GEMV, 1), ("lut", binding.KERNEL_GEMV, 2), ("few", binding.KERNEL_FEW, 5), ("few", binding.KERNEL_FEW, 20),
-           ("tile", binding.KERNEL_GEMM, 40), ("persistent", binding.KERNEL_GEMM, 300), ("simple", binding.KERNEL_GEMV_SIMPLE, 3),
+           ("tmem", binding.KERNEL_GEMM, 40), ("prefill", binding.KERNEL_GEMM, 300), ("simple", binding.KERNEL_GEMV_SIMPLE, 3),
            ("auto", binding.KERNEL_AUTO, 9)]
 
 
@@ -48,7 +48,7 @@ def test_permutation_rejects_what_is_not_one_and_works_in_a_batch():
     assert ei.value.code == binding.ERR_INVALID
     perm = _group_perm(640, g, 511)
     layers[1][0].bpdq_set_input_permutation(perm)                        # one linear of the batch is permuted, the other is not
-    for Mb in (1, M):                                                    # look-up-table launch, few-token launch
+    for Mb in (1, M):                                                    # look-up-table launch, tensor-core launch
         x = synth.activations(512 + Mb, Mb, 640)
         xt = G.x_tensor(x)
         ys = [torch.full((Mb, o), float("nan"), dtype=torch.float16, device="cuda") for o, _ in shapes]
@@ -63,7 +63,7 @@ def test_permutation_rejects_what_is_not_one_and_works_in_a_batch():
 @pytest.mark.parametrize("name,kernel,M", KERNELS + [("split", binding.KERNEL_GEMM, 24)])
 def test_bias_in_every_kernel(name, kernel, M):
     K, g = 2, 128
-    out, in_ = (256, 4096) if name == "split" else (272, 896)           # few row tiles and long rows: the tile kernel splits the input dimension
+    out, in_ = (256, 4096) if name == "split" else (272, 896)           # few row tiles and long rows: tiles are cut between CTAs
     h, bits, coef = G.make_layer(520, out, in_, K, g, max_M=M)
     x = synth.activations(521 + M, M, in_)
     bias = (np.random.default_rng(522).normal(0, 0.5, out)).astype(np.float16)
@@ -82,7 +82,7 @@ def test_bias_in_every_kernel(name, kernel, M):
 @pytest.mark.parametrize("M,with_bias,with_perm", [(1, False, False), (2, True, True), (8, False, False), (16, True, True), (40, True, False),
                                                     (300, False, True)])
 def test_gated_unit_of_a_gate_up_pair(M, with_bias, with_perm):
-    """h = silu(x Wg^T) * (x Wu^T): one launch up to the few-token threshold, three above; twice in a row (the second
+    """h = silu(x Wg^T) * (x Wu^T): one launch up to 128 tokens, three above; twice in a row (the second
     call finds workspaces and counters as the first left them)."""
     K, g, out, in_ = 2, 128, 400, 1152
     hg, bg, cg = G.make_layer(530, out, in_, K, g, max_M=M)

@@ -72,19 +72,87 @@ def test_few_token_kernel_full_size_sampled(name, out, in_, K, M):
     assert np.all(np.isfinite(y))
 
 
-def test_dispatcher_sends_3_to_16_tokens_to_the_few_token_kernel():
-    K, g, out, in_ = 2, 128, 272, 896
-    h, bits, coef = G.make_layer(171, out, in_, K, g, max_M=40)
-    for M, same_as in ((2, binding.KERNEL_GEMV), (3, binding.KERNEL_FEW), (16, binding.KERNEL_FEW), (17, binding.KERNEL_GEMM)):
+@pytest.mark.parametrize("K,g", [(2, 128), (3, 64), (4, 128), (4, 64)])
+def test_dispatcher_on_default_settings(K, g):
+    """Which kernel takes how many tokens: the look-up-table kernel up to 2 (3 at K = 4 and g >= 128; two tokens per pass), the
+    tensor-core kernels above.  Bit for bit: rows of 14 blocks are not cut between CTAs, and the kernels that a wrong choice would take
+    add in another order (some of 2064 x M results differ)."""
+    out, in_ = 2064, 1792
+    h, bits, coef = G.make_layer(171 + K, out, in_, K, g, max_M=129)
+    lut = 3 if K == 4 and g >= 128 else 2
+    rows = np.unique(np.concatenate([np.arange(0, out, 61), [127, 128, out - 1]]))
+    for M in (1, 2, 3, 4, 16, 17, 33, 128, 129):
         x = synth.activations(172 + M, M, in_)
-        G.check_linear(h, bits, coef, x, g, binding.KERNEL_AUTO, what=f"auto M={M}")
         n0 = h.bpdq_launch_count()
         ya = G.run_linear(h, x, binding.KERNEL_AUTO)
-        assert h.bpdq_launch_count() == n0 + 1
-        assert np.allclose(ya, G.run_linear(h, x, same_as), rtol=2.0 ** -9, atol=1e-5)
-    h.bpdq_set_few_max_m(0)                                               # switched off: the tcgen05 kernel takes over
-    x = synth.activations(180, 8, in_)
-    assert np.array_equal(G.run_linear(h, x, binding.KERNEL_AUTO), G.run_linear(h, x, binding.KERNEL_GEMM))
+        assert h.bpdq_launch_count() - n0 == ((M + 1) // 2 if M <= lut else 1)
+        y_ref, a_ref = oracle.linear(bits[:, rows], coef[:, rows], x, g)
+        G.assert_linear_close(ya[:, rows], y_ref, a_ref, f"auto M={M}")
+        gemm = G.run_linear(h, x, binding.KERNEL_GEMM)
+        if M > lut:
+            assert np.array_equal(ya, gemm)
+            if 16 <= M <= binding.FEW_MAX_M:
+                assert not np.array_equal(ya, G.run_linear(h, x, binding.KERNEL_FEW))
+        else:
+            assert not np.array_equal(ya, gemm)
+            # four slices meet in binary32 adds in the order of their arrival: the last binary16 digit may differ
+            assert np.allclose(ya, G.run_linear(h, x, binding.KERNEL_GEMV), rtol=2.0 ** -9, atol=1e-5)
+
+
+def test_few_token_kernel_on_request():
+    """bpdq_set_few_max_m: single, batched and gated calls with a bias and a permutation, twice in a row, against the checker; one launch
+    each beside the gathers.  The kernel's own sums: a batch equals single calls but for the order of adds."""
+    import torch
+    K, g, M, in_ = 3, 128, 13, 896
+    outs = (2064, 144, 2064)
+    layers = [G.make_layer(181 + k, o, in_, K, g, max_M=20) for k, o in enumerate(outs)]
+    hs = [L[0] for L in layers]
+    perm = np.random.RandomState(5).permutation(in_).astype(np.int32)
+    bias = np.random.RandomState(6).randn(outs[1]).astype(np.float16)
+    hs[0].bpdq_set_input_permutation(perm)
+    hs[1].bpdq_set_bias(bias.view(np.uint16))
+    x = synth.activations(185, M, in_)
+    refs, sums = [], []
+    for k, (_, bits, coef) in enumerate(layers):
+        y, a = oracle.linear(bits, coef, np.ascontiguousarray(x[:, perm]) if k == 0 else x, g)
+        refs.append(y + (bias.astype(np.float64) if k == 1 else 0.0))
+        sums.append(a + (np.abs(bias.astype(np.float64)) if k == 1 else 0.0))
+    default = [G.run_linear(h, x) for h in hs]
+    for h in hs:
+        h.bpdq_set_few_max_m(16)
+    few = [G.run_linear(h, x, binding.KERNEL_FEW) for h in hs]
+    assert any(not np.array_equal(f, d) for f, d in zip(few, default))
+    xt = G.x_tensor(x)
+    launches = lambda: sum(h.bpdq_launch_count() for h in hs)          # noqa: E731
+    for _ in range(2):
+        for h, y, a, f in zip(hs, refs, sums, few):
+            ya = G.run_linear(h, x)
+            G.assert_linear_close(ya, y, a, "single")
+            assert np.allclose(ya, f, rtol=2.0 ** -9, atol=1e-5)
+        ys = [torch.full((M, o), float("nan"), dtype=torch.float16, device="cuda") for o in outs]
+        n0 = launches()
+        binding.bpdq_linear_batch(hs, [xt.data_ptr()] * 3, [y.data_ptr() for y in ys], M, G.stream_ptr())
+        torch.cuda.synchronize()
+        hs[0].bpdq_get_status(G.stream_ptr())
+        assert launches() - n0 == 2                                     # one gather, one launch over the three
+        for y, r, a, f in zip(ys, refs, sums, few):
+            y = y.cpu().numpy().astype(np.float64)
+            G.assert_linear_close(y, r, a, "batch")
+            assert np.allclose(y, f, rtol=2.0 ** -9, atol=1e-5)
+        unit = torch.full((M, outs[0]), float("nan"), dtype=torch.float16, device="cuda")
+        n0 = launches()
+        binding.bpdq_gate_up_swiglu(hs[0], hs[2], xt.data_ptr(), unit.data_ptr(), M, G.stream_ptr())
+        torch.cuda.synchronize()
+        hs[0].bpdq_get_status(G.stream_ptr())
+        assert launches() - n0 == 2
+        want = oracle.swiglu(refs[0], refs[2])
+        dg, du = G.TOL_REL * sums[0] + G.TOL_ABS, G.TOL_REL * sums[2] + G.TOL_ABS
+        silu_g = oracle.swiglu(refs[0], np.ones_like(refs[0]))
+        bound = 1.1 * (np.abs(refs[2]) + du) * dg + (np.abs(silu_g) + 1.1 * dg) * du + 2.0 ** -10 * np.abs(want) + 1e-4
+        assert np.all(np.abs(unit.cpu().numpy().astype(np.float64) - want) <= bound)
+    for h in hs:
+        h.bpdq_set_few_max_m(0)                                         # switched off: the tensor-core kernel takes over
+        assert np.array_equal(G.run_linear(h, x), G.run_linear(h, x, binding.KERNEL_GEMM))
 
 
 def test_few_token_kernel_rejects_what_it_cannot_take():
@@ -100,8 +168,8 @@ def test_few_token_kernel_rejects_what_it_cannot_take():
 
 @pytest.mark.parametrize("g", [128, 64])
 def test_dispatcher_with_sixteen_candidates(g):
-    """K = 4 through bpdq_linear at the token counts either side of its thresholds (look-up-table kernel up to 3 tokens,
-    2 at g = 64; few-token kernel to 16; tcgen05 beyond): every choice within the checker's bound."""
+    """K = 4 through bpdq_linear at the token counts either side of its threshold (look-up-table kernel up to 3 tokens, 2 at
+    g = 64; tensor-core kernel beyond): every choice within the checker's bound."""
     K, out, in_ = 4, 272, 1536
     h, bits, coef = G.make_layer(190 + g, out, in_, K, g, max_M=20)
     for M in (1, 2, 3, 4, 16, 17):

@@ -12,35 +12,35 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("K,g,out,in_,M", [
     (2, 128, 128, 128, 16),      # one tile, one 128-column block, two stages
     (2, 128, 128, 1024, 32),     # more k-blocks than pipeline stages: every barrier wraps
-    (3, 128, 256, 512, 33),      # token tile of 64 with a ragged tail
+    (3, 128, 256, 512, 33),      # 48 token columns, the last fifteen beyond M
     (1, 128, 128, 256, 5),
     (2, 64, 128, 384, 64),       # a coefficient group per k-block
-    (3, 256, 256, 768, 100),     # a coefficient group every four k-blocks, token tile 128
-    (2, 128, 160, 640, 130),     # ragged last row tile (160 = 128 + 32), token tile 256 with a ragged tail
-    (3, 128, 384, 2048, 257),    # two token tiles of 256, the second holds one token
+    (3, 256, 256, 768, 100),     # a coefficient group every four k-blocks, 112 token columns
+    (2, 128, 160, 640, 130),     # ragged last row tile (160 = 128 + 32), several token tiles, the last one ragged
+    (3, 128, 384, 2048, 257),    # an odd number of tokens, the last tile ragged
     (2, 128, 1024, 1024, 300),
     (2, 128, 128, 128, 1),       # a single token through the tensor-core path
     (4, 128, 256, 512, 40),      # sixteen candidates per group (the paper's W4-G128): two byte-permutes and a select
     (4, 64, 128, 384, 300),
-    (2, 128, 256, 4096, 40),     # few row tiles, long rows: four CTAs share an output tile (split over the input dimension)
-    (3, 64, 128, 8192, 64),      # eight-way split
-    (4, 128, 384, 2048, 7),      # two-way split, ragged token tile
-    (2, 128, 256, 4096, 100),    # 128-token tile shared by four CTAs (split over the input dimension), two CTAs per SM
-    (3, 128, 384, 2048, 128),    # 128-token tile, two-way split, all 128 token columns in use
-    (2, 256, 160, 640, 24),      # g = 256 with a short last group: tile kernel
-    (3, 256, 272, 1152, 200),    # ... 256-token kernel
-    (2, 256, 160, 1664, 600),    # ... 512-token kernel (six and a half groups)
-    (2, 128, 256, 384, 20500),   # 162 output tiles for 148 persistent CTAs: a second tile per CTA, odd number of blocks per tile
-    (4, 128, 128, 640, 38000),   # 149 tiles, three-stage ring (K = 4), odd number of blocks per tile
-    (3, 64, 160, 640, 24),       # tile kernel, ragged last row tile (the tensor maps fill the missing rows), two groups per block
-    (1, 256, 144, 1024, 100),    # tile kernel with the 128-token tile, ragged row tile, a group every two blocks
-    (2, 128, 400, 1152, 9),      # 16-token tile, odd number of blocks, rings wrap at different stages
-    (2, 128, 256, 512, 256),     # the most tokens the 256-token kernel takes
-    (3, 128, 384, 2048, 200),    # 256-token kernel, ragged token tile
-    (2, 64, 160, 640, 700),      # 512-token kernel: two token tiles (the second holds 188), ragged row tile, a group per half block
-    (3, 256, 272, 1024, 513),    # 512-token kernel: the second token tile holds one token; a group every two blocks
-    (1, 128, 128, 256, 1030),    # 512-token kernel: two blocks per tile, three token tiles
-    (4, 128, 256, 384, 300),     # 512-token kernel with sixteen candidates (largest packed blocks), odd number of blocks per tile
+    (2, 128, 256, 4096, 40),     # few row tiles, long rows: four CTAs share a tile
+    (3, 64, 128, 8192, 64),      # eight shares
+    (4, 128, 384, 2048, 7),      # two shares per tile, ragged token columns
+    (2, 128, 256, 4096, 100),    # 112 token columns: one accumulator pair, four shares per tile
+    (3, 128, 384, 2048, 128),    # two shares per tile, all 128 token columns in use
+    (2, 256, 160, 640, 24),      # g = 256 with a short last group: TMEM kernel
+    (3, 256, 272, 1152, 200),    # ... prefill kernel, one token tile
+    (2, 256, 160, 1664, 600),    # ... several token tiles (six and a half groups)
+    (2, 128, 256, 384, 20500),   # more token tiles than SMs: a second tile for some CTAs, odd number of blocks per tile
+    (4, 128, 128, 640, 38000),   # the same with the largest packed blocks (K = 4)
+    (3, 64, 160, 640, 24),       # TMEM kernel, ragged last row tile (the tensor maps fill the missing rows), two groups per block
+    (1, 256, 144, 1024, 100),    # TMEM kernel with 112 token columns, ragged row tile, a group every two blocks
+    (2, 128, 400, 1152, 9),      # 16 token columns, odd number of blocks, rings wrap at different blocks
+    (2, 128, 256, 512, 256),     # prefill kernel, 64-column stages
+    (3, 128, 384, 2048, 200),    # prefill kernel, ragged token tile
+    (2, 64, 160, 640, 700),      # prefill kernel, several token tiles, ragged row tile, a group per half block
+    (3, 256, 272, 1024, 513),    # an odd number of tokens over 512; a group every two blocks
+    (1, 128, 128, 256, 1030),    # two blocks per tile, several token tiles
+    (4, 128, 256, 384, 300),     # prefill kernel with sixteen candidates (largest packed blocks), odd number of blocks per tile
 ])
 def test_gemm_kernel(K, g, out, in_, M):
     h, bits, coef = G.make_layer(60 + K, out, in_, K, g, max_M=M)

@@ -1,7 +1,7 @@
 """A decoder layer's launches recorded once into a CUDA graph and replayed: the calls of the C ABI enqueue kernels on the
 caller's stream and nothing else once a handle has been used (no allocation, no host wait), so a stream capture
 takes them as they are.  The replayed graph must give what the direct calls give, for new activations written into
-the same buffers, with each of the three kernel families (look-up-table, few-token, tcgen05)."""
+the same buffers, with each of the three kernels that the dispatcher picks from (look-up-table, TMEM, prefill)."""
 import numpy as np
 import pytest
 import torch
