@@ -26,6 +26,9 @@
  *     that take a stream only enqueue work and do not synchronise, unless stated;
  *   - a handle owns its device copy of the packed weights and a scratch workspace.  Two calls
  *     on the same handle must not overlap on the GPU (issue them on one stream);
+ *   - a row whose columns are cut between several thread blocks is summed by binary32 adds in the order of their arrival:
+ *     repeated calls of any linear call may differ in the last bit of a result (never by more than binary32 sums in another
+ *     order give).  bpdq_dequant and, above 128 tokens, every linear call return the same bits every time;
  *   - threads: calls that name the same handle (for bpdq_linear_batch: the same first handle,
  *     which keeps the launch plan) and all calls of bpdq_linear_noalloc on one device must be
  *     serialised by the caller; calls on different handles may run concurrently from

@@ -193,14 +193,12 @@ extern "C" int bpdq_create(bpdq_handle_t* hp, int out, int in, int K, int group,
     h->blob_bytes = h->planes_bytes + coefs_bytes(out, in, K, group);
     h->ws_bytes = gemv_workspace_bytes(out, in, K, group, max_M, h->sm_count);
     h->n_counters = gemv_counter_count(out);
-    // Measured on 72B-shaped layers: one two-token pass of the look-up-table kernel (37 us on the largest projections)
-    // beats every other kernel; a second pass (64 us) does not beat the few-token kernel.
-    h->gemv_max_m = 2;
+    // One pass of the look-up-table kernel takes two tokens and does not round the weights.  72B-shaped gate, look-up-table / TMEM kernel,
+    // us back to back: one token 16.3 / 34.2 (K = 2), 23.9 / 38.3 (K = 3), 31.1 / 72.0 (K = 4), two tokens 24.4 / 34.2, 37.5 / 38.3, 45.4 / 72.0;
+    // a second pass loses, three tokens 40.6 / 34.3, 62.3 / 38.3, and so does one with a coefficient group per half block at K = 3, two
+    // tokens (50.3 / 40.0), which stays for its weights' sake.  So does a second pass at K = 4, three tokens: 76.1 / 72.1 (4096 x 4096: 12.9 / 10.0).
+    h->gemv_max_m = K == 4 && group != 64 ? 3 : 2;
     h->few_max_m = 0;                                    // the few-token kernel runs for callers that ask for it
-    // sixteen candidates (the few-token kernel then takes tasks of two row groups): 83-88 us on the largest projections for
-    // 3 to 16 tokens against 77 / 92 us for two look-up-table passes at 3 / 4 tokens (103 / 120 us at g = 64) and 118 us
-    // for the tile kernel
-    if (K == 4) h->gemv_max_m = group == 64 ? 2 : 3;
 
     const size_t stage_x = (size_t)max_M * in * 2, stage_y = (size_t)max_M * out * 2;
     if ((e = cudaMalloc(&h->d_blob, h->blob_bytes)) != cudaSuccess ||

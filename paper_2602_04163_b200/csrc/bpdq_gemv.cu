@@ -682,10 +682,9 @@ bool gemv_supported(int out, int in, int K, int group) {
     return (unsigned long long)planes_bytes(out, in, K) + coefs_bytes(out, in, K, group) < (1ull << 32);
 }
 
-// binary32 row sums: kMaxMT tokens for the look-up-table kernel; up to 64 tokens for the tensor-core kernel's split
-// over the input dimension
+// binary32 row sums: kMaxMT tokens for the look-up-table kernel; up to 128 for the few-token and the TMEM kernel, which share it
 size_t gemv_workspace_bytes(int out, int, int, int, int max_M, int) {
-    const int tokens = max_M < kMaxMT ? kMaxMT : (max_M > 128 ? 128 : max_M);   // the tile kernel's split over the input dimension shares it, up to its largest token tile
+    const int tokens = max_M < kMaxMT ? kMaxMT : (max_M > 128 ? 128 : max_M);
     return (size_t)tokens * out * sizeof(float);
 }
 
