@@ -436,4 +436,5 @@ __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_con
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }
+    if (*abort_flag) linger();
 }

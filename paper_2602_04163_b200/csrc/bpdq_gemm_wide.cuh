@@ -285,4 +285,5 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         tc_fence_after();
         tmem_dealloc(tmem_d, 512);
     }
+    if (*abort_flag) linger();
 }

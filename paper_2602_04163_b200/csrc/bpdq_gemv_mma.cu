@@ -481,6 +481,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_mma_kernel(const __grid_consta
         tsk += rg_end - rg_begin;
     }
     if (pend_li >= 0) hand_over(p.lin[pend_li], pend_begin, pend_end, pend_nsl);
+    if (*abort_flag) bpdq::tma::linger();
 }
 
 template <int K, int MT, bool G64, int NJ, int W, bool EXT>

@@ -75,6 +75,13 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned parity, volatile int* abort_flag, int* status) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status)) != 0;
 }
+// A CTA that gave up may have copies under way, and its shared memory must outlive them: it stays for a millisecond, a thousand times
+// what a copy takes.  (Waiting on the rings' barriers instead cost every launch up to 1 % in registers or polls.)
+constexpr unsigned long long kLingerNanos = 1000000ull;
+__device__ __forceinline__ void linger() {
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < kLingerNanos) {}
+}
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 

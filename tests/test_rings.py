@@ -281,3 +281,14 @@ def test_the_work_split_of_rows_of_different_lengths(driver, blocks, sms):
     out = subprocess.run([driver, str(len(blocks)), str(units), "0", str(sms)], check=True, capture_output=True, text=True).stdout
     grid, whole, cut_begin, cut_units, step = (int(v) for v in out.split())
     assert (whole, cut_begin, cut_units, step) == (0, 0, units, 1) and 1 <= grid <= min(sms, (units + 7) // 8)
+
+
+def test_a_cta_that_gave_up_outlives_its_copies():
+    """The last thing every kernel with bounded waits and copies does: in the tensor-core kernels once all roles have met, in the few-token
+    kernel, whose warps wait for their own copies only, in each warp."""
+    for name in ("bpdq_gemm_ts.cuh", "bpdq_gemm_wide.cuh"):
+        with open(os.path.join(HEADER_DIR, name)) as f:
+            text = f.read()
+        assert re.search(r"__syncthreads\(\);\s*if \(warp == 1\) \{[^}]*\}\s*if \(\*abort_flag\) linger\(\);\s*\}\s*$", text), name
+    with open(os.path.join(HEADER_DIR, "bpdq_gemv_mma.cu")) as f:
+        assert re.search(r"pend_nsl\);\s*if \(\*abort_flag\) bpdq::tma::linger\(\);\s*\}\s*template", f.read())
