@@ -191,10 +191,10 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
     return BPDQ_OK;
 }
 
-template <int K, int BKW>
+template <int K, int BKW, int NG>
 int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaStream_t stream) {
     static bpdq::SmemOptin optin;
-    if (const int rc = bpdq::ensure_smem_optin(gemm_wide_kernel<K, BKW>, optin, h->device, kWideSmem, "gemm"); rc != BPDQ_OK) return rc;
+    if (const int rc = bpdq::ensure_smem_optin(gemm_wide_kernel<K, BKW, NG>, optin, h->device, kWideSmem, "gemm"); rc != BPDQ_OK) return rc;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: cuTensorMapEncodeTiled is not available from this driver");
     const int nrt = (h->out + BM - 1) / BM;
@@ -219,7 +219,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaS
     const long long ntiles = (long long)nrt * ((M + 2 * p.half - 1) / (2 * p.half));
     const int grid = ntiles < h->sm_count ? (int)ntiles : h->sm_count;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kWideThreads); cfg.dynamicSmemBytes = kWideSmem; cfg.stream = stream;
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(WideCfg<K, BKW, NG>::kThreads); cfg.dynamicSmemBytes = kWideSmem; cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     // Short launches: SMs that the kernel before has left set up and fetch packed blocks (a permuted 7B-shaped layer with 777 tokens
     // 512 us, 479 with this and what was changed beside it).  Long ones run into the power limit, and CTAs that wait beside them cost
@@ -227,7 +227,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaS
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = ntiles <= 4LL * h->sm_count ? 1 : 0;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_wide_kernel<K, BKW>, map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_wide_kernel<K, BKW, NG>, map, *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[0]),
                                        *reinterpret_cast<const CUtensorMap*>(h->gemm_maps[1]), p);
     h->launches += 1;
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -239,7 +239,9 @@ template <int K>
 int launch_k(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
     if (M <= kTsMaxM && !bpdq::ts_drain_bound((h->out + BM - 1) / BM, h->in / 128, M, h->sm_count)) return launch_ts<K>(&h, &x, &y, 1, M, stream, false);
     const int half = bpdq::wide_half(M, (h->out + BM - 1) / BM, h->in / 128, K, h->sm_count);
-    return half <= kWideLongHalf ? launch_wide<K, 64>(h, x, y, M, half, stream) : launch_wide<K, 32>(h, x, y, M, half, stream);
+    if constexpr (K < 4)
+        if (bpdq::wide_groups(K, half) == 4) return launch_wide<K, 64, 4>(h, x, y, M, half, stream);
+    return half <= kWideLongHalf ? launch_wide<K, 64, 2>(h, x, y, M, half, stream) : launch_wide<K, 32, 2>(h, x, y, M, half, stream);
 }
 
 // Diagnostic: the library's bounded wait on a barrier that nothing arrives at.  It must give up after its limit, record

@@ -1,27 +1,27 @@
 // Included by bpdq_gemm.cu (inside its unnamed namespace, after the PTX wrappers): the prefill kernel for many tokens.
 //
-// gemm_wide_kernel: one decoded weight stage feeds TWO halves (of up to 256 tokens each) of a token tile.  Two warps issue, each into
-// a 128 x half accumulator of its own (the two halves of TMEM's 512 columns) from the same A stage and its own x half, so a weight is
-// decoded once per tile: the decode's energy is what the 1 kW cap charges (every further plane costs 8-20 %).  TMEM is full with one
-// tile, so the epilogue does not overlap the next tile's MMAs (about 3 % of a 72B-shaped tile's time); producer and decode warps run
+// gemm_wide_kernel: one decoded weight stage feeds a token tile of two halves (of up to 256 tokens each), so a weight is decoded once per tile:
+// the decode's energy is what the 1 kW cap charges (every further plane costs 8-20 %).  Two warps issue, each into an accumulator of its own
+// (the two halves of TMEM's 512 columns).  Halves above 128 tokens: each issuer multiplies every stage with its own half of x.  Up to
+// 128: one issuer multiplies with the whole tile, and tiles alternate between the accumulators, so that one is drained while the other
+// fills.  (An MMA reads 4 KB of A from shared memory: two of 80 tokens take 2 x 52 clocks where one of 160 takes 80.)  Above, TMEM is full with
+// one tile, so the epilogue does not overlap the next tile's MMAs (about 3 % of a 72B-shaped tile's time); producer and decode warps run
 // ahead into the next tile's stages meanwhile.
 //
 // Stages are 64 columns (128-byte swizzle rows) while four of them fit, i.e. for halves of up to 128 tokens, else 32 columns
 // (64-byte rows: five stages of the widest tile): a stage costs its issuers about 330 clocks beside the decode warps that
 // share their schedulers, a block of four 32-column ones 1320, which is more than the MMAs of halves below 160 tokens take.
-// Packed 128-column blocks (two tensor-map boxes each) come in a ring of two to eight.  Roles (640 threads): warps 0 and 3
-// producers (x, packed), warps 1-2 MMA issuers (half 0, half 1), warps 4-11 decode (two groups of four warps, thread =
-// output row, alternating 128-column blocks of the stage sequence, which continues across tiles), warps 12-19 epilogue (four
-// per half).  Barriers per stage: full (both x halves' bytes and one arrival per warp of the owning decode group), empty (one
-// tcgen05.commit per issuer); per packed slot: full_p, empty_p; acc_full (one commit per issuer), acc_empty (one arrival per
+// Packed 128-column blocks (two tensor-map boxes each) come in a ring of two to eight.  Roles (640 threads, 896 with four decode
+// groups): warps 0 and 3 producers (x, packed), warps 1-2 MMA issuers, two or four decode groups of four warps (thread =
+// output row, taking 128-column blocks of the stage sequence in turn, which continues across tiles), eight epilogue warps (four
+// per half).  Barriers per stage: full (both x halves' bytes and one arrival per warp of the owning decode group), two that
+// release it in turn (one tcgen05.commit per issuer); per packed slot: full_p, empty_p; acc_full (one commit per issuer), acc_empty (one arrival per
 // epilogue warp).  All waits are bounded.
 using bpdq::kWideMaxHalf;
 using bpdq::kWideLongHalf;
 using bpdq::kWideSmem;
 constexpr int kWideEpiWarps = 8;
-constexpr int kWideGroups = 2;                                // decode groups, alternating blocks
-constexpr int kWideFirstDecode = 4, kWideFirstEpi = kWideFirstDecode + 4 * kWideGroups;
-constexpr int kWideThreads = 32 * (kWideFirstEpi + kWideEpiWarps);
+constexpr int kWideFirstDecode = 4;
 
 struct WideParams {
     GemmParams g;
@@ -29,10 +29,14 @@ struct WideParams {
     int stages, sp;            // slots of the stage ring and of the packed ring
 };
 
-// BKW: columns per stage, 32 (64-byte swizzle rows) or 64 (128-byte ones).
-template <int K, int BKW> struct WideCfg {
+// BKW: columns per stage, 32 (64-byte swizzle rows) or 64 (128-byte ones).  NG: decode groups (wide_groups, bpdq_rings.h).
+template <int K, int BKW, int NG> struct WideCfg {
     static constexpr int kATile = BM * BKW * 2;                // 8 or 16 KB
     static constexpr int kPerBlock = 128 / BKW;                // stages per packed block
+    static constexpr int kGroups = NG;                         // decode groups; they take blocks in turn
+    static constexpr int kFirstEpi = kWideFirstDecode + 4 * kGroups, kThreads = 32 * (kFirstEpi + kWideEpiWarps);
+    static constexpr bool kWhole = BKW == 64;                  // a MMA takes the whole token tile (two halves of up to 128)
+    static constexpr int kIssuers = kWhole ? 1 : 2;
     static constexpr int kPlaneBytes = bpdq::wide_plane_bytes(K), kCoefBytes = bpdq::wide_coef_bytes(K);
     static constexpr int kBlockBytes = bpdq::wide_block_bytes(K);
     static_assert(kATile == bpdq::wide_a_bytes(BKW), "bytes of a stage's weights");
@@ -46,13 +50,14 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(unsigned addr) {
            ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
-template <int K, int BKW>
-__global__ void __launch_bounds__(kWideThreads, 1)
+template <int K, int BKW, int NG>
+__global__ void __launch_bounds__(WideCfg<K, BKW, NG>::kThreads, 1)
 gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap planes_map,
                  const __grid_constant__ CUtensorMap coefs_map, const WideParams wp) {
     const GemmParams& p = wp.g;
-    using C = WideCfg<K, BKW>;
+    using C = WideCfg<K, BKW, NG>;
     constexpr int kPerBlock = C::kPerBlock;
+    constexpr bool kWhole = C::kWhole;
     const int S = wp.stages, SP = wp.sp, half = wp.half;
     const unsigned bhalf = (unsigned)half * (BKW * 2), stage = C::kATile + 2u * bhalf;
     extern __shared__ unsigned char smem_raw[];
@@ -62,11 +67,16 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     const unsigned p_base = st_base + (unsigned)S * stage;              // SP x packed block
     const unsigned bar_base = p_base + SP * C::kBlockBytes;
     auto full = [&](int s) { return bar_base + 8u * s; };
-    auto empty = [&](int s) { return bar_base + 8u * (S + s); };
-    auto full_p = [&](int s) { return bar_base + 8u * (2 * S + s); };
-    auto empty_p = [&](int s) { return bar_base + 8u * (2 * S + SP + s); };
-    const unsigned acc_full = bar_base + 8u * (2 * S + 2 * SP), acc_empty = acc_full + 8u;
-    unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * (2 * S + 2 * SP + 2));
+    // a stage slot's release: uses of a slot alternate between two barriers (wide_rings, bpdq_rings.h); n = 0, 1, ... counts them
+    auto empty = [&](int s, int n) { return bar_base + 8u * (S + 2 * s + (n & 1)); };
+    auto released = [&](int s, int n) { return empty(s, n - 1); };           // what use n waits for, by parity ((n - 1) >> 1) & 1
+    auto full_p = [&](int s) { return bar_base + 8u * (3 * S + s); };
+    auto empty_p = [&](int s) { return bar_base + 8u * (3 * S + SP + s); };
+    // an accumulator's barriers: one set of both halves' (kIssuers commits), or two that tiles j = 0, 1, ... take in turn
+    auto acc_full = [&](int j) { return bar_base + 8u * (3 * S + 2 * SP + (kWhole ? j & 1 : 0)); };
+    auto acc_empty = [&](int j) { return acc_full(j) + 16u; };
+    auto acc_parity = [&](int j) { return (unsigned)(kWhole ? j >> 1 : j) & 1u; };
+    unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * (3 * S + 2 * SP + 4));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -80,11 +90,11 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(full(s), 1 + 4);                   // the producer (with both x halves' bytes) and four decode warps
-            mbar_init(empty(s), 2);
+            mbar_init(empty(s, 0), C::kIssuers);
+            mbar_init(empty(s, 1), C::kIssuers);
         }
         for (int s = 0; s < SP; ++s) { mbar_init(full_p(s), 1); mbar_init(empty_p(s), 4); }
-        mbar_init(acc_full, 2);
-        mbar_init(acc_empty, kWideEpiWarps);
+        for (int j = 0; j < 2; ++j) { mbar_init(acc_full(j), C::kIssuers); mbar_init(acc_empty(j), kWideEpiWarps); }
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -106,18 +116,17 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         asm volatile("griddepcontrol.wait;" ::: "memory");   // the kernel before this one may have written x
         if (elect_one()) {
             const int boxes = 2 * half <= 256 ? 1 : 2;
-            int s = 0;                                   // stage slot, continuing across tiles
-            unsigned ph = 1u;
+            int s = 0, n = 0;                            // stage slot and its use, continuing across tiles
             bool ok = true;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                 const int tok0 = (tile / nrt) * (2 * half);
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(empty(s), ph, abort_flag, p.status)) { ok = false; break; }
+                    if (!mbar_wait(released(s, n), (unsigned)((n - 1) >> 1) & 1u, abort_flag, p.status)) { ok = false; break; }
                     mbar_expect_tx(full(s), 2u * bhalf);
                     const unsigned bdst = st_base + (unsigned)s * stage + C::kATile;
                     tma_load_2d(bdst, &x_map, kb * BKW, tok0, full(s));
                     if (boxes == 2) tma_load_2d(bdst + bhalf, &x_map, kb * BKW, tok0 + half, full(s));
-                    if (++s == S) { s = 0; ph ^= 1u; }
+                    if (++s == S) { s = 0; ++n; }
                 }
             }
         }
@@ -142,41 +151,40 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         }
         __syncwarp();
     } else if (warp <= 2) {
-        // ---------------- MMA issuers: warp 1 + h multiplies every stage with x half h into accumulator h ----------------
+        // ---------------- MMA issuers: warp 1 + h multiplies every stage with x half h into accumulator h; or warp 1 with all of x ----------------
         // One thread throughout: it has 256 clocks per stage beside the decode warps that share its scheduler, so a stage has
         // one barrier for weights and activations together and nothing in the loop involves the rest of the warp.
-        if (elect_one()) {
-            const unsigned idesc = instr_desc_f16(BM, half);
+        if (warp <= C::kIssuers && elect_one()) {
+            const unsigned idesc = instr_desc_f16(BM, kWhole ? 2 * half : half);
             const int h = warp - 1;
-            const unsigned d = tmem_d + (unsigned)(h * 256);
-            int s = 0, j = 0;
-            unsigned ph = 0u;
+            int s = 0, n = 0, j = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++j) {
                 // the epilogue must have drained the accumulators of the tile before
-                if (!mbar_wait(acc_empty, ((unsigned)j & 1u) ^ 1u, abort_flag, p.status)) break;
+                if (!mbar_wait(acc_empty(j), acc_parity(j) ^ 1u, abort_flag, p.status)) break;
+                const unsigned d = tmem_d + (unsigned)((kWhole ? j & 1 : h) * 256);
                 unsigned more = 0u;
                 for (int kb = 0; kb < nkb; ++kb) {
-                    ok = mbar_wait(full(s), ph, abort_flag, p.status);
+                    ok = mbar_wait(full(s), (unsigned)n & 1u, abort_flag, p.status);
                     if (!ok) break;
                     tc_fence_after();
                     const unsigned a_addr = st_base + (unsigned)s * stage;
-                    const unsigned b_addr = a_addr + C::kATile + (unsigned)h * bhalf;
+                    const unsigned b_addr = a_addr + C::kATile + (kWhole ? 0u : (unsigned)h * bhalf);
                     const uint64_t adesc = BKW == 32 ? smem_desc_sw64(a_addr) : smem_desc_sw128(a_addr);
                     const uint64_t bdesc = BKW == 32 ? smem_desc_sw64(b_addr) : smem_desc_sw128(b_addr);
 #pragma unroll
                     for (int k = 0; k < BKW / 16; ++k)                // 16 columns = 32 bytes further along the swizzled row
                         umma_f16(d, adesc + 2u * k, bdesc + 2u * k, idesc, k == 0 ? more : 1u);
-                    umma_commit(empty(s));
+                    umma_commit(empty(s, n));
                     more = 1u;
-                    if (++s == S) { s = 0; ph ^= 1u; }
+                    if (++s == S) { s = 0; ++n; }
                 }
-                if (ok) umma_commit(acc_full);
+                if (ok) umma_commit(acc_full(j));
             }
         }
         __syncwarp();
-    } else if (warp < kWideFirstEpi) {
-        // ---------------- decode warps: thread = output row; a group takes every other block ----------------
+    } else if (warp < C::kFirstEpi) {
+        // ---------------- decode warps: thread = output row; groups take blocks in turn ----------------
         const int grp = (warp - kWideFirstDecode) >> 2;
         const int rl = ((warp - kWideFirstDecode) & 3) * 32 + lane;     // row inside the tile; row tiles start at multiples of 128
         unsigned a_off[BKW / 8];                         // swizzled byte offset of each 16-byte chunk of this thread's 64- or 128-byte row
@@ -190,12 +198,13 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         // Stage slots are shared by the groups; why their waits by parity are safe stands at wide_rings (bpdq_rings.h).
         const int my_tiles = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
         int s = 0, sp = grp;
-        unsigned ph = 1u, pp = 0u;
-        auto advance = [&](int n) { s += n; while (s >= S) { s -= S; ph ^= 1u; } };
+        int n = 0;
+        unsigned pp = 0u;
+        auto advance = [&](int by) { s += by; while (s >= S) { s -= S; ++n; } };
         advance(kPerBlock * grp);
         bool ok = true;
         const long long nbseq = (long long)my_tiles * nblk;
-        for (long long bseq = grp; bseq < nbseq && ok; bseq += kWideGroups) {
+        for (long long bseq = grp; bseq < nbseq && ok; bseq += C::kGroups) {
             if (!mbar_wait_warp(full_p(sp), pp, abort_flag, p.status)) break;
             const unsigned so = (unsigned)(sp * C::kBlockBytes);
             unsigned a[K][4];
@@ -228,7 +237,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 #pragma unroll
                     for (int u = 0; u < 4; ++u) v8[4 * e + u] = bpdq::decode8<K>(sel[u], tab);
                 }
-                if (!mbar_wait_warp(empty(s), ph, abort_flag, p.status)) { ok = false; break; }
+                if (!mbar_wait_warp(released(s, n), (unsigned)((n - 1) >> 1) & 1u, abort_flag, p.status)) { ok = false; break; }
                 const unsigned dst = st_base + (unsigned)s * stage;
 #pragma unroll
                 for (int ch = 0; ch < BKW / 8; ++ch)
@@ -242,21 +251,21 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 }
                 advance(1);
             }
-            advance(kPerBlock * (kWideGroups - 1));              // the other group's block
-            sp += kWideGroups;
+            advance(kPerBlock * (C::kGroups - 1));              // the other groups' blocks
+            sp += C::kGroups;
             if (sp >= SP) { sp -= SP; pp ^= 1u; }
         }
     } else {
         // ---------------- epilogue warps: four per accumulator ----------------
-        const int quad = warp & 3, h = (warp - kWideFirstEpi) >> 2;   // TMEM lane quadrant this warp may access; half
+        const int quad = warp & 3, h = (warp - C::kFirstEpi) >> 2;   // TMEM lane quadrant this warp may access; half
         const int rl = quad * 32 + lane;
-        const unsigned taddr = tmem_d + ((unsigned)(quad * 32) << 16) + (unsigned)(h * 256);
         const size_t out = (size_t)p.out;
         asm volatile("griddepcontrol.wait;" ::: "memory");   // ... or may still be reading what y overwrites
         int j = 0;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++j) {
-            if (!mbar_wait_warp(acc_full, (unsigned)j & 1u, abort_flag, p.status)) break;
+            if (!mbar_wait_warp(acc_full(j), acc_parity(j), abort_flag, p.status)) break;
             tc_fence_after();
+            const unsigned taddr = tmem_d + ((unsigned)(quad * 32) << 16) + (unsigned)(kWhole ? (j & 1) * 256 + h * half : h * 256);
             const int row0 = (tile % nrt) * BM, tok0 = (tile / nrt) * (2 * half) + h * half;
             const int r = row0 + rl;
             const bool row_ok = r < p.out;
@@ -276,7 +285,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty);       // one arrival per epilogue warp: the accumulators may be overwritten
+            if (lane == 0) mbar_arrive(acc_empty(j));       // one arrival per epilogue warp: the accumulators may be overwritten
         }
     }
     tc_fence_before();

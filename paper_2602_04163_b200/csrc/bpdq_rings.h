@@ -78,31 +78,39 @@ constexpr int wide_release_stage(int stages_per_block) { return stages_per_block
 constexpr int kWideMaxHalf = 256;                             // most tokens of a half tile
 constexpr int kWideLongHalf = 128;                            // ... with 64-column stages
 constexpr int kWideSmem = 227 * 1024;
-constexpr int kWideMinSP = 2, kWideMaxSP = 8, kWideMaxStages = 12;
+constexpr int kWideMaxSP = 8, kWideMaxStages = 12;
 constexpr int wide_plane_bytes(int K) { return K * 2048; }
 constexpr int wide_coef_bytes(int K) { return (K + 1) * 256; }
 constexpr int wide_block_bytes(int K) { return (wide_plane_bytes(K) + 2 * wide_coef_bytes(K) + 1023) / 1024 * 1024; }
 constexpr int wide_a_bytes(int bkw) { return 128 * bkw * 2; }                              // a stage's weights
 constexpr int wide_stage_bytes(int bkw, int half) { return wide_a_bytes(bkw) + 2 * half * bkw * 2; }   // ... and both halves of x
 
+// Decode groups of the prefill kernel.  A group's block is a chain of some 290 instructions per lane; with few tokens the MMAs wait for
+// it, and four groups are faster than two: K = 2, ns per block with halves of 16 / 48 tokens 487 / 517 and 443 / 468, K = 3 857 / 867 and 519 /
+// 572; with 80 and more the two are (K = 2: 606 and 637 with 80, 801 and 828 with 128, the columns of a stage shared by two issuers).  K = 4 needs
+// more registers than four groups leave.
+constexpr int wide_groups(int K, int half) { return half <= 64 && K < 4 ? 4 : 2; }
+
 struct WideRings {
     int stages, sp;                                   // slots of the stage ring and of the packed ring
 };
 
-// `bkw` columns per stage, 32 or 64.  Packed slots: an even number, so that a slot belongs to one of the two decode groups, which
-// has waited for every use of it.  Stage slots are shared by the groups: the group that waits for the release of stage it - S has
-// waited, for the last stage of its block before, it - (stages per block + 1), for MMAs no later than S stages before that one, and MMAs
-// complete in order; so the release before, of stage it - 2 S, is over if S >= stages per block + 1.  The narrowest ring is the
-// widest tile's at K = 4: five stages of 32 columns.
+// `bkw` columns per stage, 32 or 64.  Packed slots: a multiple of the decode groups, so that a slot belongs to one of them, which
+// has waited for every use of it.  Stage slots are shared by the groups.  The group that waits for the release of stage it - S has
+// waited, for the last stage of its block before, it - (groups - 1) * (stages per block) - 1, for MMAs no later than S stages before that
+// one, and MMAs complete in order; uses of a slot are released through two barriers in turn, so the phase before the awaited one is
+// stage it - 3 S, and it is over if 2 S >= (groups - 1) * (stages per block) + 1.  The narrowest rings are three stages of 64 columns with two groups, five
+// of 32 with two, and six of 64 with four.
 constexpr WideRings wide_rings(int K, int bkw, int half) {
-    const int stage = wide_stage_bytes(bkw, half), budget = kWideSmem - kWideMinSP * wide_block_bytes(K) - 2048;   // 2048: alignment slack, barriers
+    const int least = wide_groups(K, half);
+    const int stage = wide_stage_bytes(bkw, half), budget = kWideSmem - least * wide_block_bytes(K) - 2048;   // 2048: alignment slack, barriers
     int stages = budget / stage;
     if (stages > kWideMaxStages) stages = kWideMaxStages;
-    int sp = kWideMinSP + (budget - stages * stage) / wide_block_bytes(K);
-    sp = sp > kWideMaxSP ? kWideMaxSP : sp / 2 * 2;
+    int sp = least + (budget - stages * stage) / wide_block_bytes(K);
+    sp = sp > kWideMaxSP ? kWideMaxSP : sp / least * least;
     return {stages, sp};
 }
-static_assert(wide_rings(4, 32, kWideMaxHalf).stages >= 5 && wide_rings(4, 64, kWideLongHalf).stages >= 3, "the widest tiles");
+static_assert(wide_rings(4, 32, kWideMaxHalf).stages >= 5 && wide_rings(4, 64, kWideLongHalf).stages >= 3 && wide_rings(3, 64, 64).stages >= 5, "the widest tiles");
 
 // Tokens of a half tile: the cut of M tokens into equal tiles that takes the least time by a model of the kernel.  A 128-column
 // block takes 8.5 clocks per token of a half (the MMAs), but no less than the decode and the hand-over of its stages: 1150 clocks

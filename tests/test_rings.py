@@ -292,3 +292,49 @@ def test_a_cta_that_gave_up_outlives_its_copies():
         assert re.search(r"__syncthreads\(\);\s*if \(warp == 1\) \{[^}]*\}\s*if \(\*abort_flag\) linger\(\);\s*\}\s*$", text), name
     with open(os.path.join(HEADER_DIR, "bpdq_gemv_mma.cu")) as f:
         assert re.search(r"pend_nsl\);\s*if \(\*abort_flag\) bpdq::tma::linger\(\);\s*\}\s*template", f.read())
+
+
+def wide_order_two_releases(stages, sp, per_block, blocks, groups, issuers, release):
+    """gemm_wide_kernel with any number of decode groups (group b mod groups takes block b); a stage slot's uses are released
+    through two barriers in turn, so the phase before the awaited one is three uses back."""
+    o = Order()
+
+    def ev(kind, q):
+        return (kind, q) if q >= 0 else None
+    for b in range(blocks):
+        o.event(("packed asked", b), ev("packed asked", b - 1), ev("stored", (b - sp) * per_block + release) if b >= sp else None)
+        o.wait("packed producer", ev("packed asked", b - 1), ev("stored", (b - 2 * sp) * per_block + release) if b >= 2 * sp else None)
+        o.event(("packed landed", b), ("packed asked", b))
+        for it in range(b * per_block, (b + 1) * per_block):
+            o.event(("x asked", it), ev("x asked", it - 1), ev("multiplied", it - stages))
+            o.wait("x producer", ev("x asked", it - 1), ev("multiplied", it - 3 * stages))
+            o.event(("x landed", it), ("x asked", it))
+            before = ev("stored", it - 1) if it % per_block else ev("stored", (b - groups + 1) * per_block - 1)
+            if it % per_block == 0:
+                o.wait("group, packed", before, ev("packed landed", b - sp))
+            o.wait("group, stage", before, ev("multiplied", it - 3 * stages))
+            o.event(("stored", it), before, ("packed landed", b), ev("multiplied", it - stages))
+            for i in range(issuers):
+                o.wait("issuer", ev(f"issued {i}", it - 1), ev("full", it - stages))
+                o.event((f"issued {i}", it), ev(f"issued {i}", it - 1), ("full", it))
+            o.event(("full", it), ("stored", it), ("x landed", it))
+            o.event(("multiplied", it), *((f"issued {i}", it) for i in range(issuers)), ev("multiplied", it - 1))
+    return o
+
+
+def test_rings_of_the_prefill_kernel_with_its_decode_groups(rings):
+    """As above, with the groups that a tile has (four up to halves of 64 tokens below K = 4) and one issuer or two."""
+    (release,) = [r for kind, r in rings if kind == "release"]
+    four = 0
+    for kind, r in rings:
+        if kind != "wide":
+            continue
+        K, half, per_block, stages, sp, left = r
+        groups = 4 if half <= 64 and K < 4 else 2
+        four += groups == 4
+        assert sp % groups == 0 and left >= 1024 + 8 * (3 * stages + 2 * sp + 4) + 8, r
+        o = wide_order_two_releases(stages, sp, per_block, 2 * sp + 2 * stages + 8, groups, 1 if half <= 128 else 2, release[0 if per_block == 4 else 1])
+        assert o.open_waits() == [], r
+    assert four == 12
+    assert wide_order_two_releases(3, 4, 2, 40, 4, 1, 1).open_waits()           # three stages and four groups would not do
+    assert wide_order_two_releases(6, 6, 2, 40, 4, 1, 1).open_waits()           # nor a packed ring that is no multiple of the groups
