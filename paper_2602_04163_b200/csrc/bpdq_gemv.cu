@@ -42,6 +42,7 @@ constexpr int kMaxMT = 2;                             // tokens per pass (64 KB 
 constexpr int kChunkRgs = 8;                          // row groups (of 16 rows) per completion counter
 constexpr int kMiscBytes = 4096;                      // xsum + completion list, at the start of shared memory
 constexpr int kMaxDone = 512;                         // completed chunks handled per batch
+constexpr int kExtPair = 1, kExtBias = 2, kExtPerm = 4;   // what a launch uses beyond plain linears
 
 // One linear of a launch.  A launch covers one or several linears (same K, same token count): their
 // (slice, row group) task spaces are concatenated and every CTA takes a contiguous share of the whole.
@@ -153,10 +154,10 @@ __device__ __forceinline__ float2 unpack2(unsigned long long v) {
     return f;
 }
 
-// EXT: the launch uses an input permutation, a bias or a (gate, up) pair somewhere.  The plain instantiation carries none of
-// that code: the streaming loop sits at the 128-register cap, and the extra live values cost it spills (5 % of the
-// headline, up to 50 % at g = 64) although they are only used outside the loop.
-template <int K, int MT, int D, int W, bool G64, bool EXT>
+// EXT: what the launch uses somewhere of kExtPair, kExtBias, kExtPerm.  An instantiation carries no other code: the streaming loop sits
+// at the 128-register cap, and the extra live values cost it spills (5 % of the headline, up to 50 % at g = 64) although they
+// are only used outside the loop.  Launches with one of pair and bias are common and have instantiations of their own, all else shares one.
+template <int K, int MT, int D, int W, bool G64, int EXT>
 __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_constant__ GemvParams p) {
     constexpr int kThreads = W * 32;
     constexpr int NS = K * MT;                        // look-up streams per step: (plane, token) pairs
@@ -227,8 +228,10 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
         if (nd > 0) {
             __threadfence();
             // items of four consecutive rows; a thread reads several before it writes, so that the
-            // L2 round trips of a CTA that completes many chunks overlap
-            constexpr int kQuads = kChunkRgs * 16 / 4, kAhead = 4;
+            // L2 round trips of a CTA that completes many chunks overlap (two of a pair, which has two sums of each: four spilled
+            // registers of the next segment's weights, 72B-shaped pair with two tokens 119 -> 104 us at K = 3, g = 64, 100 -> 72 at g = 128,
+            // 152 -> 111 at K = 4, g = 64; with one token 34.6 -> 32.7 at K = 2)
+            constexpr int kQuads = kChunkRgs * 16 / 4, kAhead = (EXT & kExtPair) ? 2 : 4;
             const int nitems = nd * MT * kQuads;
             for (int i0 = tid; i0 < nitems; i0 += kThreads * kAhead) {
                 float4 v[kAhead], vb[kAhead];
@@ -247,24 +250,25 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                             live[u] = true;
                             row[u] = r;
                             at[u] = (size_t)(rem / kQuads) * L.out + r;
-                            v[u] = __ldcg(reinterpret_cast<const float4*>((EXT ? L.conv_a : L.ws) + at[u]));
-                            if (EXT && L.conv_b) vb[u] = __ldcg(reinterpret_cast<const float4*>(L.conv_b + at[u]));
+                            v[u] = __ldcg(reinterpret_cast<const float4*>(((EXT & kExtPair) ? L.conv_a : L.ws) + at[u]));
+                            if ((EXT & kExtPair) && L.conv_b) vb[u] = __ldcg(reinterpret_cast<const float4*>(L.conv_b + at[u]));
                         }
                     }
                 }
 #pragma unroll
                 for (int u = 0; u < kAhead; ++u) {
                     if (live[u]) {
-                        if (EXT) {
-                            bpdq::finish_quad(v[u], vb[u], L.bias_a, L.bias_b, L.conv_b != nullptr, row[u]);
-                            if (L.conv_b) __stcg(reinterpret_cast<float4*>(L.conv_b + at[u]), make_float4(0.f, 0.f, 0.f, 0.f));
+                        if (EXT & (kExtPair | kExtBias)) {
+                            const bool pair = (EXT & kExtPair) && L.conv_b != nullptr;
+                            bpdq::finish_quad(v[u], vb[u], (EXT & kExtBias) ? L.bias_a : nullptr, (EXT & kExtBias) ? L.bias_b : nullptr, pair, row[u]);
+                            if (pair) __stcg(reinterpret_cast<float4*>(L.conv_b + at[u]), make_float4(0.f, 0.f, 0.f, 0.f));
                         }
                         const __half2 h01 = __floats2half2_rn(v[u].x, v[u].y), h23 = __floats2half2_rn(v[u].z, v[u].w);
                         uint2 o;
                         o.x = *reinterpret_cast<const unsigned*>(&h01);
                         o.y = *reinterpret_cast<const unsigned*>(&h23);
                         *reinterpret_cast<uint2*>(L.y + at[u]) = o;
-                        __stcg(reinterpret_cast<float4*>((EXT ? L.conv_a : L.ws) + at[u]), make_float4(0.f, 0.f, 0.f, 0.f));
+                        __stcg(reinterpret_cast<float4*>(((EXT & kExtPair) ? L.conv_a : L.ws) + at[u]), make_float4(0.f, 0.f, 0.f, 0.f));
                     }
                 }
             }
@@ -284,7 +288,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                 const int lo = max(rg_begin, ck * kChunkRgs), hi = min(rg_end, (ck + 1) * kChunkRgs);
                 const int size = min(L.nrg, (ck + 1) * kChunkRgs) - ck * kChunkRgs;
                 const unsigned before = atomicAdd(&L.counters[ck], (unsigned)(hi - lo));
-                if (before + (unsigned)(hi - lo) == (unsigned)(size * L.nslices * (EXT ? L.target_mul : 1))) {
+                if (before + (unsigned)(hi - lo) == (unsigned)(size * L.nslices * ((EXT & kExtPair) ? L.target_mul : 1))) {
                     L.counters[ck] = 0u;
                     done[atomicAdd(ndone, 1)] = ck;
                 }
@@ -381,7 +385,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 xraw[m][u] = col >= L.in ? 0u
-                             : !(EXT && L.perm) ? ldg_x4(L.x + (size_t)m * L.in + col + 8 * u)
+                             : !((EXT & kExtPerm) && L.perm) ? ldg_x4(L.x + (size_t)m * L.in + col + 8 * u)
                                          : (unsigned)ldg_x2(L.x + (size_t)m * L.in + __ldg(L.perm + col + 8 * u)) |
                                                ((unsigned)ldg_x2(L.x + (size_t)m * L.in + __ldg(L.perm + col + 8 * u + 1)) << 16);
         if (!early) {
@@ -576,7 +580,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
     if (pend_li >= 0) hand_over(p.lin[pend_li], pend_begin, pend_end);
 }
 
-template <int K, int MT, int D, int W, bool G64, bool EXT>
+template <int K, int MT, int D, int W, bool G64, int EXT>
 int launch_cfg(bpdq_handle_s* h, GemvParams p, cudaStream_t stream) {
     static bpdq::SmemOptin optin;
     const int smem = 65536 + MT * kTableBytes;        // tables start at the first 64 KB boundary of the shared window
@@ -630,11 +634,18 @@ int launch_cfg(bpdq_handle_s* h, GemvParams p, cudaStream_t stream) {
 // for every K); one where two tasks do not fit the register file (K = 4).
 template <int K, int MT>
 int launch_one(bpdq_handle_s* h, const GemvParams& p, cudaStream_t stream) {
-    bool ext = false;
-    for (int k = 0; k < p.n; ++k) ext = ext || p.lin[k].perm || p.lin[k].bias_a || p.lin[k].conv_b;
+    int ext = 0;
+    for (int k = 0; k < p.n; ++k)
+        ext |= (p.lin[k].conv_b ? kExtPair : 0) | (p.lin[k].bias_a || p.lin[k].bias_b ? kExtBias : 0) | (p.lin[k].perm ? kExtPerm : 0);
     constexpr int D = K <= 3 ? 2 : 1;
-    if (p.lin[0].group == 64) return ext ? launch_cfg<K, MT, D, 16, true, true>(h, p, stream) : launch_cfg<K, MT, D, 16, true, false>(h, p, stream);
-    return ext ? launch_cfg<K, MT, D, 16, false, true>(h, p, stream) : launch_cfg<K, MT, D, 16, false, false>(h, p, stream);
+    constexpr int kAll = kExtPair | kExtBias | kExtPerm;
+    if (p.lin[0].group == 64)
+        return ext == 0 ? launch_cfg<K, MT, D, 16, true, 0>(h, p, stream)
+             : ext == kExtPair ? launch_cfg<K, MT, D, 16, true, kExtPair>(h, p, stream)
+             : ext == kExtBias ? launch_cfg<K, MT, D, 16, true, kExtBias>(h, p, stream) : launch_cfg<K, MT, D, 16, true, kAll>(h, p, stream);
+    return ext == 0 ? launch_cfg<K, MT, D, 16, false, 0>(h, p, stream)
+         : ext == kExtPair ? launch_cfg<K, MT, D, 16, false, kExtPair>(h, p, stream)
+         : ext == kExtBias ? launch_cfg<K, MT, D, 16, false, kExtBias>(h, p, stream) : launch_cfg<K, MT, D, 16, false, kAll>(h, p, stream);
 }
 
 void fill_linear(GemvLinear& L, const bpdq_handle_s* h) {
