@@ -14,7 +14,7 @@
 // groups; it builds the 64 chunk tables of its slice once (64 KB per token) and then streams
 // planes.  A warp takes 16 rows x 4 blocks per task: lane (h, a) = (lane/16, lane%16) owns row a
 // and the two blocks of parity h.  Its 16-byte plane units and binary16 coefficients come straight
-// from global memory into registers (16 lanes x 16 bytes = 256 contiguous bytes per request), two
+// from global memory into registers (16 lanes x 16 bytes = 256 contiguous bytes per request), up to three
 // tasks ahead, so that HBM latency is covered by loads in flight and shared memory
 // carries nothing but the look-ups.  The blob stores, at byte p of row r, the 8-column chunk
 // ("logical byte") (p + r) mod 16, and table entries are laid out as [entry][slot],
@@ -435,9 +435,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
 
         // ---- stream the row groups of this slice ----
         // n_next >= 0: the task that takes this one's registers; each half is requested as soon as the half it
-        // replaces has been used, so that nearly D tasks per warp are in flight rather than D - 1 (three planes
-        // for two tokens keep the whole-task request: the other order costs that instantiation spills)
-        constexpr bool kReloadHalves = !(K == 3 && MT == 2);
+        // replaces has been used, so that nearly D tasks per warp are in flight rather than D - 1
         auto process_task = [&](Task<K, NG>& tk, int n, int n_next) {
             float yacc[MT];
 #pragma unroll
@@ -545,7 +543,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                         for (int m = 0; m < MT; ++m) yacc[m] = fmaf(ci, S[i * MT + m], yacc[m]);
                     }
                 }
-                if (kReloadHalves && n_next >= 0) load_half(tk, n_next, q);
+                if (n_next >= 0) load_half(tk, n_next, q);
             }
             // the two half-warps hold the even-block and odd-block parts of the same 16 rows
 #pragma unroll
@@ -560,14 +558,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
 #pragma unroll
             for (int d = 0; d < D; ++d) {
                 const int n = n0 + d;
-                if (n < ntask) {                      // warp-uniform
-                    if constexpr (kReloadHalves) {
-                        process_task(tk[d], n, n + D < ntask ? n + D : -1);
-                    } else {
-                        process_task(tk[d], n, -1);
-                        if (n + D < ntask) load_task(tk[d], n + D);
-                    }
-                }
+                if (n < ntask) process_task(tk[d], n, n + D < ntask ? n + D : -1);      // warp-uniform
             }
         }
 
@@ -630,22 +621,33 @@ int launch_cfg(bpdq_handle_s* h, GemvParams p, cudaStream_t stream) {
     return BPDQ_OK;
 }
 
-// Tasks kept in flight per lane: two (a third costs more in registers than it hides in latency: measured slower
-// for every K); one where two tasks do not fit the register file (K = 4).
+// Warps of a CTA and tasks kept in flight per lane.  Sixteen warps of 128 registers with two tasks, or with one where two do not fit the
+// registers; eight of 255 where the planes of one task already crowd 128.  72B-shaped gate, us: K = 3, two tokens 37.9 with two tasks (requested
+// as a whole; 38.8 by halves), 36.3 with one, at g = 64 50.3 (55.4) and 41.9; K = 4, one token 32.0 with one task, 30.9 with eight warps and
+// three; K = 4, g = 64, two tokens 59.0 and, with eight warps and two tasks, 54.8.  All others are slower in the other forms (K = 2, one
+// token 17.9 with sixteen warps and two tasks, 20.9 with one, 21.0 with eight warps and three; K = 4, g = 64, one token: the pair 68.8 and 72.5).
+template <int K, int MT, bool G64> struct Flight {
+    static constexpr bool kFew = K == 4 && (MT == 2) == G64;
+    static constexpr int W = kFew ? 8 : 16, D = kFew ? (G64 ? 2 : 3) : K == 4 || (K == 3 && MT == 2) ? 1 : 2;
+};
+
+template <int K, int MT, bool G64>
+int launch_ext(bpdq_handle_s* h, const GemvParams& p, cudaStream_t stream, int ext) {
+    constexpr int D = Flight<K, MT, G64>::D, W = Flight<K, MT, G64>::W;
+    switch (ext) {
+        case 0: return launch_cfg<K, MT, D, W, G64, 0>(h, p, stream);
+        case kExtPair: return launch_cfg<K, MT, D, W, G64, kExtPair>(h, p, stream);
+        case kExtBias: return launch_cfg<K, MT, D, W, G64, kExtBias>(h, p, stream);
+        default: return launch_cfg<K, MT, D, W, G64, kExtPair | kExtBias | kExtPerm>(h, p, stream);
+    }
+}
+
 template <int K, int MT>
 int launch_one(bpdq_handle_s* h, const GemvParams& p, cudaStream_t stream) {
     int ext = 0;
     for (int k = 0; k < p.n; ++k)
         ext |= (p.lin[k].conv_b ? kExtPair : 0) | (p.lin[k].bias_a || p.lin[k].bias_b ? kExtBias : 0) | (p.lin[k].perm ? kExtPerm : 0);
-    constexpr int D = K <= 3 ? 2 : 1;
-    constexpr int kAll = kExtPair | kExtBias | kExtPerm;
-    if (p.lin[0].group == 64)
-        return ext == 0 ? launch_cfg<K, MT, D, 16, true, 0>(h, p, stream)
-             : ext == kExtPair ? launch_cfg<K, MT, D, 16, true, kExtPair>(h, p, stream)
-             : ext == kExtBias ? launch_cfg<K, MT, D, 16, true, kExtBias>(h, p, stream) : launch_cfg<K, MT, D, 16, true, kAll>(h, p, stream);
-    return ext == 0 ? launch_cfg<K, MT, D, 16, false, 0>(h, p, stream)
-         : ext == kExtPair ? launch_cfg<K, MT, D, 16, false, kExtPair>(h, p, stream)
-         : ext == kExtBias ? launch_cfg<K, MT, D, 16, false, kExtBias>(h, p, stream) : launch_cfg<K, MT, D, 16, false, kAll>(h, p, stream);
+    return p.lin[0].group == 64 ? launch_ext<K, MT, true>(h, p, stream, ext) : launch_ext<K, MT, false>(h, p, stream, ext);
 }
 
 void fill_linear(GemvLinear& L, const bpdq_handle_s* h) {

@@ -150,3 +150,33 @@ def test_a_wait_that_runs_out_is_reported_and_leaves_the_handle_usable():
     h.bpdq_get_status(sp)                                                # reading the word cleared it
     for M, kernel in ((1, binding.KERNEL_GEMV), (5, binding.KERNEL_FEW), (40, binding.KERNEL_GEMM)):
         G.check_linear(h, bits, coef, synth.activations(602 + M, M, 640), 128, kernel, what=f"after the probe M={M}")
+
+
+@pytest.mark.parametrize("K,g,out,in_,M", [(4, 128, 4112, 1152, 1), (4, 64, 4112, 1152, 2), (3, 128, 4112, 1152, 2), (3, 64, 20000, 640, 2), (4, 64, 16, 128, 2),
+                                           (4, 128, 30000, 512, 1)])
+def test_lut_kernel_with_other_flights(K, g, out, in_, M):
+    """Formats whose instantiations have eight warps, or one task in flight where there are two registers' worth: ragged slices, a single
+    task, a hundred tasks per warp.  Plain, with a bias, and the gated unit over two of them."""
+    layers = [G.make_layer(880 + k, out, in_, K, g, max_M=M) for k in range(2)]
+    x = synth.activations(881, M, in_)
+    rows = np.unique(np.concatenate([np.arange(0, out, 1 + out // 200), [out - 16, out - 1]]))
+    refs = [oracle.linear(b[:, rows], c[:, rows], x, g) for _, b, c in layers]
+    for (h, _, _), (y_ref, a_ref) in zip(layers, refs):
+        G.assert_linear_close(G.run_linear(h, x, binding.KERNEL_GEMV)[:, rows], y_ref, a_ref, "plain")
+    (hg, _, _), (hu, _, _) = layers
+    (gy, ga), (uy, ua) = refs
+    want = oracle.swiglu(gy, uy)
+    dg, du = G.TOL_REL * ga + G.TOL_ABS, G.TOL_REL * ua + G.TOL_ABS
+    silu_g = oracle.swiglu(gy, np.ones_like(gy))
+    # first-order propagation of the two linears' accepted errors through the unit (|silu'| <= 1.1), plus the output's rounding
+    bound = 1.1 * (np.abs(uy) + du) * dg + (np.abs(silu_g) + 1.1 * dg) * du + 2.0 ** -10 * np.abs(want) + 1e-4
+    xt = G.x_tensor(x)
+    for _ in range(2):
+        out_t = torch.full((M, out), float("nan"), dtype=torch.float16, device="cuda")
+        binding.bpdq_gate_up_swiglu(hg, hu, xt.data_ptr(), out_t.data_ptr(), M, G.stream_ptr())
+        torch.cuda.synchronize()
+        assert np.all(np.abs(out_t.cpu().numpy().astype(np.float64)[:, rows] - want) <= bound)
+    bias = np.random.RandomState(3).randn(out).astype(np.float16)
+    hg.bpdq_set_bias(bias.view(np.uint16))
+    b = bias[rows].astype(np.float64)
+    G.assert_linear_close(G.run_linear(hg, x, binding.KERNEL_GEMV)[:, rows], gy + b, ga + np.abs(b), "bias")
