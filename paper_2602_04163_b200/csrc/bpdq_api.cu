@@ -55,31 +55,52 @@ __global__ void gather_kernel(const __grid_constant__ GatherParams p) {
     }
 }
 
-// Activations in stored-column order: dst[m][j] = src[m][perm[j]].  A CTA takes a token: its row comes in once with full
-// lines and is picked apart in shared memory (2-byte reads from global memory at random took 45 us for 777 x 18944 values).
-// Rows that do not fit shared memory are read from L2.
-template <bool STAGED>
+// Activations in stored-column order: dst[m][j] = src[m][perm[j]].  A CTA takes kTokens tokens: their rows come in once with full
+// lines and are picked apart in shared memory (2-byte reads from global memory at random took 45 us for 777 x 18944 values).  Two
+// tokens lie side by side there, so that an index and a random access (3.5 bank conflicts on average) serve both.
+// Rows that do not fit shared memory are read from L2 (kTokens = 0).
+template <int kTokens>
 __global__ void __launch_bounds__(512) gather_columns_kernel(const __half* __restrict__ src, const int* __restrict__ perm, __half* __restrict__ dst,
                                                              int M, int in) {
     extern __shared__ __align__(16) unsigned char gather_smem[];
-    const __half* staged = reinterpret_cast<const __half*>(gather_smem);
+    constexpr int kStep = kTokens == 2 ? 2 : 1;
     const int chunks = in / 8;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");            // the kernel before this one may have written src, or still read dst
-    for (int m = blockIdx.x; m < M; m += gridDim.x) {
+    for (int m = blockIdx.x * kStep; m < M; m += gridDim.x * kStep) {
         const __half* row = src + (size_t)m * in;
-        if (STAGED) {
-            for (int c = threadIdx.x; c < chunks; c += blockDim.x)
-                reinterpret_cast<uint4*>(gather_smem)[c] = __ldcg(reinterpret_cast<const uint4*>(row) + c);
+        const bool second = kTokens == 2 && m + 1 < M;
+        if (kTokens > 0) {
+            for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
+                const uint4 v = __ldcg(reinterpret_cast<const uint4*>(row) + c);
+                if (kTokens == 1) {
+                    reinterpret_cast<uint4*>(gather_smem)[c] = v;
+                } else {
+                    const uint4 w = second ? __ldcg(reinterpret_cast<const uint4*>(row + in) + c) : v;
+                    uint4* to = reinterpret_cast<uint4*>(gather_smem) + 2 * c;
+                    to[0] = make_uint4(__byte_perm(v.x, w.x, 0x5410u), __byte_perm(v.x, w.x, 0x7632u), __byte_perm(v.y, w.y, 0x5410u), __byte_perm(v.y, w.y, 0x7632u));
+                    to[1] = make_uint4(__byte_perm(v.z, w.z, 0x5410u), __byte_perm(v.z, w.z, 0x7632u), __byte_perm(v.w, w.w, 0x5410u), __byte_perm(v.w, w.w, 0x7632u));
+                }
+            }
             __syncthreads();
         }
-        const __half* from = STAGED ? staged : row;
         for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
             const int4 p0 = __ldg(reinterpret_cast<const int4*>(perm + c * 8)), p1 = __ldg(reinterpret_cast<const int4*>(perm + c * 8 + 4));
-            __align__(16) __half v[8] = {from[p0.x], from[p0.y], from[p0.z], from[p0.w], from[p1.x], from[p1.y], from[p1.z], from[p1.w]};
-            *reinterpret_cast<uint4*>(dst + (size_t)m * in + c * 8) = *reinterpret_cast<const uint4*>(v);
+            uint4* out = reinterpret_cast<uint4*>(dst + (size_t)m * in + c * 8);
+            if (kTokens == 2) {
+                const unsigned* both = reinterpret_cast<const unsigned*>(gather_smem);
+                const unsigned b[8] = {both[p0.x], both[p0.y], both[p0.z], both[p0.w], both[p1.x], both[p1.y], both[p1.z], both[p1.w]};
+                *out = make_uint4(__byte_perm(b[0], b[1], 0x5410u), __byte_perm(b[2], b[3], 0x5410u), __byte_perm(b[4], b[5], 0x5410u), __byte_perm(b[6], b[7], 0x5410u));
+                if (second)
+                    *reinterpret_cast<uint4*>(dst + (size_t)(m + 1) * in + c * 8) =
+                        make_uint4(__byte_perm(b[0], b[1], 0x7632u), __byte_perm(b[2], b[3], 0x7632u), __byte_perm(b[4], b[5], 0x7632u), __byte_perm(b[6], b[7], 0x7632u));
+            } else {
+                const __half* from = kTokens == 1 ? reinterpret_cast<const __half*>(gather_smem) : row;
+                __align__(16) __half v[8] = {from[p0.x], from[p0.y], from[p0.z], from[p0.w], from[p1.x], from[p1.y], from[p1.z], from[p1.w]};
+                *out = *reinterpret_cast<const uint4*>(v);
+            }
         }
-        if (STAGED) __syncthreads();
+        if (kTokens > 0) __syncthreads();
     }
 }
 
@@ -471,19 +492,25 @@ struct PdlConfig {
 };
 
 int launch_gather_columns(bpdq_handle_s* h, const void* x, int M, cudaStream_t stream) {
-    const size_t smem = (size_t)h->in * 2;
-    const bool staged = smem <= (size_t)h->smem_optin && smem <= 200 * 1024;
+    // two tokens per CTA where their rows fit and every SM still has one; else one, else none in shared memory
+    const size_t room = (size_t)h->smem_optin < 200 * 1024 ? (size_t)h->smem_optin : 200 * 1024, row = (size_t)h->in * 2;
+    const int tokens = 2 * row <= room && M >= 2 * h->sm_count ? 2 : row <= room ? 1 : 0;
+    const size_t smem = tokens * row;
     unsigned blocks = 4u * (unsigned)h->sm_count;
-    if ((long long)M < (long long)blocks) blocks = (unsigned)M;
-    static SmemOptin optin;
-    if (staged)
-        if (const int rc = ensure_smem_optin(gather_columns_kernel<true>, optin, h->device, (int)smem, "gather"); rc != BPDQ_OK) return rc;
-    PdlConfig c(blocks, 512, staged ? smem : 0, stream);
+    const int groups = tokens == 2 ? (M + 1) / 2 : M;
+    if ((long long)groups < (long long)blocks) blocks = (unsigned)groups;
+    static SmemOptin optin1, optin2;
+    if (tokens == 2)
+        if (const int rc = ensure_smem_optin(gather_columns_kernel<2>, optin2, h->device, (int)smem, "gather"); rc != BPDQ_OK) return rc;
+    if (tokens == 1)
+        if (const int rc = ensure_smem_optin(gather_columns_kernel<1>, optin1, h->device, (int)smem, "gather"); rc != BPDQ_OK) return rc;
+    PdlConfig c(blocks, 512, smem, stream);
     const __half* src = static_cast<const __half*>(x);
     __half* dst = static_cast<__half*>(h->d_xperm);
     const int* perm = h->d_perm;
-    cudaError_t e = staged ? cudaLaunchKernelEx(&c.cfg, gather_columns_kernel<true>, src, perm, dst, M, h->in)
-                           : cudaLaunchKernelEx(&c.cfg, gather_columns_kernel<false>, src, perm, dst, M, h->in);
+    cudaError_t e = tokens == 2 ? cudaLaunchKernelEx(&c.cfg, gather_columns_kernel<2>, src, perm, dst, M, h->in)
+                  : tokens == 1 ? cudaLaunchKernelEx(&c.cfg, gather_columns_kernel<1>, src, perm, dst, M, h->in)
+                                : cudaLaunchKernelEx(&c.cfg, gather_columns_kernel<0>, src, perm, dst, M, h->in);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(BPDQ_ERR_CUDA, "gather launch: %s", cudaGetErrorString(e));
     h->launches += 1;

@@ -176,3 +176,15 @@ def test_permuted_rows_staged_and_not(in_, M):
         assert np.array_equal(got, want)
     else:
         assert np.allclose(got, want, rtol=2.0 ** -9, atol=1e-4)
+
+
+@pytest.mark.parametrize("in_,M", [(128, 297), (1152, 701), (50304, 300), (51328, 300)])
+def test_permuted_rows_two_tokens_side_by_side(in_, M):
+    """The gather with two tokens per CTA: an odd number of tokens, the longest rows that two fit of, and the shortest that they do not."""
+    K, g, out = 1, 128, 16
+    h = binding.Handle(out, in_, K, g, None, 78, M)
+    x = synth.activations(79, M, in_)
+    perm = np.random.RandomState(80).permutation(in_).astype(np.int32)
+    want = G.run_linear(h, np.ascontiguousarray(x[:, perm]), binding.KERNEL_GEMM)
+    h.bpdq_set_input_permutation(perm)
+    assert np.array_equal(G.run_linear(h, x, binding.KERNEL_GEMM), want)
