@@ -215,9 +215,9 @@ extern "C" int bpdq_create(bpdq_handle_t* hp, int out, int in, int K, int group,
     h->ws_bytes = gemv_workspace_bytes(out, in, K, group, max_M, h->sm_count);
     h->n_counters = gemv_counter_count(out);
     // One pass of the look-up-table kernel takes two tokens and does not round the weights.  72B-shaped gate, look-up-table / TMEM kernel,
-    // us back to back: one token 16.3 / 34.2 (K = 2), 23.9 / 38.3 (K = 3), 31.1 / 72.0 (K = 4), two tokens 24.4 / 34.2, 37.5 / 38.3, 45.4 / 72.0;
+    // us back to back: one token 16.3 / 34.2 (K = 2), 23.9 / 38.3 (K = 3), 30.9 / 72.0 (K = 4), two tokens 24.4 / 34.2, 36.3 / 38.3, 45.4 / 72.0;
     // a second pass loses, three tokens 40.6 / 34.3, 62.3 / 38.3, and so does one with a coefficient group per half block at K = 3, two
-    // tokens (50.3 / 40.0), which stays for its weights' sake.  So does a second pass at K = 4, three tokens: 76.1 / 72.1 (4096 x 4096: 12.9 / 10.0).
+    // tokens (41.9 / 40.0), which stays for its weights' sake.  So does a second pass at K = 4, three tokens: 76.1 / 72.1 (4096 x 4096: 12.9 / 10.0).
     h->gemv_max_m = K == 4 && group != 64 ? 3 : 2;
     h->few_max_m = 0;                                    // the few-token kernel runs for callers that ask for it
 

@@ -115,11 +115,12 @@ static_assert(wide_rings(4, 32, kWideMaxHalf).stages >= 5 && wide_rings(4, 64, k
 // Tokens of a half tile: the cut of M tokens into equal tiles that takes the least time by a model of the kernel.  A 128-column
 // block takes 8.5 clocks per token of a half (the MMAs), but no less than the decode and the hand-over of its stages: 1150 clocks
 // with 64-column stages, 1320 with 32-column ones (1600 and 1700 with sixteen candidates); a tile is paid for in whole rounds over
-// the SMs.  Measured, ns per block with one tile per SM, 12288 and 4096 columns, back to back (the 1 kW cap slows the larger halves; g = 128):
+// the SMs.  Measured, ns per block with one tile per SM, 12288 and 4096 columns, back to back (the 1 kW cap slows the larger halves; g = 128;
+// K = 1 and 4 up to 128 from the kernel with two MMAs per 16 columns):
 //   half      16    48    80   112   128 |  144   160   192   224   256
 //   K = 1    479   524   697   764   825 | 1006  1055  1144  1326  1541
-//   K = 2    507   548   658   800   872 | 1179  1121  1232  1473  1602
-//   K = 3    830   866   779   948  1028 | 1311  1307  1324  1503  1722
+//   K = 2    443   468   654   774   831 | 1179  1121  1232  1473  1602
+//   K = 3    519   572   746   906   936 | 1311  1307  1324  1503  1722
 //   K = 4   1069  1078   974  1167  1517 | 1383  1453  1578  1632  1833
 // Always 512 tokens per tile left most SMs idle on short token counts: 3584 x 18944 (28 row tiles) with 777 tokens took 199 us in
 // 56 tiles, in 140 it takes 94.
