@@ -37,6 +37,7 @@ template <int K, int BKW, int NG> struct WideCfg {
     static constexpr int kFirstEpi = kWideFirstDecode + 4 * kGroups, kThreads = 32 * (kFirstEpi + kWideEpiWarps);
     static constexpr bool kWhole = BKW == 64;                  // a MMA takes the whole token tile (two halves of up to 128)
     static constexpr int kIssuers = kWhole ? 1 : 2;
+    static constexpr int kAccs = kWhole ? 2 : 1;               // accumulator barrier sets, which tiles take in turn
     static constexpr int kPlaneBytes = bpdq::wide_plane_bytes(K), kCoefBytes = bpdq::wide_coef_bytes(K);
     static constexpr int kBlockBytes = bpdq::wide_block_bytes(K);
     static_assert(kATile == bpdq::wide_a_bytes(BKW), "bytes of a stage's weights");
@@ -73,9 +74,9 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     auto full_p = [&](int s) { return bar_base + 8u * (3 * S + s); };
     auto empty_p = [&](int s) { return bar_base + 8u * (3 * S + SP + s); };
     // an accumulator's barriers: one set of both halves' (kIssuers commits), or two that tiles j = 0, 1, ... take in turn
-    auto acc_full = [&](int j) { return bar_base + 8u * (3 * S + 2 * SP + (kWhole ? j & 1 : 0)); };
+    auto acc_full = [&](int j) { return bar_base + 8u * (3 * S + 2 * SP + j % C::kAccs); };
     auto acc_empty = [&](int j) { return acc_full(j) + 16u; };
-    auto acc_parity = [&](int j) { return (unsigned)(kWhole ? j >> 1 : j) & 1u; };
+    auto acc_parity = [&](int j) { return (unsigned)(j / C::kAccs) & 1u; };
     unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * (3 * S + 2 * SP + 4));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -94,7 +95,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             mbar_init(empty(s, 1), C::kIssuers);
         }
         for (int s = 0; s < SP; ++s) { mbar_init(full_p(s), 1); mbar_init(empty_p(s), 4); }
-        for (int j = 0; j < 2; ++j) { mbar_init(acc_full(j), C::kIssuers); mbar_init(acc_empty(j), kWideEpiWarps); }
+        for (int j = 0; j < C::kAccs; ++j) { mbar_init(acc_full(j), C::kIssuers); mbar_init(acc_empty(j), kWideEpiWarps); }   // a live barrier must not be initialised again
         *abort_flag = 0;
         fence_barrier_init();
     }

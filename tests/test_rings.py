@@ -338,3 +338,73 @@ def test_rings_of_the_prefill_kernel_with_its_decode_groups(rings):
     assert four == 12
     assert wide_order_two_releases(3, 4, 2, 40, 4, 1, 1).open_waits()           # three stages and four groups would not do
     assert wide_order_two_releases(6, 6, 2, 40, 4, 1, 1).open_waits()           # nor a packed ring that is no multiple of the groups
+
+
+BARRIERS = r"""
+#include <cstdio>
+#include "bpdq_rings.h"
+constexpr int kWideEpiWarps = %(epi)s;
+template <int BKW> struct Cfg {
+    %(config)s
+};
+static void mbar_init(unsigned addr, int count) { printf("init %%u %%d\n", addr, count); }
+static void fence_barrier_init() {}
+template <int BKW> void layout(int K, int half) {
+    using C = Cfg<BKW>;
+    constexpr bool kWhole = C::kWhole;
+    (void)kWhole;
+    const bpdq::WideRings r = bpdq::wide_rings(K, BKW, half);
+    const int S = r.stages, SP = r.sp, tid = 0;
+    const unsigned bar_base = 0;
+    int aborted = 0, *abort_flag = &aborted;
+    printf("tile %%d %%d\n", K, half);
+    %(names)s
+    %(init)s
+    // what the roles use: three uses of every stage slot, both packed barriers, the accumulators of six tiles
+    for (int n = 0; n < 3; ++n)
+        for (int s = 0; s < S; ++s) printf("use %%u\nuse %%u\nuse %%u\n", full(s), empty(s, n), released(s, n));
+    for (int s = 0; s < SP; ++s) printf("use %%u\nuse %%u\n", full_p(s), empty_p(s));
+    for (int j = 0; j < 6; ++j) printf("use %%u\nuse %%u\nacc %%u %%u %%u\n", acc_full(j), acc_empty(j), acc_full(j), acc_empty(j), acc_parity(j));
+    printf("end %%d\n", %(end)s);
+}
+int main() {
+    for (int K = 1; K <= 4; ++K)
+        for (int half = 16; half <= bpdq::kWideMaxHalf; half += 16)
+            if (half <= bpdq::kWideLongHalf) layout<64>(K, half); else layout<32>(K, half);
+    return 0;
+}
+"""
+
+
+def test_every_barrier_of_the_prefill_kernel_is_initialised_once(tmp_path):
+    """The kernel's own lines that lay out and initialise its barriers, run on the host: every address that a role uses is initialised, none
+    twice (a second initialisation of a live mbarrier is undefined), all lie below the TMEM address, and one accumulator's barriers serve every
+    tile, or two sets serve tiles in turn."""
+    with open(os.path.join(HEADER_DIR, "bpdq_gemm_wide.cuh")) as f:
+        text = f.read()
+    kernel = text[text.index("gemm_wide_kernel(const"):]
+    parts = {
+        "epi": re.search(r"kWideEpiWarps = (\d+);", text).group(1),
+        "config": "\n".join(re.findall(r"static constexpr (?:bool kWhole|int kIssuers|int kAccs) = [^;]*;", text)),
+        "names": kernel[kernel.index("auto full ="):kernel.index("unsigned* tmem_slot")],
+        "init": re.search(r"if \(tid == 0\) \{.*?fence_barrier_init\(\);\s*\}", kernel, re.S).group(),
+        "end": re.search(r"\(bar_base - base\) \+ (8 \* \([^;]*\))\);", kernel).group(1),
+    }
+    src, exe = tmp_path / "barriers.cpp", tmp_path / "barriers"
+    src.write_text(BARRIERS % parts)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-I", HEADER_DIR, str(src), "-o", str(exe)], check=True)
+    out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
+    tiles = out.split("tile ")[1:]
+    assert len(tiles) == 64
+    for tile in tiles:
+        rows = [line.split() for line in tile.splitlines()]
+        half = int(rows[0][1])
+        inits = [int(r[1]) for r in rows if r[0] == "init"]
+        used = {int(r[1]) for r in rows if r[0] == "use"}
+        (end,) = [int(r[1]) for r in rows if r[0] == "end"]
+        assert len(set(inits)) == len(inits) and used == set(inits), rows[0]
+        assert all(a % 8 == 0 and a + 8 <= end for a in used), rows[0]
+        acc = [tuple(int(v) for v in r[1:]) for r in rows if r[0] == "acc"]
+        sets = 2 if half <= 128 else 1
+        assert [a[:2] for a in acc] == [acc[j % sets][:2] for j in range(6)] and len({a[:2] for a in acc}) == sets
+        assert [a[2] for a in acc] == [j // sets % 2 for j in range(6)]
