@@ -6,6 +6,7 @@
 
 #include "bpdq_internal.h"
 #include "bpdq_finish.cuh"
+#include "bpdq_rings.h"
 
 #include <cuda_fp16.h>
 
@@ -492,10 +493,8 @@ struct PdlConfig {
 };
 
 int launch_gather_columns(bpdq_handle_s* h, const void* x, int M, cudaStream_t stream) {
-    // two tokens per CTA where their rows fit and every SM still has one; else one, else none in shared memory
-    const size_t room = (size_t)h->smem_optin < 200 * 1024 ? (size_t)h->smem_optin : 200 * 1024, row = (size_t)h->in * 2;
-    const int tokens = 2 * row <= room && M >= 2 * h->sm_count ? 2 : row <= room ? 1 : 0;
-    const size_t smem = tokens * row;
+    const int tokens = gather_tokens(h->in, M, h->sm_count, h->smem_optin);
+    const size_t smem = (size_t)tokens * h->in * 2;
     unsigned blocks = 4u * (unsigned)h->sm_count;
     const int groups = tokens == 2 ? (M + 1) / 2 : M;
     if ((long long)groups < (long long)blocks) blocks = (unsigned)groups;

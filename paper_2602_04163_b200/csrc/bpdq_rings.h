@@ -1,5 +1,5 @@
 // Host side of the tensor-core kernels (plain C++, no CUDA): lengths of the rings in shared memory that their roles hand blocks
-// round in, the split of the work over CTAs, the size of token tiles.
+// round in, the split of the work over CTAs, the size of token tiles; and the rows that a CTA of the gather stages.
 #pragma once
 
 namespace bpdq {
@@ -136,6 +136,17 @@ inline int wide_half(int M, int nrt, int nblocks, int K, int sms) {
         if (best == 0 || cost < best) { best = cost; half = h; }
     }
     return half;
+}
+
+// Tokens whose rows a CTA of the gather in stored-column order holds in shared memory.  Two where every SM still has a CTA and two CTAs fit an
+// SM (a CTA's rows and its 1 KB that the system takes, twice, in one CTA's largest opt-in and 1 KB): with one resident CTA the load, the barrier and the
+// scatter are in series.  One where a row fits, else none.  us on top of the plain linear, one token and two: 18944 columns with 777 tokens
+// 16.6 and 12.7, with 4096 85 and 71; 24576 columns with 4096 113 and 93; 29568 columns (one CTA of two rows per SM) 28 and 38, 142 and 191.
+constexpr int gather_tokens(int in, int M, int sms, int smem_optin) {
+    const int room = smem_optin < 200 * 1024 ? smem_optin : 200 * 1024;
+    const long long row = 2LL * in;
+    if (M >= 2 * sms && 2 * (2 * row + 1024) <= smem_optin + 1024LL) return 2;
+    return row <= room ? 1 : 0;
 }
 
 }  // namespace bpdq

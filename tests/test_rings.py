@@ -28,6 +28,10 @@ int main(int argc, char** argv) {
         printf("%d\n", bpdq::wide_half(atoi(argv[1]), atoi(argv[2]), atoi(argv[3]), atoi(argv[4]), atoi(argv[5])));
         return 0;
     }
+    if (argc == 4) {
+        printf("%d\n", bpdq::gather_tokens(atoi(argv[1]), atoi(argv[2]), 148, atoi(argv[3])));
+        return 0;
+    }
     for (int K = 1; K <= 4; ++K)
         for (int half = 16; half <= 256; half += 16) {
             const int bkw = half <= bpdq::kWideLongHalf ? 64 : 32;
@@ -408,3 +412,18 @@ def test_every_barrier_of_the_prefill_kernel_is_initialised_once(tmp_path):
         sets = 2 if half <= 128 else 1
         assert [a[:2] for a in acc] == [acc[j % sets][:2] for j in range(6)] and len({a[:2] for a in acc}) == sets
         assert [a[2] for a in acc] == [j // sets % 2 for j in range(6)]
+
+
+@pytest.mark.parametrize("in_,M,smem_optin", [(128, 295, 232448), (128, 296, 232448), (18944, 777, 232448), (24576, 4096, 232448), (28928, 4096, 232448),
+                                              (29056, 4096, 232448), (29568, 4096, 232448), (51200, 4096, 232448), (102400, 500, 232448),
+                                              (102528, 500, 232448), (24576, 500, 101376)])
+def test_a_gather_that_stages_two_tokens_leaves_room_for_a_second_cta(driver, in_, M, smem_optin):
+    """Rows that a CTA of the gather holds fit its shared memory, and two tokens are staged only where two such CTAs share an SM (whose shared
+    memory is a CTA's largest opt-in and the 1 KB that every CTA costs beside its own)."""
+    tokens = int(subprocess.run([driver, str(in_), str(M), str(smem_optin)], check=True, capture_output=True, text=True).stdout)
+    cta = 2 * in_ * tokens
+    two_ctas = 2 * (4 * in_ + 1024) <= smem_optin + 1024
+    assert tokens == (2 if M >= 296 and two_ctas else 1 if 2 * in_ <= 200 * 1024 and 2 * in_ <= smem_optin else 0)
+    assert cta <= smem_optin and (tokens < 2 or 2 * (cta + 1024) <= smem_optin + 1024)
+    if in_ == 29568:
+        assert tokens == 1                                   # the 72B-shaped down projection: 142 us with one, 191 with two
