@@ -14,8 +14,8 @@
 // Packed 128-column blocks (two tensor-map boxes each) come in a ring of two to eight.  Roles (640 threads, 896 with four decode
 // groups): warps 0 and 3 producers (x, packed), warps 1-2 MMA issuers, two or four decode groups of four warps (thread =
 // output row, taking 128-column blocks of the stage sequence in turn, which continues across tiles), eight epilogue warps (four
-// per half).  Barriers per stage: full (both x halves' bytes and one arrival per warp of the owning decode group), two that
-// release it in turn (one tcgen05.commit per issuer); per packed slot: full_p, empty_p; acc_full (one commit per issuer), acc_empty (one arrival per
+// per half).  Barriers per stage: full (both x halves' bytes and one arrival per warp of the owning decode group), one or
+// two that release it in turn (one tcgen05.commit per issuer); per packed slot: full_p, empty_p; acc_full (one commit per issuer), acc_empty (one arrival per
 // epilogue warp).  All waits are bounded.
 using bpdq::kWideMaxHalf;
 using bpdq::kWideLongHalf;
@@ -37,6 +37,7 @@ template <int K, int BKW, int NG> struct WideCfg {
     static constexpr int kFirstEpi = kWideFirstDecode + 4 * kGroups, kThreads = 32 * (kFirstEpi + kWideEpiWarps);
     static constexpr bool kWhole = BKW == 64;                  // a MMA takes the whole token tile (two halves of up to 128)
     static constexpr int kIssuers = kWhole ? 1 : 2;
+    static constexpr int kReleases = bpdq::wide_releases(NG);  // release barriers of a stage slot
     static constexpr int kAccs = kWhole ? 2 : 1;               // accumulator barrier sets, which tiles take in turn
     static constexpr int kPlaneBytes = bpdq::wide_plane_bytes(K), kCoefBytes = bpdq::wide_coef_bytes(K);
     static constexpr int kBlockBytes = bpdq::wide_block_bytes(K);
@@ -68,16 +69,18 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     const unsigned p_base = st_base + (unsigned)S * stage;              // SP x packed block
     const unsigned bar_base = p_base + SP * C::kBlockBytes;
     auto full = [&](int s) { return bar_base + 8u * s; };
-    // a stage slot's release: uses of a slot alternate between two barriers (wide_rings, bpdq_rings.h); n = 0, 1, ... counts them
-    auto empty = [&](int s, int n) { return bar_base + 8u * (S + 2 * s + (n & 1)); };
-    auto released = [&](int s, int n) { return empty(s, n - 1); };           // what use n waits for, by parity ((n - 1) >> 1) & 1
-    auto full_p = [&](int s) { return bar_base + 8u * (3 * S + s); };
-    auto empty_p = [&](int s) { return bar_base + 8u * (3 * S + SP + s); };
+    // a stage slot's release: uses n = 0, 1, ... of a slot take its R barriers in turn (wide_releases, bpdq_rings.h)
+    constexpr int R = C::kReleases;
+    auto empty = [&](int s, int n) { return bar_base + 8u * (S + R * s + (n & (R - 1))); };
+    auto released = [&](int s, int n) { return empty(s, n - 1); };           // what use n waits for
+    auto released_parity = [&](int n) { return (unsigned)((n - 1) >> (R - 1)) & 1u; };
+    auto full_p = [&](int s) { return bar_base + 8u * ((1 + R) * S + s); };
+    auto empty_p = [&](int s) { return bar_base + 8u * ((1 + R) * S + SP + s); };
     // an accumulator's barriers: one set of both halves' (kIssuers commits), or two that tiles j = 0, 1, ... take in turn
-    auto acc_full = [&](int j) { return bar_base + 8u * (3 * S + 2 * SP + j % C::kAccs); };
+    auto acc_full = [&](int j) { return bar_base + 8u * ((1 + R) * S + 2 * SP + j % C::kAccs); };
     auto acc_empty = [&](int j) { return acc_full(j) + 16u; };
     auto acc_parity = [&](int j) { return (unsigned)(j / C::kAccs) & 1u; };
-    unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * (3 * S + 2 * SP + 4));
+    unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * ((1 + R) * S + 2 * SP + 4));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -91,8 +94,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(full(s), 1 + 4);                   // the producer (with both x halves' bytes) and four decode warps
-            mbar_init(empty(s, 0), C::kIssuers);
-            mbar_init(empty(s, 1), C::kIssuers);
+            for (int n = 0; n < R; ++n) mbar_init(empty(s, n), C::kIssuers);
         }
         for (int s = 0; s < SP; ++s) { mbar_init(full_p(s), 1); mbar_init(empty_p(s), 4); }
         for (int j = 0; j < C::kAccs; ++j) { mbar_init(acc_full(j), C::kIssuers); mbar_init(acc_empty(j), kWideEpiWarps); }   // a live barrier must not be initialised again
@@ -122,7 +124,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                 const int tok0 = (tile / nrt) * (2 * half);
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait(released(s, n), (unsigned)((n - 1) >> 1) & 1u, abort_flag, p.status)) { ok = false; break; }
+                    if (!mbar_wait(released(s, n), released_parity(n), abort_flag, p.status)) { ok = false; break; }
                     mbar_expect_tx(full(s), 2u * bhalf);
                     const unsigned bdst = st_base + (unsigned)s * stage + C::kATile;
                     tma_load_2d(bdst, &x_map, kb * BKW, tok0, full(s));
@@ -238,7 +240,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 #pragma unroll
                     for (int u = 0; u < 4; ++u) v8[4 * e + u] = bpdq::decode8<K>(sel[u], tab);
                 }
-                if (!mbar_wait_warp(released(s, n), (unsigned)((n - 1) >> 1) & 1u, abort_flag, p.status)) { ok = false; break; }
+                if (!mbar_wait_warp(released(s, n), released_parity(n), abort_flag, p.status)) { ok = false; break; }
                 const unsigned dst = st_base + (unsigned)s * stage;
 #pragma unroll
                 for (int ch = 0; ch < BKW / 8; ++ch)

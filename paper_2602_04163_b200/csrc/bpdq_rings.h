@@ -95,11 +95,15 @@ struct WideRings {
     int stages, sp;                                   // slots of the stage ring and of the packed ring
 };
 
+// Barriers that release a stage slot, its uses taking them in turn: two with four decode groups, whose waits one barrier would leave
+// open (below); two groups need one.  A second one beside two groups slowed the issuers: halves of 144 tokens by 2 to 4 %.
+constexpr int wide_releases(int groups) { return groups == 4 ? 2 : 1; }
+
 // `bkw` columns per stage, 32 or 64.  Packed slots: a multiple of the decode groups, so that a slot belongs to one of them, which
 // has waited for every use of it.  Stage slots are shared by the groups.  The group that waits for the release of stage it - S has
 // waited, for the last stage of its block before, it - (groups - 1) * (stages per block) - 1, for MMAs no later than S stages before that
-// one, and MMAs complete in order; uses of a slot are released through two barriers in turn, so the phase before the awaited one is
-// stage it - 3 S, and it is over if 2 S >= (groups - 1) * (stages per block) + 1.  The narrowest rings are three stages of 64 columns with two groups, five
+// one, and MMAs complete in order; with R barriers that release a slot in turn the phase before the awaited one is stage it - (1 + R) S, and
+// it is over if R S >= (groups - 1) * (stages per block) + 1.  The narrowest rings are three stages of 64 columns with two groups, five
 // of 32 with two, and six of 64 with four.
 constexpr WideRings wide_rings(int K, int bkw, int half) {
     const int least = wide_groups(K, half);

@@ -36,8 +36,9 @@ int main(int argc, char** argv) {
         for (int half = 16; half <= 256; half += 16) {
             const int bkw = half <= bpdq::kWideLongHalf ? 64 : 32;
             const bpdq::WideRings r = bpdq::wide_rings(K, bkw, half);
-            printf("wide %d %d %d %d %d %d\n", K, half, 128 / bkw, r.stages, r.sp,
-                   bpdq::kWideSmem - r.stages * bpdq::wide_stage_bytes(bkw, half) - r.sp * bpdq::wide_block_bytes(K));
+            const int groups = bpdq::wide_groups(K, half);
+            printf("wide %d %d %d %d %d %d %d %d\n", K, half, 128 / bkw, r.stages, r.sp,
+                   bpdq::kWideSmem - r.stages * bpdq::wide_stage_bytes(bkw, half) - r.sp * bpdq::wide_block_bytes(K), groups, bpdq::wide_releases(groups));
         }
     for (int K = 1; K <= 4; ++K)
         for (int cols = 16; cols <= 128; cols += 16) {
@@ -140,9 +141,10 @@ def test_the_order_model_sees_an_odd_ring():
     assert ts_order(8, 23, 100).open_waits() == []           # an odd ring that the x ring covers
 
 
-def wide_order(stages, sp, per_block, blocks, release):
-    """gemm_wide_kernel: x producer, packed producer, two decode groups (group b mod 2 takes block b), two issuers that multiply every
-    stage."""
+def wide_order(stages, sp, per_block, blocks, groups, releases, issuers, release, tile=5, accs=2):
+    """gemm_wide_kernel: x producer, packed producer, decode groups (group b mod groups takes block b), issuers that all multiply every
+    stage, epilogue.  A stage slot's uses are released through `releases` barriers in turn, so the phase before the awaited one is
+    releases + 1 uses back; tiles of `tile` blocks take `accs` accumulators with barriers of their own in turn."""
     o = Order()
 
     def ev(kind, q):
@@ -151,35 +153,61 @@ def wide_order(stages, sp, per_block, blocks, release):
         o.event(("packed asked", b), ev("packed asked", b - 1), ev("stored", (b - sp) * per_block + release) if b >= sp else None)
         o.wait("packed producer", ev("packed asked", b - 1), ev("stored", (b - 2 * sp) * per_block + release) if b >= 2 * sp else None)
         o.event(("packed landed", b), ("packed asked", b))
+        j = b // tile
         for it in range(b * per_block, (b + 1) * per_block):
             o.event(("x asked", it), ev("x asked", it - 1), ev("multiplied", it - stages))
-            o.wait("x producer", ev("x asked", it - 1), ev("multiplied", it - 2 * stages))
+            o.wait("x producer", ev("x asked", it - 1), ev("multiplied", it - (releases + 1) * stages))
             o.event(("x landed", it), ("x asked", it))
-            before = ev("stored", it - 1) if it % per_block else ev("stored", (b - 1) * per_block - 1)    # the group's stage before
+            before = ev("stored", it - 1) if it % per_block else ev("stored", (b - groups + 1) * per_block - 1)    # the group's stage before
             if it % per_block == 0:
                 o.wait("group, packed", before, ev("packed landed", b - sp))
-            o.wait("group, stage", before, ev("multiplied", it - 2 * stages))
+            o.wait("group, stage", before, ev("multiplied", it - (releases + 1) * stages))
             o.event(("stored", it), before, ("packed landed", b), ev("multiplied", it - stages))
-            for i in range(2):
-                o.wait("issuer", ev(f"issued {i}", it - 1), ev("full", it - stages))
-                o.event((f"issued {i}", it), ev(f"issued {i}", it - 1), ("full", it))
+            for i in range(issuers):
+                last = ev(f"issued {i}", it - 1)
+                if it == j * tile * per_block:              # a tile's first stage: its accumulator has been drained of tile j - accs
+                    o.wait("issuer, accumulator", last, ev("drained", j - 2 * accs))
+                    o.event((f"accumulator {i}", j), last, ev("drained", j - accs))
+                    last = (f"accumulator {i}", j)
+                o.wait("issuer", last, ev("full", it - stages))
+                o.event((f"issued {i}", it), last, ("full", it))
             o.event(("full", it), ("stored", it), ("x landed", it))
-            o.event(("multiplied", it), ("issued 0", it), ("issued 1", it), ev("multiplied", it - 1))
+            o.event(("multiplied", it), *((f"issued {i}", it) for i in range(issuers)), ev("multiplied", it - 1))
+        if b % tile == tile - 1:                            # the tile's last commits fill its accumulator, the epilogue drains it
+            o.event(("filled", j), ("multiplied", (b + 1) * per_block - 1))
+            o.wait("epilogue", ev("drained", j - 1), ev("filled", j - accs))
+            o.event(("drained", j), ev("drained", j - 1), ("filled", j))
     return o
 
 
 def test_rings_of_the_prefill_kernel(rings):
+    """Every K and half tile, with the groups and issuers that it has, tiles of one block and of several: no wait can pass by a phase that is
+    still open, the rings and barriers fit shared memory, and the release barriers of a slot are no more than the shortest ring takes."""
     (release,) = [r for kind, r in rings if kind == "release"]
-    seen = 0
+    seen, needed = 0, set()
     for kind, r in rings:
         if kind != "wide":
             continue
-        K, half, per_block, stages, sp, left = r
+        K, half, per_block, stages, sp, left, groups, releases = r
         seen += 1
-        assert left >= 1024 + 8 * (2 * stages + 2 * sp + 2) + 8, r             # alignment slack, barriers, TMEM address and flag
-        assert wide_order(stages, sp, per_block, 2 * sp + 2 * stages + 4, release[0 if per_block == 4 else 1]).open_waits() == [], r
-    assert seen == 64
-    assert wide_order(4, 2, 4, 20, 2).open_waits()                              # four stages of 32 columns would not do
+        assert groups == 4 or releases == 1, r
+        assert groups in (2, 4) and sp % groups == 0 and (K < 4 or groups == 2), r
+        assert left >= 1024 + 8 * ((1 + releases) * stages + 2 * sp + 4) + 8, r     # alignment slack, barriers, TMEM address and flag
+        whole = half <= 128                                  # one issuer and two accumulators, else two and one
+        shape = (stages, sp, per_block, 2 * sp + 3 * stages + 8, groups)
+        last = (1 if whole else 2, release[0 if per_block == 4 else 1])
+        for tile in (1, 5):
+            assert wide_order(*shape, releases, *last, tile, 2 if whole else 1).open_waits() == [], r
+        if releases > 1 and wide_order(*shape, releases - 1, *last).open_waits():
+            needed.add(groups)
+    assert seen == 64 and needed == {4}
+
+
+def test_the_order_model_of_the_prefill_kernel_sees_what_would_not_do():
+    assert wide_order(4, 2, 4, 20, 2, 1, 2, 2).open_waits()                     # four stages of 32 columns
+    assert wide_order(3, 4, 2, 40, 4, 2, 1, 1).open_waits()                     # three of 64 with four groups
+    assert wide_order(6, 6, 2, 40, 4, 2, 1, 1).open_waits()                     # a packed ring that is no multiple of the groups
+    assert {role for role, _ in wide_order(6, 4, 2, 40, 4, 1, 1, 1).open_waits()} == {"group, stage"}     # one release barrier
 
 
 @pytest.mark.parametrize("M,nrt,nblocks,K", [(129, 28, 28, 2), (777, 28, 148, 2), (777, 4, 28, 2), (4096, 231, 64, 3), (4096, 1, 1, 4), (513, 148, 32, 4),
@@ -298,63 +326,17 @@ def test_a_cta_that_gave_up_outlives_its_copies():
         assert re.search(r"pend_nsl\);\s*if \(\*abort_flag\) bpdq::tma::linger\(\);\s*\}\s*template", f.read())
 
 
-def wide_order_two_releases(stages, sp, per_block, blocks, groups, issuers, release):
-    """gemm_wide_kernel with any number of decode groups (group b mod groups takes block b); a stage slot's uses are released
-    through two barriers in turn, so the phase before the awaited one is three uses back."""
-    o = Order()
-
-    def ev(kind, q):
-        return (kind, q) if q >= 0 else None
-    for b in range(blocks):
-        o.event(("packed asked", b), ev("packed asked", b - 1), ev("stored", (b - sp) * per_block + release) if b >= sp else None)
-        o.wait("packed producer", ev("packed asked", b - 1), ev("stored", (b - 2 * sp) * per_block + release) if b >= 2 * sp else None)
-        o.event(("packed landed", b), ("packed asked", b))
-        for it in range(b * per_block, (b + 1) * per_block):
-            o.event(("x asked", it), ev("x asked", it - 1), ev("multiplied", it - stages))
-            o.wait("x producer", ev("x asked", it - 1), ev("multiplied", it - 3 * stages))
-            o.event(("x landed", it), ("x asked", it))
-            before = ev("stored", it - 1) if it % per_block else ev("stored", (b - groups + 1) * per_block - 1)
-            if it % per_block == 0:
-                o.wait("group, packed", before, ev("packed landed", b - sp))
-            o.wait("group, stage", before, ev("multiplied", it - 3 * stages))
-            o.event(("stored", it), before, ("packed landed", b), ev("multiplied", it - stages))
-            for i in range(issuers):
-                o.wait("issuer", ev(f"issued {i}", it - 1), ev("full", it - stages))
-                o.event((f"issued {i}", it), ev(f"issued {i}", it - 1), ("full", it))
-            o.event(("full", it), ("stored", it), ("x landed", it))
-            o.event(("multiplied", it), *((f"issued {i}", it) for i in range(issuers)), ev("multiplied", it - 1))
-    return o
-
-
-def test_rings_of_the_prefill_kernel_with_its_decode_groups(rings):
-    """As above, with the groups that a tile has (four up to halves of 64 tokens below K = 4) and one issuer or two."""
-    (release,) = [r for kind, r in rings if kind == "release"]
-    four = 0
-    for kind, r in rings:
-        if kind != "wide":
-            continue
-        K, half, per_block, stages, sp, left = r
-        groups = 4 if half <= 64 and K < 4 else 2
-        four += groups == 4
-        assert sp % groups == 0 and left >= 1024 + 8 * (3 * stages + 2 * sp + 4) + 8, r
-        o = wide_order_two_releases(stages, sp, per_block, 2 * sp + 2 * stages + 8, groups, 1 if half <= 128 else 2, release[0 if per_block == 4 else 1])
-        assert o.open_waits() == [], r
-    assert four == 12
-    assert wide_order_two_releases(3, 4, 2, 40, 4, 1, 1).open_waits()           # three stages and four groups would not do
-    assert wide_order_two_releases(6, 6, 2, 40, 4, 1, 1).open_waits()           # nor a packed ring that is no multiple of the groups
-
-
 BARRIERS = r"""
 #include <cstdio>
 #include "bpdq_rings.h"
 constexpr int kWideEpiWarps = %(epi)s;
-template <int BKW> struct Cfg {
+template <int BKW, int NG> struct Cfg {
     %(config)s
 };
 static void mbar_init(unsigned addr, int count) { printf("init %%u %%d\n", addr, count); }
 static void fence_barrier_init() {}
-template <int BKW> void layout(int K, int half) {
-    using C = Cfg<BKW>;
+template <int BKW, int NG> void layout(int K, int half) {
+    using C = Cfg<BKW, NG>;
     constexpr bool kWhole = C::kWhole;
     (void)kWhole;
     const bpdq::WideRings r = bpdq::wide_rings(K, BKW, half);
@@ -374,7 +356,9 @@ template <int BKW> void layout(int K, int half) {
 int main() {
     for (int K = 1; K <= 4; ++K)
         for (int half = 16; half <= bpdq::kWideMaxHalf; half += 16)
-            if (half <= bpdq::kWideLongHalf) layout<64>(K, half); else layout<32>(K, half);
+            if (half > bpdq::kWideLongHalf) layout<32, 2>(K, half);
+            else if (bpdq::wide_groups(K, half) == 4) layout<64, 4>(K, half);
+            else layout<64, 2>(K, half);
     return 0;
 }
 """
@@ -389,7 +373,7 @@ def test_every_barrier_of_the_prefill_kernel_is_initialised_once(tmp_path):
     kernel = text[text.index("gemm_wide_kernel(const"):]
     parts = {
         "epi": re.search(r"kWideEpiWarps = (\d+);", text).group(1),
-        "config": "\n".join(re.findall(r"static constexpr (?:bool kWhole|int kIssuers|int kAccs) = [^;]*;", text)),
+        "config": "\n".join(re.findall(r"static constexpr (?:bool kWhole|int kIssuers|int kAccs|int kReleases) = [^;]*;", text)),
         "names": kernel[kernel.index("auto full ="):kernel.index("unsigned* tmem_slot")],
         "init": re.search(r"if \(tid == 0\) \{.*?fence_barrier_init\(\);\s*\}", kernel, re.S).group(),
         "end": re.search(r"\(bar_base - base\) \+ (8 \* \([^;]*\))\);", kernel).group(1),
