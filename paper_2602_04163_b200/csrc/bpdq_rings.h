@@ -86,10 +86,14 @@ constexpr int wide_a_bytes(int bkw) { return 128 * bkw * 2; }                   
 constexpr int wide_stage_bytes(int bkw, int half) { return wide_a_bytes(bkw) + 2 * half * bkw * 2; }   // ... and both halves of x
 
 // Decode groups of the prefill kernel.  A group's block is a chain of some 290 instructions per lane; with few tokens the MMAs wait for
-// it, and four groups are faster than two: K = 2, ns per block with halves of 16 / 48 tokens 487 / 517 and 443 / 468, K = 3 857 / 867 and 519 /
-// 572; with 80 and more the two are (K = 2: 606 and 637 with 80, 801 and 828 with 128, the columns of a stage shared by two issuers).  K = 4 needs
-// more registers than four groups leave.
-constexpr int wide_groups(int K, int half) { return half <= 64 && K < 4 ? 4 : 2; }
+// it, and four groups are faster than two.  ns per block with two / four groups, one tile per SM, 12288 and 4096 columns, sustained (g = 128):
+//   half        16         32         48         64         80         96        112        128
+//   K = 1    631 / 581  791 / 602  722 / 651  762 / 692  925 / 720  792 / 733  820 / 792  858 / 854
+//   K = 2    622 / 588  639 / 593  684 / 663  754 / 717  736 / 743  778 / 783  813 / 791  866 / 850
+//   K = 3   1090 / 676  695 / 700 1060 / 771  853 / 802  865 / 830 1183 / 876  978 / 909  948 / 936
+// (with g = 64, K = 2: 799 / 819 at 80, 841 / 859 at 96, 884 / 864 at 128).  3584 x 18944 with 900 tokens (halves of 96) 123.8 and 102.6 us at
+// K = 3, 29568 x 8192 with 129 (80) 86.8 and 65.5 at K = 1.  K = 4 needs more registers than four groups leave.
+constexpr int wide_groups(int K, int half) { return half <= (K == 2 ? 64 : kWideLongHalf) && K < 4 ? 4 : 2; }
 
 struct WideRings {
     int stages, sp;                                   // slots of the stage ring and of the packed ring
@@ -104,7 +108,7 @@ constexpr int wide_releases(int groups) { return groups == 4 ? 2 : 1; }
 // waited, for the last stage of its block before, it - (groups - 1) * (stages per block) - 1, for MMAs no later than S stages before that
 // one, and MMAs complete in order; with R barriers that release a slot in turn the phase before the awaited one is stage it - (1 + R) S, and
 // it is over if R S >= (groups - 1) * (stages per block) + 1.  The narrowest rings are three stages of 64 columns with two groups, five
-// of 32 with two, and six of 64 with four.
+// of 32 with two, and four of 64 with four.
 constexpr WideRings wide_rings(int K, int bkw, int half) {
     const int least = wide_groups(K, half);
     const int stage = wide_stage_bytes(bkw, half), budget = kWideSmem - least * wide_block_bytes(K) - 2048;   // 2048: alignment slack, barriers
@@ -114,7 +118,7 @@ constexpr WideRings wide_rings(int K, int bkw, int half) {
     sp = sp > kWideMaxSP ? kWideMaxSP : sp / least * least;
     return {stages, sp};
 }
-static_assert(wide_rings(4, 32, kWideMaxHalf).stages >= 5 && wide_rings(4, 64, kWideLongHalf).stages >= 3 && wide_rings(3, 64, 64).stages >= 5, "the widest tiles");
+static_assert(wide_rings(4, 32, kWideMaxHalf).stages >= 5 && wide_rings(4, 64, kWideLongHalf).stages >= 3 && wide_rings(3, 64, kWideLongHalf).stages >= 4, "the widest tiles");
 
 // Tokens of a half tile: the cut of M tokens into equal tiles that takes the least time by a model of the kernel.  A 128-column
 // block takes 8.5 clocks per token of a half (the MMAs), but no less than the decode and the hand-over of its stages: 1150 clocks
