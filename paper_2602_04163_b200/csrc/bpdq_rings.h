@@ -120,27 +120,27 @@ constexpr WideRings wide_rings(int K, int bkw, int half) {
 }
 static_assert(wide_rings(4, 32, kWideMaxHalf).stages >= 5 && wide_rings(4, 64, kWideLongHalf).stages >= 3 && wide_rings(3, 64, kWideLongHalf).stages >= 4, "the widest tiles");
 
-// Tokens of a half tile: the cut of M tokens into equal tiles that takes the least time by a model of the kernel.  A 128-column
-// block takes 8.5 clocks per token of a half (the MMAs), but no less than the decode and the hand-over of its stages: 1150 clocks
-// with 64-column stages, 1320 with 32-column ones (1600 and 1700 with sixteen candidates); a tile is paid for in whole rounds over
-// the SMs.  Measured, ns per block with one tile per SM, 12288 and 4096 columns, back to back (the 1 kW cap slows the larger halves; g = 128;
-// K = 1 and 4 up to 128 from the kernel with two MMAs per 16 columns):
-//   half      16    48    80   112   128 |  144   160   192   224   256
-//   K = 1    479   524   697   764   825 | 1006  1055  1144  1326  1541
-//   K = 2    443   468   654   774   831 | 1179  1121  1232  1473  1602
-//   K = 3    519   572   746   906   936 | 1311  1307  1324  1503  1722
-//   K = 4   1069  1078   974  1167  1517 | 1383  1453  1578  1632  1833
-// Always 512 tokens per tile left most SMs idle on short token counts: 3584 x 18944 (28 row tiles) with 777 tokens took 199 us in
-// 56 tiles, in 140 it takes 94.
+// Tokens of a half tile: the cut of M tokens into equal tiles that takes the least time by a model of the kernel: rounds of tiles over the
+// SMs, each of the row's blocks and an edge (fill, drain, what of them the next tile does not cover).  A 128-column block's ns by K and
+// half, relative to one another: fitted to 3592 measured launches (layer shapes and random ones, 129 to 4096 tokens, g = 64, 128 and 256, every
+// half, sustained under the 1 kW cap, the halves within 35 % of a launch's best), checked on 1363 others: the half taken is
+// 0.4 % slower than the best on average, more than 5 % in 23.  Halves of 144 to 192 pay for their 32-column stages; the saw teeth are packed rings of two slots
+// (K = 4 but for halves of 80, 112, 176 and 208 to 224).  A model of one least time per block for all halves up to 128 and another above it
+// kept 144 to 176 where 96 to 128 or 208 to 256 are faster: 29568 x 8192 at K = 2 with 777 tokens 364 us in halves of 144, 317 in halves of 208, with 576
+// tokens 274 (144) and 220 (96); 8192 x 29568 with 2306 tokens 1093 (144) and 889 (208).  Always 512 tokens per tile left most SMs idle on short token counts:
+// 3584 x 18944 (28 row tiles) with 777 tokens took 199 us in 56 tiles, in 140 it takes 92.
+//                                            16    32    48    64    80    96   112   128   144   160   176   192   208   224   240   256
+constexpr int kWideBlockNs[4][16] = {{ 600,  610,  630,  650,  680,  750,  810,  890, 1140, 1150, 1190, 1280, 1400, 1510, 1600, 1710},
+                                     { 630,  640,  660,  710,  750,  830,  860,  900, 1200, 1160, 1250, 1280, 1400, 1490, 1590, 1690},
+                                     { 620,  640,  660,  710,  750,  780,  830,  860, 1160, 1140, 1130, 1210, 1320, 1380, 1470, 1560},
+                                     {1390, 1400, 1400, 1410, 1260, 1400, 1400, 1420, 1500, 1510, 1440, 1580, 1550, 1590, 1730, 1780}};
 inline int wide_half(int M, int nrt, int nblocks, int K, int sms) {
     long long best = 0;
     int half = kWideMaxHalf;
     for (int ntt = (M + 2 * kWideMaxHalf - 1) / (2 * kWideMaxHalf); ntt <= (M + 31) / 32; ++ntt) {
         const int h = ((M + ntt - 1) / ntt + 31) / 32 * 16;
         const long long tiles = (long long)nrt * ((M + 2 * h - 1) / (2 * h)), rounds = (tiles + sms - 1) / sms;
-        const long long least = h <= kWideLongHalf ? (K == 4 ? 1600 : 1150) : (K == 4 ? 1700 : 1320);
-        const long long block = 17LL * h / 2 > least ? 17LL * h / 2 : least;
-        const long long cost = rounds * (nblocks * block + 2000 + 30LL * h);
+        const long long cost = rounds * ((long long)nblocks * kWideBlockNs[K - 1][h / 16 - 1] + 2000 + 60LL * h);
         if (best == 0 || cost < best) { best = cost; half = h; }
     }
     return half;
