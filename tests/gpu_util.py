@@ -7,6 +7,12 @@ from paper_2602_04163_b200 import binding, synth
 
 TOL_REL, TOL_ABS = 4e-3, 1e-3     # |y - y_ref| <= 4e-3 * sum|x_j w_j| + 1e-3
 
+# Prefill launches in which a CTA of the 148 takes four tiles and the first CTA five, the last of them ragged: (K, group, columns, tokens, tokens of a half tile,
+# decode groups).  test_rings.py checks that the tile rule and the group rule give these.
+TILE_WALK_ROWS = 128 * 4 * 148 + 48
+TILE_WALKS = [(2, 128, 640, 100, 64, 4), (3, 64, 640, 129, 80, 4), (3, 128, 640, 200, 112, 4), (1, 256, 384, 250, 128, 4), (2, 128, 640, 200, 112, 2),
+              (2, 64, 384, 250, 128, 2), (4, 128, 384, 250, 128, 2), (4, 64, 256, 33, 32, 2), (2, 256, 640, 330, 176, 2), (3, 128, 384, 500, 256, 2)]
+
 
 def stream_ptr() -> int:
     return torch.cuda.current_stream().cuda_stream

@@ -182,23 +182,39 @@ def test_short_rows_in_more_tiles_than_sms(K, g, in_, M):
 
 
 @pytest.mark.parametrize("K,g,out,in_,M", [
-    (2, 128, 512, 3584, 777),        # halves of 16 tokens: four decode groups, one tile per CTA
-    (3, 64, 160, 384, 9000),         # several tiles per CTA of three blocks each, a ragged row tile and a ragged last token tile
-    (1, 256, 128, 640, 20000),       # two accumulators in turn, an odd number of blocks, a short last group
-    (2, 128, 3584, 1152, 777),       # halves of 80
+    (2, 128, 512, 3584, 777),        # halves of 16 tokens: four decode groups
+    (3, 64, 160, 384, 9000),         # halves of 64: three blocks per tile, a ragged row tile and a ragged last token tile
+    (1, 256, 128, 640, 20000),       # halves of 80: an odd number of blocks, a short last group
+    (2, 128, 3584, 1152, 777),       # halves of 80 with two decode groups
     (3, 128, 1024, 512, 4096),       # halves of 128: the widest MMA
     (4, 128, 144, 256, 2100),        # sixteen candidates: two decode groups at any half
 ])
 def test_whole_tiles_of_up_to_256_tokens(K, g, out, in_, M):
-    """One MMA for a whole token tile, drained while the next tile's accumulator fills.  Weights from bpdq_dequant, sums in binary32;
-    every call returns the same bits."""
+    """One MMA for a whole token tile, one tile per CTA.  Weights from bpdq_dequant, sums in binary32; every call returns the same bits."""
+    check_against_dequant(K, g, out, in_, M)
+
+
+@pytest.mark.parametrize("K,g,in_,M,half,groups", G.TILE_WALKS)
+def test_ctas_walk_over_several_tiles(K, g, in_, M, half, groups):
+    """Four or five tiles per CTA: stage and packed slots run on from tile to tile, the two accumulators of whole tiles are used again (from the
+    third tile on) while the other is drained, and the one of longer tiles after its drain."""
+    check_against_dequant(K, g, G.TILE_WALK_ROWS, in_, M)
+
+
+def check_against_dequant(K, g, out, in_, M):
     import torch
     h = binding.Handle(out, in_, K, g, None, 29, M)
-    x = synth.activations(30, M, in_)
+    x = G.x_tensor(synth.activations(30, M, in_))
     w = torch.from_numpy(G.run_dequant(h).view(np.float16)).cuda().float()
-    ref = (G.x_tensor(x).float() @ w.T).cpu().numpy()
-    first = G.run_linear(h, x)
-    # binary16 rounding of the result (2^-11) and binary32 sums of up to 3584 terms of size up to 0.2 in another order
-    assert np.all(np.abs(first - ref) <= 2.0 ** -10 * np.abs(ref) + 2e-3)
-    for _ in range(3):
-        assert np.array_equal(first, G.run_linear(h, x))
+    ref = x.float() @ w.T
+    first = None
+    for _ in range(4):
+        y = torch.full((M, out), float("nan"), dtype=torch.float16, device="cuda")
+        h.bpdq_linear_ex(x.data_ptr(), y.data_ptr(), M, binding.KERNEL_GEMM, G.stream_ptr())
+        torch.cuda.synchronize()
+        h.bpdq_get_status(G.stream_ptr())
+        if first is None:
+            first = y
+            # binary16 rounding of the result (2^-11) and binary32 sums of up to 3584 terms of size up to 0.2 in another order
+            assert bool(torch.all((y.float() - ref).abs() <= 2.0 ** -10 * ref.abs() + 2e-3))
+        assert torch.equal(first, y)

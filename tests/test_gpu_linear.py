@@ -153,30 +153,43 @@ def test_a_wait_that_runs_out_is_reported_and_leaves_the_handle_usable():
 
 
 @pytest.mark.parametrize("K,g,out,in_,M", [(4, 128, 4112, 1152, 1), (4, 64, 4112, 1152, 2), (3, 128, 4112, 1152, 2), (3, 64, 20000, 640, 2), (4, 64, 16, 128, 2),
-                                           (4, 128, 30000, 512, 1)])
+                                           (4, 128, 30000, 512, 1), (3, 64, 4112, 1152, 1)])
 def test_lut_kernel_with_other_flights(K, g, out, in_, M):
     """Formats whose instantiations have eight warps, or one task in flight where there are two registers' worth: ragged slices, a single
-    task, a hundred tasks per warp.  Plain, with a bias, and the gated unit over two of them."""
+    task, a hundred tasks per warp.  Every instantiation of a launch's options: plain, a bias, the gated unit over a pair, and the one that carries
+    all of it (a permutation, a permutation and a bias, a pair with a bias, a pair with both)."""
     layers = [G.make_layer(880 + k, out, in_, K, g, max_M=M) for k in range(2)]
     x = synth.activations(881, M, in_)
-    rows = np.unique(np.concatenate([np.arange(0, out, 1 + out // 200), [out - 16, out - 1]]))
-    refs = [oracle.linear(b[:, rows], c[:, rows], x, g) for _, b, c in layers]
-    for (h, _, _), (y_ref, a_ref) in zip(layers, refs):
-        G.assert_linear_close(G.run_linear(h, x, binding.KERNEL_GEMV)[:, rows], y_ref, a_ref, "plain")
-    (hg, _, _), (hu, _, _) = layers
-    (gy, ga), (uy, ua) = refs
-    want = oracle.swiglu(gy, uy)
-    dg, du = G.TOL_REL * ga + G.TOL_ABS, G.TOL_REL * ua + G.TOL_ABS
-    silu_g = oracle.swiglu(gy, np.ones_like(gy))
-    # first-order propagation of the two linears' accepted errors through the unit (|silu'| <= 1.1), plus the output's rounding
-    bound = 1.1 * (np.abs(uy) + du) * dg + (np.abs(silu_g) + 1.1 * dg) * du + 2.0 ** -10 * np.abs(want) + 1e-4
-    xt = G.x_tensor(x)
-    for _ in range(2):
-        out_t = torch.full((M, out), float("nan"), dtype=torch.float16, device="cuda")
-        binding.bpdq_gate_up_swiglu(hg, hu, xt.data_ptr(), out_t.data_ptr(), M, G.stream_ptr())
-        torch.cuda.synchronize()
-        assert np.all(np.abs(out_t.cpu().numpy().astype(np.float64)[:, rows] - want) <= bound)
+    perm = np.random.RandomState(4).permutation(in_).astype(np.int32)
     bias = np.random.RandomState(3).randn(out).astype(np.float16)
-    hg.bpdq_set_bias(bias.view(np.uint16))
+    rows = np.unique(np.concatenate([np.arange(0, out, 1 + out // 200), [out - 16, out - 1]]))
     b = bias[rows].astype(np.float64)
-    G.assert_linear_close(G.run_linear(hg, x, binding.KERNEL_GEMV)[:, rows], gy + b, ga + np.abs(b), "bias")
+    (hg, _, _), (hu, _, _) = layers
+    xt = G.x_tensor(x)
+
+    def check(x_stored, with_bias, what):
+        (gy, ga), (uy, ua) = (oracle.linear(bits[:, rows], c[:, rows], x_stored, g) for _, bits, c in layers)
+        if with_bias:
+            gy, ga = gy + b, ga + np.abs(b)
+        G.assert_linear_close(G.run_linear(hg, x, binding.KERNEL_GEMV)[:, rows], gy, ga, what)
+        G.assert_linear_close(G.run_linear(hu, x, binding.KERNEL_GEMV)[:, rows], uy, ua, what)
+        want = oracle.swiglu(gy, uy)
+        dg, du = G.TOL_REL * ga + G.TOL_ABS, G.TOL_REL * ua + G.TOL_ABS
+        silu_g = oracle.swiglu(gy, np.ones_like(gy))
+        # first-order propagation of the two linears' accepted errors through the unit (|silu'| <= 1.1), plus the output's rounding
+        bound = 1.1 * (np.abs(uy) + du) * dg + (np.abs(silu_g) + 1.1 * dg) * du + 2.0 ** -10 * np.abs(want) + 1e-4
+        for _ in range(2):
+            out_t = torch.full((M, out), float("nan"), dtype=torch.float16, device="cuda")
+            binding.bpdq_gate_up_swiglu(hg, hu, xt.data_ptr(), out_t.data_ptr(), M, G.stream_ptr())
+            torch.cuda.synchronize()
+            assert np.all(np.abs(out_t.cpu().numpy().astype(np.float64)[:, rows] - want) <= bound), "pair, " + what
+
+    check(x, False, "plain")
+    hg.bpdq_set_bias(bias.view(np.uint16))
+    check(x, True, "bias")
+    for h in (hg, hu):
+        h.bpdq_set_input_permutation(perm)
+    x_stored = np.ascontiguousarray(x[:, perm])
+    check(x_stored, True, "permutation and bias")
+    hg.bpdq_set_bias(None)
+    check(x_stored, False, "permutation")

@@ -249,6 +249,20 @@ def test_the_half_tile_that_is_taken_is_measured_fast(driver, M, out, in_, K, us
     assert half in us and us[half] <= 1.05 * min(us.values())
 
 
+def test_launches_of_several_tiles_per_cta_are_what_their_gpu_test_says(driver, rings):
+    """The GPU test of CTAs that walk over tiles is only worth something while the rules give its launches these tiles."""
+    from tests import gpu_util as G
+    groups_of = {(r[0], r[1]): r[6] for kind, r in rings if kind == "wide"}
+    nrt = -(-G.TILE_WALK_ROWS // 128)
+    for K, g, in_, M, half, groups in G.TILE_WALKS:
+        out = subprocess.run([driver, *map(str, (M, nrt, in_ // 128, K, 148))], check=True, capture_output=True, text=True).stdout
+        assert int(out) == half and groups_of[K, half] == groups, (K, g, in_, M)
+        assert nrt * -(-M // (2 * half)) > 4 * 148
+        # not a call of the kernel for up to 128 tokens (ts_drain_bound)
+        assert M > 128 or (M > 16 and in_ // 128 <= (8 if M > 64 else 2))
+    assert {(half > 128, groups) for _, _, _, _, half, groups in G.TILE_WALKS} == {(False, 4), (False, 2), (True, 2)}
+
+
 def test_prefill_slots_are_given_back_after_the_last_use(rings):
     """The stage behind which a decode group of the prefill kernel gives a packed slot back: by then every plane word and every
     coefficient group that it has loaded is part of a stored stage, for both stage widths and for one or two groups per block."""
