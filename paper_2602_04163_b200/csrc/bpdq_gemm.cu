@@ -13,9 +13,9 @@
 // itself; the decode threads reproduce it by hand.
 //
 // Two kernels: gemm_ts_kernel (up to 128 tokens: decoded weights in TMEM, one or several linears per launch;
-// bpdq_gemm_ts.cuh) and gemm_wide_kernel (more than 128 tokens, fewer where rows are short and tiles many: token tiles of up to 512,
-// two issuing warps; bpdq_gemm_wide.cuh).  In the second the decoded operand goes through shared memory: there the MMAs, not the decode, are
-// the bound, and TMEM is full of accumulators.
+// bpdq_gemm_ts.cuh) and gemm_wide_kernel (more than 128 tokens, fewer where rows are short and tiles many: token tiles of up to 512;
+// bpdq_gemm_wide.cuh).  In the second the decoded operand goes through shared memory and feeds one MMA of up to 256 tokens or two; tiles of 512 tokens are
+// bound by the MMAs, tiles of up to 160 by the decode.
 //
 // Decode: a thread reads its row's units and coefficients from the stage, builds the 2^K candidate values of the group
 // (Eq. 7, the decode rule's exact arithmetic) as byte tables, and then eight columns cost one shift-and-mask per plane to

@@ -1,10 +1,13 @@
 // Included by bpdq_gemm.cu (inside its unnamed namespace, after the PTX wrappers): the prefill kernel for many tokens.
 //
 // gemm_wide_kernel: one decoded weight stage feeds a token tile of two halves (of up to 256 tokens each), so a weight is decoded once per tile:
-// the decode's energy is what the 1 kW cap charges (every further plane costs 8-20 %).  Two warps issue, each into an accumulator of its own
-// (the two halves of TMEM's 512 columns).  Halves above 128 tokens: each issuer multiplies every stage with its own half of x.  Up to
+// the decode's energy is what the 1 kW cap charges (every further plane costs 8-20 %).  The two halves of TMEM's 512 columns are accumulators.
+// Halves above 128 tokens: two warps issue, each multiplies every stage with its own half of x into an accumulator of its own.  Up to
 // 128: one issuer multiplies with the whole tile, and tiles alternate between the accumulators, so that one is drained while the other
-// fills.  (An MMA reads 4 KB of A from shared memory: two of 80 tokens take 2 x 52 clocks where one of 160 takes 80.)  Above, TMEM is full with
+// fills.  (An MMA reads 4 KB of A from shared memory: two of 80 tokens take 2 x 52 clocks of the pipe where one of 160 takes 80.  The pipe is not what
+// bounds that tile: 3584 x 18944 with 777 tokens, K = 2, went from 94.6 to 92.2 us, and a block still takes 980 clocks for 640 of MMAs, the rest
+// being the two decode groups' chain and hand-over.  Where drains overlap it gives more: K = 2, halves of 128, 8192 x 8192 with 4096 tokens 3 %,
+// 20480 x 1024 with 512 tokens 9 %.)  Above, TMEM is full with
 // one tile, so the epilogue does not overlap the next tile's MMAs (about 3 % of a 72B-shaped tile's time); producer and decode warps run
 // ahead into the next tile's stages meanwhile.
 //
@@ -85,7 +88,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int nkb = p.in / BKW;                  // stages per tile
-    const int nblk = p.in / 128;                     // packed blocks per tile (four stages each)
+    const int nblk = p.in / 128;                     // packed blocks per tile (two or four stages each)
     const int nrt = (p.out + BM - 1) / BM;
     const int ntt = (p.M + 2 * half - 1) / (2 * half);
     const int ntiles = nrt * ntt;

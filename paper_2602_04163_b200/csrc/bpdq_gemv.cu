@@ -155,8 +155,8 @@ __device__ __forceinline__ float2 unpack2(unsigned long long v) {
 }
 
 // EXT: what the launch uses somewhere of kExtPair, kExtBias, kExtPerm.  An instantiation carries no other code: the streaming loop sits
-// at the 128-register cap, and the extra live values cost it spills (5 % of the headline, up to 50 % at g = 64) although they
-// are only used outside the loop.  Launches with one of pair and bias are common and have instantiations of their own, all else shares one.
+// at the 128-register cap, and the extra live values cost it time (5 % of the headline, up to 50 % at g = 64) although they
+// are only used outside the loop; how many rows the completion reads ahead matters as much (kAhead).  Launches with one of pair and bias are common and have instantiations of their own, all else shares one.
 template <int K, int MT, int D, int W, bool G64, int EXT>
 __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_constant__ GemvParams p) {
     constexpr int kThreads = W * 32;
@@ -228,9 +228,10 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
         if (nd > 0) {
             __threadfence();
             // items of four consecutive rows; a thread reads several before it writes, so that the
-            // L2 round trips of a CTA that completes many chunks overlap (two of a pair, which has two sums of each: four spilled
-            // registers of the next segment's weights, 72B-shaped pair with two tokens 119 -> 104 us at K = 3, g = 64, 100 -> 72 at g = 128,
-            // 152 -> 111 at K = 4, g = 64; with one token 34.6 -> 32.7 at K = 2)
+            // L2 round trips of a CTA that completes many chunks overlap: four, or two of a pair, which has two sums of each and spilled the
+            // next segment's weights with four.  72B-shaped pair, us with the shared instantiation, with its own and four, with its own and two:
+            // two tokens 119.5 / 112.9 / 104.2 at K = 3, g = 64, 101.2 / 93.9 / 72.8 at g = 128, 152.2 / 121.2 / 112.3 at K = 4, g = 64; one token 34.7 / 34.0 / 33.0
+            // at K = 2, 69.9 / 65.6 / 45.2 at K = 3.  (Instantiations without a pair spill 4 to 36 bytes with four at g = 64, most of which two would end.)
             constexpr int kQuads = kChunkRgs * 16 / 4, kAhead = (EXT & kExtPair) ? 2 : 4;
             const int nitems = nd * MT * kQuads;
             for (int i0 = tid; i0 < nitems; i0 += kThreads * kAhead) {
