@@ -182,9 +182,17 @@ int check_batch_handles(const bpdq_handle_t* hs, int n, int M, const char* who) 
     return M == 0 ? BPDQ_OK : check_device(hs[0], who);
 }
 
-// Whether a launch goes to the look-up-table kernel: up to the first linear's threshold.  (Two tokens at K = 3, g = 64 are
-// faster through the tensor-core kernel, but it rounds the weights to binary16 and this one does not.)
-bool prefer_lut(bpdq_handle_s* const* hs, int M) { return M <= hs[0]->gemv_max_m; }
+// Whether a launch goes to the look-up-table kernel: up to the first linear's threshold, but for large launches that the kernel with the planes as a
+// sparse operand, which does not round the weights either, is faster at.  (Not where a caller has set a threshold, and not through a permutation, which only the
+// look-up-table kernel folds into its load of x.)
+bool prefer_lut(bpdq_handle_s* const* hs, int n, int M) {
+    const bpdq_handle_s* h = hs[0];
+    if (M > h->gemv_max_m) return false;
+    if (h->gemv_set || h->few_set) return true;
+    for (int k = 0; k < n; ++k)
+        if (hs[k]->d_perm || !gemm_batch_supported(hs[k], M)) return true;
+    return !sp_before_lut(h->K, h->group == 64, M, sp_units(hs, n), h->sm_count);
+}
 
 }  // namespace
 
@@ -219,6 +227,7 @@ extern "C" int bpdq_create(bpdq_handle_t* hp, int out, int in, int K, int group,
     // us back to back: one token 16.3 / 34.2 (K = 2), 23.9 / 38.3 (K = 3), 30.9 / 72.0 (K = 4), two tokens 24.4 / 34.2, 36.3 / 38.3, 45.4 / 72.0;
     // a second pass loses, three tokens 40.6 / 34.3, 62.3 / 38.3, and so does one with a coefficient group per half block at K = 3, two
     // tokens (41.9 / 40.0), which stays for its weights' sake.  So does a second pass at K = 4, three tokens: 76.1 / 72.1 (4096 x 4096: 12.9 / 10.0).
+    // (Large launches at K = 3, g = 64 and at K = 4 leave it earlier for a kernel that does not round either: prefer_lut.)
     h->gemv_max_m = K == 4 && group != 64 ? 3 : 2;
     h->few_max_m = 0;                                    // the few-token kernel runs for callers that ask for it
 
@@ -279,7 +288,7 @@ extern "C" int bpdq_linear_ex(bpdq_handle_t h, const void* x, void* y, int M, in
         const bool gv = gemv_supported(h->out, h->in, h->K, h->group);
         const bool gm = gemm_supported(h->out, h->in, h->K, h->group);
         const bool fw = gemv_mma_supported(h->out, h->in, h->K, h->group);
-        if (gv && (prefer_lut(&h, M) || !gm) && M <= BPDQ_GEMV_MAX_M) kernel = BPDQ_KERNEL_GEMV;
+        if (gv && (prefer_lut(&h, 1, M) || !gm) && M <= BPDQ_GEMV_MAX_M) kernel = BPDQ_KERNEL_GEMV;
         else if (fw && h->few_max_m && M <= h->few_max_m && M <= BPDQ_FEW_MAX_M) kernel = BPDQ_KERNEL_FEW;
         else if (gm) kernel = BPDQ_KERNEL_GEMM;
         else kernel = BPDQ_KERNEL_GEMV_SIMPLE;
@@ -324,7 +333,7 @@ extern "C" int bpdq_linear_batch(const bpdq_handle_t* hs, const void* const* xs,
     // above the look-up-table threshold the tensor-core kernel (or the few-token kernel, if asked for) takes the whole batch,
     // when every linear allows it.  A caller who has set the few-token threshold has also set where the rounding of weights to
     // binary16 ends: above it come passes of the look-up-table kernel, which does not round them.
-    bool gemm = !prefer_lut(hs, M) && !hs[0]->few_set;
+    bool gemm = !prefer_lut(hs, n, M) && !hs[0]->few_set;
     bool few = M > hs[0]->gemv_max_m && M <= hs[0]->few_max_m && M <= BPDQ_FEW_MAX_M;
     for (int k = 0; few && k < n; ++k)
         few = hs[k]->d_few_maps && gemv_mma_supported(hs[k]->out, hs[k]->in, hs[k]->K, hs[k]->group) &&
@@ -433,6 +442,7 @@ extern "C" int bpdq_set_gemv_max_m(bpdq_handle_t h, int max_gemv_m) {
     if (max_gemv_m < 0 || max_gemv_m > BPDQ_GEMV_MAX_M)
         return set_error(BPDQ_ERR_INVALID, "bpdq_set_gemv_max_m: %d outside [0, %d]", max_gemv_m, BPDQ_GEMV_MAX_M);
     h->gemv_max_m = max_gemv_m;
+    h->gemv_set = 1;
     return BPDQ_OK;
 }
 
@@ -597,7 +607,7 @@ extern "C" int bpdq_gate_up_swiglu(bpdq_handle_t hg, bpdq_handle_t hu, const voi
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     bpdq_handle_s* hs[2] = {hg, hu};
     const bool same_g64 = (hg->group == 64) == (hu->group == 64);
-    const bool lut = same_g64 && prefer_lut(hs, M) && M <= BPDQ_GEMV_MAX_M && gemv_supported(hg->out, hg->in, hg->K, hg->group) &&
+    const bool lut = same_g64 && prefer_lut(hs, 2, M) && M <= BPDQ_GEMV_MAX_M && gemv_supported(hg->out, hg->in, hg->K, hg->group) &&
                      gemv_supported(hu->out, hu->in, hu->K, hu->group);
     bool few = same_g64 && !lut && M <= hg->few_max_m && M <= BPDQ_FEW_MAX_M && hg->d_few_maps && hu->d_few_maps &&
                (size_t)M * hg->out * sizeof(float) <= hg->ws_bytes && (size_t)M * hu->out * sizeof(float) <= hu->ws_bytes;

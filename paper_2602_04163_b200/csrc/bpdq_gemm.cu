@@ -12,9 +12,10 @@
 // 16-byte chunk c of row r is stored at chunk position c ^ (r mod 8).  TMA writes that layout by
 // itself; the decode threads reproduce it by hand.
 //
-// Two kernels: gemm_ts_kernel (up to 128 tokens: decoded weights in TMEM, one or several linears per launch;
+// Three kernels: gemm_sp_kernel (up to 16 tokens on large linears: the planes themselves as a sparse operand, nothing is decoded;
+// bpdq_gemm_sp.cuh), gemm_ts_kernel (up to 128 tokens: decoded weights in TMEM, one or several linears per launch;
 // bpdq_gemm_ts.cuh) and gemm_wide_kernel (more than 128 tokens, fewer where rows are short and tiles many: token tiles of up to 512;
-// bpdq_gemm_wide.cuh).  In the second the decoded operand goes through shared memory and feeds one MMA of up to 256 tokens or two; tiles of 512 tokens are
+// bpdq_gemm_wide.cuh).  In the last the decoded operand goes through shared memory and feeds one MMA of up to 256 tokens or two; tiles of 512 tokens are
 // bound by the MMAs, tiles of up to 160 by the decode.
 //
 // Decode: a thread reads its row's units and coefficients from the stage, builds the 2^K candidate values of the group
@@ -95,6 +96,7 @@ __host__ __device__ constexpr unsigned instr_desc_f16(int m, int n) {
 
 #include "bpdq_gemm_wide.cuh"
 #include "bpdq_gemm_ts.cuh"
+#include "bpdq_gemm_sp.cuh"
 
 // ---- host side ------------------------------------------------------------------------------
 using bpdq::EncodeTiledFn;
@@ -124,6 +126,55 @@ int ensure_packed_maps(bpdq_handle_s* h, EncodeTiledFn enc) {
     if (r1 != CUDA_SUCCESS || r2 != CUDA_SUCCESS)
         return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: tensor map encode of the packed weights failed (CUresult %d, %d)", (int)r1, (int)r2);
     h->gemm_maps_ready = 1;
+    return BPDQ_OK;
+}
+
+// Few tokens: one or several linears (same K, all or none with group 64); pair: the gated unit of two.
+template <int K, int NG>
+int launch_sp(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair) {
+    static bpdq::SmemOptin optin;
+    bpdq_handle_s* h0 = hs[0];
+    const int smem = bpdq::sp_smem(M);
+    if (kSpSmem > h0->smem_optin)
+        return bpdq::set_error(BPDQ_ERR_UNSUPPORTED, "gemm: %d bytes of shared memory needed, device offers %d", kSpSmem, h0->smem_optin);
+    if (const int rc = bpdq::ensure_smem_optin(gemm_sp_kernel<K, NG, 16>, optin, h0->device, kSpSmem, "gemm"); rc != BPDQ_OK) return rc;
+    SpParams p;
+    p.n = n; p.M = M;
+    p.status = h0->d_status;
+    long long units = 0;
+    for (int k = 0; k < n; ++k) {
+        const bpdq_handle_s* h = hs[k];
+        if (!h->d_few_maps)
+            return bpdq::set_error(BPDQ_ERR_UNSUPPORTED, "gemm: linear %d has no tensor maps (the driver did not offer cuTensorMapEncodeTiled)", k);
+        SpLinear& L = p.lin[k];
+        L.maps = static_cast<const CUtensorMap*>(h->d_few_maps) + 2;
+        L.x = static_cast<const __half*>(xs[k]);
+        L.y = static_cast<__half*>(ys[pair ? 0 : k]);
+        L.ws = h->d_ws; L.counters = pair ? h0->d_counters : h->d_counters;
+        L.conv_a = pair ? h0->d_ws : h->d_ws; L.conv_b = pair ? hs[1]->d_ws : nullptr;
+        L.bias_a = static_cast<const __half*>(pair ? h0->d_bias : h->d_bias);
+        L.bias_b = pair ? static_cast<const __half*>(hs[1]->d_bias) : nullptr;
+        L.out = h->out; L.in = h->in; L.nblocks = h->in / 128; L.ntiles = (h->out + BM - 1) / BM;
+        L.gsh = h->group == 64 ? 0 : (h->group == 128 ? 1 : 2);
+        L.u_begin = (int)units;
+        units += (long long)L.ntiles * L.nblocks;
+    }
+    const bpdq::SpRings rings = bpdq::sp_rings(K, 16, smem);
+    p.sb = rings.sb;
+    for (int k = 0; k < n; ++k) p.lin[k].ns = bpdq::sp_slices(p.lin[k].nblocks, rings.sb);
+    p.sp = rings.sp;
+    p.units = (int)units;
+    const long long ctas = (units + 3) / 4;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(ctas < h0->sm_count ? ctas : h0->sm_count)); cfg.blockDim = dim3(kSpThreads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the first packed blocks are requested under the tail of the kernel before
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_sp_kernel<K, NG, 16>, p);
+    h0->launches += 1;
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
     return BPDQ_OK;
 }
 
@@ -191,6 +242,13 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
     return BPDQ_OK;
 }
 
+// Up to 128 tokens: the few-token kernel where it is the faster one, else the TMEM kernel.
+template <int K>
+int launch_up_to_128(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair) {
+    if (!bpdq::sp_takes(K, M, bpdq::sp_units(hs, n), hs[0]->sm_count)) return launch_ts<K>(hs, xs, ys, n, M, stream, pair);
+    return hs[0]->group == 64 ? launch_sp<K, 2>(hs, xs, ys, n, M, stream, pair) : launch_sp<K, 1>(hs, xs, ys, n, M, stream, pair);
+}
+
 template <int K, int BKW, int NG>
 int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaStream_t stream) {
     static bpdq::SmemOptin optin;
@@ -237,7 +295,7 @@ int launch_wide(bpdq_handle_s* h, const void* x, void* y, int M, int half, cudaS
 
 template <int K>
 int launch_k(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_t stream) {
-    if (M <= kTsMaxM && !bpdq::ts_drain_bound((h->out + BM - 1) / BM, h->in / 128, M, h->sm_count)) return launch_ts<K>(&h, &x, &y, 1, M, stream, false);
+    if (M <= kTsMaxM && !bpdq::ts_drain_bound((h->out + BM - 1) / BM, h->in / 128, M, h->sm_count)) return launch_up_to_128<K>(&h, &x, &y, 1, M, stream, false);
     const int half = bpdq::wide_half(M, (h->out + BM - 1) / BM, h->in / 128, K, h->sm_count);
     if constexpr (K < 4)
         if (bpdq::wide_groups(K, half) == 4) return launch_wide<K, 64, 4>(h, x, y, M, half, stream);
@@ -275,6 +333,12 @@ bool gemm_supported(int, int, int K, int group) {
     return K >= 1 && K <= 4 && (group == 64 || group == 128 || group == 256);
 }
 
+long long sp_units(const bpdq_handle_s* const* hs, int n) {
+    long long units = 0;
+    for (int k = 0; k < n; ++k) units += (long long)((hs[k]->out + BM - 1) / BM) * (hs[k]->in / 128);
+    return units;
+}
+
 bool gemm_batch_supported(const bpdq_handle_s* h, int M) { return h->d_few_maps && M <= kTsMaxM && gemm_supported(h->out, h->in, h->K, h->group); }
 
 int launch_gemm_batch(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair) {
@@ -284,10 +348,10 @@ int launch_gemm_batch(bpdq_handle_s* const* hs, const void* const* xs, void* con
         if (hs[k]->K != hs[0]->K || (hs[k]->group == 64) != (hs[0]->group == 64) || !gemm_batch_supported(hs[k], M))
             return set_error(BPDQ_ERR_INVALID, "gemm: linear %d does not go into one launch with linear 0 (M=%d)", k, M);
     switch (hs[0]->K) {
-        case 1: return launch_ts<1>(hs, xs, ys, n, M, stream, pair);
-        case 2: return launch_ts<2>(hs, xs, ys, n, M, stream, pair);
-        case 3: return launch_ts<3>(hs, xs, ys, n, M, stream, pair);
-        case 4: return launch_ts<4>(hs, xs, ys, n, M, stream, pair);
+        case 1: return launch_up_to_128<1>(hs, xs, ys, n, M, stream, pair);
+        case 2: return launch_up_to_128<2>(hs, xs, ys, n, M, stream, pair);
+        case 3: return launch_up_to_128<3>(hs, xs, ys, n, M, stream, pair);
+        case 4: return launch_up_to_128<4>(hs, xs, ys, n, M, stream, pair);
         default: return set_error(BPDQ_ERR_UNSUPPORTED, "gemm: K=%d", hs[0]->K);
     }
 }

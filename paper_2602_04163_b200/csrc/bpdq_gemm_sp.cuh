@@ -1,0 +1,537 @@
+// Included by bpdq_gemm.cu (inside its unnamed namespace, after bpdq_gemm_ts.cuh): the kernel for few tokens.
+//
+// gemm_sp_kernel: the bit planes themselves are the MMA's operand, as the positions of a 2:4 sparse matrix.  Per plane i and row
+//
+//     sum_j b_ij c_i x_j  =  A B,   B = (0, x_0, 0, x_1, 0, x_2, ...) along K,   A = c_i in every group of four at one of
+//                                   positions 0, 1 (b = 0, 1) and at one of positions 2, 3:
+//
+// the compressed A is c_i everywhere (8 TMEM columns per plane and 128-column block, whatever the bits) and the sparsity metadata,
+// four bits per group of four, is "1 b 0 b": one mask of a packed word gives the metadata of sixteen columns.  So a block of 128
+// columns costs a thread some 20 instructions per plane where decoding its weights into binary16 takes 186 (K = 2) to 450 (K = 4),
+// and the weights are not rounded.  c_0 sum_j x_j is one dense MMA per block: K = four 32-column sums of x, each as binary16 parts
+// (high, low, what exceeds binary16 / 64).  Bound: with 16 token columns a block's 8 K + 1 MMAs take 10 clocks each, less than its
+// packed bytes take from HBM; from 32 on the MMAs (16 clocks at 32, 24 at 48).
+//
+// A sparse MMA (K = 32, i.e. 16 columns of a plane) takes its metadata from one TMEM column: lane 16 a + 8 h + b holds the 16 bits
+// of K half h of rows 16 a + b (low) and 16 a + b + 8 (high).  So the thread of row r reads, of rows r & ~8 and r | 8, the words
+// 2 h and 2 h + 1 (h = bit 3 of r): K half h of a block's MMAs comes from the words 2 h, 2 h + 1, which is also the coefficient group of
+// g = 64.  MMA (e, x, d) of a plane: word 2 h + e, bits 16 x + 2 s + d for s = 0..7.
+//
+// Work split: units are (row tile, block) pairs, slice by slice (a slice: `sb` blocks of columns), in a slice tile by tile; every CTA
+// takes an equal contiguous share.  x of a slice stays in shared memory, zeros and all, while the CTA walks over the slice's row
+// tiles; the sums of a (tile, slice) go into the handle's binary32 workspace, and when a CTA leaves a slice it counts the blocks it
+// has delivered; who delivers a tile's last block rounds the sums to y.
+//
+// Roles (768 threads): two pipelines, one for the even and one for the odd blocks of a slice, each with a ring of packed blocks
+// (one producer warp), two decode groups of four warps, an operand slot in TMEM per group and an MMA issuer with an accumulator of
+// its own; four warps expand x and drain.  A pipeline's rings belong to it alone, so that waits by parity follow their phases:
+// the group that waits for packed block q has waited for the MMAs of block q - 4 (its operand slot, two blocks before), and an issuer's MMAs
+// complete in order, so with four slots or more the copy of the slot's last use has landed.
+using bpdq::kSpSmem;
+constexpr int kSpFirstDecode = 4, kSpFirstEpi = 20;
+constexpr int kSpThreads = 32 * (kSpFirstEpi + 4);
+constexpr unsigned kSpSumBytes = bpdq::kSpSumBytes;
+constexpr int kSpMaxDone = 64;
+
+struct SpLinear {
+    const CUtensorMap* maps;   // planes and coefficients of one 128-row x 128-column block
+    const __half* x;           // [M][in]
+    __half* y;                 // [M][out]
+    float* ws;                 // [M][out] binary32, zero between calls
+    unsigned* counters;        // blocks delivered per 128-row tile, zero between calls (a pair: the gate's)
+    float* conv_a;             // a pair: the gate's and the up projection's sums
+    float* conv_b;             // null unless paired
+    const __half* bias_a;      // binary16 [out] added before the rounding, or null
+    const __half* bias_b;
+    int out, in, nblocks, ntiles, gsh;   // rows, columns, 128-column blocks per row, row tiles, log2(group / 64)
+    int ns;                    // slices
+    int u_begin;               // first unit
+};
+struct SpParams {
+    SpLinear lin[BPDQ_BATCH_MAX];
+    int n, M;                  // linears; tokens
+    int* status;
+    int units;
+    int sb, sp;                // blocks of a slice at most; packed slots per pipeline
+};
+// A stretch of one row tile inside a slice: blocks s0 + o .. s0 + o + n - 1 of the row, units u .. u + n - 1.  [seg_begin, seg_end): the
+// CTA's units in this slice; a block's next use is w units on.
+struct SpPiece {
+    int li, tile, s0, w, o, n, u, seg_begin, seg_end;
+};
+__device__ __forceinline__ int sp_share(const SpParams& p, int s) { return (int)((long long)p.units * s / gridDim.x); }
+// The first piece at unit u: linear, slice, tile and block come from divisions, a thousand clocks of them ...
+__device__ __forceinline__ void sp_seek(const SpParams& p, const int begin, const int end, const int u, SpPiece& c) {
+    c.li = 0;
+    while (c.li + 1 < p.n && u >= p.lin[c.li + 1].u_begin) ++c.li;
+    const SpLinear& L = p.lin[c.li];
+    const int rel = u - L.u_begin, s = bpdq::sp_slice_of(rel / L.ntiles, L.nblocks, L.ns);
+    c.s0 = bpdq::sp_slice(s, L.nblocks, L.ns);
+    c.w = bpdq::sp_slice(s + 1, L.nblocks, L.ns) - c.s0;
+    const int in_slice = rel - c.s0 * L.ntiles, first = L.u_begin + c.s0 * L.ntiles;
+    c.tile = in_slice / c.w;
+    c.o = in_slice - c.tile * c.w;
+    c.n = min(c.w - c.o, end - u);
+    c.u = u;
+    c.seg_begin = max(begin, first);
+    c.seg_end = min(end, first + c.w * L.ntiles);
+}
+// ... so pieces of the same slice follow from the one before.
+__device__ __forceinline__ bool sp_next(const SpParams& p, const int begin, const int end, SpPiece& c) {
+    const int u = c.u + c.n;
+    if (u >= end) return false;
+    if (u >= c.seg_end) {
+        sp_seek(p, begin, end, u, c);
+    } else {
+        ++c.tile;
+        c.o = 0;
+        c.u = u;
+        c.n = min(c.w, end - u);
+    }
+    return true;
+}
+
+// K-major tile with 32-byte swizzle: rows 32 bytes apart, eight rows per 256-byte atom, layout type 6
+__device__ __forceinline__ uint64_t smem_desc_sw32(unsigned addr) {
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
+}
+// Instruction descriptor bits of a sparse MMA: sparse flag, and which of the two metadata columns at the (even) address
+constexpr unsigned kSparse = 4u;
+__device__ __forceinline__ void umma_f16_sp(unsigned d, unsigned a, uint64_t bdesc, unsigned meta, unsigned idesc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, 1, 0;\n\t"
+        "tcgen05.mma.sp.cta_group::1.kind::f16 [%0], [%1], %2, [%3], %4, p;\n\t}"
+        ::"r"(d), "r"(a), "l"(bdesc), "r"(meta), "r"(idesc) : "memory");
+}
+__device__ __forceinline__ void tmem_st8(unsigned t, const unsigned (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"r"(t), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+
+// adds `bytes` of binary32 from shared memory to global memory; bulk_wait: this thread's adds have arrived
+__device__ __forceinline__ void bulk_add(float* dst, unsigned src, unsigned bytes) {
+    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_wait() {
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    asm volatile("fence.proxy.async;" ::: "memory");
+}
+__device__ __forceinline__ unsigned shf_left(unsigned lo, unsigned hi, unsigned sh) {
+    unsigned v;
+    asm("shf.l.wrap.b32 %0, %1, %2, %3;" : "=r"(v) : "r"(lo), "r"(hi), "r"(sh));
+    return v;
+}
+__device__ __forceinline__ unsigned lds32(unsigned addr) {
+    unsigned v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ unsigned lds16(unsigned addr) {
+    unsigned v;
+    asm volatile("{\n\t.reg .u16 t;\n\tld.shared.u16 t, [%1];\n\tcvt.u32.u16 %0, t;\n\t}" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void tmem_st4(unsigned t, unsigned a, unsigned b, unsigned c, unsigned d) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(t), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
+// NG: coefficient groups per block, 1 or 2 (a branch on it in the decode costs K = 2 1.8 us of 30 on a 72 MB projection)
+template <int K, int NG, int N>
+__global__ void __launch_bounds__(kSpThreads, 1) gemm_sp_kernel(const __grid_constant__ SpParams p) {
+    using C = TsCfg<K>;
+    constexpr int kSlotCols = bpdq::sp_slot_cols(K);               // TMEM: metadata (8 per plane), then c_0's operand and the planes'
+    constexpr int NA = bpdq::sp_slots(K);                          // operand slots of a pipeline
+    constexpr int kBarX = 4 * NA + 4;
+    extern __shared__ unsigned char smem_raw[];
+    const unsigned base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
+    const int SB = p.sb, SP = p.sp;
+    constexpr unsigned xs = (unsigned)N * 512u, zs = (unsigned)N * 32u;     // a block's expanded x and its sums
+    const unsigned x_base = base, z_base = base + (unsigned)SB * xs, r_base = z_base + (unsigned)SB * zs, p_base = r_base + 2u * kSpSumBytes;
+    const unsigned bar_base = p_base + (unsigned)(2 * SP) * C::kSlotBytes;
+    auto full_a = [&](int s) { return bar_base + 8u * s; };                 // operand slots: pipeline * NA + slot
+    auto empty_a = [&](int s) { return bar_base + 8u * (2 * NA + s); };
+    auto acc_full = [&](int b) { return bar_base + 8u * (4 * NA + b); };
+    auto acc_empty = [&](int b) { return bar_base + 8u * (4 * NA + 2 + b); };
+    auto full_x = [&](int s) { return bar_base + 8u * (kBarX + s); };
+    auto empty_x = [&](int s) { return bar_base + 8u * (kBarX + SB + s); };
+    auto full_p = [&](int s) { return bar_base + 8u * (kBarX + 2 * SB + s); };       // packed slots: pipeline * SP + slot
+    auto empty_p = [&](int s) { return bar_base + 8u * (kBarX + 2 * SB + 2 * SP + s); };
+    const int nbars = kBarX + 2 * SB + 4 * SP;
+    unsigned* tmem_slot = reinterpret_cast<unsigned*>(smem + (bar_base - base) + 8 * nbars);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* ndone = reinterpret_cast<volatile int*>(tmem_slot + 2);
+    volatile int* full = reinterpret_cast<volatile int*>(tmem_slot + 3);    // [2] the list is full, as of this piece and the one before
+    volatile int* done = reinterpret_cast<volatile int*>(tmem_slot + 5);    // [kSpMaxDone] complete tiles: linear << 24 | tile
+
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int begin = sp_share(p, blockIdx.x), end = sp_share(p, blockIdx.x + 1);
+
+    if (tid == 0) {
+        for (int s = 0; s < 2 * NA; ++s) { mbar_init(full_a(s), 4); mbar_init(empty_a(s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), 2); mbar_init(acc_empty(b), 4); }
+        for (int s = 0; s < SB; ++s) { mbar_init(full_x(s), 4); mbar_init(empty_x(s), 1); }
+        for (int s = 0; s < 2 * SP; ++s) { mbar_init(full_p(s), 1); mbar_init(empty_p(s), 4); }
+        *abort_flag = 0;
+        *ndone = full[0] = full[1] = 0;
+        fence_barrier_init();
+    }
+    if (warp == 2) {
+        tmem_alloc(smem_u32(tmem_slot), 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    // only now: a CTA of the next kernel that took this SM's TMEM first and then waited for this kernel would keep it
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const unsigned tmem = *tmem_slot, tmem_d = tmem + 2u * NA * kSlotCols;       // accumulators: (2 * buffer + pipeline) * N columns
+    const unsigned quad_lanes = (unsigned)((warp & 3) * 32) << 16;          // TMEM lane quadrant this warp may access
+
+    // Complete tiles are rounded, written to y and their sums zeroed by `threads` threads; an item is four rows of one token.
+    auto convert = [&](const int first, const int threads) {
+        const int nd = *ndone, M = p.M;
+        if (nd == 0) return;
+        __threadfence();
+        constexpr int kAhead = 2;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k0 = first; k0 < nd * M * 32; k0 += threads * kAhead) {
+            float4 v[kAhead], vb[kAhead];
+#pragma unroll
+            for (int e = 0; e < kAhead; ++e) {
+                const int k = k0 + e * threads, d = (k >> 5) / M, t = (k >> 5) - d * M;
+                if (k >= nd * M * 32) break;
+                const SpLinear& L = p.lin[done[d] >> 24];
+                const int q = (done[d] & 0xFFFFFF) * 128 + (k & 31) * 4;
+                if (q >= L.out) continue;
+                v[e] = __ldcg(reinterpret_cast<const float4*>(L.conv_a + (size_t)t * L.out + q));
+                if (L.conv_b) vb[e] = __ldcg(reinterpret_cast<const float4*>(L.conv_b + (size_t)t * L.out + q));
+            }
+#pragma unroll
+            for (int e = 0; e < kAhead; ++e) {
+                const int k = k0 + e * threads, d = (k >> 5) / M, t = (k >> 5) - d * M;
+                if (k >= nd * M * 32) break;
+                const SpLinear& L = p.lin[done[d] >> 24];
+                const int q = (done[d] & 0xFFFFFF) * 128 + (k & 31) * 4;
+                if (q >= L.out) continue;
+                const size_t at = (size_t)t * L.out + q;
+                bpdq::finish_quad(v[e], vb[e], L.bias_a, L.bias_b, L.conv_b != nullptr, q);
+                const __half2 h01 = __floats2half2_rn(v[e].x, v[e].y), h23 = __floats2half2_rn(v[e].z, v[e].w);
+                uint2 o;
+                o.x = *reinterpret_cast<const unsigned*>(&h01);
+                o.y = *reinterpret_cast<const unsigned*>(&h23);
+                *reinterpret_cast<uint2*>(L.y + at) = o;
+                __stcg(reinterpret_cast<float4*>(L.conv_a + at), zero);
+                if (L.conv_b) __stcg(reinterpret_cast<float4*>(L.conv_b + at), zero);
+            }
+        }
+    };
+    if (warp < 2) {
+        // ---------------- packed blocks of one pipeline ----------------
+        if (elect_one()) {
+            const int pipe = warp;
+            int sl = 0;
+            unsigned ph = 1u;
+            bool ok = true;
+            SpPiece c;
+            sp_seek(p, begin, end, begin, c);
+            do {
+                const CUtensorMap* maps = p.lin[c.li].maps;
+                const int gsh = p.lin[c.li].gsh;
+                for (int o = c.o + ((c.o ^ pipe) & 1); o < c.o + c.n; o += 2) {
+                    const int s = pipe * SP + sl, b = c.s0 + o;
+                    if (!mbar_wait(empty_p(s), ph, abort_flag, p.status)) { ok = false; break; }
+                    const unsigned dst = p_base + (unsigned)s * C::kSlotBytes, bar = full_p(s);
+                    mbar_expect_tx(bar, (unsigned)(C::kPlaneBytes + NG * C::kCoefBytes));
+                    tma_load_2d(dst, &maps[0], c.tile * 256, b * K, bar);                    // 8-byte elements: two per row
+                    tma_load_2d(dst + C::kPlaneBytes, &maps[1], c.tile * 32, ((2 * b) >> gsh) * (K + 1), bar);
+                    if (++sl == SP) { sl = 0; ph ^= 1u; }
+                }
+            } while (ok && sp_next(p, begin, end, c));
+        }
+        __syncwarp();
+    } else if (warp < kSpFirstDecode) {
+        // ---------------- MMA issuer of one pipeline ----------------
+        if (elect_one()) {
+            const int pipe = warp - 2;
+            constexpr unsigned idesc = instr_desc_f16(BM, N);
+            int sa = 0, buf = 0;
+            unsigned pa = 0u, pacc = 1u, px = 0u;        // px: a bit per x slot
+            bool ok = true;
+            SpPiece c;
+            sp_seek(p, begin, end, begin, c);
+            do {
+                ok = mbar_wait(acc_empty(buf), pacc, abort_flag, p.status);
+                const unsigned d = tmem_d + (unsigned)((2 * buf + pipe) * N);
+                unsigned more = 0u;
+                for (int o = c.o + ((c.o ^ pipe) & 1); o < c.o + c.n && ok; o += 2) {
+                    const int ub = c.u + o - c.o;
+                    if (ub - c.w < c.seg_begin) {        // first use of this block's x
+                        ok = mbar_wait(full_x(o), (px >> o) & 1u, abort_flag, p.status);
+                        px ^= 1u << o;
+                    }
+                    ok = ok && mbar_wait(full_a(pipe * NA + sa), pa, abort_flag, p.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const unsigned meta = tmem + (unsigned)((pipe * NA + sa) * kSlotCols), a = meta + 8 * K;
+                    umma_f16_ts(d, a, smem_desc_sw32(z_base + (unsigned)o * zs), idesc, more);
+                    more = 1u;
+                    const uint64_t b0 = smem_desc_sw128(x_base + (unsigned)o * xs);
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) {
+                        const uint64_t b = b0 + (uint64_t)((m >> 1) * (N * 8) + (m & 1) * 4);
+#pragma unroll
+                        for (int i = 0; i < K; ++i)
+                            umma_f16_sp(d, a + 8 * (i + 1), b, meta + 8 * i + (m & 6), idesc | kSparse | (m & 1));
+                    }
+                    umma_commit(empty_a(pipe * NA + sa));
+                    if (ub + c.w >= c.seg_end) umma_commit(empty_x(o));      // last use
+                    if (++sa == NA) { sa = 0; pa ^= 1u; }
+                }
+                if (ok) umma_commit(acc_full(buf));
+                buf ^= 1;
+                if (buf == 0) pacc ^= 1u;
+            } while (ok && sp_next(p, begin, end, c));
+        }
+        __syncwarp();
+    } else if (warp < kSpFirstEpi) {
+        // ---------------- decode warps: from packed blocks to metadata and coefficient operands ----------------
+        const int wd = warp - kSpFirstDecode, pipe = wd >> 3, grp = (wd >> 2) & 1;
+        const int rl = (warp & 3) * 32 + lane, ra = rl & ~8, h = (rl >> 3) & 1, M = p.M;
+        const unsigned sh = (unsigned)(rl & 3) * 8u;
+        // logical word k of row r takes the bytes of physical words k - wrot and k - wrot - 1, wrot = (r / 4) mod 4; words 2 h and 2 h + 1 need
+        // three of them, and row r + 8 has them two words on
+        unsigned off_a[3], off_b[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const unsigned w = (unsigned)(2 * h + j - 1 - (ra >> 2)) & 3u, at = p_base + (unsigned)(pipe * SP) * C::kSlotBytes + (unsigned)ra * 16u;
+            off_a[j] = at + 4u * w;
+            off_b[j] = at + 128u + 4u * (w ^ 2u);
+        }
+        const unsigned off_c = p_base + (unsigned)(pipe * SP) * C::kSlotBytes + C::kPlaneBytes + (unsigned)rl * 2u;
+        unsigned ex = 0u;                                // a bit per x slot: its phase
+        // x of a segment's blocks, in the order of their first use.  Block o of a slice belongs to group o mod 4 (pipeline + 2 * group), which alone
+        // waits for its slot's releases, one phase after the other.  A thread takes (token, 32-column word, parity d of the bits): columns
+        // 8 d .. + 7 and 8 (d + 2) .. + 7 of the word, i.e. bits 4 j + d and 4 j + d + 2, which go side by side.
+        const int mine = pipe + 2 * grp, xt = (warp & 3) * 4 + (lane >> 3), xd = lane & 1, xe = (lane >> 1) & 1, xk = (lane >> 2) & 1;
+        auto load_x = [&](const SpLinear& L, const int s0, const int o, uint4 (&va)[N / 16], uint4 (&vb)[N / 16]) {
+            const __half* src = L.x + (size_t)xt * L.in + (size_t)(s0 + o) * 128 + 64 * xk + 32 * xe + 8 * xd;
+#pragma unroll
+            for (int q = 0; q < N / 16; ++q, src += (size_t)16 * L.in) {
+                va[q] = vb[q] = make_uint4(0u, 0u, 0u, 0u);
+                if (xt + 16 * q < M) {
+                    va[q] = __ldcg(reinterpret_cast<const uint4*>(src));
+                    vb[q] = __ldcg(reinterpret_cast<const uint4*>(src) + 2);
+                }
+            }
+        };
+        auto store_x = [&](const int o, const uint4 (&va)[N / 16], const uint4 (&vb)[N / 16]) -> bool {
+            if (!mbar_wait_warp(empty_x(o), ((ex >> o) & 1u) ^ 1u, abort_flag, p.status)) return false;
+            ex ^= 1u << o;
+#pragma unroll
+            for (int q = 0; q < N / 16; ++q) {
+                const int t = xt + 16 * q;
+                const unsigned ua[4] = {va[q].x, va[q].y, va[q].z, va[q].w}, ub[4] = {vb[q].x, vb[q].y, vb[q].z, vb[q].w};
+                float sums[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {            // e = 2 * (bits 16..31 of the word) + chunk
+                    const unsigned dst = x_base + (unsigned)o * xs + (unsigned)((2 * xe + (e >> 1)) * N + t) * 128u +
+                                         ((unsigned)((4 * xd + 2 * xk + (e & 1)) ^ (t & 7)) << 4);
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(ua[e] << 16), "r"(ub[e] << 16),
+                                 "r"(ua[e] & 0xFFFF0000u), "r"(ub[e] & 0xFFFF0000u) : "memory");
+                    const float2 fa = __half22float2(*reinterpret_cast<const __half2*>(&ua[e])), fb = __half22float2(*reinterpret_cast<const __half2*>(&ub[e]));
+                    sums[e] = (fa.x + fa.y) + (fb.x + fb.y);
+                }
+                float sum = (sums[0] + sums[1]) + (sums[2] + sums[3]);
+                sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                if (xd == 0) {
+                    // sum = hi + lo + 64 big; an infinite or undefined one is in `big` alone
+                    const float bigf = fabsf(sum) <= 32768.f ? 0.f : sum * (1.f / 64.f);
+                    const __half bg = __float2half_rn(bigf);
+                    const bool finite = fabsf(sum) <= 3.0e38f;
+                    const float rest = finite ? sum - 64.f * __half2float(bg) : 0.f;
+                    const __half hi = __float2half_rn(rest), lo = __float2half_rn(rest - __half2float(hi));
+                    const unsigned dst = z_base + (unsigned)o * zs + (unsigned)t * 32u + ((unsigned)(xk ^ ((t >> 2) & 1)) << 4) + 8u * xe;
+                    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(dst),
+                                 "r"((unsigned)__half_as_ushort(hi) | ((unsigned)__half_as_ushort(lo) << 16)), "r"((unsigned)__half_as_ushort(bg)) : "memory");
+                }
+            }
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full_x(o));
+            return true;
+        };
+        // blocks of this pipeline among the first v units of a slice of w blocks
+        auto below = [&](int v, int w) { return v / w * ((w + 1 - pipe) >> 1) + ((v % w + 1 - pipe) >> 1); };
+        int sl = grp, sa = grp, q = grp, nblk = 0;       // q: this group's next block of its pipeline's nblk so far
+        unsigned ph = 0u, pa = 1u;
+        bool ok = true;
+        unsigned even = 0x55555555u, ones = 0x88888888u;
+        asm volatile("" : "+r"(even), "+r"(ones));       // kept in registers
+        auto block = [&]() -> bool {
+            const int s = pipe * SP + sl;
+            if (!mbar_wait_warp(full_p(s), ph, abort_flag, p.status)) return false;
+            const unsigned so = (unsigned)sl * C::kSlotBytes;
+            unsigned md[K][8];
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                unsigned a[3], b[3];
+#pragma unroll
+                for (int e = 0; e < 3; ++e) {
+                    a[e] = lds32(so + off_a[e] + i * 2048);
+                    b[e] = lds32(so + off_b[e] + i * 2048);
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const unsigned wa = shf_left(a[e], a[e + 1], sh), wb = shf_left(b[e], b[e + 1], sh);
+                    const unsigned x0 = bpdq::prmt_raw(wa, wb, 0x5410u), x1 = bpdq::prmt_raw(wa, wb, 0x7632u);
+                    md[i][4 * e] = (x0 & even) | ones;
+                    md[i][4 * e + 1] = ((x0 >> 1) & even) | ones;
+                    md[i][4 * e + 2] = (x1 & even) | ones;
+                    md[i][4 * e + 3] = ((x1 >> 1) & even) | ones;
+                }
+            }
+            // coefficients in both halves of a register, c_0 with its 64-fold, kept finite since it multiplies zero but for sums above 32768
+            auto coefs = [&](const int g, unsigned (&cf)[K + 2]) {
+#pragma unroll
+                for (int i = 0; i <= K; ++i)
+                    cf[i] = bpdq::prmt_raw(lds16(so + off_c + (g * (K + 1) + i) * 256), 0u, 0x1010u);
+                const __half2 most = __half2half2(__ushort_as_half((unsigned short)0x7BFF));
+                const __half2 big = __hmin2(__hmax2(__hmul2(*reinterpret_cast<const __half2*>(&cf[0]), __half2half2(__ushort_as_half((unsigned short)0x5400))), __hneg2(most)), most);
+                cf[K + 1] = *reinterpret_cast<const unsigned*>(&big);
+            };
+            unsigned cf[K + 2];
+            coefs(0, cf);
+            if (!mbar_wait_warp(empty_a(pipe * NA + sa), pa, abort_flag, p.status)) return false;
+            tc_fence_after();
+            const unsigned slot = tmem + quad_lanes + (unsigned)((pipe * NA + sa) * kSlotCols);
+#pragma unroll
+            for (int i = 0; i < K; ++i) tmem_st8(slot + 8 * i, md[i]);
+            const unsigned c0 = slot + 8 * K;
+            tmem_st4(c0, cf[0], cf[K + 1], cf[0], cf[K + 1]);
+#pragma unroll
+            for (int i = 1; i <= K; ++i) tmem_st4(c0 + 8 * i, cf[i], cf[i], cf[i], cf[i]);
+            if (NG == 2) coefs(1, cf);
+            tmem_st4(c0 + 4, cf[0], cf[K + 1], cf[0], cf[K + 1]);
+#pragma unroll
+            for (int i = 1; i <= K; ++i) tmem_st4(c0 + 8 * i + 4, cf[i], cf[i], cf[i], cf[i]);
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(full_a(pipe * NA + sa));
+                mbar_arrive(empty_p(s));         // everything read from the slot has been stored as an operand
+            }
+            sa += 2;
+            if (sa >= NA) { sa -= NA; pa ^= 1u; }
+            q += 2;
+            sl += 2;
+            if (sl >= SP) { sl -= SP; ph ^= 1u; }
+            return true;
+        };
+        SpPiece c;
+        for (int u = begin; ok && u < end; u = c.seg_end) {
+            sp_seek(p, begin, end, u, c);
+            const SpLinear& L = p.lin[c.li];
+            const bpdq::SpFirstUses xb = bpdq::sp_first_uses(mine, c.o, c.w, c.seg_end - c.seg_begin);
+            const int nx = xb.n;
+            // two of the group's blocks of x first, then one ahead of every packed block: a pipeline's k-th block needs the x that some group
+            // has stored ahead of its own block k + 1 at the latest, for which that group waits no further than the MMAs of block k - 1
+            const int first = c.u - c.tile * c.w - c.o;          // the slice's first unit
+            nblk += below(c.seg_end - first, c.w) - below(c.seg_begin - first, c.w);
+            if (u == begin) {
+                if (q < nblk) ok = block();                      // needs nothing of the kernel before,
+                asm volatile("griddepcontrol.wait;" ::: "memory");   // which may have written x
+            }
+            uint4 va[N / 16], vb[N / 16], va2[N / 16], vb2[N / 16];
+            if (nx > 0) load_x(L, c.s0, xb.block(0), va, vb);
+            if (nx > 1) load_x(L, c.s0, xb.block(1), va2, vb2);
+            if (nx > 0) ok = ok && store_x(xb.block(0), va, vb);
+            if (nx > 1) ok = ok && store_x(xb.block(1), va2, vb2);
+            for (int j = 2; ok && (q < nblk || j < nx); ++j) {
+                if (j < nx) load_x(L, c.s0, xb.block(j), va, vb);
+                if (q < nblk) ok = block();
+                if (j < nx) ok = ok && store_x(xb.block(j), va, vb);
+            }
+        }
+    } else {
+        // ---------------- four warps drain finished pieces ----------------
+        const int et = tid - 32 * kSpFirstEpi, rl = (warp & 3) * 32 + lane, M = p.M;
+        // A piece's sums go through one of two buffers in shared memory and are added to the workspace by bulk copies, a lane of the first warp per
+        // token.  They are counted under the next piece's MMAs, when the adds have long arrived; who counts a tile's last block completes the tile,
+        // at the end of its work together with the decode warps (or when its list is full).
+        int buf = 0, li = -1, tile = 0;                  // linear, tile and blocks of the piece before (li < 0: none)
+        unsigned n = 0u, pacc = 0u;
+        SpPiece c;
+        sp_seek(p, begin, end, begin, c);
+        asm volatile("griddepcontrol.wait;" ::: "memory");   // the kernel before may still be reading what y overwrites
+        bool more = true;
+        while (true) {
+            if (li >= 0 && et < 32) {
+                bulk_wait();
+                __syncwarp();
+                if (et == 0) {
+                    const SpLinear& L = p.lin[li];
+                    __threadfence();
+                    const unsigned before = atomicAdd(&L.counters[tile], n);
+                    const bool all = before + n == (unsigned)(L.conv_b != nullptr ? 2 * L.nblocks : L.nblocks);
+                    if (all) L.counters[tile] = 0u;
+                    if (all) {
+                        done[*ndone] = (li << 24) | tile;
+                        *ndone = *ndone + 1;
+                    }
+                    full[buf] = *ndone == kSpMaxDone;
+                }
+                __syncwarp();
+            }
+            const bool got = more && mbar_wait_warp(acc_full(buf), pacc, abort_flag, p.status);
+            if (got) {
+                tc_fence_after();
+                // a piece of one block has one pipeline's sum only: it is taken for both and halved (exactly)
+                const float half = c.n > 1 ? 1.f : 0.5f;
+                const unsigned d = tmem_d + quad_lanes + (unsigned)(2 * buf * N);
+                const unsigned d0 = c.n > 1 ? d : d + (unsigned)((c.o & 1) * N), d1 = c.n > 1 ? d + (unsigned)N : d0;
+                unsigned v[N], v2[N];
+                static_assert(N == 16, "one load per accumulator");
+                tmem_ld16(d0, v);
+                tmem_ld16(d1, v2);
+                tmem_ld_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acc_empty(buf));
+                const unsigned at = r_base + (unsigned)buf * kSpSumBytes + (unsigned)rl * 4u;
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(at + j * 512), "f"((__uint_as_float(v[j]) + __uint_as_float(v2[j])) * half) : "memory");
+                fence_proxy_async();
+            }
+            bar_sync(1, 128);
+            if (got && et < M) {                         // (M <= 16: lanes of the first warp)
+                const SpLinear& L = p.lin[c.li];
+                bulk_add(L.ws + (size_t)et * L.out + c.tile * 128, r_base + (unsigned)buf * kSpSumBytes + (unsigned)et * 512u, (unsigned)min(128, L.out - c.tile * 128) * 4u);
+            }
+            if (full[buf]) {
+                convert(et, 128);
+                bar_sync(1, 128);
+                if (et == 0) *ndone = 0;
+                bar_sync(1, 128);
+            }
+            if (!more) break;
+            buf ^= 1;
+            if (buf == 0) pacc ^= 1u;
+            li = c.li; tile = c.tile; n = (unsigned)c.n;
+            more = sp_next(p, begin, end, c);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp >= kSpFirstDecode) convert(tid - 32 * kSpFirstDecode, kSpThreads - 32 * kSpFirstDecode);
+    if (warp == 2) {
+        tc_fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+    if (*abort_flag) linger();
+}

@@ -84,6 +84,7 @@ struct bpdq_handle_s {
     void* d_xstage;           // staging for bpdq_linear_host
     void* d_ystage;
     int gemv_max_m;
+    int gemv_set;             // the caller chose it (bpdq_set_gemv_max_m)
     uint64_t launches;
     int few_max_m;            // largest M the dispatcher sends to the few-token kernel
     int few_set;              // the caller chose it (bpdq_set_few_max_m)
@@ -112,6 +113,7 @@ int launch_gemv_mma(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_
 int launch_gemv_mma_batch(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair = false);
 int launch_gemm_batch(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair = false);
 bool gemm_batch_supported(const bpdq_handle_s* h, int M);
+long long sp_units(const bpdq_handle_s* const* hs, int n);          // 128-row x 128-column blocks of these linears
 bool gemv_mma_supported(int out, int in, int K, int group);
 int few_prepare(bpdq_handle_s* h);
 size_t gemv_workspace_bytes(int out, int in, int K, int group, int max_M, int sm_count);

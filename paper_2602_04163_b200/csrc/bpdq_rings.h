@@ -60,6 +60,76 @@ constexpr TsSplit ts_split(int tiles, int units, int nb0, int sms) {
     return w;
 }
 
+// Kernel for few tokens (planes as a sparse operand): `sb` blocks of expanded x (512 bytes per token and block, and 32 of sums) stay in shared
+// memory, the two pipelines share the rest for their packed rings of `sp` slots each.  sb is even, so that a slice begins with an even block.
+constexpr int kSpSmem = 227 * 1024;
+// Up to two tokens, which the look-up-table kernel takes in other launches of the same layer, the same split of an SM's memory into L1 cache and shared memory as
+// that kernel's at two tokens (192 KB): each change of the split between launches waits for an idle SM (72B-shaped layer, K = 3, g = 64, two tokens, {q, k, v}
+// and o there, the rest here: 147.3 us with 227 KB, 142.9 with 195; all of it there 154).
+constexpr int kSpSmemLow = 195 * 1024;
+constexpr int sp_smem(int M) { return M <= 2 ? kSpSmemLow : kSpSmem; }
+constexpr int kSpMaxSB = 16, kSpMaxSP = 12;
+constexpr int kSpSumBytes = 16 * 512;                          // a piece's sums on their way to the workspace, twice
+#if defined(__CUDACC__)
+#define BPDQ_RINGS_FN __host__ __device__ constexpr
+#else
+#define BPDQ_RINGS_FN constexpr
+#endif
+// A row's blocks in `ns` slices of at most sb blocks, as equal as whole pairs of blocks allow (unequal ones would leave the CTAs of a short last
+// slice with most of the drains): slice s begins with block sp_slice(s); sp_slice_of(b) is the slice of block b.
+BPDQ_RINGS_FN int sp_slices(int nblocks, int sb) { return ((nblocks + 1) / 2 + sb / 2 - 1) / (sb / 2); }
+BPDQ_RINGS_FN int sp_slice(int s, int nblocks, int ns) { return s == ns ? nblocks : (int)((unsigned)((nblocks + 1) / 2) * (unsigned)s / (unsigned)ns) * 2; }
+BPDQ_RINGS_FN int sp_slice_of(int b, int nblocks, int ns) { return (int)(((unsigned)(b / 2 + 1) * (unsigned)ns - 1u) / (unsigned)((nblocks + 1) / 2)); }
+constexpr int sp_slot_cols(int K) { return 16 * K + 8; }       // TMEM columns of an operand slot
+constexpr int sp_slots(int K) { return K < 4 ? 4 : 3; }        // operand slots of a pipeline, next to four accumulators of 16 columns in 512
+static_assert(2 * sp_slots(3) * sp_slot_cols(3) + 4 * 16 <= 512 && 2 * sp_slots(4) * sp_slot_cols(4) + 4 * 16 <= 512, "TMEM");
+// x of the blocks o with o mod 4 == mine that a CTA meets in a slice of w blocks when it begins with block o and takes `units` blocks, tile after tile: n of
+// them, in the order of their first use.
+struct SpFirstUses {
+    int a0, na, mine, n;
+    BPDQ_RINGS_FN int block(int j) const { return j < na ? a0 + 4 * j : mine + 4 * (j - na); }
+};
+BPDQ_RINGS_FN SpFirstUses sp_first_uses(int mine, int o, int w, int units) {
+    const int stop = o + (units < w ? units : w), mid = stop < w ? stop : w;   // blocks o .. mid - 1, then 0 .. stop - w - 1
+    const int a0 = o + ((mine - o) & 3), na = (mid - a0 + 3) >> 2, nb = (stop - w - mine + 3) >> 2;
+    return {a0, na, mine, na + (nb > 0 ? nb : 0)};
+}
+struct SpRings {
+    int sb, sp;
+};
+constexpr SpRings sp_rings(int K, int cols, int smem) {
+    int sb = (smem - 3584 - 2 * kSpSumBytes - 2 * (sp_slots(K) + 2) * ts_slot_bytes(K)) / (cols * 544) / 2 * 2;
+    if (sb > kSpMaxSB) sb = kSpMaxSB;
+    int sp = (smem - 3584 - 2 * kSpSumBytes - sb * cols * 544) / (2 * ts_slot_bytes(K));      // 3584: alignment slack, barriers, list of finished tiles
+    if (sp > kSpMaxSP) sp = kSpMaxSP;
+    return {sb, sp};
+}
+
+// Few tokens: which launches go to the kernel with the planes as a sparse operand, by blocks per SM.  Its start and end cost some 1.5 us more
+// than the TMEM kernel's, a block less: per block and SM 0.20 us with 4 tokens and 0.22 with 16 at K = 2 (TMEM kernel 0.27), 0.25 and
+// 0.30 at K = 3 (0.31), 0.29 and 0.33 at K = 4 (0.64).  us there and here, 4 / 16 tokens: K = 2, 29568 x 8192 (100 blocks) 35.0 / 35.6
+// and 28.6 / 31.8, 8192 x 8192 (28) 15.4 / 15.8 and 14.5 / 15.7, 18944 x 3584 (28, a tile per SM) 13.1 / 13.3 and 14.4 / 15.3; K = 3, 100 blocks 38.8 / 39.4 and
+// 34.7 / 39.6, 28 16.7 / 17.1 and 16.6 / 17.8; K = 4 72.4 / 72.9 and 38.3 / 42.4, 26.0 / 26.2 and 17.5 / 18.7, 3584 x 3584 (5) 9.4 / 9.8 and
+// 9.6 / 10.4.  (K = 1 decodes fastest and has not been measured here.)
+constexpr int kSpMaxM = 16;
+constexpr bool sp_takes(int K, int M, long long units, int sms) {
+    if (M > kSpMaxM || K == 1 || units >= (1ll << 30)) return false;
+    const int least = K == 4 ? 8 : K == 3 ? (M <= 8 ? 28 : 64) : M <= 8 ? 16 : 28;
+    return units >= (long long)least * sms;
+}
+// ... and which of those that the look-up-table kernel would take: it has a pass for two tokens (at K = 4 three tokens are two passes), whose time grows
+// with the planes, and with the groups at g = 64.  Neither kernel rounds the weights.  us there and here with two tokens, launches by themselves: (gate, up) of
+// 29568 x 8192 (200 blocks per SM) at K = 3, g = 64 77.4 and 65.5, at K = 4 111.5 and 73.2 (g = 64), 86.9 and 68.6; 8192 x 29568 (100) 44.3 and 37.6, 57.9 and 41.7,
+// 48.4 and 40.1; 8192 x 8192 (28) 15.9 and 16.7, 19.8 and 17.9, 16.7 and 17.6.  A launch behind one of the other kernel costs some 2 us more, which takes
+// what 18944 x 3584 twice (56) would gain: a 7B-shaped layer at K = 3, g = 64 58.2 and, with its larger launches here, 59.7, a 72B-shaped one 154 and 143.  At K = 3,
+// g = 128 a 72B-shaped layer gains 1 us of 138.8, at K = 2 it loses.
+constexpr bool sp_before_lut(int K, bool g64, int M, long long units, int sms) {
+    if (M < 2 || !sp_takes(K, M, units, sms)) return false;
+    if (M > 2) return true;
+    if (K < 3 || (K == 3 && !g64)) return false;
+    return units >= (K == 4 && g64 ? 27LL : 80LL) * sms;
+}
+
 // Linears of up to 128 tokens that go to the prefill kernel all the same: more tiles than SMs with rows so short that a tile's
 // drain, by four warps and above 64 tokens with no second accumulator, takes longer than its blocks; the prefill kernel drains
 // with eight.  K = 2, us here and there: 20480 x 1024 (8 blocks) with 128 tokens 17.7 and 12.4, with 72 tokens 14.0 and 11.3; 20480 x 256 with

@@ -1,0 +1,194 @@
+"""Host logic of the kernel with the planes as a sparse operand (csrc/bpdq_rings.h): slices, the order in which x is stored, rings.
+
+Two properties of the roles' order: no wait by parity begins while the phase before the awaited one is open (the model of test_rings.py), and a CTA's
+roles, each of which does its steps in its own order, always get to their end."""
+import os
+import subprocess
+
+import pytest
+
+from tests.test_rings import HEADER_DIR, Order
+
+DRIVER = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "bpdq_rings.h"
+int main(int argc, char** argv) {
+    if (argc == 3) {
+        const int nb = atoi(argv[1]), ns = bpdq::sp_slices(nb, atoi(argv[2]));
+        for (int s = 0; s <= ns; ++s) printf("%d ", bpdq::sp_slice(s, nb, ns));
+        printf("\n");
+        for (int b = 0; b < nb; ++b) printf("%d ", bpdq::sp_slice_of(b, nb, ns));
+        printf("\n");
+        return 0;
+    }
+    if (argc == 2) {
+        for (int w = 1; w <= bpdq::kSpMaxSB; ++w)
+            for (int o = 0; o < w; ++o)
+                for (int n = 1; n <= 2 * w; ++n)
+                    for (int mine = 0; mine < 4; ++mine) {
+                        const bpdq::SpFirstUses u = bpdq::sp_first_uses(mine, o, w, n);
+                        printf("%d %d %d %d", w, o, n, mine);
+                        for (int j = 0; j < u.n; ++j) printf(" %d", u.block(j));
+                        printf("\n");
+                    }
+        return 0;
+    }
+    for (int K = 1; K <= 4; ++K) {
+        for (int M = 2; M <= 3; ++M) {
+        const bpdq::SpRings r = bpdq::sp_rings(K, 16, bpdq::sp_smem(M));
+        printf("%d %d %d %d %d\n", K, r.sb, r.sp, bpdq::sp_slots(K),
+               bpdq::sp_smem(M) - 2 * bpdq::kSpSumBytes - r.sb * 16 * 544 - 2 * r.sp * bpdq::ts_slot_bytes(K) - 1024 - 8 * (4 * bpdq::sp_slots(K) + 4 + 2 * r.sb + 4 * r.sp) - 4 * (5 + 64));
+        }
+        for (int M = 1; M <= 17; ++M)
+            for (int least = 1; least <= 256; ++least)
+                if (bpdq::sp_takes(K, M, least * 148LL, 148)) { printf("takes %d %d %d\n", K, M, least); break; }
+    }
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def driver(tmp_path_factory):
+    d = tmp_path_factory.mktemp("sp")
+    src, exe = d / "driver.cpp", d / "driver"
+    src.write_text(DRIVER)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", HEADER_DIR, str(src), "-o", str(exe)], check=True)
+    return lambda *a: subprocess.run([str(exe), *map(str, a)], check=True, capture_output=True, text=True).stdout.splitlines()
+
+
+@pytest.mark.parametrize("sb", [2, 12, 14, 16])
+def test_slices_cover_a_row_in_whole_pairs(driver, sb):
+    for nb in (1, 2, 3, 11, 16, 17, 28, 63, 64, 71, 231, 4097):
+        starts, of = [[int(v) for v in line.split()] for line in driver(nb, sb)]
+        assert starts[0] == 0 and starts[-1] == nb and all(0 < b - a <= sb for a, b in zip(starts, starts[1:]))
+        assert all(s % 2 == 0 for s in starts[:-1])                       # a slice begins with an even block: pipelines are parities
+        widths = [b - a for a, b in zip(starts, starts[1:])]
+        assert max(widths) - min(widths) <= 3                             # a pair, and the odd block at the end
+        assert all(starts[s] <= b < starts[s + 1] for b, s in enumerate(of))
+
+
+def test_x_is_stored_in_the_order_of_its_first_use(driver):
+    for line in driver("first"):
+        w, o, n, mine, *got = [int(v) for v in line.split()]
+        assert got == [(o + i) % w for i in range(min(w, n)) if (o + i) % w % 4 == mine], line
+
+
+def test_rings_and_rule(driver):
+    rows = [line.split() for line in driver()]
+    for K, sb, sp, na, left in [[int(v) for v in r] for r in rows if r[0] != "takes"]:
+        assert sb % 2 == 0 and sb >= 8 and sp >= na + 2 and left >= 0, (K, sb, sp, left)
+    takes = {(int(k), int(m)): int(n) for _, k, m, n in [r for r in rows if r[0] == "takes"]}
+    assert all((1, m) not in takes for m in range(1, 18)) and all((k, 17) not in takes for k in range(1, 5))
+    assert takes[4, 16] == 8 and takes[2, 4] == 16 and takes[3, 16] == 64
+
+
+def pipeline_order(na, sp, blocks):
+    """One pipeline: producer, two decode groups (group q mod 2 takes block q), one issuer, `na` operand slots and `sp` packed slots."""
+    o = Order()
+
+    def ev(kind, q):
+        return (kind, q) if q >= 0 else None
+    for q in range(blocks):
+        o.event(("asked", q), ev("asked", q - 1), ev("decoded", q - sp))
+        o.wait("producer", ev("asked", q - 1), ev("decoded", q - 2 * sp))
+        o.event(("landed", q), ("asked", q))
+        o.wait("group, packed", ev("decoded", q - 2), ev("landed", q - sp))
+        o.wait("group, operand", ev("decoded", q - 2), ev("multiplied", q - 2 * na))
+        o.event(("decoded", q), ev("decoded", q - 2), ("landed", q), ev("multiplied", q - na))
+        o.wait("issuer", ev("issued", q - 1), ev("decoded", q - na))
+        o.event(("issued", q), ev("issued", q - 1), ("decoded", q))
+        o.event(("multiplied", q), ("issued", q), ev("multiplied", q - 1))
+    return o
+
+
+def test_no_wait_passes_by_an_open_phase(driver):
+    for K, sb, sp, na, left in [[int(v) for v in line.split()] for line in driver() if not line.startswith("takes")]:
+        assert pipeline_order(na, sp, 60).open_waits() == []
+    assert pipeline_order(4, 5, 60).open_waits() != []                    # a shorter packed ring would not do
+
+
+def ends(begin, end, ntiles, starts, na, first_blocks=1):
+    """Whether a CTA with units begin .. end - 1 gets through: groups decode and store x in their order, issuers multiply in theirs."""
+    units, u = [], 0
+    for s, (b0, b1) in enumerate(zip(starts, starts[1:])):
+        units += [(s, t, o, b1 - b0) for t in range(ntiles) for o in range(b1 - b0)]
+    units = units[begin:end]
+    segs = []
+    for s, t, o, w in units:
+        if not segs or segs[-1][0] != s:
+            segs.append([s, o, w, 0])
+        segs[-1][3] += 1
+    seq = [[(s, t, o) for s, t, o, _ in units if o % 2 == pipe] for pipe in (0, 1)]
+    pieces = sorted(set((s, t) for s, t, _, _ in units))
+    last = {}
+    for pipe in (0, 1):
+        for k, (s, t, o) in enumerate(seq[pipe]):
+            last[s, o] = k
+    prog = {}
+    for pipe in (0, 1):
+        for grp in (0, 1):
+            steps, q, before = [], grp, {}
+            for i, (s, o, w, n) in enumerate(segs):
+                xs = [(o + j) % w for j in range(min(w, n)) if (o + j) % w % 4 == pipe + 2 * grp]
+                nblk = sum(1 for a in seq[pipe] if a[0] <= s)
+                if i == 0:
+                    for _ in range(first_blocks):
+                        if q < nblk:
+                            steps.append(("decode", q))
+                            q += 2
+                steps += [("x", s, b) for b in xs[:2]]
+                j = 2
+                while q < nblk or j < len(xs):
+                    if q < nblk:
+                        steps.append(("decode", q))
+                        q += 2
+                    if j < len(xs):
+                        steps.append(("x", s, xs[j]))
+                    j += 1
+            prog[pipe, grp] = steps
+    at, done, multiplied, stored, moved = {k: 0 for k in prog}, [set(), set()], [0, 0], set(), True
+    while moved:
+        moved = False
+        drained = 0
+        while drained < len(pieces) and all(multiplied[p] >= sum(1 for s, t, _ in seq[p] if (s, t) <= pieces[drained]) for p in (0, 1)):
+            drained += 1
+        for (pipe, grp), steps in prog.items():
+            while at[pipe, grp] < len(steps):
+                step = steps[at[pipe, grp]]
+                if step[0] == "decode":
+                    if step[1] >= na and multiplied[pipe] <= step[1] - na:
+                        break
+                    done[pipe].add(step[1])
+                else:
+                    earlier = [k for (s, o), k in last.items() if o == step[2] and s < step[1]]
+                    if earlier and multiplied[pipe] <= max(earlier):
+                        break
+                    stored.add(step[1:])
+                at[pipe, grp] += 1
+                moved = True
+        for pipe in (0, 1):
+            while multiplied[pipe] < len(seq[pipe]):
+                s, t, o = seq[pipe][multiplied[pipe]]
+                if multiplied[pipe] not in done[pipe] or (s, o) not in stored or pieces.index((s, t)) - 2 >= drained:
+                    break
+                multiplied[pipe] += 1
+                moved = True
+    return all(multiplied[p] == len(seq[p]) for p in (0, 1))
+
+
+@pytest.mark.parametrize("nb,ntiles,ctas", [(64, 3, 11), (71, 2, 9), (28, 5, 7), (5, 9, 6), (2, 40, 8)])
+def test_every_cta_gets_to_its_end(driver, nb, ntiles, ctas):
+    for K, sb, sp, na, left in [[int(v) for v in line.split()] for line in driver() if not line.startswith("takes")]:
+        starts = [int(v) for v in driver(nb, sb)[0].split()]
+        total = nb * ntiles
+        for c in range(ctas):
+            assert ends(total * c // ctas, total * (c + 1) // ctas, ntiles, starts, na), (K, c)
+
+
+def test_the_model_sees_two_blocks_ahead_of_x_with_three_slots(driver):
+    """Two packed blocks per group ahead of the first x fill all three operand slots of K = 4; the group that has the fourth waits for the MMAs of the first, and
+    those for x that it has yet to store where the CTA begins with block 2 or 3 of four."""
+    starts = [int(v) for v in driver(64, 12)[0].split()]
+    assert not ends(2, 60, 10, starts, 3, first_blocks=2) and ends(2, 60, 10, starts, 3)

@@ -1,0 +1,116 @@
+"""The kernel with the planes as a sparse operand (up to 16 tokens of large linears) through the public entry points, against binary64 sums of the
+unrounded weights."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2602_04163_b200 import binding, synth
+from tests import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+
+
+def exact(seed, out, in_, K, g, x, rows):
+    """Sums of x times c0 + sum ci bi in binary64 and the sums of the terms' sizes."""
+    bits = synth.plane_bits(seed, out, in_, K, rows).astype(np.float64)
+    coef = synth.coefficients(seed, out, in_, K, g, rows).view(np.float16).astype(np.float64)
+    group = np.arange(in_) // g
+    xd = x.view(np.float16).astype(np.float64)
+    terms = [coef[0][:, group]] + [coef[i + 1][:, group] * bits[i] for i in range(K)]
+    return xd @ sum(terms).T, np.abs(xd) @ sum(np.abs(t) for t in terms).T
+
+
+def bound(y, a):
+    """binary16 rounding of the result, and binary32 sums (a tensor core's keep 2^-23 of the running sum) of up to a few hundred MMAs: 2^-15 of the terms' sizes."""
+    return 2.0 ** -11 * np.abs(y) + 2.0 ** -15 * a + 2.0 ** -24
+
+
+def sample(out):
+    return np.unique(np.concatenate([np.arange(0, out, 131), [7, 8, 15, 16, 127, 128, out - 129, out - 128, out - 17, out - 1]]))
+
+
+@pytest.mark.parametrize("K,g,out,in_,M", [
+    (4, 128, 2064, 9088, 3),         # a ragged last tile (16 rows), 71 blocks: an odd block at the end of a row, at the rule's line
+    (4, 64, 2176, 8960, 16),         # a coefficient group per half block, every token column
+    (4, 256, 18944, 1152, 5),        # nine blocks per row: a single slice; a short last group
+    (4, 128, 151568, 128, 16),       # one block per row: pieces of one block, eight complete tiles per CTA
+    (2, 128, 4112, 9344, 8),         # 73 blocks, five slices
+    (2, 256, 6160, 11136, 15),       # 87 blocks, half a group at the end
+    (3, 64, 8208, 8192, 7),          # 64 blocks, five slices
+    (3, 128, 18944, 8192, 13),
+    (4, 128, 8192, 8192, 2),         # two tokens: ahead of the look-up-table kernel only by the rule, here on request
+])
+def test_planes_as_a_sparse_operand(K, g, out, in_, M):
+    h = binding.Handle(out, in_, K, g, None, 700 + K, M)
+    rows = sample(out)
+    x = synth.activations(701, M, in_)
+    y, a = exact(700 + K, out, in_, K, g, x, rows)
+    for _ in range(3):               # later calls find the workspace and the counters as the call before left them
+        got = G.run_linear(h, x, binding.KERNEL_GEMM)
+        assert np.all(np.isfinite(got))
+        err = np.abs(got[:, rows] - y)
+        assert np.all(err <= bound(y, a)), float(np.max(err / bound(y, a)))
+    # sums of 32 activations beyond binary16, on both sides of the line where their high part is split off, and at its far end
+    x = synth.activations(702, M, in_).view(np.float16).copy()
+    sign = 1.0 - 2.0 * (np.arange(in_) // 32 % 2)        # the words' sums cancel, so that results stay inside binary16
+    x[0, :] = 2000.0 * sign
+    x[1, :] = np.where(np.arange(in_) // 64 % 2, 1023.0, 1025.0) * sign
+    if M > 2:
+        x[2, :64] = 65504.0 * sign[:64]
+        x[2, 64:] = 0.0
+    y, a = exact(700 + K, out, in_, K, g, x.view(np.uint16), rows)
+    got = G.run_linear(h, x.view(np.uint16), binding.KERNEL_GEMM)[:, rows]
+    inside = np.abs(y) + bound(y, a) < 65504.0
+    assert np.all(np.abs(got - y)[inside] <= bound(y, a)[inside]) and inside.mean() > 0.9
+
+
+@pytest.mark.parametrize("K,g,M", [(4, 128, 3), (4, 64, 2), (3, 64, 2), (2, 128, 16)])
+def test_batches_pairs_and_the_rule(K, g, M):
+    """Linears of different lengths in one launch, one with a bias, and a (gate, up) pair; below the rule's line and where a caller has set the look-up-table
+    threshold, calls go where they went."""
+    import torch
+    shapes = ((12304, 8192), (144, 11392), (2064, 640)) if K < 4 else ((8208, 8192), (144, 11392), (2064, 640))
+    hs = [binding.Handle(o, i, K, g, None, 710 + k, M) for k, (o, i) in enumerate(shapes)]
+    bias = np.random.RandomState(1).randn(shapes[1][0]).astype(np.float16)
+    hs[1].bpdq_set_bias(bias.view(np.uint16))
+    xs = [synth.activations(720 + k, M, i) for k, (_, i) in enumerate(shapes)]
+    for _ in range(2):
+        ys = [torch.full((M, o), float("nan"), dtype=torch.float16, device="cuda") for o, _ in shapes]
+        xt = [G.x_tensor(x) for x in xs]
+        n0 = sum(h.bpdq_launch_count() for h in hs)
+        binding.bpdq_linear_batch(hs, [x.data_ptr() for x in xt], [y.data_ptr() for y in ys], M, G.stream_ptr())
+        torch.cuda.synchronize()
+        hs[0].bpdq_get_status(G.stream_ptr())
+        assert sum(h.bpdq_launch_count() for h in hs) == n0 + 1
+        for k, (o, i) in enumerate(shapes):
+            rows = sample(o) if o > 300 else np.arange(o)
+            y, a = exact(710 + k, o, i, K, g, xs[k], rows)
+            y = y + (bias[rows].astype(np.float64) if k == 1 else 0.0)
+            assert np.all(np.abs(ys[k].cpu().numpy().astype(np.float64)[:, rows] - y) <= bound(y, a) + 2.0 ** -11 * 4.0)
+    # a pair: the unit on unrounded sums
+    o, i = shapes[0]
+    up = binding.Handle(o, i, K, g, None, 730, M)
+    rows = sample(o)
+    gy, ga = exact(710, o, i, K, g, xs[0], rows)
+    uy, ua = exact(730, o, i, K, g, xs[0], rows)
+    want = oracle.swiglu(gy, uy)
+    dg, du = 2.0 ** -15 * ga, 2.0 ** -15 * ua
+    silu = oracle.swiglu(gy, np.ones_like(gy))
+    for _ in range(2):
+        unit = torch.full((M, o), float("nan"), dtype=torch.float16, device="cuda")
+        binding.bpdq_gate_up_swiglu(hs[0], up, G.x_tensor(xs[0]).data_ptr(), unit.data_ptr(), M, G.stream_ptr())
+        torch.cuda.synchronize()
+        hs[0].bpdq_get_status(G.stream_ptr())
+        err = np.abs(unit.cpu().numpy().astype(np.float64)[:, rows] - want)
+        assert np.all(err <= 1.1 * (np.abs(uy) + du) * dg + (np.abs(silu) + 1.1 * dg) * du + 2.0 ** -10 * np.abs(want) + 2.0 ** -24)
+    # small ones stay with the look-up-table kernel up to its threshold, and so does everything once a caller has set it
+    if M <= 3:
+        small = hs[2]
+        assert np.allclose(G.run_linear(small, xs[2]), G.run_linear(small, xs[2], binding.KERNEL_GEMV), rtol=2.0 ** -9, atol=1e-5)
+        n0 = hs[0].bpdq_launch_count()
+        G.run_linear(hs[0], xs[0])
+        assert hs[0].bpdq_launch_count() == n0 + 1
+        hs[0].bpdq_set_gemv_max_m(M)
+        n0 = hs[0].bpdq_launch_count()
+        G.run_linear(hs[0], xs[0])
+        assert hs[0].bpdq_launch_count() == n0 + (M + 1) // 2
