@@ -188,7 +188,7 @@ int check_batch_handles(const bpdq_handle_t* hs, int n, int M, const char* who) 
 bool prefer_lut(bpdq_handle_s* const* hs, int n, int M) {
     const bpdq_handle_s* h = hs[0];
     if (M > h->gemv_max_m) return false;
-    if (h->gemv_set || h->few_set) return true;
+    if (M < 2 || h->gemv_set || h->few_set) return true;
     for (int k = 0; k < n; ++k)
         if (hs[k]->d_perm || !gemm_batch_supported(hs[k], M)) return true;
     return !sp_before_lut(h->K, h->group == 64, M, sp_units(hs, n), h->sm_count);

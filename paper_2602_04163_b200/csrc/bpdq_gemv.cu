@@ -22,7 +22,7 @@
 // the data: table loads are conflict-free by construction.  The tables start at a multiple of
 // 64 KB in the shared window, so the byte-permute that splices the plane byte into bits 8..15 of
 // the lane's slot address yields the final address.  Look-up results are accumulated two at a
-// time with packed binary32 adds.
+// time with packed binary32 adds (with two tokens: one 64-bit look-up brings both tokens' sums).
 // Row sums are combined across slices with binary32 atomic adds into a small workspace
 // [token][row] that lives in L2; per 128 rows an arrival counter tells the CTA that delivers the
 // last contribution to round those rows to binary16, write y and zero the workspace again.
@@ -148,6 +148,15 @@ __device__ __forceinline__ void lookup2_add(unsigned long long& acc, unsigned ad
         "add.rn.f32x2 %0, %0, t;\n\t}"
         : "+l"(acc) : "r"(addr0), "r"(addr1), "n"(IMM0), "n"(IMM1));
 }
+// The same for two tokens, whose tables lie side by side: one 64-bit look-up brings both.
+template <int IMM>
+__device__ __forceinline__ void lookup_pair_add(unsigned long long& acc, unsigned addr) {
+    asm("{\n\t.reg .f32 a, b;\n\t.reg .b64 t;\n\t"
+        "ld.shared.v2.f32 {a, b}, [%1+%2];\n\t"
+        "mov.b64 t, {a, b};\n\t"
+        "add.rn.f32x2 %0, %0, t;\n\t}"
+        : "+l"(acc) : "r"(addr), "n"(IMM));
+}
 __device__ __forceinline__ float2 unpack2(unsigned long long v) {
     float2 f;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
@@ -185,10 +194,16 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
     float* xsum = reinterpret_cast<float*>(smem);                         // [MT][kSliceBlocks][2]: per 64-column half block
     int* done = reinterpret_cast<int*>(smem + 64);                        // [kMaxDone]
     int* ndone = done + kMaxDone;
-    float* lut = reinterpret_cast<float*>(smem + (lut0 - smem0));         // [MT][256][kSlots]
+    // One token: [256][kSlots].  Two: block pair by block pair [kSliceBlocks / 2][256][kSlots / 2][2 tokens], so that a look-up is one 64-bit load for both
+    // (half the load instructions of the streaming loop: 72B-shaped gate 26.2 -> 25.5 us at K = 2, 31.5 -> 30.2 at g = 64, 36.3 -> 34.4 at K = 3 with the warps that
+    // now fit, 54.8 -> 52.8 at K = 4, g = 64; the lanes of a half-warp still meet sixteen different bank pairs).
+    float* lut = reinterpret_cast<float*>(smem + (lut0 - smem0));
+    auto table_at = [&](int m, int entry, int slot) {                     // index of token m's entry in slot 16 * block + chunk
+        return MT == 1 ? entry * kSlots + slot : (slot >> 5) * (kTableBytes / 4) + entry * kSlots + (slot & 31) * 2 + m;
+    };
 
-    // The lane's table address at step s is lut0 + 256 * (plane byte) + slot(s), slot(s) = 4*((s + a) mod 16) + 64*h
-    // (< 128).  lut0 is a multiple of 64 KB below 16 MB, so the address is four bytes: [slot][plane byte]
+    // The lane's table address at step s is lut0 + 256 * (plane byte) + slot(s), slot(s) = 4*((s + a) mod 16) + 64*h (two tokens: twice that)
+    // (< 256).  lut0 is a multiple of 64 KB below 16 MB, so the address is four bytes: [slot][plane byte]
     // [lut0 >> 16][0], which one byte-permute assembles from the plane word and a register that holds
     // lut0 >> 16 in byte 0 and the slots of three consecutive steps in bytes 1..3 (the zero top byte is
     // the replicated sign of byte 0).
@@ -202,7 +217,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
             // g = 64: the eight steps of each half stay in one 64-column half of the block, lanes a < 8 beginning with the
             // first and the others with the second, so that the sixteen lanes still meet sixteen chunks at every step
             const unsigned chunk = G64 ? ((s + a) & 7) + 8 * (((a >> 3) ^ (s >> 3)) & 1) : (s + a) & 15;
-            if (s < 16) slots[j] |= (4u * chunk + 64u * h) << (8 * (e + 1));
+            if (s < 16) slots[j] |= (4u * MT * chunk + 64u * MT * h) << (8 * (e + 1));
         }
     }
 #pragma unroll
@@ -420,7 +435,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                 if (eh & 1) base += xs[5];
                 if (eh & 2) base += xs[6];
                 if (eh & 4) base += xs[7];
-                float* dst = lut + m * (kTableBytes / 4) + (eh * 32) * kSlots + slot;
+                float* dst = lut + table_at(m, eh * 32, slot);
 #pragma unroll
                 for (int j = 0; j < 32; ++j) dst[j * kSlots] = base + lo[j];
             }
@@ -429,7 +444,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
         if (tid < MT * kSliceBlocks * 2) {            // sums of x over the two 64-column halves of every block
             const int m = tid / (kSliceBlocks * 2), hb = tid % (kSliceBlocks * 2);
             float acc = 0.f;
-            for (int c = 0; c < 8; ++c) acc += lut[m * (kTableBytes / 4) + 255 * kSlots + hb * 8 + c];
+            for (int c = 0; c < 8; ++c) acc += lut[table_at(m, 255, hb * 8 + c)];
             xsum[m * (kSliceBlocks * 2) + hb] = acc;
         }
         __syncthreads();
@@ -480,11 +495,11 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                         addr[i] = prmt(word_of(tk.pl[q][i], st >> 2), slots[st / 3], 0xC400u | ((st & 3) << 4) | (5 + st % 3));   // the selector is a constant once the step loop is unrolled
                     constexpr int QI = 128;               // the block pair and the token's table go into the immediate
                     if constexpr (MT == 2) {
-                        // pair = the two tokens of one plane: one address, two tables
+                        // pair = the two tokens of one plane: one address, one load
 #pragma unroll
                         for (int i = 0; i < K; ++i) {
-                            if (q == 0) lookup2_add<0, kTableBytes>(acc[i][st & 1], addr[i], addr[i]);
-                            else lookup2_add<QI, kTableBytes + QI>(acc[i][st & 1], addr[i], addr[i]);
+                            if (q == 0) lookup_pair_add<0>(acc[i][st & 1], addr[i]);
+                            else lookup_pair_add<kTableBytes>(acc[i][st & 1], addr[i]);
                         }
                     } else {
                         // one token: pair = two planes; an odd plane left over pairs two consecutive steps
@@ -625,10 +640,11 @@ int launch_cfg(bpdq_handle_s* h, GemvParams p, cudaStream_t stream) {
 // Warps of a CTA and tasks kept in flight per lane.  Sixteen warps of 128 registers with two tasks, or with one where two do not fit the
 // registers; eight of 255 where the planes of one task already crowd 128.  72B-shaped gate, us: K = 3, two tokens 37.9 with two tasks (requested
 // as a whole; 38.8 by halves), 36.3 with one, at g = 64 50.3 (55.4) and 41.9; K = 4, one token 32.0 with one task, 30.9 with eight warps and
-// three; K = 4, g = 64, two tokens 59.0 and, with eight warps and two tasks, 54.8.  All others are slower in the other forms (K = 2, one
+// three; K = 4, g = 64, two tokens 59.0 and, with eight warps and two tasks, 54.8.  With one 64-bit load for both tokens' look-ups: K = 3, two tokens 36.1 with sixteen
+// warps, 34.4 with eight and three tasks (8192 x 8192 14.0 and 13.3), at g = 64 41.5 and 43.9 (its pair 77.3 and 83.7).  All others are slower in the other forms (K = 2, one
 // token 17.9 with sixteen warps and two tasks, 20.9 with one, 21.0 with eight warps and three; K = 4, g = 64, one token: the pair 68.8 and 72.5).
 template <int K, int MT, bool G64> struct Flight {
-    static constexpr bool kFew = K == 4 && (MT == 2) == G64;
+    static constexpr bool kFew = (K == 4 && (MT == 2) == G64) || (K == 3 && MT == 2 && !G64);
     static constexpr int W = kFew ? 8 : 16, D = kFew ? (G64 ? 2 : 3) : K == 4 || (K == 3 && MT == 2) ? 1 : 2;
 };
 
