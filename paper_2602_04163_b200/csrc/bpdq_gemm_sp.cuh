@@ -9,8 +9,13 @@
 // four bits per group of four, is "1 b 0 b": one mask of a packed word gives the metadata of sixteen columns.  So a block of 128
 // columns costs a thread some 20 instructions per plane where decoding its weights into binary16 takes 186 (K = 2) to 450 (K = 4),
 // and the weights are not rounded.  c_0 sum_j x_j is one dense MMA per block: K = four 32-column sums of x, each as binary16 parts
-// (high, low, what exceeds binary16 / 64).  Bound: with 16 token columns a block's 8 K + 1 MMAs take 10 clocks each, less than its
-// packed bytes take from HBM; from 32 on the MMAs (16 clocks at 32, 24 at 48).
+// (high, low, what exceeds binary16 / 64).
+// Bound: no single unit (29568 x 8192, K = 2, 16 tokens, of active cycles: tensor pipe 25 %, ALU 37 %, issue 57 %, DRAM 23 %), but the roles' chains.  Of 28.6 us
+// with 4 tokens 22.8 are left without decode, most MMAs and the completion of tiles (timing-only copies: masks and shifts 2.5, operand stores 1.3, coefficients
+// 0.5, MMAs 0.5, the coefficients' copies 0.6): start and end of a launch some 9, the packed blocks' way through their ring the rest; HBM needs 11.  What did
+// not help: two issuers per pipeline with half of a block's MMAs each (32.5 -> 36.3), the adds and the counting in a warp of their own (29.9 -> 32.5), narrower
+// slices for a longer packed ring (10 blocks instead of 16: 33.9, with 16 tokens 41.0, since every piece costs a drain and an add of 128 x 16 sums).  What
+// did: complete tiles finished at the end by all warps and not one by one by the draining ones (32.8 -> 30.5, with 16 tokens 38.7 -> 33.5).
 //
 // A sparse MMA (K = 32, i.e. 16 columns of a plane) takes its metadata from one TMEM column: lane 16 a + 8 h + b holds the 16 bits
 // of K half h of rows 16 a + b (low) and 16 a + b + 8 (high).  So the thread of row r reads, of rows r & ~8 and r | 8, the words
@@ -19,14 +24,15 @@
 //
 // Work split: units are (row tile, block) pairs, slice by slice (a slice: `sb` blocks of columns), in a slice tile by tile; every CTA
 // takes an equal contiguous share.  x of a slice stays in shared memory, zeros and all, while the CTA walks over the slice's row
-// tiles; the sums of a (tile, slice) go into the handle's binary32 workspace, and when a CTA leaves a slice it counts the blocks it
-// has delivered; who delivers a tile's last block rounds the sums to y.
+// tiles; the sums of a (tile, slice) are added to the handle's binary32 workspace by bulk copies and their blocks counted a piece later; who counts a tile's last
+// block completes the tile at the end of its work: rounds the sums to y (a pair: applies the gated unit) and zeroes them.
 //
 // Roles (768 threads): two pipelines, one for the even and one for the odd blocks of a slice, each with a ring of packed blocks
-// (one producer warp), two decode groups of four warps, an operand slot in TMEM per group and an MMA issuer with an accumulator of
-// its own; four warps expand x and drain.  A pipeline's rings belong to it alone, so that waits by parity follow their phases:
-// the group that waits for packed block q has waited for the MMAs of block q - 4 (its operand slot, two blocks before), and an issuer's MMAs
-// complete in order, so with four slots or more the copy of the slot's last use has landed.
+// (one producer warp), two decode groups of four warps, NA operand slots in TMEM that its blocks take in turn, and an MMA issuer with an accumulator of
+// its own (two, taken in turn by pieces); four warps drain.  The decode groups also expand x: every block of a slice has a slot of its own and belongs to one group.
+// A pipeline's rings belong to it alone, so that waits by parity follow their phases: the group that waits for packed block q has waited, two blocks
+// before, for the MMAs of block q - 2 - NA (its operand slot), and an issuer's MMAs complete in order, so with NA + 2 packed slots the copy of the slot's last use
+// has landed; the wait for the operand slot of block q, whose phase before is over with the MMAs of block q - 2 NA, follows from the same (NA >= 2).
 using bpdq::kSpSmem;
 constexpr int kSpFirstDecode = 4, kSpFirstEpi = 20;
 constexpr int kSpThreads = 32 * (kSpFirstEpi + 4);
@@ -461,8 +467,8 @@ __global__ void __launch_bounds__(kSpThreads, 1) gemm_sp_kernel(const __grid_con
         // ---------------- four warps drain finished pieces ----------------
         const int et = tid - 32 * kSpFirstEpi, rl = (warp & 3) * 32 + lane, M = p.M;
         // A piece's sums go through one of two buffers in shared memory and are added to the workspace by bulk copies, a lane of the first warp per
-        // token.  They are counted under the next piece's MMAs, when the adds have long arrived; who counts a tile's last block completes the tile,
-        // at the end of its work together with the decode warps (or when its list is full).
+        // token.  They are counted under the next piece's MMAs, when the adds have long arrived; complete tiles are listed, and finished here only
+        // where the list is full.
         int buf = 0, li = -1, tile = 0;                  // linear, tile and blocks of the piece before (li < 0: none)
         unsigned n = 0u, pacc = 0u;
         SpPiece c;
