@@ -179,19 +179,18 @@ int launch_sp(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
 }
 
 // Up to 128 tokens: one or several linears (same K, all or none with group 64); pair: the gated unit of two.
-template <int K>
+template <int K, int NG>
 int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair) {
     static bpdq::SmemOptin optin;
     bpdq_handle_s* h0 = hs[0];
     if (kTsSmem > h0->smem_optin)
         return bpdq::set_error(BPDQ_ERR_UNSUPPORTED, "gemm: %d bytes of shared memory needed, device offers %d", kTsSmem, h0->smem_optin);
-    if (const int rc = bpdq::ensure_smem_optin(gemm_ts_kernel<K>, optin, h0->device, kTsSmem, "gemm"); rc != BPDQ_OK) return rc;
+    if (const int rc = bpdq::ensure_smem_optin(gemm_ts_kernel<K, NG>, optin, h0->device, kTsSmem, "gemm"); rc != BPDQ_OK) return rc;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm: cuTensorMapEncodeTiled is not available from this driver");
     TsParams p;
     p.n = n; p.M = M; p.cols = (M + 15) / 16 * 16;
     p.status = h0->d_status;
-    p.ng = h0->group == 64 ? 2 : 1;
     long long units = 0, tiles = 0;
     bool same = true;                                    // rows of one length
     for (int k = 0; k < n; ++k) {
@@ -235,7 +234,7 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the first packed blocks are requested under the tail of the kernel before
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_ts_kernel<K>, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_ts_kernel<K, NG>, p);
     h0->launches += 1;
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return bpdq::set_error(BPDQ_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
@@ -245,8 +244,10 @@ int launch_ts(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, 
 // Up to 128 tokens: the few-token kernel where it is the faster one, else the TMEM kernel.
 template <int K>
 int launch_up_to_128(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair) {
-    if (!bpdq::sp_takes(K, M, bpdq::sp_units(hs, n), hs[0]->sm_count)) return launch_ts<K>(hs, xs, ys, n, M, stream, pair);
-    return hs[0]->group == 64 ? launch_sp<K, 2>(hs, xs, ys, n, M, stream, pair) : launch_sp<K, 1>(hs, xs, ys, n, M, stream, pair);
+    const bool g64 = hs[0]->group == 64;
+    if (!bpdq::sp_takes(K, M, bpdq::sp_size(hs, n), hs[0]->sm_count))
+        return g64 ? launch_ts<K, 2>(hs, xs, ys, n, M, stream, pair) : launch_ts<K, 1>(hs, xs, ys, n, M, stream, pair);
+    return g64 ? launch_sp<K, 2>(hs, xs, ys, n, M, stream, pair) : launch_sp<K, 1>(hs, xs, ys, n, M, stream, pair);
 }
 
 template <int K, int BKW, int NG>
@@ -333,10 +334,14 @@ bool gemm_supported(int, int, int K, int group) {
     return K >= 1 && K <= 4 && (group == 64 || group == 128 || group == 256);
 }
 
-long long sp_units(const bpdq_handle_s* const* hs, int n) {
-    long long units = 0;
-    for (int k = 0; k < n; ++k) units += (long long)((hs[k]->out + BM - 1) / BM) * (hs[k]->in / 128);
-    return units;
+SpSize sp_size(const bpdq_handle_s* const* hs, int n) {
+    SpSize z = {0, 0};
+    for (int k = 0; k < n; ++k) {
+        const int row = hs[k]->in / 128;
+        z.units += (long long)((hs[k]->out + BM - 1) / BM) * row;
+        if (row > z.row) z.row = row;
+    }
+    return z;
 }
 
 bool gemm_batch_supported(const bpdq_handle_s* h, int M) { return h->d_few_maps && M <= kTsMaxM && gemm_supported(h->out, h->in, h->K, h->group); }

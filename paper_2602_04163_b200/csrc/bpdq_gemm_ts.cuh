@@ -53,7 +53,6 @@ struct TsParams {
     int cut_step;              // ... of whole multiples of this many (a row's blocks when rows are not cut)
     int sp, sx;                // slots of the packed and of the x ring
     int nbuf, dcols;           // accumulator pairs; TMEM columns of one accumulator
-    int ng;                    // coefficient groups per block
 };
 // A CTA's work as pieces of row tiles: its share of the cut units, then its whole tiles.
 struct TsPieces {
@@ -106,7 +105,9 @@ __device__ __forceinline__ void tmem_st32(unsigned t, const unsigned (&v)[32]) {
           "r"(v[30]), "r"(v[31]) : "memory");
 }
 
-template <int K>
+// NG: coefficient groups per block, 1 or 2 (as a parameter of the launch, beside a packed slot that was advanced step by step, it cost 2 to 4 %: 18944 x 3584 at K = 2
+// with 24 tokens 13.8 us and 13.3, K = 3 15.1 and 14.7, K = 4, g = 64 25.2 and 24.2)
+template <int K, int NG>
 __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_constant__ TsParams p) {
     using C = TsCfg<K>;
     constexpr int NA = kTsGroups;
@@ -128,7 +129,6 @@ __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_con
     volatile int* finish = reinterpret_cast<volatile int*>(tmem_slot + 2);
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-    const int ng = p.ng;
     TsPieces work = ts_pieces(p);
     TsPiece pc;
 
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_con
                 for (int b = pc.b0; b < pc.b0 + pc.n; ++b) {
                     if (!mbar_wait(empty_p0 + 8u * sl, ph, abort_flag, p.status)) { ok = false; break; }
                     const unsigned dst = p_base + (unsigned)sl * C::kSlotBytes, bar = full_p0 + 8u * sl;
-                    mbar_expect_tx(bar, (unsigned)(C::kPlaneBytes + ng * C::kCoefBytes));
+                    mbar_expect_tx(bar, (unsigned)(C::kPlaneBytes + NG * C::kCoefBytes));
                     tma_load_2d(dst, &maps[0], pc.tile * 256, b * K, bar);                    // 8-byte elements: two per row
                     tma_load_2d(dst + C::kPlaneBytes, &maps[1], pc.tile * 32, ((2 * b) >> gsh) * (K + 1), bar);
                     if (++sl == SP) { sl = 0; ph ^= 1u; }
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_con
             bool ok = true;
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
-                if (half == 0 || ng == 2) {              // candidate tables of the coefficient group that starts here
+                if (half == 0 || NG == 2) {              // candidate tables of the coefficient group that starts here
                     float c[K + 1];
 #pragma unroll
                     for (int i = 0; i <= K; ++i) {
@@ -387,8 +387,8 @@ __global__ void __launch_bounds__(kTsThreads, 1) gemm_ts_kernel(const __grid_con
                 mbar_arrive(empty_p0 + 8u * sl);         // everything read from the slot has been stored as an operand
             }
             pa ^= 1u;
-            for (int e = 0; e < kTsGroups; ++e)
-                if (++sl == SP) { sl = 0; ph ^= 1u; }
+            sl += kTsGroups;                             // (the ring is longer)
+            if (sl >= SP) { sl -= SP; ph ^= 1u; }
         }
     } else if (warp >= kTsFirstEpi) {
         // ---------------- epilogue warps: every piece, the last one together with the decode warps ----------------

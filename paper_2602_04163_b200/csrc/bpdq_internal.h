@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "bpdq.h"
+#include "bpdq_rings.h"
 
 #if defined(__CUDACC__)
 #define BPDQ_HD __host__ __device__ __forceinline__
@@ -113,7 +114,7 @@ int launch_gemv_mma(bpdq_handle_s* h, const void* x, void* y, int M, cudaStream_
 int launch_gemv_mma_batch(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair = false);
 int launch_gemm_batch(bpdq_handle_s* const* hs, const void* const* xs, void* const* ys, int n, int M, cudaStream_t stream, bool pair = false);
 bool gemm_batch_supported(const bpdq_handle_s* h, int M);
-long long sp_units(const bpdq_handle_s* const* hs, int n);          // 128-row x 128-column blocks of these linears
+SpSize sp_size(const bpdq_handle_s* const* hs, int n);
 bool gemv_mma_supported(int out, int in, int K, int group);
 int few_prepare(bpdq_handle_s* h);
 size_t gemv_workspace_bytes(int out, int in, int K, int group, int max_M, int sm_count);

@@ -111,11 +111,16 @@ constexpr SpRings sp_rings(int K, int cols, int smem) {
 // and 28.6 / 31.8, 8192 x 8192 (28) 15.4 / 15.8 and 14.5 / 15.7, 18944 x 3584 (28, a tile per SM) 13.1 / 13.3 and 14.4 / 15.3; K = 3, 100 blocks 38.8 / 39.4 and
 // 34.7 / 39.6, 28 16.7 / 17.1 and 16.6 / 17.8; K = 4 72.4 / 72.9 and 38.3 / 42.4, 26.0 / 26.2 and 17.5 / 18.7, 3584 x 3584 (5) 9.4 / 9.8 and
 // 9.6 / 10.4.  (K = 1 decodes fastest and has not been measured here.)
+// Rows of fewer than 48 blocks make the TMEM kernel's tiles short and mostly whole, which it does without adds: 18944 x 3584 above.
 constexpr int kSpMaxM = 16;
-constexpr bool sp_takes(int K, int M, long long units, int sms) {
-    if (M > kSpMaxM || K == 1 || units >= (1ll << 30)) return false;
-    const int least = K == 4 ? 8 : K == 3 ? (M <= 8 ? 28 : 64) : M <= 8 ? 16 : 28;
-    return units >= (long long)least * sms;
+struct SpSize {
+    long long units;                                  // 128-row x 128-column blocks of a launch
+    int row;                                          // blocks of its longest row
+};
+constexpr bool sp_takes(int K, int M, SpSize z, int sms) {
+    if (M > kSpMaxM || K == 1 || z.units >= (1ll << 30)) return false;
+    const int least = K == 4 ? 8 : z.row < 48 ? (K == 3 ? (M <= 8 ? 48 : 150) : M <= 8 ? 40 : 100) : K == 3 ? (M <= 8 ? 28 : 64) : M <= 8 ? 16 : 28;
+    return z.units >= (long long)least * sms;
 }
 // ... and which of those that the look-up-table kernel would take: it has a pass for two tokens (at K = 4 three tokens are two passes), whose time grows
 // with the planes, and with the groups at g = 64.  Neither kernel rounds the weights.  us there and here with two tokens, launches by themselves: (gate, up) of
@@ -123,11 +128,11 @@ constexpr bool sp_takes(int K, int M, long long units, int sms) {
 // 48.4 and 40.1; 8192 x 8192 (28) 15.9 and 16.7, 19.8 and 17.9, 16.7 and 17.6.  A launch behind one of the other kernel costs some 2 us more, which takes
 // what 18944 x 3584 twice (56) would gain: a 7B-shaped layer at K = 3, g = 64 58.2 and, with its larger launches here, 59.7, a 72B-shaped one 154 and 143.  At K = 3,
 // g = 128 a 72B-shaped layer gains 1 us of 138.8, at K = 2 it loses.
-constexpr bool sp_before_lut(int K, bool g64, int M, long long units, int sms) {
-    if (M < 2 || !sp_takes(K, M, units, sms)) return false;
+constexpr bool sp_before_lut(int K, bool g64, int M, SpSize z, int sms) {
+    if (M < 2 || !sp_takes(K, M, z, sms)) return false;
     if (M > 2) return true;
     if (K < 3 || (K == 3 && !g64)) return false;
-    return units >= (K == 4 && g64 ? 27LL : 80LL) * sms;
+    return z.units >= (K == 4 && g64 ? 27LL : 80LL) * sms;
 }
 
 // Linears of up to 128 tokens that go to the prefill kernel all the same: more tiles than SMs with rows so short that a tile's

@@ -42,7 +42,7 @@ int main(int argc, char** argv) {
         }
         for (int M = 1; M <= 17; ++M)
             for (int least = 1; least <= 256; ++least)
-                if (bpdq::sp_takes(K, M, least * 148LL, 148)) { printf("takes %d %d %d\n", K, M, least); break; }
+                if (bpdq::sp_takes(K, M, bpdq::SpSize{least * 148LL, 64}, 148)) { printf("takes %d %d %d\n", K, M, least); break; }
     }
     return 0;
 }
@@ -81,7 +81,7 @@ def test_rings_and_rule(driver):
         assert sb % 2 == 0 and sb >= 8 and sp >= na + 2 and left >= 0, (K, sb, sp, left)
     takes = {(int(k), int(m)): int(n) for _, k, m, n in [r for r in rows if r[0] == "takes"]}
     assert all((1, m) not in takes for m in range(1, 18)) and all((k, 17) not in takes for k in range(1, 5))
-    assert takes[4, 16] == 8 and takes[2, 4] == 16 and takes[3, 16] == 64
+    assert takes[4, 16] == 8 and takes[2, 4] == 16 and takes[3, 16] == 64                   # rows of 64 blocks
 
 
 def pipeline_order(na, sp, blocks):
