@@ -198,9 +198,6 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
     // (half the load instructions of the streaming loop: 72B-shaped gate 26.2 -> 25.5 us at K = 2, 31.5 -> 30.2 at g = 64, 36.3 -> 34.4 at K = 3 with the warps that
     // now fit, 54.8 -> 52.8 at K = 4, g = 64; the lanes of a half-warp still meet sixteen different bank pairs).
     float* lut = reinterpret_cast<float*>(smem + (lut0 - smem0));
-    auto table_at = [&](int m, int entry, int slot) {                     // index of token m's entry in slot 16 * block + chunk
-        return MT == 1 ? entry * kSlots + slot : (slot >> 5) * (kTableBytes / 4) + entry * kSlots + (slot & 31) * 2 + m;
-    };
 
     // The lane's table address at step s is lut0 + 256 * (plane byte) + slot(s), slot(s) = 4*((s + a) mod 16) + 64*h (two tokens: twice that)
     // (< 256).  lut0 is a multiple of 64 KB below 16 MB, so the address is four bytes: [slot][plane byte]
@@ -217,7 +214,7 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
             // g = 64: the eight steps of each half stay in one 64-column half of the block, lanes a < 8 beginning with the
             // first and the others with the second, so that the sixteen lanes still meet sixteen chunks at every step
             const unsigned chunk = G64 ? ((s + a) & 7) + 8 * (((a >> 3) ^ (s >> 3)) & 1) : (s + a) & 15;
-            if (s < 16) slots[j] |= (4u * MT * chunk + 64u * MT * h) << (8 * (e + 1));
+            if (s < 16) slots[j] |= (MT == 1 ? 4u * chunk + 64u * h : 8u * chunk + 128u * h) << (8 * (e + 1));
         }
     }
 #pragma unroll
@@ -435,7 +432,8 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
                 if (eh & 1) base += xs[5];
                 if (eh & 2) base += xs[6];
                 if (eh & 4) base += xs[7];
-                float* dst = lut + table_at(m, eh * 32, slot);
+                float* dst = MT == 1 ? lut + m * (kTableBytes / 4) + (eh * 32) * kSlots + slot
+                                     : lut + (slot >> 5) * (kTableBytes / 4) + (eh * 32) * kSlots + (slot & 31) * 2 + m;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) dst[j * kSlots] = base + lo[j];
             }
@@ -444,7 +442,9 @@ __global__ void __launch_bounds__(W * 32, 1) gemv_lut_kernel(const __grid_consta
         if (tid < MT * kSliceBlocks * 2) {            // sums of x over the two 64-column halves of every block
             const int m = tid / (kSliceBlocks * 2), hb = tid % (kSliceBlocks * 2);
             float acc = 0.f;
-            for (int c = 0; c < 8; ++c) acc += lut[table_at(m, 255, hb * 8 + c)];
+            for (int c = 0; c < 8; ++c)
+                acc += MT == 1 ? lut[m * (kTableBytes / 4) + 255 * kSlots + hb * 8 + c]
+                               : lut[(hb >> 2) * (kTableBytes / 4) + 255 * kSlots + ((hb & 3) * 8 + c) * 2 + m];
             xsum[m * (kSliceBlocks * 2) + hb] = acc;
         }
         __syncthreads();
